@@ -11,13 +11,16 @@
 //   k_scale       grid scale (2^21-1)/extent, one thread
 //   k_quant       every vertex to the grid (double, rounded once per operation)
 //   k_snap        every texture coordinate to 1/256 texel (round half to even)
-//   k_raster      one thread per triangle: set-up record, area weight, and the texels of
-//                 small triangles (atomicMin of the triangle id: smallest id wins); big
-//                 triangles are split into 16x16-texel blocks appended to a work list
+//   k_raster      one thread per triangle: position planes, area weight, and the texels of
+//                 small triangles; big triangles are split into 16x16-texel blocks appended to a
+//                 work list
 //   k_raster_big  one CTA per (triangle, block) entry
-//   k_resolve     one CTA per tile, one texel per thread and step: exact barycentric position of
-//                 every covered texel, coverage bits, tile box
+//   k_resolve     one CTA per tile, one texel per thread and step: position of every covered texel
+//                 (from the triangle's planes where their rounding cannot matter, else exact
+//                 barycentrics), coverage bits, tile box
 //   k_super       one CTA per super-tile: union of its tile boxes
+// Where triangles overlap in the texture (found by counting), k_raster to k_super run once more, with
+// atomicMin: the smallest id wins.
 #include <algorithm>
 #include <cstring>
 
@@ -42,39 +45,59 @@ __global__ void k_init(uint32_t *__restrict__ tri, int64_t n_texels, uint32_t *_
         }
         hdr->flags = 0;
         hdr->n_big = 0;
+        hdr->n_covered = 0;
+        for (int a = 0; a < 8; ++a) hdr->n_hits[a] = 0;
     }
 }
 
-__global__ void k_bbox(const float *__restrict__ pos, int64_t n_pos, AtlasHdr *hdr) {
+// Four vertices (three 16-byte loads) per thread and step; one set of atomics per CTA.
+__global__ void __launch_bounds__(kThreads) k_bbox(const float *__restrict__ pos, int64_t n_pos, AtlasHdr *hdr) {
     float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
     bool bad = false;
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n_pos; v += (int64_t)gridDim.x * blockDim.x) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (!LCL_IN(3 * v + a, 3 * n_pos)) continue;
-            float p = pos[3 * v + a];
-            bad |= !isfinite(p);
-            mn[a] = fminf(mn[a], p);
-            mx[a] = fmaxf(mx[a], p);
-        }
+    auto take = [&](int axis, float p) {
+        bad |= !isfinite(p);
+        mn[axis] = fminf(mn[axis], p);
+        mx[axis] = fmaxf(mx[axis], p);
+    };
+    const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t n_quads = (reinterpret_cast<uintptr_t>(pos) & 15) == 0 ? n_pos / 4 : 0;  // the array may start anywhere
+    for (int64_t v = first; v < n_quads; v += stride) {
+        if (!LCL_IN(12 * v + 11, 3 * n_pos)) continue;
+        const float4 *p = reinterpret_cast<const float4 *>(pos) + 3 * v;
+        const float4 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
+        take(0, a.x), take(1, a.y), take(2, a.z), take(0, a.w);
+        take(1, b.x), take(2, b.y), take(0, b.z), take(1, b.w);
+        take(2, c.x), take(0, c.y), take(1, c.z), take(2, c.w);
     }
+    for (int64_t v = 4 * n_quads + first; v < n_pos; v += stride)
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            if (LCL_IN(3 * v + a, 3 * n_pos)) take(a, pos[3 * v + a]);
+    __shared__ float red[6][kThreads / 32];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         for (int o = 16; o; o >>= 1) {
             mn[a] = fminf(mn[a], __shfl_xor_sync(0xffffffffu, mn[a], o));
             mx[a] = fmaxf(mx[a], __shfl_xor_sync(0xffffffffu, mx[a], o));
         }
-    }
-    bad = __any_sync(0xffffffffu, bad);
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (mn[a] <= mx[a]) {
-                atomicMin(&hdr->key_min[a], float_key(mn[a]));
-                atomicMax(&hdr->key_max[a], float_key(mx[a]));
-            }
+        if ((threadIdx.x & 31) == 0) {
+            red[a][threadIdx.x >> 5] = mn[a];
+            red[3 + a][threadIdx.x >> 5] = mx[a];
         }
-        if (bad) atomicOr(&hdr->flags, kBadPos);
+    }
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x < 3) {
+        const int a = threadIdx.x;
+        float lo = red[a][0], hi = red[3 + a][0];
+        for (int w = 1; w < kThreads / 32; ++w) {
+            lo = fminf(lo, red[a][w]);
+            hi = fmaxf(hi, red[3 + a][w]);
+        }
+        if (lo <= hi) {
+            atomicMin(&hdr->key_min[a], float_key(lo));
+            atomicMax(&hdr->key_max[a], float_key(hi));
+        }
+        if (a == 0 && bad) atomicOr(&hdr->flags, kBadPos);
     }
 }
 
@@ -92,20 +115,33 @@ __global__ void k_scale(AtlasHdr *hdr) {
     } else {
         hdr->scale = __ddiv_rn((double)kGridMax, ext);
     }
+    hdr->pair = scale_pair(hdr->scale);
 }
 
 __global__ void k_quant(const float *__restrict__ pos, int64_t n_pos, const AtlasHdr *__restrict__ hdr,
                         int4 *__restrict__ q) {
     int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (v >= n_pos) return;
-    double S = hdr->scale;
+    const double S = hdr->scale;
+    const ScalePair sp = hdr->pair;
     if (!LCL_IN(3 * v + 2, 3 * n_pos)) return;
     int4 r;
-    r.x = quantize_coord(pos[3 * v + 0], hdr->mn[0], S);
-    r.y = quantize_coord(pos[3 * v + 1], hdr->mn[1], S);
-    r.z = quantize_coord(pos[3 * v + 2], hdr->mn[2], S);
+    r.x = quantize_coord(pos[3 * v + 0], hdr->mn[0], S, sp);
+    r.y = quantize_coord(pos[3 * v + 1], hdr->mn[1], S, sp);
+    r.z = quantize_coord(pos[3 * v + 2], hdr->mn[2], S, sp);
     r.w = 0;
     q[v] = r;
+}
+
+// rint(u * K), ties to even, for |u| <= 2 and an integer K <= 2^22 (exact in binary32): ph + pl is the
+// product exactly (FMA), r = rint(ph) and d = ph - r are exact, and d is a multiple of ulp(ph) while
+// |pl| is at most half of that, so pl changes the outcome only where d is a tie; a tie of ph that pl
+// leaves alone goes to even as in rint.  (In binary64 the two products per vertex took 62 us for 4 M,
+// FP64 being slow on this part.)
+__device__ __forceinline__ int32_t snap_coord(float u, float K) {
+    const float ph = __fmul_rn(u, K), pl = __fmaf_rn(u, K, -ph);
+    const float r = rintf(ph), d = __fsub_rn(ph, r);
+    return (int32_t)r + (d == 0.5f && pl > 0.0f ? 1 : 0) - (d == -0.5f && pl < 0.0f ? 1 : 0);
 }
 
 __global__ void k_snap(const float *__restrict__ uv, int64_t n_uv, int32_t w, int32_t h, AtlasHdr *hdr,
@@ -120,17 +156,14 @@ __global__ void k_snap(const float *__restrict__ uv, int64_t n_uv, int32_t w, in
         out[v] = make_int2(0, 0);
         return;
     }
-    // u * 256 * extent is exact in double (24 + 22 significant bits); rint = ties to even.
-    long long X = __double2ll_rn(__dmul_rn((double)u, (double)(256 * (int64_t)w)));
-    long long Y = __double2ll_rn(__dmul_rn((double)t, (double)(256 * (int64_t)h)));
-    out[v] = make_int2((int32_t)X, (int32_t)Y);
+    out[v] = make_int2(snap_coord(u, (float)(256 * w)), snap_coord(t, (float)(256 * h)));
 }
 
 // floor(sqrt(n)) for n < 2^88 (the squared length of a cross product of 21-bit differences,
 // at most 3 * 2^86): a binary64 estimate, then exact integer corrections.  Converting n to binary64
 // and the correctly rounded square root each err by at most half an ulp, so the estimate is within
 // 2^-8 of sqrt(n) < 2^44, and its floor within one of the result.
-__device__ uint64_t isqrt_u88(unsigned __int128 n) {
+__device__ __noinline__ uint64_t isqrt_u88(unsigned __int128 n) {
     const double d = (double)(uint64_t)(n >> 64) * 18446744073709551616.0 + (double)(uint64_t)n;
     uint64_t r = (uint64_t)__dsqrt_rn(d);
 #pragma unroll 1
@@ -140,14 +173,108 @@ __device__ uint64_t isqrt_u88(unsigned __int128 n) {
     return r;
 }
 
-struct RasterArgs {
+// A 64-bit integer below 2^62 as a float to within 2^-22 of itself (a 64-bit conversion runs on the slow
+// FP64 pipe).
+__device__ __forceinline__ float to_float_fast(int64_t n) {
+    return __fmaf_rn(__int2float_rn((int32_t)(n >> 31)), 2147483648.0f, __int2float_rn((int32_t)(n & 0x7FFFFFFF)));
+}
+
+// The same for n < 2^62 from binary32: the estimate is within 2^-21 sqrt(n) of sqrt(n) (2^10), and one
+// Newton step with the exact remainder leaves an error below 2^20 / (2 sqrt(n)) of the squared term, 1/2
+// of the rounding and 2^-20 of the step: two at most for n >= 2^38; smaller n have estimates within
+// two to begin with.
+__device__ __forceinline__ uint64_t isqrt_u62(uint64_t n) {
+    const float f = __fsqrt_rn(to_float_fast((int64_t)n));
+    int64_t r = (int64_t)(uint32_t)f;
+    if (n >= (uint64_t(1) << 38)) r += __float2int_rn(__fdividef(__fmul_rn(0.5f, to_float_fast((int64_t)n - r * r)), f));
+#pragma unroll 1
+    for (int k = 0; k < 4 && (uint64_t)(r * r) > n; ++k) --r;
+#pragma unroll 1
+    for (int k = 0; k < 4 && (uint64_t)((r + 1) * (r + 1)) <= n; ++k) ++r;
+    return (uint64_t)r;
+}
+
+// floor(r / A) for r < 2^39 given as r_float too, 0 < A < 2^31, inv = RN(1 / RN(A)), by a binary32 estimate and corrections
+// (quotients up to 2^24 come out within 3 of it, those up to 2^8 within 1); r becomes the remainder.
+__device__ __forceinline__ uint32_t div_step(uint64_t &r, uint32_t A, float r_float, float inv) {
+    uint32_t q = (uint32_t)__fmul_rn(r_float, inv);
+    int64_t rem = (int64_t)r - (int64_t)q * (int64_t)A;
+#pragma unroll 1
+    for (int k = 0; k < 4 && rem < 0; ++k) { --q; rem += A; }
+#pragma unroll 1
+    for (int k = 0; k < 4 && rem >= (int64_t)A; ++k) { ++q; rem -= A; }
+    r = (uint64_t)rem;
+    return q;
+}
+
+// floor(a 2^24 / A) for a < 2^24, 0 < A < 2^31: an integer quotient and three of eight bits each.
+__device__ __forceinline__ uint64_t area_quotient(uint32_t a, uint32_t A, float inv) {
+    uint64_t r = a;
+    uint64_t q = div_step(r, A, __uint2float_rn(a), inv);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float f = __fmul_rn(__uint2float_rn((uint32_t)r), 256.0f);  // r < A < 2^31
+        r <<= 8;
+        q = (q << 8) + div_step(r, A, f, inv);
+    }
+    return q;
+}
+
+// The mesh as the kernels gather it: indices, grid positions and snapped texture coordinates.
+struct MeshRefs {
     const uint32_t *tri_pos, *tri_uv;
-    int64_t n_tri, n_pos, n_uv;
     const int4 *q;
     const int2 *uvs;
-    int32_t w, h;        // texture size (h: rows of the whole texture)
+    int64_t n_tri, n_pos, n_uv;
+};
+
+// Corners of a triangle, counter-clockwise in the texture: snapped texture coordinates, grid
+// positions, and A, twice the texture area in sub-pixel units (0: it covers nothing).  Sub-pixel
+// coordinates lie within [-2^22, 2^23] (sides <= 2^14, UVs in [-1, 2]): differences fit in 32 bits.
+struct Corners {
+    int32_t x[3], y[3], qx[3], qy[3], qz[3];
+    int64_t A;
+};
+
+// False for an index out of range.
+__device__ __forceinline__ bool load_corners(const MeshRefs &m, int64_t t, Corners &c) {
+    uint32_t ip[3], iu[3];
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        ip[k] = m.tri_pos[3 * t + k];
+        iu[k] = m.tri_uv[3 * t + k];
+        ok &= ip[k] < (uint64_t)m.n_pos && iu[k] < (uint64_t)m.n_uv;
+    }
+    if (!ok) return false;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int2 u = m.uvs[iu[k]];
+        const int4 q = m.q[ip[k]];
+        c.x[k] = u.x;
+        c.y[k] = u.y;
+        c.qx[k] = q.x;
+        c.qy[k] = q.y;
+        c.qz[k] = q.z;
+    }
+    c.A = edge_fn32(c.x[0], c.y[0], c.x[1], c.y[1], c.x[2], c.y[2]);
+    if (c.A < 0) {  // swap corners 1 and 2
+        int32_t tmp;
+        tmp = c.x[1]; c.x[1] = c.x[2]; c.x[2] = tmp;
+        tmp = c.y[1]; c.y[1] = c.y[2]; c.y[2] = tmp;
+        tmp = c.qx[1]; c.qx[1] = c.qx[2]; c.qx[2] = tmp;
+        tmp = c.qy[1]; c.qy[1] = c.qy[2]; c.qy[2] = tmp;
+        tmp = c.qz[1]; c.qz[1] = c.qz[2]; c.qz[2] = tmp;
+        c.A = -c.A;
+    }
+    return true;
+}
+
+struct RasterArgs {
+    MeshRefs m;
+    int32_t w;           // texture width
     int32_t row0, rows;  // the rows this atlas holds: [row0, row0 + rows)
-    TriSetup *setup;
+    TriPlane *planes;
     uint64_t *area_w;
     uint32_t *tri_plane;
     AtlasHdr *hdr;
@@ -156,12 +283,74 @@ struct RasterArgs {
 };
 
 // Texel-centre range [i0, i1] of sub-pixel interval [lo, hi] clamped to [first, last].
-__device__ __forceinline__ void texel_range(int64_t lo, int64_t hi, int64_t first, int64_t last, int64_t &i0,
-                                            int64_t &i1) {
-    i0 = -floordiv(-(lo - 128), 256);
-    i1 = floordiv(hi - 128, 256);
-    i0 = i0 < first ? first : i0;
-    i1 = i1 > last ? last : i1;
+__device__ __forceinline__ void texel_range(int32_t lo, int32_t hi, int32_t first, int32_t last, int32_t &i0,
+                                            int32_t &i1) {
+    i0 = max((lo + 127) >> 8, first);   // ceil((lo - 128) / 256)
+    i1 = min((hi - 128) >> 8, last);    // floor((hi - 128) / 256)
+}
+
+// n as a sum of two floats, the second the first one's rounding error.
+__device__ __forceinline__ void split_int(int64_t n, float &h, float &l) {
+    if (n <= (1 << 30) && n >= -(1 << 30)) {
+        const int32_t k = (int32_t)n;
+        h = __int2float_rn(k);
+        l = __int2float_rn(k - __float2int_rn(h));
+    } else {
+        h = __ll2float_rn(n);
+        l = __ll2float_rn(n - __float2ll_rn(h));
+    }
+}
+
+// The position planes of a triangle.  The slopes num / A (integers) are computed as float pairs, q plus
+// the remainder's quotient, good to about 2^-44 of themselves, then rounded to 2^-s as integers below
+// 2^30 in magnitude, so each errs by at most 1.01 * 2^-s (two roundings to an integer); over the
+// triangle's extent (ex, ey) a position then errs by at most 1.01 (ex + ey) 2^-s, about 2^-18 for
+// triangles of a few texels.  Triangles too steep for that (s < 8, or a margin of 1/2) get a margin
+// that sends every texel to exact_position.
+__device__ __forceinline__ TriPlane make_plane(const Corners &c, int32_t ex, int32_t ey) {
+    TriPlane p;
+    p.x0 = c.x[0];
+    p.y0 = c.y[0];
+    const int32_t ax = c.y[2] - c.y[0], ay = c.x[0] - c.x[2];  // d w1 / dx, d w1 / dy
+    const int32_t bx = c.y[0] - c.y[1], by = c.x[1] - c.x[0];  // d w2 / dx, d w2 / dy
+    float ah, al;
+    split_int(c.A, ah, al);
+    const float inv = __frcp_rn(ah);
+    float g[6], gl[6], most = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int32_t *const q = k == 0 ? c.qx : k == 1 ? c.qy : c.qz;
+        const int32_t d1 = q[1] - q[0], d2 = q[2] - q[0];
+        p.q0[k] = q[0];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            float h, l;
+            split_int(e ? (int64_t)ay * d1 + (int64_t)by * d2 : (int64_t)ax * d1 + (int64_t)bx * d2, h, l);
+            const float v = __fmul_rn(h, inv);
+            g[2 * k + e] = v;
+            gl[2 * k + e] = __fmul_rn(__fadd_rn(__fmaf_rn(-v, ah, h), __fmaf_rn(-v, al, l)), inv);
+            most = fmaxf(most, fabsf(v));
+        }
+    }
+    const int32_t s = min(30, 29 - ((int32_t)(__float_as_uint(most) >> 23) - 127));  // most 2^s < 2^30
+    const float scale = __uint_as_float((uint32_t)(127 + max(s, 0)) << 23);
+    const float margin = __fmul_rn(1.02f * 4294967296.0f, __fdividef((float)(ex + ey), scale));
+    const bool usable = s >= 8 && margin < 2147483000.0f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        p.gx[k] = usable ? __float2int_rn(__fmul_rn(g[2 * k], scale)) + __float2int_rn(__fmul_rn(gl[2 * k], scale)) : 0;
+        p.gy[k] = usable ? __float2int_rn(__fmul_rn(g[2 * k + 1], scale)) + __float2int_rn(__fmul_rn(gl[2 * k + 1], scale)) : 0;
+    }
+    p.fine = usable ? ((((uint32_t)margin + 64u) & ~31u) | (uint32_t)s) : (0x80000000u | 8u);
+    return p;
+}
+
+// Marks a texel as covered by triangle t.  MIN: by the smallest id (texels that several triangles
+// cover); otherwise by whichever triangle comes last.
+template <bool MIN>
+__device__ __forceinline__ void mark_texel(uint32_t *texel, uint32_t t) {
+    if (MIN) atomicMin(texel, t);
+    else *texel = t;
 }
 
 // raster_rect for a triangle whose corners span at most 2^14 sub-pixels (64 texels) on each axis.
@@ -169,25 +358,29 @@ __device__ __forceinline__ void texel_range(int64_t lo, int64_t hi, int64_t firs
 // and the values computed one texel past the last column or row within one texel of it, so with
 // ex, ey <= 2^14 the extents: |edge value| <= ex (ey + 256) + ey (ex + 256) + 1 < 2^30, and the
 // steps are at most 256 * 2^14.  The scan therefore runs in 32-bit integers after an exact start.
-__device__ void raster_rect_small(const TriSetup &s, uint32_t t, int64_t i0, int64_t i1, int64_t j0, int64_t j1,
+template <bool MIN>
+__device__ __forceinline__ uint32_t raster_rect_small(const Corners &s, uint32_t t, int32_t i0, int32_t i1, int32_t j0, int32_t j1,
                                   int32_t w, int32_t row0, int32_t rows, uint32_t *__restrict__ tri_plane) {
     const int32_t X0 = s.x[0], X1 = s.x[1], X2 = s.x[2], Y0 = s.y[0], Y1 = s.y[1], Y2 = s.y[2];
-    const int32_t px = 256 * (int32_t)i0 + 128, py = 256 * (int32_t)j0 + 128;
+    const int32_t px = 256 * i0 + 128, py = 256 * j0 + 128;
     int32_t e0 = (int32_t)(edge_fn32(X1, Y1, X2, Y2, px, py) + edge_bias(X2 - X1, Y2 - Y1));
     int32_t e1 = (int32_t)(edge_fn32(X2, Y2, X0, Y0, px, py) + edge_bias(X0 - X2, Y0 - Y2));
     int32_t e2 = (int32_t)(edge_fn32(X0, Y0, X1, Y1, px, py) + edge_bias(X1 - X0, Y1 - Y0));
     const int32_t dx0 = -(Y2 - Y1) * 256, dy0 = (X2 - X1) * 256;
     const int32_t dx1 = -(Y0 - Y2) * 256, dy1 = (X0 - X2) * 256;
     const int32_t dx2 = -(Y1 - Y0) * 256, dy2 = (X1 - X0) * 256;
-    const int32_t n_i = (int32_t)(i1 - i0);
+    const int32_t n_i = i1 - i0;
+    uint32_t hits = 0;
 #pragma unroll 1
-    for (int64_t j = j0; j <= j1; ++j) {
+    for (int32_t j = j0; j <= j1; ++j) {
         int32_t r0 = e0, r1 = e1, r2 = e2;
         uint32_t *row = tri_plane + (j - row0) * (int64_t)w + i0;
 #pragma unroll 1
         for (int32_t i = 0; i <= n_i; ++i) {
-            if (min(r0, min(r1, r2)) > 0 && LCL_IN((j - row0) * (int64_t)w + i0 + i, (int64_t)w * rows))
-                atomicMin(row + i, t);
+            if (min(r0, min(r1, r2)) > 0 && LCL_IN((j - row0) * (int64_t)w + i0 + i, (int64_t)w * rows)) {
+                mark_texel<MIN>(row + i, t);
+                ++hits;
+            }
             r0 += dx0;
             r1 += dx1;
             r2 += dx2;
@@ -196,11 +389,13 @@ __device__ void raster_rect_small(const TriSetup &s, uint32_t t, int64_t i0, int
         e1 += dy1;
         e2 += dy2;
     }
+    return hits;
 }
 
 // Rasterises texels [i0, i1] x [j0, j1] (texture rows j) of a set-up triangle into a plane that
-// holds rows [row0, row0 + rows): atomicMin of its id.
-__device__ void raster_rect(const TriSetup &s, uint32_t t, int64_t i0, int64_t i1, int64_t j0, int64_t j1, int32_t w,
+// holds rows [row0, row0 + rows).  Returns the texels it covers there.
+template <bool MIN>
+__device__ __noinline__ uint32_t raster_rect(const Corners &s, uint32_t t, int64_t i0, int64_t i1, int64_t j0, int64_t j1, int32_t w,
                             int32_t row0, int32_t rows, uint32_t *__restrict__ tri_plane) {
     int64_t X0 = s.x[0], X1 = s.x[1], X2 = s.x[2], Y0 = s.y[0], Y1 = s.y[1], Y2 = s.y[2];
     int64_t px = 256 * i0 + 128, py = 256 * j0 + 128;
@@ -212,14 +407,17 @@ __device__ void raster_rect(const TriSetup &s, uint32_t t, int64_t i0, int64_t i
     int64_t dx0 = -(Y2 - Y1) * 256, dy0 = (X2 - X1) * 256;
     int64_t dx1 = -(Y0 - Y2) * 256, dy1 = (X0 - X2) * 256;
     int64_t dx2 = -(Y1 - Y0) * 256, dy2 = (X1 - X0) * 256;
+    uint32_t hits = 0;
 #pragma unroll 1
     for (int64_t j = j0; j <= j1; ++j) {
         int64_t r0 = e0, r1 = e1, r2 = e2;
         uint32_t *row = tri_plane + (j - row0) * (int64_t)w;
 #pragma unroll 1
         for (int64_t i = i0; i <= i1; ++i) {
-            if (r0 > 0 && r1 > 0 && r2 > 0 && LCL_IN((j - row0) * (int64_t)w + i, (int64_t)w * rows))
-                atomicMin(row + i, t);
+            if (r0 > 0 && r1 > 0 && r2 > 0 && LCL_IN((j - row0) * (int64_t)w + i, (int64_t)w * rows)) {
+                mark_texel<MIN>(row + i, t);
+                ++hits;
+            }
             r0 += dx0;
             r1 += dx1;
             r2 += dx2;
@@ -228,127 +426,135 @@ __device__ void raster_rect(const TriSetup &s, uint32_t t, int64_t i0, int64_t i
         e1 += dy1;
         e2 += dy2;
     }
+    return hits;
 }
 
-__global__ void k_raster(RasterArgs a) {
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= a.n_tri) return;
-    TriSetup s;
-    s.rden = 0.0f;
-    uint32_t ip[3], iu[3];
-    bool ok = true;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        ip[k] = a.tri_pos[3 * t + k];
-        iu[k] = a.tri_uv[3 * t + k];
-        ok &= ip[k] < (uint64_t)a.n_pos && iu[k] < (uint64_t)a.n_uv;
-    }
-    if (!ok) {
+// Triangle t's planes and area weight (not MIN), and its texels: returns how many if it is a small
+// triangle (the texels of big ones are added to the header's counts).
+template <bool MIN>
+__device__ __forceinline__ uint32_t raster_triangle(const RasterArgs &a, int64_t t) {
+    Corners c;
+    if (!load_corners(a.m, t, c)) {
         atomicOr(&a.hdr->flags, kBadIndex);
-        s.x[0] = INT32_MIN;
-        a.setup[t] = s;
         a.area_w[t] = 0;
-        return;
+        return 0;
     }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        int2 c = a.uvs[iu[k]];
-        int4 q = a.q[ip[k]];
-        s.x[k] = c.x;
-        s.y[k] = c.y;
-        s.qx[k] = q.x;
-        s.qy[k] = q.y;
-        s.qz[k] = q.z;
-    }
-    int64_t A = edge_fn(s.x[0], s.y[0], s.x[1], s.y[1], s.x[2], s.y[2]);
-    // area weight: 3D area over UV area, floor(isqrt(|n|^2) * 2^(16+F) / |A|), capped
-    {
-        int64_t d1x = (int64_t)s.qx[1] - s.qx[0], d1y = (int64_t)s.qy[1] - s.qy[0], d1z = (int64_t)s.qz[1] - s.qz[0];
-        int64_t d2x = (int64_t)s.qx[2] - s.qx[0], d2y = (int64_t)s.qy[2] - s.qy[0], d2z = (int64_t)s.qz[2] - s.qz[0];
-        int64_t nx = d1y * d2z - d1z * d2y, ny = d1z * d2x - d1x * d2z, nz = d1x * d2y - d1y * d2x;
-        unsigned __int128 nn = (unsigned __int128)((__int128)nx * nx) + (unsigned __int128)((__int128)ny * ny) +
-                               (unsigned __int128)((__int128)nz * nz);
-        uint64_t wgt = 0;
-        if (A != 0) {
-            uint64_t a3 = isqrt_u88(nn);
-            unsigned __int128 num = (unsigned __int128)a3 << (16 + LCL_AREA_FRAC_BITS);
-            uint64_t den = (uint64_t)(A < 0 ? -A : A);
-            unsigned __int128 wq = num / den;
-            wgt = wq > kWeightCap ? kWeightCap : (uint64_t)wq;
+    // area weight: 3D area over UV area, floor(isqrt(|n|^2) * 2^(16+F) / A), capped
+    if (!MIN) {
+        const int32_t d1x = c.qx[1] - c.qx[0], d1y = c.qy[1] - c.qy[0], d1z = c.qz[1] - c.qz[0];
+        const int32_t d2x = c.qx[2] - c.qx[0], d2y = c.qy[2] - c.qy[0], d2z = c.qz[2] - c.qz[0];
+        const int64_t nx = (int64_t)d1y * d2z - (int64_t)d1z * d2y, ny = (int64_t)d1z * d2x - (int64_t)d1x * d2z,
+                      nz = (int64_t)d1x * d2y - (int64_t)d1y * d2x;
+        uint64_t a3, wgt = 0;
+        // components below 2^30: the sum of their squares is below 2^62
+        const int64_t most = max(max(nx < 0 ? -nx : nx, ny < 0 ? -ny : ny), nz < 0 ? -nz : nz);
+        if (most < (1 << 30)) {
+            const int32_t sx = (int32_t)nx, sy = (int32_t)ny, sz = (int32_t)nz;
+            a3 = isqrt_u62((uint64_t)((int64_t)sx * sx + (int64_t)sy * sy + (int64_t)sz * sz));
+        } else {
+            a3 = isqrt_u88((unsigned __int128)((__int128)nx * nx) + (unsigned __int128)((__int128)ny * ny) +
+                           (unsigned __int128)((__int128)nz * nz));
+        }
+        if (c.A != 0) {
+            if (a3 < (1u << 24) && c.A < (int64_t(1) << 31)) {
+                wgt = area_quotient((uint32_t)a3, (uint32_t)c.A, __frcp_rn((float)(uint32_t)c.A));
+            } else if (a3 < (uint64_t(1) << 40)) {
+                wgt = (a3 << (16 + LCL_AREA_FRAC_BITS)) / (uint64_t)c.A;
+            } else {
+                const unsigned __int128 wq = ((unsigned __int128)a3 << (16 + LCL_AREA_FRAC_BITS)) / (uint64_t)c.A;
+                wgt = wq > kWeightCap ? kWeightCap : (uint64_t)wq;
+            }
+            wgt = wgt > kWeightCap ? kWeightCap : wgt;
         }
         a.area_w[t] = wgt;
     }
-    if (A == 0) {
-        s.x[0] = INT32_MIN;
-        a.setup[t] = s;
-        return;
-    }
-    s.rden = __frcp_rn((float)(2 * (A < 0 ? -A : A)));
-    if (A < 0) {  // counter-clockwise: swap corners 1 and 2
-        int32_t tmp;
-        tmp = s.x[1]; s.x[1] = s.x[2]; s.x[2] = tmp;
-        tmp = s.y[1]; s.y[1] = s.y[2]; s.y[2] = tmp;
-        tmp = s.qx[1]; s.qx[1] = s.qx[2]; s.qx[2] = tmp;
-        tmp = s.qy[1]; s.qy[1] = s.qy[2]; s.qy[2] = tmp;
-        tmp = s.qz[1]; s.qz[1] = s.qz[2]; s.qz[2] = tmp;
-    }
-    a.setup[t] = s;
-    int64_t xmin = min(s.x[0], min(s.x[1], s.x[2])), xmax = max(s.x[0], max(s.x[1], s.x[2]));
-    int64_t ymin = min(s.y[0], min(s.y[1], s.y[2])), ymax = max(s.y[0], max(s.y[1], s.y[2]));
-    int64_t i0, i1, j0, j1;
+    if (c.A == 0) return 0;
+    const int32_t xmin = min(c.x[0], min(c.x[1], c.x[2])), xmax = max(c.x[0], max(c.x[1], c.x[2]));
+    const int32_t ymin = min(c.y[0], min(c.y[1], c.y[2])), ymax = max(c.y[0], max(c.y[1], c.y[2]));
+    int32_t i0, i1, j0, j1;
     texel_range(xmin, xmax, 0, a.w - 1, i0, i1);
-    texel_range(ymin, ymax, a.row0, (int64_t)a.row0 + a.rows - 1, j0, j1);  // this atlas's rows only
-    if (i0 > i1 || j0 > j1) return;
-    int64_t nx = i1 - i0 + 1, ny = j1 - j0 + 1;
+    texel_range(ymin, ymax, a.row0, a.row0 + a.rows - 1, j0, j1);  // this atlas's rows only
+    if (i0 > i1 || j0 > j1) return 0;
+    if (!MIN) a.planes[t] = make_plane(c, xmax - xmin, ymax - ymin);
+    const int32_t nx = i1 - i0 + 1, ny = j1 - j0 + 1;  // up to 2^14 each
     if (nx * ny <= kSmallRaster) {
         if (xmax - xmin <= (1 << 14) && ymax - ymin <= (1 << 14))
-            raster_rect_small(s, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
-        else
-            raster_rect(s, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
-        return;
+            return raster_rect_small<MIN>(c, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
+        return raster_rect<MIN>(c, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
     }
-    int64_t nbx = (nx + kBlockSide - 1) / kBlockSide, nby = (ny + kBlockSide - 1) / kBlockSide;
-    int64_t nb = nbx * nby;
+    const int64_t nb = (int64_t)((nx + kBlockSide - 1) / kBlockSide) * ((ny + kBlockSide - 1) / kBlockSide);
     unsigned long long base = atomicAdd(&a.hdr->n_big, (unsigned long long)nb);
     if ((int64_t)base + nb <= a.big_cap) {
         for (int64_t b = 0; b < nb; ++b)
             if (LCL_IN((int64_t)base + b, a.big_cap)) a.big[base + b] = make_uint2((uint32_t)t, (uint32_t)b);
-    } else {
+        return 0;
+    }
+    {
         // list full: the reserved slots that lie below the capacity are read by k_raster_big, so they
         // get empty entries, and this thread rasterises the triangle itself
         for (int64_t b = 0; b < nb && (int64_t)base + b < a.big_cap; ++b)
             if (LCL_IN((int64_t)base + b, a.big_cap)) a.big[base + b] = make_uint2(kNone, 0u);
-        raster_rect(s, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
+        const uint32_t hits = raster_rect<MIN>(c, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
+        if (!MIN) atomicAdd(&a.hdr->n_hits[0], (unsigned long long)hits);
+        return 0;
     }
 }
 
-__global__ void k_raster_big(const uint2 *__restrict__ big, const AtlasHdr *__restrict__ hdr, int64_t cap,
-                             const TriSetup *__restrict__ setup, int64_t n_tri, int32_t w, int32_t row0,
-                             int32_t rows, uint32_t *__restrict__ tri_plane) {
-    int64_t n = min((int64_t)hdr->n_big, cap);
+// A thread per triangle.  Texels that no two triangles share, as in most unwraps, need no atomics, whose
+// rate of about one lane a cycle and SM bounds the scattered writes (268 M of them took 1.05 ms).  So
+// the first run (not MIN) stores ids as they come and counts the texels each triangle covers; when the
+// counts add up to the covered texels, every texel has one triangle and the plane is right.  Otherwise
+// atlas_build_impl runs MIN over the result: of the triangles that cover a texel the smallest id.
+template <bool MIN>
+__global__ void __launch_bounds__(128) k_raster(const __grid_constant__ RasterArgs a) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    uint32_t hits = t < a.m.n_tri ? raster_triangle<MIN>(a, t) : 0u;
+    if (!MIN) {
+        __shared__ uint32_t s_hits[4];
+        hits = __reduce_add_sync(0xffffffffu, hits);
+        if ((threadIdx.x & 31) == 0) s_hits[threadIdx.x >> 5] = hits;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const unsigned long long n = (unsigned long long)s_hits[0] + s_hits[1] + s_hits[2] + s_hits[3];
+            if (n) atomicAdd(&a.hdr->n_hits[blockIdx.x & 7u], n);
+        }
+    }
+}
+
+template <bool MIN>
+__global__ void __launch_bounds__(kThreads) k_raster_big(const uint2 *__restrict__ big, AtlasHdr *hdr, int64_t cap,
+                             const MeshRefs m, int32_t w, int32_t row0, int32_t rows,
+                             uint32_t *__restrict__ tri_plane) {
+    const int64_t n = min((int64_t)hdr->n_big, cap);
+    uint32_t hits = 0;
     for (int64_t e = blockIdx.x; e < n; e += gridDim.x) {
         if (!LCL_IN(e, cap)) break;
         uint2 ent = big[e];
         if (ent.x == kNone) continue;  // a slot of a reservation that did not fit
-        if (!LCL_IN(ent.x, n_tri)) continue;
-        TriSetup s = setup[ent.x];
-        int64_t xmin = min(s.x[0], min(s.x[1], s.x[2])), xmax = max(s.x[0], max(s.x[1], s.x[2]));
-        int64_t ymin = min(s.y[0], min(s.y[1], s.y[2])), ymax = max(s.y[0], max(s.y[1], s.y[2]));
-        int64_t i0, i1, j0, j1;
+        if (!LCL_IN(ent.x, m.n_tri)) continue;
+        Corners s;
+        if (!load_corners(m, ent.x, s)) continue;  // uniform
+        const int32_t xmin = min(s.x[0], min(s.x[1], s.x[2])), xmax = max(s.x[0], max(s.x[1], s.x[2]));
+        const int32_t ymin = min(s.y[0], min(s.y[1], s.y[2])), ymax = max(s.y[0], max(s.y[1], s.y[2]));
+        int32_t i0, i1, j0, j1;
         texel_range(xmin, xmax, 0, w - 1, i0, i1);
-        texel_range(ymin, ymax, row0, (int64_t)row0 + rows - 1, j0, j1);  // as k_raster cut the blocks
-        int64_t nbx = (i1 - i0 + 1 + kBlockSide - 1) / kBlockSide;
-        int64_t bx = ent.y % nbx, by = ent.y / nbx;
-        int64_t i = i0 + bx * kBlockSide + (threadIdx.x % kBlockSide);
-        int64_t j = j0 + by * kBlockSide + (threadIdx.x / kBlockSide);
+        texel_range(ymin, ymax, row0, row0 + rows - 1, j0, j1);  // as k_raster cut the blocks
+        const uint32_t nbx = (uint32_t)(i1 - i0 + 1 + kBlockSide - 1) / kBlockSide;
+        const int32_t i = i0 + (int32_t)(ent.y % nbx) * kBlockSide + (int32_t)(threadIdx.x % kBlockSide);
+        const int32_t j = j0 + (int32_t)(ent.y / nbx) * kBlockSide + (int32_t)(threadIdx.x / kBlockSide);
         if (i > i1 || j > j1) continue;
-        int64_t px = 256 * i + 128, py = 256 * j + 128;
-        int64_t X0 = s.x[0], X1 = s.x[1], X2 = s.x[2], Y0 = s.y[0], Y1 = s.y[1], Y2 = s.y[2];
-        int64_t e0 = edge_fn(X1, Y1, X2, Y2, px, py) + edge_bias(X2 - X1, Y2 - Y1);
-        int64_t e1 = edge_fn(X2, Y2, X0, Y0, px, py) + edge_bias(X0 - X2, Y0 - Y2);
-        int64_t e2 = edge_fn(X0, Y0, X1, Y1, px, py) + edge_bias(X1 - X0, Y1 - Y0);
-        if (e0 > 0 && e1 > 0 && e2 > 0 && LCL_IN((j - row0) * (int64_t)w + i, (int64_t)w * rows))
-            atomicMin(tri_plane + (j - row0) * (int64_t)w + i, ent.x);
+        const int32_t px = 256 * i + 128, py = 256 * j + 128;
+        const int64_t e0 = edge_fn32(s.x[1], s.y[1], s.x[2], s.y[2], px, py) + edge_bias(s.x[2] - s.x[1], s.y[2] - s.y[1]);
+        const int64_t e1 = edge_fn32(s.x[2], s.y[2], s.x[0], s.y[0], px, py) + edge_bias(s.x[0] - s.x[2], s.y[0] - s.y[2]);
+        const int64_t e2 = edge_fn32(s.x[0], s.y[0], s.x[1], s.y[1], px, py) + edge_bias(s.x[1] - s.x[0], s.y[1] - s.y[0]);
+        if (e0 > 0 && e1 > 0 && e2 > 0 && LCL_IN((j - row0) * (int64_t)w + i, (int64_t)w * rows)) {
+            mark_texel<MIN>(tri_plane + (j - row0) * (int64_t)w + i, ent.x);
+            ++hits;
+        }
+    }
+    if (!MIN && n > 0) {
+        hits = __reduce_add_sync(0xffffffffu, hits);
+        if ((threadIdx.x & 31) == 0 && hits) atomicAdd(&hdr->n_hits[blockIdx.x & 7u], (unsigned long long)hits);
     }
 }
 
@@ -386,8 +592,53 @@ __device__ __forceinline__ int32_t interp_axis(int64_t w1, int64_t w2, int64_t A
     return q0 + (int32_t)est;
 }
 
-__global__ void __launch_bounds__(kThreads, 4) k_resolve(const TriSetup *__restrict__ setup, int64_t n_tri, int32_t w,
-                                                      int32_t h, int32_t row0, int32_t T,
+// The position of triangle t's texel centre (cx, cy), exactly, from the mesh.
+__device__ __noinline__ int3 exact_position(const MeshRefs &m, uint32_t t, int32_t cx, int32_t cy) {
+    Corners c;
+    if (!load_corners(m, t, c)) return make_int3(INT32_MIN, 0, 0);  // not a triangle that covers a texel
+    const int64_t w1 = edge_fn32(c.x[2], c.y[2], c.x[0], c.y[0], cx, cy);
+    const int64_t w2 = edge_fn32(c.x[0], c.y[0], c.x[1], c.y[1], cx, cy);
+    const float rden = __frcp_rn((float)(2 * c.A));
+    return make_int3(interp_axis(w1, w2, c.A, rden, c.qx[0], c.qx[1], c.qx[2]),
+                     interp_axis(w1, w2, c.A, rden, c.qy[0], c.qy[1], c.qy[2]),
+                     interp_axis(w1, w2, c.A, rden, c.qz[0], c.qz[1], c.qz[2]));
+}
+
+// The position of triangle t's texel (x, y): q0 + floor(v), v = (gx (cx - x0) + gy (cy - y0)) 2^-s + 1/2
+// per axis as a 64-bit integer with s fraction bits; where the fraction is further than the planes'
+// error from 0 and 1 the exact v has the same floor.
+__device__ __forceinline__ int3 plane_position(const TriPlane *__restrict__ planes, const MeshRefs &mesh, uint32_t t,
+                                               int32_t x, int32_t y) {
+    const int4 *const r = reinterpret_cast<const int4 *>(planes + t);
+    const int4 ra = __ldg(r), rb = __ldg(r + 1), rc = __ldg(r + 2);
+    const int32_t cx = 256 * x + 128, cy = 256 * y + 128;
+    const int32_t dx = cx - ra.x, dy = cy - ra.y;  // within +-2^24
+    const uint32_t s = (uint32_t)rc.w & 31u, margin = (uint32_t)rc.w & ~31u;
+    const int64_t half = (int64_t)(1u << (s - 1u));
+    const int64_t vx = (int64_t)ra.z * dx + ((int64_t)rb.y * dy + half);
+    const int64_t vy = (int64_t)ra.w * dx + ((int64_t)rb.z * dy + half);
+    const int64_t vz = (int64_t)rb.x * dx + ((int64_t)rb.w * dy + half);
+    const uint32_t lim = 0u - 2u * margin;  // settled: margin <= fraction < 2^32 - margin
+    if (((uint32_t)vx << (32u - s)) - margin >= lim || ((uint32_t)vy << (32u - s)) - margin >= lim ||
+        ((uint32_t)vz << (32u - s)) - margin >= lim)
+        return exact_position(mesh, t, cx, cy);
+    return make_int3(rc.x + (int32_t)__funnelshift_r((uint32_t)vx, (uint32_t)(vx >> 32), s),
+                     rc.y + (int32_t)__funnelshift_r((uint32_t)vy, (uint32_t)(vy >> 32), s),
+                     rc.z + (int32_t)__funnelshift_r((uint32_t)vz, (uint32_t)(vz >> 32), s));
+}
+
+// One CTA per tile.  WORDS (tile side 32 or more, width a multiple of 32): a warp takes 32-texel row
+// segments, each one aligned coverage word, a texel per lane.  Otherwise one texel per thread and
+// step, a tile row after the other.  Either way warps read the triangle plane and write the position
+// planes in long rows, and the texels of one triangle, which lie together, find its planes in L1.
+// Bound by the latency of the chain triangle id -> planes (47% of issue slots, a third of DRAM): 1.83 ms
+// at 16384^2 with 8 M triangles, where exact barycentrics for every texel (290 instructions) took 2.79.
+// Slower: planes in binary32 (their error sent a tenth of the warps to exact_position: 2.28 ms), four
+// segments in flight per warp (1.95 ms, spills), five or six CTAs per SM (spills).
+template <bool WORDS>
+__global__ void __launch_bounds__(kThreads, 4) k_resolve(const TriPlane *__restrict__ planes,
+                                                      const __grid_constant__ MeshRefs mesh, int32_t w, int32_t h,
+                                                      int32_t row0, int32_t T,
                                                       const uint32_t *__restrict__ tri_plane,
                                                       int32_t *__restrict__ px, int32_t *__restrict__ py,
                                                       int32_t *__restrict__ pz, uint32_t *__restrict__ cover,
@@ -395,72 +646,56 @@ __global__ void __launch_bounds__(kThreads, 4) k_resolve(const TriSetup *__restr
     const int32_t tx = blockIdx.x, ty = blockIdx.y;
     int32_t mn[3] = {INT32_MAX, INT32_MAX, INT32_MAX}, mx[3] = {INT32_MIN, INT32_MIN, INT32_MIN};
     int32_t cnt = 0;
-    // one texel per thread and step, a tile row after the other: warps read the triangle plane and
-    // write the position planes in whole 128-byte rows, and the texels of one triangle, which lie
-    // together, find its set-up record in L1
-    const int32_t n_tex_tile = T * T;
-    const int iters = (n_tex_tile + kThreads - 1) / kThreads;
-    // tiles of 32 texels or more on a width that is a multiple of 32: each warp's 32 texels are one
-    // aligned coverage word (uniform over the grid)
-    const bool aligned = T >= 32 && (w & 31) == 0;
-    // the triangle id of the thread's texel in step it + 1 is loaded during step it; T is a power of
-    // two, so the texel's row and column in the tile come from a shift and a mask
-    const int tshift = __ffs(T) - 1;
-    auto texel = [&](int step, int32_t &x, int32_t &y, int64_t &l) {
-        const int32_t i = step * kThreads + threadIdx.x;
-        x = tx * T + (i & (T - 1));
-        y = ty * T + (i >> tshift);
-        const bool v = i < n_tex_tile && x < w && y < h && LCL_IN((int64_t)y * w + x, (int64_t)w * h);
-        l = v ? (int64_t)y * w + x : -1;
+    const int tshift = __ffs(T) - 1;  // T is a power of two
+    auto resolve = [&](uint32_t t, int32_t x, int32_t y, int32_t l) {  // writes the texel, returns whether it is covered
+        int3 o = make_int3(INT32_MIN, 0, 0);
+        const bool covered = t != kNone && LCL_IN(t, mesh.n_tri);
+        if (covered) {
+            o = plane_position(planes, mesh, t, x, y + row0);
+            mn[0] = min(mn[0], o.x); mx[0] = max(mx[0], o.x);
+            mn[1] = min(mn[1], o.y); mx[1] = max(mx[1], o.y);
+            mn[2] = min(mn[2], o.z); mx[2] = max(mx[2], o.z);
+        }
+        __stcs(px + l, o.x);
+        __stcs(py + l, o.y);
+        __stcs(pz + l, o.z);
+        return covered;
     };
-    int32_t nx, ny;
-    int64_t nl;
-    texel(0, nx, ny, nl);
-    uint32_t nt = nl >= 0 ? __ldcs(tri_plane + nl) : kNone;
-    for (int it = 0; it < iters; ++it) {
-        const int32_t x = nx, y = ny;
-        const bool valid = nl >= 0;
-        const int64_t l = valid ? nl : 0;
-        const uint32_t t = nt;
-        if (it + 1 < iters) {
-            texel(it + 1, nx, ny, nl);
-            nt = nl >= 0 ? __ldcs(tri_plane + nl) : kNone;
-        }
-        bool covered = false;
-        if (valid) {
-            int32_t ox = INT32_MIN, oy = 0, oz = 0;
-            if (t != kNone && LCL_IN(t, n_tri)) {
-                const TriSetup s = setup[t];
-                // sub-pixel coordinates and texel centres lie within [-2^22, 2^23] (sides <= 2^14,
-                // UVs in [-1, 2]): differences fit in 32 bits, products in 64
-                const int32_t cx = 256 * x + 128, cy = 256 * (y + row0) + 128;
-                const int64_t A = edge_fn32(s.x[0], s.y[0], s.x[1], s.y[1], s.x[2], s.y[2]);
-                const int64_t w1 = edge_fn32(s.x[2], s.y[2], s.x[0], s.y[0], cx, cy);
-                const int64_t w2 = edge_fn32(s.x[0], s.y[0], s.x[1], s.y[1], cx, cy);
-                const float rden = s.rden;
-                ox = interp_axis(w1, w2, A, rden, s.qx[0], s.qx[1], s.qx[2]);
-                oy = interp_axis(w1, w2, A, rden, s.qy[0], s.qy[1], s.qy[2]);
-                oz = interp_axis(w1, w2, A, rden, s.qz[0], s.qz[1], s.qz[2]);
-                mn[0] = min(mn[0], ox); mx[0] = max(mx[0], ox);
-                mn[1] = min(mn[1], oy); mx[1] = max(mx[1], oy);
-                mn[2] = min(mn[2], oz); mx[2] = max(mx[2], oz);
-                ++cnt;
-                covered = true;
-            }
-            __stcs(px + l, ox);
-            __stcs(py + l, oy);
-            __stcs(pz + l, oz);
-        }
-        // coverage bits
-        const uint32_t word = (uint32_t)(l >> 5);
-        if (aligned) {
-            // the warp holds one whole 32-texel word of one tile row (lane k = texel k): a ballot is
-            // the word, written by lane 0 (the tile's CTA is its only writer)
+    if (WORDS) {
+        const int lane = threadIdx.x & 31, slog = tshift - 5;  // segments per row: 1 << slog
+        const int n_words = 1 << (tshift + slog);
+        // the triangle ids of the warp's next segment are loaded during this one
+        auto place = [&](int i, int32_t &x, int32_t &y) {
+            x = (tx << tshift) + ((i & ((1 << slog) - 1)) << 5);
+            y = (ty << tshift) + (i >> slog);
+            return i < n_words && x < w && y < h;  // x < w implies x + 31 < w
+        };
+        int32_t nx, ny;
+        bool nv = place((int)(threadIdx.x >> 5), nx, ny);
+        uint32_t nt = nv ? __ldcs(tri_plane + (ny * w + nx + lane)) : kNone;
+        for (int i = (int)(threadIdx.x >> 5); i < n_words; i += kThreads / 32) {  // uniform over the warp
+            const int32_t x = nx, y = ny;
+            const bool v = nv;
+            const uint32_t t = nt;
+            nv = place(i + kThreads / 32, nx, ny);
+            nt = nv ? __ldcs(tri_plane + (ny * w + nx + lane)) : kNone;
+            if (!v) continue;
+            const int32_t l = y * w + x + lane;  // below 2^28
+            const bool covered = LCL_IN(l, (int64_t)w * h) && resolve(t, x + lane, y, l);
             const uint32_t bits = __ballot_sync(0xffffffffu, covered);
-            if (valid && (threadIdx.x & 31) == 0 && LCL_IN(word, ((int64_t)w * h + 31) / 32)) cover[word] = bits;
-        } else {
+            cnt += __popc(bits);  // the warp's count, in every lane
+            if (lane == 0) cover[l >> 5] = bits;  // the tile's CTA is the word's only writer
+        }
+        if (lane) cnt = 0;
+    } else {
+        for (int i = threadIdx.x; i - (int)(threadIdx.x & 31) < T * T; i += kThreads) {  // whole warps together
+            const int32_t x = tx * T + (i & (T - 1)), y = ty * T + (i >> tshift);
+            const bool valid = i < T * T && x < w && y < h && LCL_IN((int64_t)y * w + x, (int64_t)w * h);
+            const int32_t l = valid ? y * w + x : 0;
+            const bool covered = valid && resolve(__ldcs(tri_plane + l), x, y, l);
+            cnt += covered;
             // lanes writing the same 32-bit word combine, one atomicOr per word
-            const uint32_t val = covered ? 1u << (uint32_t)(l & 31) : 0u;
+            const uint32_t word = (uint32_t)(l >> 5), val = covered ? 1u << (uint32_t)(l & 31) : 0u;
             const uint32_t peers = __match_any_sync(0xffffffffu, valid ? word : 0xFFFFFFFFu);
             const uint32_t orv = __reduce_or_sync(peers, val);
             if (valid && orv != 0 && (threadIdx.x & 31) == (__ffs(peers) - 1) &&
@@ -470,27 +705,29 @@ __global__ void __launch_bounds__(kThreads, 4) k_resolve(const TriSetup *__restr
     }
     // tile box: block reduction
     __shared__ int32_t red[7][kThreads / 32];
-    int32_t v[7] = {mn[0], mn[1], mn[2], cnt, mx[0], mx[1], mx[2]};
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        v[0] = min(v[0], __shfl_xor_sync(0xffffffffu, v[0], o));
-        v[1] = min(v[1], __shfl_xor_sync(0xffffffffu, v[1], o));
-        v[2] = min(v[2], __shfl_xor_sync(0xffffffffu, v[2], o));
-        v[3] += __shfl_xor_sync(0xffffffffu, v[3], o);
-        v[4] = max(v[4], __shfl_xor_sync(0xffffffffu, v[4], o));
-        v[5] = max(v[5], __shfl_xor_sync(0xffffffffu, v[5], o));
-        v[6] = max(v[6], __shfl_xor_sync(0xffffffffu, v[6], o));
-    }
+    int32_t v[7];
+    v[0] = __reduce_min_sync(0xffffffffu, mn[0]);
+    v[1] = __reduce_min_sync(0xffffffffu, mn[1]);
+    v[2] = __reduce_min_sync(0xffffffffu, mn[2]);
+    v[3] = __reduce_add_sync(0xffffffffu, cnt);
+    v[4] = __reduce_max_sync(0xffffffffu, mx[0]);
+    v[5] = __reduce_max_sync(0xffffffffu, mx[1]);
+    v[6] = __reduce_max_sync(0xffffffffu, mx[2]);
     const int wid = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0)
         for (int k = 0; k < 7; ++k) red[k][wid] = v[k];
     __syncthreads();
+    if (threadIdx.x < 32) {  // lane j holds warp j's values
+        const int j = threadIdx.x & (kThreads / 32 - 1);
+        v[0] = __reduce_min_sync(0xffffffffu, red[0][j]);
+        v[1] = __reduce_min_sync(0xffffffffu, red[1][j]);
+        v[2] = __reduce_min_sync(0xffffffffu, red[2][j]);
+        v[3] = __reduce_add_sync(0xffffffffu, threadIdx.x < kThreads / 32 ? red[3][j] : 0);
+        v[4] = __reduce_max_sync(0xffffffffu, red[4][j]);
+        v[5] = __reduce_max_sync(0xffffffffu, red[5][j]);
+        v[6] = __reduce_max_sync(0xffffffffu, red[6][j]);
+    }
     if (threadIdx.x == 0) {
-        for (int j = 1; j < kThreads / 32; ++j) {
-            v[0] = min(v[0], red[0][j]); v[1] = min(v[1], red[1][j]); v[2] = min(v[2], red[2][j]);
-            v[3] += red[3][j];
-            v[4] = max(v[4], red[4][j]); v[5] = max(v[5], red[5][j]); v[6] = max(v[6], red[6][j]);
-        }
         if (LCL_IN((int64_t)ty * gridDim.x + tx, (int64_t)((w + T - 1) / T) * ((h + T - 1) / T))) {
             int32_t *b = tile_box + 8 * ((int64_t)ty * gridDim.x + tx);
             reinterpret_cast<int4 *>(b)[0] = make_int4(v[0], v[1], v[2], v[3]);
@@ -500,7 +737,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_resolve(const TriSetup *__restr
 }
 
 __global__ void __launch_bounds__(kThreads) k_super(const int32_t *__restrict__ tile_box, int32_t tiles_x,
-                                                    int32_t tiles_y, int32_t *__restrict__ super_box) {
+                                                    int32_t tiles_y, int32_t *__restrict__ super_box,
+                                                    unsigned long long *n_covered) {
     const int32_t sx = blockIdx.x, sy = blockIdx.y;
     const int32_t tx = sx * LCL_SUPER + (threadIdx.x % LCL_SUPER), ty = sy * LCL_SUPER + (threadIdx.x / LCL_SUPER);
     int32_t v[7] = {INT32_MAX, INT32_MAX, INT32_MAX, 0, INT32_MIN, INT32_MIN, INT32_MIN};
@@ -536,12 +774,13 @@ __global__ void __launch_bounds__(kThreads) k_super(const int32_t *__restrict__ 
             b[0] = make_int4(v[0], v[1], v[2], v[3]);
             b[1] = make_int4(v[4], v[5], v[6], 0);
         }
+        if (v[3]) atomicAdd(n_covered, (unsigned long long)v[3]);
         (void)n_sup;
     }
 }
 
 struct WsLayout {
-    size_t hdr, q, uvs, setup, big, total;
+    size_t hdr, q, uvs, planes, big, total;
 };
 
 WsLayout ws_layout(int64_t n_pos, int64_t n_uv, int64_t n_tri, int32_t w, int32_t h) {
@@ -549,8 +788,8 @@ WsLayout ws_layout(int64_t n_pos, int64_t n_uv, int64_t n_tri, int32_t w, int32_
     L.hdr = 0;
     L.q = align256(sizeof(AtlasHdr));
     L.uvs = L.q + align256((size_t)n_pos * sizeof(int4));
-    L.setup = L.uvs + align256((size_t)n_uv * sizeof(int2));
-    L.big = L.setup + align256((size_t)n_tri * sizeof(TriSetup));
+    L.planes = L.uvs + align256((size_t)n_uv * sizeof(int2));
+    L.big = L.planes + align256((size_t)n_tri * 64);  // 64 bytes a triangle, of which its planes take 48
     L.total = L.big + align256((size_t)big_capacity(n_tri, w, h) * sizeof(uint2));
     return L;
 }
@@ -573,7 +812,7 @@ lcl_status atlas_build_impl(const lcl_mesh *mesh, lcl_atlas *at, void *ws, size_
     AtlasHdr *hdr = reinterpret_cast<AtlasHdr *>(base + L.hdr);
     int4 *q = reinterpret_cast<int4 *>(base + L.q);
     int2 *uvs = reinterpret_cast<int2 *>(base + L.uvs);
-    TriSetup *setup = reinterpret_cast<TriSetup *>(base + L.setup);
+    TriPlane *planes = reinterpret_cast<TriPlane *>(base + L.planes);
     uint2 *big = reinterpret_cast<uint2 *>(base + L.big);
     const int64_t n_tex = (int64_t)at->width * at->height;
     const int64_t n_words = (n_tex + 31) / 32;
@@ -588,42 +827,60 @@ lcl_status atlas_build_impl(const lcl_mesh *mesh, lcl_atlas *at, void *ws, size_
     k_snap<<<(unsigned)((mesh->n_uv + kThreads - 1) / kThreads), kThreads, 0, st>>>(mesh->uv, mesh->n_uv, at->width,
                                                                                    tex_h, hdr, uvs);
     count_launches(5);
+    MeshRefs mr;
+    mr.tri_pos = mesh->tri_pos;
+    mr.tri_uv = mesh->tri_uv;
+    mr.q = q;
+    mr.uvs = uvs;
+    mr.n_tri = mesh->n_tri;
+    mr.n_pos = mesh->n_pos;
+    mr.n_uv = mesh->n_uv;
+    RasterArgs ra;
+    ra.m = mr;
+    ra.w = at->width;
+    ra.row0 = at->row0;
+    ra.rows = at->height;
+    ra.planes = planes;
+    ra.area_w = at->area_w;
+    ra.tri_plane = at->tri;
+    ra.hdr = hdr;
+    ra.big = big;
+    ra.big_cap = (int64_t)big_capacity(mesh->n_tri, at->width, at->height);  // blocks of this atlas's rows
+    const unsigned rg = (unsigned)((mesh->n_tri + 127) / 128);
+    const dim3 tg(at->tiles_x, at->tiles_y), sg(at->supers_x, at->supers_y);
+    auto resolve = [&]() {
+        auto kernel = at->tile >= 32 && (at->width & 31) == 0 ? k_resolve<true> : k_resolve<false>;
+        kernel<<<tg, kThreads, 0, st>>>(planes, mr, at->width, at->height, at->row0, at->tile, at->tri, at->pos_x,
+                                        at->pos_y, at->pos_z, at->cover, at->tile_box);
+        k_super<<<sg, kThreads, 0, st>>>(at->tile_box, at->tiles_x, at->tiles_y, at->super_box, &hdr->n_covered);
+        count_launches(2);
+    };
     if (mesh->n_tri > 0) {
-        RasterArgs ra;
-        ra.tri_pos = mesh->tri_pos;
-        ra.tri_uv = mesh->tri_uv;
-        ra.n_tri = mesh->n_tri;
-        ra.n_pos = mesh->n_pos;
-        ra.n_uv = mesh->n_uv;
-        ra.q = q;
-        ra.uvs = uvs;
-        ra.w = at->width;
-        ra.h = tex_h;
-        ra.row0 = at->row0;
-        ra.rows = at->height;
-        ra.setup = setup;
-        ra.area_w = at->area_w;
-        ra.tri_plane = at->tri;
-        ra.hdr = hdr;
-        ra.big = big;
-        ra.big_cap = (int64_t)big_capacity(mesh->n_tri, at->width, at->height);  // blocks of this atlas's rows
-        k_raster<<<(unsigned)((mesh->n_tri + 127) / 128), 128, 0, st>>>(ra);
-        k_raster_big<<<sms * 8, kThreads, 0, st>>>(big, hdr, ra.big_cap, setup, mesh->n_tri, at->width, at->row0,
-                                                   at->height, at->tri);
+        k_raster<false><<<rg, 128, 0, st>>>(ra);
+        k_raster_big<false><<<sms * 8, kThreads, 0, st>>>(big, hdr, ra.big_cap, mr, at->width, at->row0, at->height,
+                                                          at->tri);
         count_launches(2);
     }
-    dim3 tg(at->tiles_x, at->tiles_y);
-    k_resolve<<<tg, kThreads, 0, st>>>(setup, mesh->n_tri, at->width, at->height, at->row0, at->tile, at->tri,
-                                       at->pos_x, at->pos_y, at->pos_z, at->cover, at->tile_box);
-    dim3 sg(at->supers_x, at->supers_y);
-    k_super<<<sg, kThreads, 0, st>>>(at->tile_box, at->tiles_x, at->tiles_y, at->super_box);
-    count_launches(2);
+    resolve();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "atlas build launch");
     AtlasHdr host;
     e = cudaMemcpyAsync(&host, hdr, sizeof(AtlasHdr), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "atlas build");
+    unsigned long long hits = 0;
+    for (const unsigned long long n : host.n_hits) hits += n;
+    if (hits != host.n_covered) {  // some texel has several triangles: the smallest id
+        // the big triangles' list is filled again from its start
+        e = cudaMemsetAsync(&hdr->n_big, 0, sizeof(hdr->n_big), st);
+        k_raster<true><<<rg, 128, 0, st>>>(ra);
+        k_raster_big<true><<<sms * 8, kThreads, 0, st>>>(big, hdr, ra.big_cap, mr, at->width, at->row0, at->height, at->tri);
+        count_launches(2);
+        resolve();
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return cuda_fail(e, "atlas build");
+    }
     if (host.flags & kBadPos) return fail(LCL_ERR_INVALID_ARG, "mesh positions contain a non-finite value");
     if (host.flags & kFlatBBox) return fail(LCL_ERR_INVALID_ARG, "mesh bounding box has zero extent");
     if (host.flags & kBadIndex) return fail(LCL_ERR_INVALID_ARG, "triangle index out of range");

@@ -62,7 +62,8 @@ struct Mat16 {
 };
 
 __global__ void k_vertex(const float *__restrict__ pos, int64_t n_pos, const Mat16 mat, float mn0, float mn1,
-                         float mn2, double scale, float fw, float fh, PVert *__restrict__ out) {
+                         float mn2, double scale, ScalePair sp, float fw, float fh,
+                         PVert *__restrict__ out) {
     const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (v >= n_pos) return;
     if (!LCL_IN(3 * v + 2, 3 * n_pos)) return;
@@ -72,9 +73,9 @@ __global__ void k_vertex(const float *__restrict__ pos, int64_t n_pos, const Mat
     r.Y = 0;
     r.z = 0.0f;
     r.pad = 0;
-    const float qx = (float)quantize_coord(pos[3 * v + 0], mn0, scale);
-    const float qy = (float)quantize_coord(pos[3 * v + 1], mn1, scale);
-    const float qz = (float)quantize_coord(pos[3 * v + 2], mn2, scale);
+    const float qx = (float)quantize_coord(pos[3 * v + 0], mn0, scale, sp);
+    const float qy = (float)quantize_coord(pos[3 * v + 1], mn1, scale, sp);
+    const float qz = (float)quantize_coord(pos[3 * v + 2], mn2, scale, sp);
     const float cw = clip_row(m + 12, qx, qy, qz);
     if (cw > 0.0f) {
         // div_rn: the correctly rounded quotient, the value of __fdiv_rn (checked by lcl_check_division)
@@ -304,7 +305,7 @@ lcl_status depth_render_impl(const lcl_mesh *mesh, const lcl_atlas *atlas, const
         Mat16 mat;
         for (int i = 0; i < 16; ++i) mat.v[i] = cam->m[i];
         k_vertex<<<(unsigned)((mesh->n_pos + kThreads - 1) / kThreads), kThreads, 0, st>>>(
-            mesh->pos, mesh->n_pos, mat, a.mn[0], a.mn[1], a.mn[2], a.scale, a.fw, a.fh, pv);
+            mesh->pos, mesh->n_pos, mat, a.mn[0], a.mn[1], a.mn[2], a.scale, scale_pair(a.scale), a.fw, a.fh, pv);
         k_raster<<<(unsigned)((mesh->n_tri + 127) / 128), 128, 0, st>>>(a);
         k_raster_big<<<sms * 8, kThreads, 0, st>>>(a);
         count_launches(3);
