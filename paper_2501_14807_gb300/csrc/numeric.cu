@@ -6,11 +6,11 @@
 //                 the 2, 4 or 8 lanes of its group, and the group's output word is merged with
 //                 shuffles and written by its first lane
 //   k_num_select  selection by value into a label layer (the lane owns its texels' label bytes)
-//   k_num_stats   zonal statistics: a contiguous range of 16-texel chunks per warp (one chunk per
-//                 lane and step); runs of equal zone labels stay in registers until the warp
-//                 meets another zone, then are reduced across the warp and flushed into a
-//                 shared-memory table (or the output, for many zones); min / max through
-//                 order-preserving 64-bit keys, sums in double
+//   k_num_stats   zonal statistics: a contiguous range of quads per warp (a quad per lane and step);
+//                 runs of equal zone labels stay in registers, as integers, until the warp meets
+//                 another zone, then are reduced across the warp, rounded to double and flushed
+//                 into a shared-memory table (or the output, for many zones); min / max through
+//                 order-preserving 64-bit keys
 #include <algorithm>
 #include <type_traits>
 
@@ -110,33 +110,37 @@ struct ArithArgs {
 // Texels of one lane's chunk: 16 / S, starting at texel c * (16 / S), inside mask word
 // (c * (16 / S)) / 32 at bit (c * (16 / S)) % 32; 2S consecutive lanes share that word.
 template <int S, int KIND>
-__global__ void __launch_bounds__(kThreads) k_num_arith(ArithArgs p) {
+__global__ void __launch_bounds__(kThreads) k_num_arith(const __grid_constant__ ArithArgs p) {
     constexpr int kPer = 16 / S;
     constexpr int kGroup = 32 / kPer;  // lanes per mask word
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // whole warps iterate together (the group merge uses shuffles over the full warp)
+    // whole warps iterate together (the group merge uses shuffles over the full warp); the next chunk is
+    // loaded while this one is worked on (out may be a or b: a thread writes only chunks it has read)
     const int64_t n_iter = (p.n_chunks + 31) & ~int64_t(31);
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c - (threadIdx.x & 31) < n_iter; c += stride) {
-        int64_t t0 = c * kPer;
-        const bool live = c < p.n_chunks && LCL_IN(t0 + kPer - 1, p.n_texels);
-        uint32_t bits = 0;
-        if (live) {
-            const uint4 A = __ldcs(p.a + c);
-            uint4 B;
+    uint4 A = make_uint4(0u, 0u, 0u, 0u), B = A;
+    uint32_t ok = 0u;
+    auto load = [&](int64_t c) {
+        const int64_t t0 = c * kPer;
+        if (c < p.n_chunks && LCL_IN(t0 + kPer - 1, p.n_texels)) {
+            A = __ldcs(p.a + c);
             if (p.b) B = __ldcs(p.b + c);
             const uint32_t word = (uint32_t)(t0 >> 5);
+            ok = __ldg(p.ma + word) & __ldg(p.cover + word);
+            if (p.b) ok &= __ldg(p.mb + word);
+        }
+    };
+    int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    load(c);
+    for (; c - (threadIdx.x & 31) < n_iter; c += stride) {
+        const int64_t t0 = c * kPer;
+        const bool live = c < p.n_chunks && LCL_IN(t0 + kPer - 1, p.n_texels);
+        const uint32_t aw[4] = {A.x, A.y, A.z, A.w}, bw[4] = {B.x, B.y, B.z, B.w};
+        const uint32_t now = ok;
+        load(c + stride);
+        uint32_t bits = 0;
+        if (live) {
             const int off = (int)(t0 & 31);
-            uint32_t valid = __ldg(p.ma + word) & __ldg(p.cover + word);
-            if (p.b) valid &= __ldg(p.mb + word);
-            valid = (valid >> off) & (kPer == 32 ? 0xFFFFFFFFu : ((1u << kPer) - 1u));
-            const uint32_t aw[4] = {A.x, A.y, A.z, A.w};
-            uint32_t bw[4] = {0u, 0u, 0u, 0u};
-            if (p.b) {
-                bw[0] = B.x;
-                bw[1] = B.y;
-                bw[2] = B.z;
-                bw[3] = B.w;
-            }
+            const uint32_t valid = (now >> off) & (kPer == 32 ? 0xFFFFFFFFu : ((1u << kPer) - 1u));
             uint32_t rw[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
             for (int k = 0; k < kPer; ++k) {
@@ -362,65 +366,6 @@ __device__ __forceinline__ double key_value(uint32_t k) {
     return (double)k;
 }
 
-// float32 bits -> double, by integer operations for normal numbers and zeros (FP64 throughput
-// on this part is a small fraction of its integer throughput); subnormals and infinities through
-// the conversion instruction.
-__device__ __forceinline__ double f32_bits_to_double(uint32_t b) {
-    const uint32_t e = (b >> 23) & 0xFFu;
-    if (e == 0 || e == 0xFFu) {
-        if ((b & 0x7FFFFFFFu) == 0) return __hiloint2double((int)(b & 0x80000000u), 0);
-        return (double)__uint_as_float(b);
-    }
-    const uint32_t m = b & 0x7FFFFFu;
-    const uint32_t hi = (b & 0x80000000u) | ((e + 896u) << 20) | (m >> 3);
-    return __hiloint2double((int)hi, (int)(m << 29));
-}
-
-// Running sums of one (zone, triangle) stretch: integers and finite float16 values (integer
-// multiples of 2^-24) exactly in int64, float32 values and float16 infinities in double; closed
-// into the zone run as sum += s and wsum += w * s.
-template <int S, int KIND>
-struct TriSum {
-    static constexpr bool kInt = !(KIND == kKindFloat && S == 4);
-    long long i;
-    double d;
-    __device__ __forceinline__ void reset() {
-        i = 0;
-        d = 0.0;
-    }
-    __device__ __forceinline__ double value() const {
-        if (!kInt) return d;
-        if (KIND == kKindFloat) return __dadd_rn(__dmul_rn((double)i, 0x1p-24), d);  // exact: |i| < 2^45; d: infinities
-        return (double)i;                                                             // exact: |i| < 2^37
-    }
-};
-
-struct StatsRun {
-    uint32_t zone;
-    uint32_t cnt;
-    unsigned long long area;
-    uint32_t kmin, kmax;  // value keys (vkey) of the smallest and largest value
-    double sum, wsum;
-};
-
-__device__ __forceinline__ void run_reset(StatsRun &r) {
-    r.cnt = 0;
-    r.area = 0;
-    r.kmin = 0xFFFFFFFFu;
-    r.kmax = 0u;
-    r.sum = 0.0;
-    r.wsum = 0.0;
-}
-
-__device__ __forceinline__ void run_merge(StatsRun &r, const StatsRun &o) {
-    r.cnt += o.cnt;
-    r.area += o.area;
-    r.kmin = min(r.kmin, o.kmin);
-    r.kmax = max(r.kmax, o.kmax);
-    r.sum = __dadd_rn(r.sum, o.sum);
-    r.wsum = __dadd_rn(r.wsum, o.wsum);
-}
-
 __device__ __forceinline__ void acc_add(ZoneAcc *z, unsigned long long cnt, unsigned long long area,
                                         unsigned long long kmin, unsigned long long kmax, double sum, double wsum) {
     atomicAdd(&z->count, cnt);
@@ -431,43 +376,69 @@ __device__ __forceinline__ void acc_add(ZoneAcc *z, unsigned long long cnt, unsi
     atomicAdd(&z->wsum, wsum);
 }
 
-template <int S, int KIND>
-__device__ __forceinline__ void flush_run(const StatsRun &r, ZoneAcc *tab, uint32_t n_zones) {
-    if (r.cnt == 0) return;
-    if (!LCL_IN(r.zone, n_zones)) return;
-    (void)n_zones;
-    acc_add(tab + r.zone, r.cnt, r.area, dkey(key_value<S, KIND>(r.kmin)), dkey(key_value<S, KIND>(r.kmax)), r.sum,
-            r.wsum);
+// x 2^k as a double (two roundings at most: the halves' sum; |k| <= 300).
+__device__ __forceinline__ double i128_to_double(__int128 x, int k) {
+    const bool neg = x < 0;
+    const unsigned __int128 m = neg ? -(unsigned __int128)x : (unsigned __int128)x;
+    const double v = __dadd_rn(__dmul_rn(__ull2double_rn((unsigned long long)(m >> 64)), 18446744073709551616.0),
+                               __ull2double_rn((unsigned long long)m));
+    const double r = __dmul_rn(v, __hiloint2double((1023 + k) << 20, 0));
+    return neg ? -r : r;
 }
 
-// Full-warp reductions (every lane gets the result).
-__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long x) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
+// The sum of v over the warp's lanes, |v| < 2^63: 26-bit pieces whose sums stay below 2^31, the top one
+// signed.
+__device__ __forceinline__ __int128 warp_sum_i64(long long v) {
+    const uint32_t a = __reduce_add_sync(0xffffffffu, (uint32_t)v & 0x3FFFFFFu);
+    const uint32_t b = __reduce_add_sync(0xffffffffu, (uint32_t)(v >> 26) & 0x3FFFFFFu);
+    const int32_t c = __reduce_add_sync(0xffffffffu, (int32_t)(v >> 52));
+    return (__int128)((long long)a + ((long long)b << 26)) + ((__int128)c << 52);
 }
-__device__ __forceinline__ double warp_sum_f64(double x) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) x = __dadd_rn(x, __shfl_xor_sync(0xffffffffu, x, o));
-    return x;
+// A signed 96-bit integer, for the weighted sums.
+struct Int96 {
+    uint32_t w0, w1, w2;
+};
+__device__ __forceinline__ void add96(Int96 &a, uint32_t b0, uint32_t b1, uint32_t b2) {
+    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+        : "+r"(a.w0), "+r"(a.w1), "+r"(a.w2)
+        : "r"(b0), "r"(b1), "r"(b2));
+}
+// Its sum over the warp's lanes, in 26-bit pieces.
+__device__ __forceinline__ __int128 warp_sum_i96(const Int96 &v) {
+    const uint32_t a = __reduce_add_sync(0xffffffffu, v.w0 & 0x3FFFFFFu);
+    const uint32_t b = __reduce_add_sync(0xffffffffu, __funnelshift_r(v.w0, v.w1, 26) & 0x3FFFFFFu);
+    const uint32_t c = __reduce_add_sync(0xffffffffu, __funnelshift_r(v.w1, v.w2, 20) & 0x3FFFFFFu);
+    const int32_t d = __reduce_add_sync(0xffffffffu, (int32_t)v.w2 >> 14);
+    return (__int128)((long long)a + ((long long)b << 26)) + ((__int128)c << 52) + ((__int128)d << 78);
 }
 
-// Adds the runs of the lanes with `take` set (all of one zone) into zone `zone` of `tab`: one warp
-// reduction per field, the atomics by lane `writer`.  Every lane of the warp calls it.
-template <int S, int KIND>
-__device__ __forceinline__ void warp_flush(const StatsRun &r, bool take, uint32_t zone, int writer, ZoneAcc *tab,
-                                           uint32_t n_zones) {
-    const bool t = take && r.cnt;
-    const unsigned long long cnt = warp_sum_u64(t ? r.cnt : 0u);
-    if (cnt == 0) return;  // uniform
-    const unsigned long long area = warp_sum_u64(t ? r.area : 0ull);
-    const uint32_t kmin = __reduce_min_sync(0xffffffffu, t ? r.kmin : 0xFFFFFFFFu);
-    const uint32_t kmax = __reduce_max_sync(0xffffffffu, t ? r.kmax : 0u);
-    const double sum = warp_sum_f64(t ? r.sum : 0.0);
-    const double wsum = warp_sum_f64(t ? r.wsum : 0.0);
-    if ((int)(threadIdx.x & 31) == writer && LCL_IN(zone, n_zones))
-        acc_add(tab + zone, cnt, area, dkey(key_value<S, KIND>(kmin)), dkey(key_value<S, KIND>(kmax)), sum, wsum);
-    (void)n_zones;
+// The exact sums of a run of texels: integers in units of 2^(base - 150), the unit of a float32 whose
+// biased exponent is `base`.  A float32 value (significand m of 24 bits, exponent e) adds m << (e - base)
+// for exponents base .. base + kWindow; integer layers and float16 (multiples of 2^-24) have a fixed
+// unit.  A lane takes at most kRunTexels texels before a flush, so |s| < 2^(24 + kWindow + 10) and the
+// weighted sum (weights below 2^35) < 2^94.
+constexpr int kWindow = 25, kRunTexels = 1024;
+// Steps of a warp at least: a warp's zones and a CTA's table are written out at the end of its work.
+constexpr int kStatsSteps = 4;
+// Times a step lets zones take over runs; a step of more than twice as many zones is noise, whose texels
+// cost less one by one.
+constexpr int kZoneRounds = 3;
+
+struct StatsRun {
+    uint32_t zone;
+    uint32_t cnt, kmin, kmax;  // value keys (vkey) of the smallest and largest value
+    unsigned long long area;
+    long long s;
+    Int96 w;
+};
+
+__device__ __forceinline__ void run_reset(StatsRun &r) {
+    r.cnt = 0;
+    r.area = 0;
+    r.kmin = 0xFFFFFFFFu;
+    r.kmax = 0u;
+    r.s = 0;
+    r.w.w0 = r.w.w1 = r.w.w2 = 0u;
 }
 
 struct StatsArgs {
@@ -478,43 +449,59 @@ struct StatsArgs {
     uint32_t n_labels;
     int64_t n_texels;
     int64_t n_tri;
+    int32_t w4, h;      // quads per row, rows
     ZoneAcc *out;
 };
 
-// Sixteen consecutive S-byte values starting at texel t (t a multiple of 16).
+// Four consecutive S-byte values of a quad.
 template <int S>
-__device__ __forceinline__ void load16(const void *data, int64_t t, uint32_t (&v)[16]) {
-    const uint4 *p = reinterpret_cast<const uint4 *>(static_cast<const uint8_t *>(data) + t * S);
-#pragma unroll
-    for (int q = 0; q < S; ++q) {
-        const uint4 w = __ldcs(p + q);
-        const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if (S == 4) {
-                v[4 * q + j] = ws[j];
-            } else if (S == 2) {
-                v[8 * q + 2 * j] = ws[j] & 0xFFFFu;
-                v[8 * q + 2 * j + 1] = ws[j] >> 16;
-            } else {
-#pragma unroll
-                for (int b = 0; b < 4; ++b) v[16 * q + 4 * j + b] = (ws[j] >> (8 * b)) & 0xFFu;
-            }
+struct Quad4 {
+    uint32_t w[S];
+    __device__ __forceinline__ void load(const void *data, int64_t q) {
+        if constexpr (S == 1) {
+            w[0] = __ldcs(static_cast<const uint32_t *>(data) + q);
+        } else if constexpr (S == 2) {
+            const uint2 v = __ldcs(static_cast<const uint2 *>(data) + q);
+            w[0] = v.x;
+            w[1] = v.y;
+        } else {
+            const uint4 v = __ldcs(static_cast<const uint4 *>(data) + q);
+            w[0] = v.x;
+            w[1] = v.y;
+            w[2] = v.z;
+            w[3] = v.w;
         }
     }
+    __device__ __forceinline__ uint32_t get(int k) const {
+        if (S == 4) return w[k];
+        if (S == 2) return (w[k >> 1] >> (16 * (k & 1))) & 0xFFFFu;
+        return (w[0] >> (8 * k)) & 0xFFu;
+    }
+};
+
+// One texel into the table.
+template <int S, int KIND>
+__device__ __noinline__ void stats_single(ZoneAcc *tab, uint32_t n_zones, uint32_t zone, uint32_t v,
+                                          unsigned long long w) {
+    if (!LCL_IN(zone, n_zones)) return;
+    (void)n_zones;
+    const double d = key_value<S, KIND>(vkey<S, KIND>(v));
+    acc_add(tab + zone, 1ull, w, dkey(d), dkey(d), d, __dmul_rn(__ull2double_rn(w), d));
 }
 
-// Zonal statistics.  A warp takes a contiguous range of iterations; in one iteration lane l takes
-// the 16-texel chunk 32 it + l.  Each lane sums its chunk into a lane run (flushed by itself with
-// atomics only if the zone changes inside the chunk): count, area, min / max as integer keys of
-// the value's own type, and per stretch of texels of one triangle the value sum (exact in int64 for
-// integer and float16 layers, in double for float32) which is closed as sum += s, wsum += w * s.
-// While every lane's chunk run has the warp's current zone, the lane merges it into its share of
-// the warp run, in registers; when an iteration brings another zone, the warp run is reduced
-// across the warp and written by one lane, the iteration's chunk runs are reduced zone by zone,
-// and the zone of lane 31 becomes the warp's zone.
+// Zonal statistics.  A warp walks down a strip of 32 texels, four rows per step, a quad of four texels
+// per lane, the next step's loads issued ahead.  Two zones have a run each, per-lane sums in registers,
+// all integers: count, area, min / max as keys of the value's own type, the values and weight x value.
+// A strip meets few zones, and along a border the same two row after row.  When a step holds a third
+// zone, a run (one that the step does not use, if there is one) is reduced into the table and taken over;
+// what is left after three such rounds goes to the table texel by texel.
+// The sums are rounded only when they go to the table.
+// Bound by instructions.  Summing in binary64 per texel was held by the FP64 pipe (1/64 of the FP32 rate
+// on this part).  8192^2 float32, 40 zones: 862 -> 390 us; strips of 64 or 128 texels, which meet more
+// zones, 470 and 680.
 template <int S, int KIND, int ZB, bool SMEM>
-__global__ void __launch_bounds__(kThreads) k_num_stats(StatsArgs p) {
+__global__ void __launch_bounds__(kThreads, 3) k_num_stats(StatsArgs p) {
+    constexpr bool kF32 = KIND == kKindFloat && S == 4;
     extern __shared__ ZoneAcc sh_zone[];
     ZoneAcc *tab = SMEM ? sh_zone : p.out;
     if (SMEM) {
@@ -528,136 +515,193 @@ __global__ void __launch_bounds__(kThreads) k_num_stats(StatsArgs p) {
         }
         __syncthreads();
     }
-    StatsRun run, wrun;
-    run.zone = kNone;
-    run_reset(run);
-    run_reset(wrun);
-    TriSum<S, KIND> ts_acc;
-    ts_acc.reset();
-    uint32_t last_t = kNone;
-    unsigned long long last_w = 0;
-    bool open = false;  // ts_acc holds texels of triangle last_t in zone run.zone
-    auto close_tri = [&]() {
-        if (!open) return;
-        const double sv = ts_acc.value();
-        run.sum = __dadd_rn(run.sum, sv);
-        run.wsum = __dadd_rn(run.wsum, __dmul_rn((double)last_w, sv));
-        ts_acc.reset();
-        open = false;
-    };
-    auto visit = [&](uint32_t z, uint32_t t, uint32_t bits, bool valid) {
-        if (!valid || t == kNone || z >= p.n_labels) return;
-        uint32_t fb = bits;  // float layers: the float32 bits of the value
-        if (KIND == kKindFloat) {
-            if (S == 2) fb = __float_as_uint(__half2float(__ushort_as_half((unsigned short)bits)));
-            if ((fb & 0x7FFFFFFFu) > 0x7F800000u) return;  // NaN
-            if ((fb & 0x7FFFFFFFu) == 0) fb = 0;           // -0 counts as +0
-        }
-        if (z != run.zone && run.cnt) {
-            close_tri();
-            flush_run<S, KIND>(run, tab, p.n_labels);
-            run_reset(run);
-        }
-        if (!LCL_IN(t, p.n_tri)) return;
-        run.zone = z;
-        if (t != last_t) {
-            close_tri();
-            last_t = t;
-            last_w = __ldg(p.area_w + t);
-        }
-        open = true;
-        run.cnt += 1;
-        run.area += last_w;
-        const uint32_t k = vkey<S, KIND>(fb);
-        run.kmin = min(run.kmin, k);
-        run.kmax = max(run.kmax, k);
-        if (KIND == kKindFloat && S == 4) ts_acc.d = __dadd_rn(ts_acc.d, f32_bits_to_double(fb));
-        else if (KIND == kKindFloat && (fb & 0x7FFFFFFFu) == 0x7F800000u) ts_acc.d = __dadd_rn(ts_acc.d, (double)__uint_as_float(fb));
-        else if (KIND == kKindFloat) ts_acc.i += __float2ll_rn(__fmul_rn(__uint_as_float(fb), 0x1p24f));  // exact
-        else if (KIND == kKindSigned) ts_acc.i += sext<S>(bits);
-        else ts_acc.i += bits;
-    };
     const int lane = threadIdx.x & 31;
-    const int64_t n_chunks = p.n_texels / 16;
-    const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t n_iter = (n_chunks + 31) / 32;
-    const int64_t per = (n_iter + n_warps - 1) / n_warps;
-    const int64_t it0 = warp * per, it1 = min(n_iter, it0 + per);
-    uint32_t wzone = kNone;
-    for (int64_t it = it0; it < it1; ++it) {
-        const int64_t c = it * 32 + lane;
-        if (c < n_chunks && LCL_IN(16 * c + 15, p.n_texels)) {
-            const int64_t t = 16 * c;
-            uint32_t v[16];
-            load16<S>(p.data, t, v);
-            const uint4 *tp = reinterpret_cast<const uint4 *>(p.tri + t);
-            const uint4 T0 = __ldcs(tp), T1 = __ldcs(tp + 1), T2 = __ldcs(tp + 2), T3 = __ldcs(tp + 3);
-            const uint32_t ts[16] = {T0.x, T0.y, T0.z, T0.w, T1.x, T1.y, T1.z, T1.w,
-                                     T2.x, T2.y, T2.z, T2.w, T3.x, T3.y, T3.z, T3.w};
-            uint32_t z[16];
-            if (p.zones) {
-                const uint4 *zp = reinterpret_cast<const uint4 *>(static_cast<const uint8_t *>(p.zones) + t * ZB);
+    // units of kStatsSteps to 32 steps: steps u / n_strips * per and on of strip u % n_strips, so that neighbouring
+    // warps read neighbouring texels, and a warp's units lie apart (borders of zones cost more)
+    constexpr int kCols = 8, kRows = 32 / kCols;  // lanes side by side, rows per step
+    const int32_t n_strips = (p.w4 + kCols - 1) / kCols, n_groups = (p.h + kRows - 1) / kRows;
+    const int32_t n_warps = (int32_t)((gridDim.x * blockDim.x) >> 5);
+    const int32_t warp = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int32_t per = max(kStatsSteps, min(32, (int32_t)((int64_t)n_groups * n_strips / n_warps)));
+    const int32_t n_units = n_strips * ((n_groups + per - 1) / per);
+    const uint32_t ntri = p.n_tri < (int64_t)0xFFFFFFFFu ? (uint32_t)p.n_tri : 0xFFFFFFFFu;
+
+    uint4 T = make_uint4(kNone, kNone, kNone, kNone);
+    Quad4<S> V;
+    Quad4<ZB> Z;
+    uint32_t bits = 0u;
 #pragma unroll
-                for (int q = 0; q < ZB; ++q) {
-                    const uint4 w = __ldcs(zp + q);
-                    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+    for (int k = 0; k < S; ++k) V.w[k] = 0u;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        if (ZB == 1) {
+    for (int k = 0; k < ZB; ++k) Z.w[k] = 0u;
+    auto load = [&](int32_t strip, int32_t group) {
+        const int32_t x = strip * kCols + (lane & (kCols - 1)), y = group * kRows + lane / kCols;
+        const int32_t q = y * p.w4 + x;  // below 2^26
+        bits = 0u;
+        if (x < p.w4 && y < p.h && LCL_IN(4 * (int64_t)q + 3, p.n_texels)) {
+            T = __ldcs(reinterpret_cast<const uint4 *>(p.tri) + q);
+            V.load(p.data, q);
+            if (p.zones) Z.load(p.zones, q);
+            bits = (__ldg(p.mask + (q >> 3)) & __ldg(p.cover + (q >> 3))) >> ((q & 7) * 4);
+        }
+    };
+
+    StatsRun run[2];
+    run_reset(run[0]);
+    run_reset(run[1]);
+    run[0].zone = run[1].zone = kNone;
+    int base = kF32 ? 1 : KIND == kKindFloat ? 126 : 150;  // float32: raised to the values met; others: fixed
+    int since = 0;                                          // steps since the runs were last empty
+    // One run's sums into the table; every lane of the warp calls it.
+    auto flush = [&](StatsRun &r) {
+        const uint32_t cnt = __reduce_add_sync(0xffffffffu, r.cnt);
+        if (cnt) {
+            const __int128 area = warp_sum_i64((long long)r.area);
+            const uint32_t kmin = __reduce_min_sync(0xffffffffu, r.kmin), kmax = __reduce_max_sync(0xffffffffu, r.kmax);
+            const __int128 sum = warp_sum_i64(r.s), wsum = warp_sum_i96(r.w);
+            if (lane == 0 && LCL_IN(r.zone, p.n_labels))
+                acc_add(tab + r.zone, cnt, (unsigned long long)area, dkey(key_value<S, KIND>(kmin)),
+                        dkey(key_value<S, KIND>(kmax)), i128_to_double(sum, base - 150), i128_to_double(wsum, base - 150));
+        }
+        run_reset(r);
+    };
+    for (int32_t u = warp; u < n_units; u += n_warps) {
+    const int32_t strip = u % n_strips, g0 = u / n_strips * per, g1 = min(n_groups, g0 + per);
+    if (g0 < g1) load(strip, g0);
+    for (int32_t g = g0; g < g1; ++g) {
+        const uint32_t ts[4] = {T.x, T.y, T.z, T.w};
+        uint32_t v[4], z[4], ok = 0u;
 #pragma unroll
-                            for (int b = 0; b < 4; ++b) z[4 * j + b] = (ws[j] >> (8 * b)) & 0xFFu;
-                        } else {
-                            z[8 * q + 2 * j] = ws[j] & 0xFFFFu;
-                            z[8 * q + 2 * j + 1] = ws[j] >> 16;
-                        }
+        for (int k = 0; k < 4; ++k) {
+            v[k] = V.get(k);
+            z[k] = p.zones ? Z.get(k) : 0u;
+        }
+        const uint32_t vb = bits;
+        // weights (a texel whose triangle is its left neighbour's shares that one's)
+        unsigned long long w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] = ts[k] < ntri && (k == 0 || ts[k] != ts[k - 1]) ? __ldg(p.area_w + ts[k]) : 0ull;
+        if (g + 1 < g1) load(strip, g + 1);
+        uint32_t emax = 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            bool good = ((vb >> k) & 1u) && ts[k] < ntri && z[k] < p.n_labels;
+            if (KIND == kKindFloat) {
+                if (S == 2) v[k] = __float_as_uint(__half2float(__ushort_as_half((unsigned short)v[k])));
+                const uint32_t mag = v[k] & 0x7FFFFFFFu;
+                good = good && mag <= 0x7F800000u;  // not NaN
+                if (mag == 0u) v[k] = 0u;           // -0 counts as +0
+                if (kF32 && good && mag < 0x7F800000u) emax = max(emax, mag >> 23);
+            }
+            ok |= (good ? 1u : 0u) << k;
+        }
+        const bool above = kF32 && __any_sync(0xffffffffu, (int)emax > base + kWindow);
+        if (above || ++since > kRunTexels / 4) {  // uniform
+            flush(run[0]);
+            flush(run[1]);
+            since = 1;
+            if (above) base = max((int)__reduce_max_sync(0xffffffffu, emax) - 20, 1);
+        }
+#pragma unroll
+        for (int k = 1; k < 4; ++k)
+            if (ts[k] == ts[k - 1]) w[k] = w[k - 1];
+        // adds the texels take0 and take1 to the lane's shares of the two runs (with1: some lane has a take1)
+        auto add = [&](uint32_t take0, uint32_t take1, bool with1) {
+            run[0].cnt += __popc(take0);
+            run[1].cnt += __popc(take1);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const bool t0 = (take0 >> k) & 1u, t1 = (take1 >> k) & 1u;
+                const uint32_t key = vkey<S, KIND>(v[k]);
+                long long f;          // the value in units
+                uint32_t b0, b1, b2;  // weight x value, 96 bits
+                if (KIND == kKindFloat) {
+                    // the value is m 2^sh units
+                    const uint32_t e = (v[k] >> 23) & 0xFFu;
+                    int32_t m = (int32_t)((v[k] & 0x7FFFFFu) | 0x800000u);
+                    int sh = (int)e - base;
+                    if (!kF32 && sh < 0) m >>= min(-sh, 31), sh = 0;  // float16: zeros are shifted out
+                    const bool fits = (uint32_t)sh < 255u - (uint32_t)base;  // else below the window, zero, or infinite
+                    m = (int32_t)v[k] < 0 ? -m : m;
+                    m = fits && (kF32 || v[k] != 0u) ? m : 0;
+                    sh = fits ? sh : 0;
+                    f = (long long)m * (long long)(1 << sh);
+                    // |m w| < 2^59: weight in parts of 30 and 5 bits, so that signed 32-bit products do
+                    const long long pw = (long long)m * (int32_t)((uint32_t)w[k] & 0x3FFFFFFFu) +
+                                         (long long)(m * (int32_t)(w[k] >> 30)) * (1 << 30);
+                    const uint32_t lo = (uint32_t)pw, hi = (uint32_t)(pw >> 32);
+                    b0 = lo << sh;
+                    b1 = __funnelshift_l(lo, hi, sh);
+                    b2 = __funnelshift_l(hi, (uint32_t)((int32_t)hi >> 31), sh);
+                    if ((t0 || t1) && !fits && v[k] != 0u) {  // in binary64, into the table
+                        const double d = (double)__uint_as_float(v[k]);
+                        ZoneAcc &za = tab[t0 ? run[0].zone : run[1].zone];
+                        atomicAdd(&za.sum, d);
+                        atomicAdd(&za.wsum, __dmul_rn(__ull2double_rn(w[k]), d));
+                    }
+                } else {
+                    f = KIND == kKindSigned ? (long long)sext<S>(v[k]) : (long long)v[k];
+                    if (S == 4) {
+                        const __int128 fw = (__int128)f * (long long)w[k];
+                        b0 = (uint32_t)fw;
+                        b1 = (uint32_t)(fw >> 32);
+                        b2 = (uint32_t)(fw >> 64);
+                    } else {
+                        const long long fw = f * (long long)w[k];
+                        b0 = (uint32_t)fw;
+                        b1 = (uint32_t)(fw >> 32);
+                        b2 = (uint32_t)(fw >> 63);
                     }
                 }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) z[k] = 0;
+                auto acc = [&](StatsRun &r, bool t) {
+                    if (!t) return;
+                    r.kmin = min(r.kmin, key);
+                    r.kmax = max(r.kmax, key);
+                    r.area += w[k];
+                    r.s += f;
+                    add96(r.w, b0, b1, b2);
+                };
+                acc(run[0], t0);
+                if (with1) acc(run[1], t1);
             }
-            const uint32_t word = (uint32_t)(t >> 5);
-            const uint32_t valid = (__ldg(p.mask + word) & __ldg(p.cover + word)) >> (t & 31);
+        };
+        uint32_t in0 = 0u, in1 = 0u;
 #pragma unroll
-            for (int k = 0; k < 16; ++k) visit(z[k], ts[k], v[k], (valid >> k) & 1u);
-            close_tri();
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t b = ok & (1u << k);
+            if (z[k] == run[0].zone) in0 |= b;
+            else if (z[k] == run[1].zone) in1 |= b;
         }
-        const uint32_t key = run.cnt ? run.zone : kNone;
-        if (__all_sync(0xffffffffu, key == wzone || key == kNone)) {
-            if (run.cnt) run_merge(wrun, run);
-        } else {
-            warp_flush<S, KIND>(wrun, true, wzone, 0, tab, p.n_labels);
-            run_reset(wrun);
-            // this iteration's chunk runs, zone by zone
-            unsigned left = __ballot_sync(0xffffffffu, key != kNone);
-            while (left) {
-                const int leader = __ffs(left) - 1;
-                const uint32_t zk = __shfl_sync(0xffffffffu, key, leader);
-                const bool mine = key == zk;
-                warp_flush<S, KIND>(run, mine, zk, leader, tab, p.n_labels);
-                left &= ~__ballot_sync(0xffffffffu, mine);
-            }
-            wzone = __shfl_sync(0xffffffffu, key, 31);
+        uint32_t odd = ok & ~(in0 | in1);
+        // a zone not yet among the runs' takes over one that the step does not use (any more)
+        auto take_over = [&](StatsRun &r, uint32_t &in) {
+            const uint32_t bal = __ballot_sync(0xffffffffu, odd != 0u);
+            if (!bal || __any_sync(0xffffffffu, in != 0u)) return;  // uniform
+            uint32_t last = kNone;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if ((odd >> k) & 1u) last = z[k];
+            flush(r);
+            r.zone = __shfl_sync(0xffffffffu, last, 31 - __clz(bal));
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (((odd >> k) & 1u) && z[k] == r.zone) in |= 1u << k;
+            odd &= ~in;
+        };
+        for (int round = 0; round < kZoneRounds; ++round) {
+            take_over(run[0], in0);
+            take_over(run[1], in1);
+            if (__any_sync(0xffffffffu, (in0 | in1) != 0u)) add(in0, in1, __any_sync(0xffffffffu, in1 != 0u));
+            in0 = in1 = 0u;
+            if (!__any_sync(0xffffffffu, odd != 0u)) break;
         }
-        run_reset(run);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)  // zones of a few texels: one by one, the lanes side by side
+            if ((odd >> k) & 1u) stats_single<S, KIND>(tab, p.n_labels, z[k], v[k], w[k]);
     }
-    warp_flush<S, KIND>(wrun, true, wzone, 0, tab, p.n_labels);
-    // tail texels (n_texels % 16), one per thread
-    for (int64_t t = n_chunks * 16 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < p.n_texels;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        if (!LCL_IN(t, p.n_texels)) break;
-        uint32_t bits, z = 0;
-        if (S == 1) bits = static_cast<const uint8_t *>(p.data)[t];
-        else if (S == 2) bits = static_cast<const uint16_t *>(p.data)[t];
-        else bits = static_cast<const uint32_t *>(p.data)[t];
-        if (p.zones) z = ZB == 1 ? static_cast<const uint8_t *>(p.zones)[t] : static_cast<const uint16_t *>(p.zones)[t];
-        const uint32_t word = (uint32_t)(t >> 5);
-        const bool valid = ((p.mask[word] & p.cover[word]) >> (t & 31)) & 1u;
-        visit(z, p.tri[t], bits, valid);
     }
-    close_tri();
-    flush_run<S, KIND>(run, tab, p.n_labels);
+    flush(run[0]);
+    flush(run[1]);
     if (SMEM) {
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < p.n_labels; i += blockDim.x) {
@@ -690,7 +734,7 @@ void launch_stats_smem(const StatsArgs &p, size_t shb, cudaStream_t st) {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, shb) != cudaSuccess || per_sm < 1)
         per_sm = 1;
-    const int64_t threads = p.n_texels / 16 + 1;
+    const int64_t threads = (int64_t)((p.w4 + 7) / 8) * ((p.h + 3) / 4) / kStatsSteps * 32 + 32;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count() * per_sm,
                                                                  (threads + kThreads - 1) / kThreads));
     kernel<<<grid, kThreads, shb, st>>>(p);
@@ -794,6 +838,8 @@ lcl_status numeric_stats_impl(const lcl_atlas *atlas, int type, const void *data
     p.n_labels = n_labels;
     p.n_texels = (int64_t)atlas->width * atlas->height;
     p.n_tri = atlas->n_tri;
+    p.w4 = atlas->width / 4;
+    p.h = atlas->height;
     p.out = reinterpret_cast<ZoneAcc *>(out);
     const unsigned zg = std::max(1u, std::min(1024u, (n_labels + kThreads - 1) / kThreads));
     k_stats_init<<<zg, kThreads, 0, st>>>(p.out, n_labels);
