@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kThreads) k_batch_pairs(const BHdr *__restrict
                 const BLasso &L = lassos[st.lasso];
                 float4 sb;
                 if (box_may_touch(L.arg, lo, hi, L.depth, &sb)) {
-                    const int cls = lasso_tile_class8<1>(L.arg, L.arg.vx, L.arg.vy, sb);
+                    const int cls = lasso_tile_class<1>(L.arg, L.arg.vx, L.arg.vy, sb);
                     hit = cls != kTileOut;
                     sure = cls == kTileIn;
                 }

@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_sphere_step(AtlasDev a, L *__re
 
 // ---- lasso ---------------------------------------------------------------------------
 
-// Super-tiles a lasso (or tool window) can touch: 8 lanes per super-tile (box_may_touch8 without
+// Super-tiles a lasso (or tool window) can touch: 8 lanes per super-tile (box_may_touch_by without
 // the depth map), appended to `list` (counter `counter`).
 __global__ void __launch_bounds__(kThreads) k_lasso_supers(AtlasDev a, const __grid_constant__ LassoArg p,
                                                            uint32_t *counter, uint32_t *list) {
@@ -296,28 +296,32 @@ __global__ void __launch_bounds__(kThreads) k_lasso_supers(AtlasDev a, const __g
     if (sidx < n_super) {  // uniform over each group of 8 lanes
         const int4 *sb = reinterpret_cast<const int4 *>(a.super_box + 8 * sidx);
         const int4 slo = sb[0], shi = sb[1];
-        cand = slo.w > 0 && box_may_touch8(p, slo, shi, nullptr);
+        cand = slo.w > 0 && box_may_touch_by<8>(p, slo, shi, nullptr);
     }
     pdl_wait();  // the counter was reset by the previous grid
     pdl_allow_next();
     append_candidate(cand && (threadIdx.x & 7u) == 0, (uint32_t)sidx, counter, list, n_super);
 }
 
-constexpr int kCullParts = LCL_SUPER * LCL_SUPER / (kThreads / 8);  // 8 parts of 32 tiles per super-tile
-
 // Candidate tiles of a lasso (or tool window) in the super-tiles k_lasso_supers listed: the CTAs take
-// (super-tile, part) units, a part being 32 tiles tested by 8 lanes each (box_may_touch8 with the
-// depth map), so the work spreads over the GPU however few super-tiles the lasso reaches.  FLAGS:
-// write a 0/1 flag per tile instead of appending candidates (first pass of a padded edit; the flags
-// of tiles in other super-tiles were cleared before).  CLASSIFY (lassos): tiles that
-// lasso_tile_class8 finds outside the polygon are dropped, and those it finds inside are listed with
+// (super-tile, part) units, a part being kThreads / G tiles tested by G lanes each (box_may_touch_by
+// with the depth map), so the work spreads over the GPU however few super-tiles the lasso reaches.
+// FLAGS: write a 0/1 flag per tile instead of appending candidates (first pass of a padded edit; the
+// flags of tiles in other super-tiles were cleared before).  CLASSIFY (lassos): tiles that
+// lasso_tile_class finds outside the polygon are dropped, and those it finds inside are listed with
 // kInsideTile set (their texels skip the edge tests).
-template <bool FLAGS, bool CLASSIFY>
+// G: a warp per tile where tiles are few, and so large on the screen: hidden ones have hundreds of
+// pixels to look at (4096^2 chart atlas, 2048^2 map: 26 us per lasso with 8 lanes a tile, each
+// scanning rows of the whole footprint); 8 lanes where there are more than kManyTiles tiles, whose
+// footprints are small.
+constexpr int64_t kManyTiles = 1 << 16;
+template <bool FLAGS, bool CLASSIFY, int G>
 __global__ void __launch_bounds__(kThreads) k_lasso_cull(AtlasDev a, const __grid_constant__ LassoArg p,
                                                          const float *__restrict__ depth,
                                                          const uint32_t *__restrict__ super_count,
                                                          const uint32_t *__restrict__ supers, uint32_t *counter,
                                                          uint32_t *list) {
+    constexpr int kCullParts = LCL_SUPER * LCL_SUPER / (kThreads / G);  // parts of a super-tile
     __shared__ float svx[LCL_MAX_LASSO_VERTICES + 1], svy[LCL_MAX_LASSO_VERTICES + 1];
     if (CLASSIFY) {
         for (int e = threadIdx.x; e <= p.nv; e += blockDim.x) {
@@ -335,25 +339,25 @@ __global__ void __launch_bounds__(kThreads) k_lasso_cull(AtlasDev a, const __gri
         if (!LCL_IN(u / kCullParts, n_super)) break;
         const uint32_t sidx = supers[u / kCullParts];
         const int32_t sx = (int32_t)(sidx % a.supers_x), sy = (int32_t)(sidx / a.supers_x);
-        const int32_t local = (int32_t)(u % kCullParts) * (kThreads / 8) + (int32_t)(threadIdx.x / 8);
+        const int32_t local = (int32_t)(u % kCullParts) * (kThreads / G) + (int32_t)(threadIdx.x / G);
         const int32_t tx = sx * LCL_SUPER + local % LCL_SUPER, ty = sy * LCL_SUPER + local / LCL_SUPER;
-        const bool in_grid = tx < a.tiles_x && ty < a.tiles_y;  // uniform over each group of 8 lanes
+        const bool in_grid = tx < a.tiles_x && ty < a.tiles_y;  // uniform over each group of G lanes
         bool cand = false;
         int cls = kTileTest;
-        // the group's 8 lanes take the same branch (in_grid and the index check are per tile)
+        // the group's lanes take the same branch (in_grid and the index check are per tile)
         if (in_grid && LCL_IN((int64_t)ty * a.tiles_x + tx, n_tiles)) {
             const int4 *tb = reinterpret_cast<const int4 *>(a.tile_box + 8 * ((int64_t)ty * a.tiles_x + tx));
             const int4 lo = tb[0], hi = tb[1];
             if (lo.w > 0) {  // uniform over the group (one tile)
-                if (CLASSIFY) cand = box_may_touch8<true>(p, lo, hi, depth, nullptr, svx, svy, &cls);
-                else cand = box_may_touch8(p, lo, hi, depth);
+                if (CLASSIFY) cand = box_may_touch_by<G, true>(p, lo, hi, depth, nullptr, svx, svy, &cls);
+                else cand = box_may_touch_by<G>(p, lo, hi, depth);
             }
         }
         const uint32_t tile = (uint32_t)(ty * a.tiles_x + tx);
         if (FLAGS) {
-            if (in_grid && (threadIdx.x & 7u) == 0 && LCL_IN(tile, n_tiles)) list[tile] = cand ? 1u : 0u;
+            if (in_grid && (threadIdx.x & (G - 1u)) == 0 && LCL_IN(tile, n_tiles)) list[tile] = cand ? 1u : 0u;
         } else {
-            append_candidate(cand && (threadIdx.x & 7u) == 0, tile | (cls == kTileIn ? kInsideTile : 0u), counter,
+            append_candidate(cand && (threadIdx.x & (G - 1u)) == 0, tile | (cls == kTileIn ? kInsideTile : 0u), counter,
                              list, n_tiles);
         }
     }
@@ -548,29 +552,26 @@ SelWs sel_ws(const lcl_atlas *a, int32_t n, void *ws) {
     return w;
 }
 
-// Launches the cull of a lasso / tool into w.list (counter w.counters[0]); with padding, the flags
-// go to w.list2 first.  Small atlases split each super-tile over up to 8 CTAs so that the grid
-// still covers the GPU.  Returns the number of launches.
-int launch_lasso_cull(const AtlasDev &a, const lcl_atlas *atlas, const LassoArg &p, const float *depth,
-                      const SelWs &w, bool pad, bool classify, cudaStream_t st) {
+// The cull's launches with G lanes per tile (launch_lasso_cull).
+template <int G>
+int launch_lasso_cull_by(const AtlasDev &a, const lcl_atlas *atlas, const LassoArg &p, const float *depth,
+                         const SelWs &w, bool pad, bool classify, cudaStream_t st) {
     // counters[1] and list3 hold the candidate super-tiles (lassos and the tool use list and list2 only)
     const int n_super = atlas->supers_x * atlas->supers_y;
-    const int grid = std::max(1, std::min(n_super * kCullParts, 8 * sm_count()));
+    const int grid = std::max(1, std::min(n_super * (LCL_SUPER * LCL_SUPER / (kThreads / G)), 8 * sm_count()));
+    const uint32_t *const super_count = w.counters + 1, *const supers = w.list3;
     if (!pad && classify) {  // the lasso's chain: each launch a programmatic dependent of the one before
         launch_pdl(k_lasso_supers, dim3((n_super + kThreads / 8 - 1) / (kThreads / 8)), st, a, p, w.counters + 1,
                    w.list3);
-        launch_pdl(k_lasso_cull<false, true>, dim3(grid), st, a, p, depth, (const uint32_t *)(w.counters + 1),
-                   (const uint32_t *)w.list3, w.counters, w.list);
+        launch_pdl(k_lasso_cull<false, true, G>, dim3(grid), st, a, p, depth, super_count, supers, w.counters, w.list);
         return 2;
     }
     k_lasso_supers<<<(n_super + kThreads / 8 - 1) / (kThreads / 8), kThreads, 0, st>>>(a, p, w.counters + 1, w.list3);
     if (!pad) {
         if (classify)
-            k_lasso_cull<false, true><<<grid, kThreads, 0, st>>>(a, p, depth, w.counters + 1, w.list3, w.counters,
-                                                                 w.list);
+            k_lasso_cull<false, true, G><<<grid, kThreads, 0, st>>>(a, p, depth, super_count, supers, w.counters, w.list);
         else
-            k_lasso_cull<false, false><<<grid, kThreads, 0, st>>>(a, p, depth, w.counters + 1, w.list3, w.counters,
-                                                                  w.list);
+            k_lasso_cull<false, false, G><<<grid, kThreads, 0, st>>>(a, p, depth, super_count, supers, w.counters, w.list);
         return 2;
     }
     // padded edits: flags for every tile that may hold a selected texel (polygon-outside tiles of a
@@ -579,13 +580,21 @@ int launch_lasso_cull(const AtlasDev &a, const lcl_atlas *atlas, const LassoArg 
     const int64_t tiles = (int64_t)atlas->tiles_x * atlas->tiles_y;
     cudaMemsetAsync(w.list2, 0, (size_t)tiles * 4, st);
     if (classify)
-        k_lasso_cull<true, true><<<grid, kThreads, 0, st>>>(a, p, depth, w.counters + 1, w.list3, w.counters, w.list2);
+        k_lasso_cull<true, true, G><<<grid, kThreads, 0, st>>>(a, p, depth, super_count, supers, w.counters, w.list2);
     else
-        k_lasso_cull<true, false><<<grid, kThreads, 0, st>>>(a, p, depth, w.counters + 1, w.list3, w.counters,
-                                                             w.list2);
+        k_lasso_cull<true, false, G><<<grid, kThreads, 0, st>>>(a, p, depth, super_count, supers, w.counters, w.list2);
     k_dilate_candidates<<<(unsigned)((tiles + kThreads - 1) / kThreads), kThreads, 0, st>>>(a, w.list2, w.counters,
                                                                                         w.list);
     return 3;
+}
+
+// Launches the cull of a lasso / tool into w.list (counter w.counters[0]); with padding, the flags
+// go to w.list2 first.  Returns the number of launches.
+int launch_lasso_cull(const AtlasDev &a, const lcl_atlas *atlas, const LassoArg &p, const float *depth,
+                      const SelWs &w, bool pad, bool classify, cudaStream_t st) {
+    return (int64_t)atlas->tiles_x * atlas->tiles_y > kManyTiles
+               ? launch_lasso_cull_by<8>(a, atlas, p, depth, w, pad, classify, st)
+               : launch_lasso_cull_by<32>(a, atlas, p, depth, w, pad, classify, st);
 }
 
 // ---- division check ----------------------------------------------------------------------

@@ -377,7 +377,7 @@ __device__ __forceinline__ void stage_lasso(LassoShared &sh, const LassoArg &p) 
 //    minimum over the box is at a corner; if that minimum (less 1e-4 for FP32 rounding) exceeds
 //    the largest depth-map value over the box's widened pixel footprint plus the bias, every texel
 //    of the box fails the depth test.  Footprints above 1024 pixels are not scanned (kept).
-// sbox (optional): as for box_may_touch8.
+// sbox (optional): as for box_may_touch_by.
 __device__ inline bool box_may_touch(const LassoArg &p, int4 lo, int4 hi, const float *__restrict__ depth = nullptr,
                                      float4 *sbox = nullptr) {
     float xmin = INFINITY, xmax = -INFINITY, ymin = INFINITY, ymax = -INFINITY, zmin = INFINITY;
@@ -413,27 +413,50 @@ __device__ inline bool box_may_touch(const LassoArg &p, int4 lo, int4 hi, const 
 }
 
 
-// box_may_touch evaluated by an aligned group of 8 lanes for one box (all 8 call it with the same
-// box): lane c projects corner c, the group reduces the screen box and the nearest depth, and the
-// depth-footprint scan is split by rows over the group.  The tests of box_may_touch, with
-// footprints of up to 2048 px scanned (1024 there) before the test gives up and keeps the box.
+// box_may_touch evaluated by an aligned group of G lanes (8 or 32) for one box (all of them call it with
+// the same box): lane c projects corner c mod 8, and the depth footprint is shared out over the group.
+// The tests of box_may_touch, with footprints of up to 2048 px scanned (1024 there) before the test
+// gives up and keeps the box.  The scan looks for a pixel that the box's nearest corner does not lie
+// behind -- max(d) + bias >= z exactly if some d + bias >= z, rounding being monotone -- and stops
+// at the first group of pixels that holds one: visible boxes take one step, hidden ones all.
 // sbox (optional): the screen box {xmin, xmax, ymin, ymax} of the projected corners when every
 // corner lies in front of the camera and projects to finite coordinates, else NaNs.
-// Tile classes for a lasso (the texels of a box projected to screen box `sb`, by box_may_touch8).
+// Tile classes for a lasso (the texels of a box projected to screen box `sb`).
 enum : int { kTileOut = 0, kTileTest = 1, kTileIn = 2 };
 
 template <int LANES>
-__device__ __forceinline__ int lasso_tile_class8(const LassoArg &p, const float *vx, const float *vy, float4 sb);
+__device__ __forceinline__ int lasso_tile_class(const LassoArg &p, const float *vx, const float *vy, float4 sb);
+
+// Some pixel of [ix0, ix1] x [iy0, iy1] with depth + bias >= z?  Every lane of the group calls it.
+template <int G>
+__device__ __forceinline__ bool depth_reaches(const LassoArg &p, const float *__restrict__ depth, int ix0, int ix1,
+                                              int iy0, int iy1, float z, unsigned gm) {
+    constexpr int kX = 8, kY = G / 8;  // the group's pixels: 8 side by side, kY rows
+    const int sub = (int)(threadIdx.x & (G - 1u));
+    for (int y = iy0; y <= iy1; y += 2 * kY)
+        for (int x = ix0; x <= ix1; x += 4 * kX) {
+            bool any = false;
+            // eight independent loads; places beyond the edge repeat the last pixel
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int ix = min(x + (sub & 7) + kX * (j & 3), ix1), iy = min(y + (sub >> 3) + kY * (j >> 2), iy1);
+                if (LCL_IN((int64_t)iy * p.w_s + ix, (int64_t)p.w_s * p.h_s))
+                    any |= __ldg(depth + (int64_t)iy * p.w_s + ix) + p.bias >= z;
+            }
+            if (__any_sync(gm, any)) return true;
+        }
+    return false;
+}
 
 // CLASSIFY (with vx, vy, *cls): between the screen-box test and the depth-footprint scan, the tile is
-// classified by lasso_tile_class8 (its class in *cls, kTileTest where it cannot be); a tile outside the
+// classified by lasso_tile_class (its class in *cls, kTileTest where it cannot be); a tile outside the
 // polygon returns false at once, without the scan.
-template <bool CLASSIFY = false>
-__device__ __forceinline__ bool box_may_touch8(const LassoArg &p, int4 lo, int4 hi, const float *__restrict__ depth,
-                                               float4 *sbox = nullptr, const float *vx = nullptr,
-                                               const float *vy = nullptr, int *cls = nullptr) {
+template <int G, bool CLASSIFY = false>
+__device__ __forceinline__ bool box_may_touch_by(const LassoArg &p, int4 lo, int4 hi, const float *__restrict__ depth,
+                                                 float4 *sbox = nullptr, const float *vx = nullptr,
+                                                 const float *vy = nullptr, int *cls = nullptr) {
     const unsigned lane = threadIdx.x & 31u, sub = lane & 7u;
-    const unsigned gm = 0xFFu << (lane & 24u);
+    const unsigned gm = G == 32 ? 0xFFFFFFFFu : 0xFFu << (lane & 24u);
     const float x = (float)((sub & 1u) ? hi.x : lo.x), y = (float)((sub & 2u) ? hi.y : lo.y);
     const float z = (float)((sub & 4u) ? hi.z : lo.z);
     const float cw = clip_row(p.m + 12, x, y, z);
@@ -456,7 +479,7 @@ __device__ __forceinline__ bool box_may_touch8(const LassoArg &p, int4 lo, int4 
     if (xmax < p.bx0 || xmin > p.bx1 || ymax < p.by0 || ymin > p.by1) return false;
     if (sbox && finite) *sbox = make_float4(xmin, xmax, ymin, ymax);
     if (CLASSIFY) {
-        *cls = finite ? lasso_tile_class8<8>(p, vx, vy, make_float4(xmin, xmax, ymin, ymax)) : kTileTest;
+        *cls = finite ? lasso_tile_class<G>(p, vx, vy, make_float4(xmin, xmax, ymin, ymax)) : kTileTest;
         if (*cls == kTileOut) return false;  // outside the polygon: no texel can be selected
     }
     if (!depth) return true;
@@ -465,18 +488,14 @@ __device__ __forceinline__ bool box_may_touch8(const LassoArg &p, int4 lo, int4 
     const int iy0 = max(0, __float2int_rd(ymin - margin)), iy1 = min(p.h_s - 1, __float2int_rd(ymax + margin));
     if (ix0 > ix1 || iy0 > iy1) return false;  // the whole footprint is off screen
     if ((ix1 - ix0 + 1) * (iy1 - iy0 + 1) > 2048) return true;
-    float dmax = -INFINITY;
-    for (int iy = iy0 + (int)sub; iy <= iy1; iy += 8)
-        for (int ix = ix0; ix <= ix1; ++ix)
-            if (LCL_IN((int64_t)iy * p.w_s + ix, (int64_t)p.w_s * p.h_s))
-                dmax = fmaxf(dmax, __ldg(depth + (int64_t)iy * p.w_s + ix));
-    for (int o = 1; o < 8; o <<= 1) dmax = fmaxf(dmax, __shfl_xor_sync(gm, dmax, o));
-    return !(zmin - 1e-4f > dmax + p.bias);
+    // NaN depths never count, as in a maximum; a NaN zmin keeps the box
+    const float near = zmin - 1e-4f;
+    return !(near == near) || depth_reaches<G>(p, depth, ix0, ix1, iy0, iy1, near, gm);
 }
 
 
-// Classifies a box whose projection lies in the screen box sb, by the aligned group of 8 lanes of
-// box_may_touch8 (all 8 call it; lane c takes edges c, c + 8, ...):
+// Classifies a box whose projection lies in the screen box sb, by the aligned group of LANES lanes of
+// box_may_touch_by (all of them call it; lane c takes edges c, c + LANES, ...):
 //   kTileOut   no edge of the polygon comes near the box and its centre is outside: no texel of the
 //              box is inside (the tile is dropped);
 //   kTileIn    no edge comes near the box, its centre is inside and the box lies on screen: every
@@ -490,12 +509,12 @@ __device__ __forceinline__ bool box_may_touch8(const LassoArg &p, int4 lo, int4 
 // same at every point of a region no edge meets -- the parity at the centre.  The segment-box test is
 // conservative: an FP32 side value whose magnitude is within its error bound counts as meeting.
 // vx, vy: the polygon's vertices (vertex nv = vertex 0), staged in shared memory by the caller so
-// that the lanes' different edges are not serialised on the parameter bank.  LANES: 8 (an aligned
-// group of 8 lanes shares the work, as after box_may_touch8) or 1 (one thread does it alone).
+// that the lanes' different edges are not serialised on the parameter bank.  LANES = 1: one thread
+// does it alone.
 template <int LANES>
-__device__ __forceinline__ int lasso_tile_class8(const LassoArg &p, const float *vx, const float *vy, float4 sb) {
-    const unsigned lane = threadIdx.x & 31u, sub = LANES == 8 ? (lane & 7u) : 0u;
-    const unsigned gm = 0xFFu << (lane & 24u);
+__device__ __forceinline__ int lasso_tile_class(const LassoArg &p, const float *vx, const float *vy, float4 sb) {
+    const unsigned lane = threadIdx.x & 31u, sub = lane & (LANES - 1u);
+    const unsigned gm = LANES == 32 ? 0xFFFFFFFFu : 0xFFu << (lane & 24u);
     if (!(isfinite(sb.x) && isfinite(sb.y) && isfinite(sb.z) && isfinite(sb.w))) return kTileTest;  // uniform
     const float m = 1.0f;
     const float x0 = sb.x - m, x1 = sb.y + m, y0 = sb.z - m, y1 = sb.w + m;
@@ -565,7 +584,7 @@ __device__ __forceinline__ bool quot_le(float a, float b, float t) {
 //    rounding is far below the 2-pixel margin;
 //  - only edges listed for the point's y-band are tested: an edge can count only if its y-range
 //    contains y, and each band lists every edge whose y-range comes within a margin of the band.
-// INSIDE: the texel's tile is known to lie inside the polygon (lasso_tile_class8): the edge tests,
+// INSIDE: the texel's tile is known to lie inside the polygon (lasso_tile_class): the edge tests,
 // whose outcome would be "inside", are skipped.
 template <bool INSIDE = false, typename Edges>
 __device__ __forceinline__ bool lasso_hit(const LassoArg &p, const Edges &sh, const float *__restrict__ depth,
@@ -633,7 +652,7 @@ constexpr uint32_t kInsideTile = 0x80000000u;
 // lasso_hit up to its band; when the quad's live texels share a band (nearly always: they are
 // neighbours on the surface) one pass over that band's edge records tests all of them.  Texels
 // that failed a step carry ys = NaN, which straddles no edge.  INSIDE: the quad's tile is known to
-// lie inside the polygon (lasso_tile_class8), so the edge tests are skipped: their outcome for
+// lie inside the polygon (lasso_tile_class), so the edge tests are skipped: their outcome for
 // every texel that reaches them is "inside".
 template <bool INSIDE>
 __device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const LassoShared &sh,
