@@ -146,10 +146,9 @@ __device__ __forceinline__ bool stroke_may_reach(const BStroke &st, const BLasso
 constexpr int kPrepWarps = kThreads / 32;  // lassos per CTA of k_batch_prep
 static_assert(kBands == 32, "k_batch_prep gives each y-band one lane");
 
-// Resets the work counters and the tile masks and builds every lasso's argument, one warp per
-// lasso: lane 0 the
-// head (bounding boxes, band mapping), then lane b counts and lists the edges of band b (the
-// same predicate, in the same edge order, as the host builder).
+// Resets the work counters and the tile masks and builds every lasso's argument, one warp per lasso:
+// the lanes copy the vertices and reduce their bounding box, then lane b counts and lists the edges of
+// band b (the same predicate, in the same edge order, as the host builder).
 __global__ void __launch_bounds__(kThreads) k_batch_prep(BHdr *hdr, const BLassoIn *__restrict__ in,
                                                          BLasso *__restrict__ out, ulonglong2 *__restrict__ tmask,
                                                          BCaps caps) {
@@ -161,24 +160,45 @@ __global__ void __launch_bounds__(kThreads) k_batch_prep(BHdr *hdr, const BLasso
     const int64_t n_tiles = hdr->n_tiles;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n_tiles; t += (int64_t)gridDim.x * blockDim.x)
         if (LCL_IN(t, caps.tiles)) tmask[t] = make_ulonglong2(0ull, 0ull);
+    __shared__ LassoArg s_arg[kPrepWarps];
     const int lane = threadIdx.x & 31;
     const int j = blockIdx.x * kPrepWarps + (int)(threadIdx.x / 32);
     if (j >= hdr->n_lassos) return;  // uniform over the warp
     if (!LCL_IN(j, caps.lassos)) return;
     (void)caps;
     const BLassoIn &L = in[j];
-    LassoArg &p = out[j].arg;
+    LassoArg &p = s_arg[threadIdx.x / 32];
+    const int nv = L.nv;
+    float x0 = INFINITY, x1 = -INFINITY, y0 = INFINITY, y1 = -INFINITY;
+    for (int i = lane; i <= LCL_MAX_LASSO_VERTICES; i += 32) {  // vertices nv and on repeat vertex 0
+        const float2 v = *reinterpret_cast<const float2 *>(L.poly + 2 * (i < nv ? i : 0));
+        p.vx[i] = v.x;
+        p.vy[i] = v.y;
+        x0 = fminf(x0, v.x);
+        x1 = fmaxf(x1, v.x);
+        y0 = fminf(y0, v.y);
+        y1 = fmaxf(y1, v.y);
+    }
+    for (int o = 16; o; o >>= 1) {
+        x0 = fminf(x0, __shfl_xor_sync(0xffffffffu, x0, o));
+        x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, o));
+        y0 = fminf(y0, __shfl_xor_sync(0xffffffffu, y0, o));
+        y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, o));
+    }
+    if (lane < 16) p.m[lane] = L.m[lane];
     if (lane == 0) {
-        lasso_arg_head(p, L.m, L.w_s, L.h_s, L.poly, L.nv, L.label, L.bias);
+        lasso_arg_scalars(p, L.w_s, L.h_s, nv, L.label, L.bias);
+        lasso_arg_box(p, x0, x1, y0, y1);
         out[j].depth = L.depth;
         out[j].pad_r = (int32_t)(L.flags & 15u);
         out[j].pad_t = (int32_t)((L.flags >> 4) & 15u);
     }
     __syncwarp();
-    const double bh = lasso_band_height(p);
-    const int nv = p.nv;
-    int c = 0;
-    for (int e = 0; e < nv; ++e) c += lasso_band_has(p, lane, e, bh) ? 1 : 0;
+    const float bh = lasso_band_height(p);
+    unsigned long long has = 0ull;  // edges of band `lane`
+    for (int e = 0; e < nv; ++e)
+        if (lasso_band_has(p, lane, e, bh)) has |= 1ull << e;
+    const int c = __popcll(has);
     int incl = c;
     for (int o = 1; o < 32; o <<= 1) {
         const int t = __shfl_up_sync(0xffffffffu, incl, o);
@@ -187,15 +207,20 @@ __global__ void __launch_bounds__(kThreads) k_batch_prep(BHdr *hdr, const BLasso
     int k = incl - c;
     p.band_off[lane] = (uint16_t)k;
     if (lane == 31) p.band_off[kBands] = (uint16_t)incl;
-    for (int e = 0; e < nv; ++e)
-        if (lasso_band_has(p, lane, e, bh)) p.band_edge[k++] = (uint8_t)e;
+    for (; has; has &= has - 1) p.band_edge[k++] = (uint8_t)(__ffsll((long long)has) - 1);
+    __syncwarp();
+    static_assert(sizeof(LassoArg) % 4 == 0, "LassoArg is copied by words");
+    for (int i = lane; i < (int)(sizeof(LassoArg) / 4); i += 32)
+        reinterpret_cast<uint32_t *>(&out[j].arg)[i] = reinterpret_cast<const uint32_t *>(&p)[i];
 }
 
 // Masks of one (super-tile, stroke) unit: unit u is super-tile u / 64 of the batch and stroke u % 64
-// of its model, so the tile tests of one super-tile and all its strokes run in parallel (a thread
-// per tile, a CTA per unit) rather than one after another in one thread.  A stroke whose test can
-// reach the super-tile tests each of its 256 tiles and ORs its bit into the tile's mask (and, for an
-// exact class, into `sure`).
+// of its model, so the tile tests of one super-tile and all its strokes run in parallel rather than
+// one after another in one thread.  A stroke whose test can reach the super-tile tests each of its 256
+// tiles and ORs its bit into the tile's mask (and, for an exact class, into `sure`): a sphere with a
+// thread per tile, a lasso with 8 lanes per tile (its eight corners, its edges and the depth footprint
+// shared out; one thread doing all of it took 8x as long), a padded stroke, whose tiles look at their
+// neighbours, with a thread per tile.
 __global__ void __launch_bounds__(kThreads) k_batch_pairs(const BHdr *__restrict__ hdr,
                                                           const BModel *__restrict__ models,
                                                           const BStroke *__restrict__ strokes,
@@ -219,38 +244,55 @@ __global__ void __launch_bounds__(kThreads) k_batch_pairs(const BHdr *__restrict
         if (!LCL_IN(sidx, (int64_t)a.supers_x * a.supers_y)) continue;
         const int32_t sx = sidx % a.supers_x, sy = sidx / a.supers_x;
         const BStroke &st = strokes[M.s0 + k];
+        const bool pads = stroke_pads(st, lassos), by_lanes = !pads && st.kind == LCL_STROKE_LASSO;
         __syncthreads();  // s_reach of the previous unit has been read
-        if (threadIdx.x == 0) s_reach = stroke_may_reach(st, lassos, a.super_box, a.supers_x, a.supers_y, sx, sy);
+        if (by_lanes) {
+            if (threadIdx.x < 32) {
+                const int4 *b = reinterpret_cast<const int4 *>(a.super_box + 8 * (int64_t)sidx);
+                const int4 lo = b[0], hi = b[1];
+                const bool reach = lo.w > 0 && box_may_touch_by<32>(lassos[st.lasso].arg, lo, hi, lassos[st.lasso].depth);
+                if (threadIdx.x == 0) s_reach = reach;
+            }
+        } else if (threadIdx.x == 0) {
+            s_reach = stroke_may_reach(st, lassos, a.super_box, a.supers_x, a.supers_y, sx, sy);
+        }
         __syncthreads();
         if (!s_reach) continue;
+        const int64_t n_tiles = (int64_t)a.tiles_x * a.tiles_y;
+        (void)n_tiles;
+        auto mark = [&](int64_t tile, bool sure) {
+            if (!LCL_IN(M.tile0 + tile, caps.tiles)) return;
+            atomicOr(&tmask[M.tile0 + tile].x, 1ull << k);
+            if (sure) atomicOr(&tmask[M.tile0 + tile].y, 1ull << k);
+        };
+        if (by_lanes) {
+            const BLasso &L = lassos[st.lasso];
+            for (int32_t i = threadIdx.x / 8; i < LCL_SUPER * LCL_SUPER; i += kThreads / 8) {
+                const int32_t tx = sx * LCL_SUPER + i % LCL_SUPER, ty = sy * LCL_SUPER + i / LCL_SUPER;
+                if (tx >= a.tiles_x || ty >= a.tiles_y) continue;  // uniform over the 8 lanes, as below
+                const int64_t tile = (int64_t)ty * a.tiles_x + tx;
+                if (!LCL_IN(tile, n_tiles)) continue;
+                const int4 *b = reinterpret_cast<const int4 *>(a.tile_box + 8 * tile);
+                const int4 lo = b[0], hi = b[1];
+                if (lo.w == 0) continue;
+                int cls = kTileTest;
+                const bool hit = box_may_touch_by<8, true>(L.arg, lo, hi, L.depth, L.arg.vx, L.arg.vy, &cls);
+                if (hit && (threadIdx.x & 7u) == 0) mark(tile, cls == kTileIn);
+            }
+            continue;
+        }
         const int32_t tx = sx * LCL_SUPER + (threadIdx.x % LCL_SUPER);
         const int32_t ty = sy * LCL_SUPER + (threadIdx.x / LCL_SUPER);
         if (tx >= a.tiles_x || ty >= a.tiles_y) continue;
         const int64_t tile = (int64_t)ty * a.tiles_x + tx;
-        bool hit = false, sure = false;
-        if (!stroke_pads(st, lassos) && LCL_IN(tile, (int64_t)a.tiles_x * a.tiles_y)) {
-            // unpadded: the tile's own box decides, with its exact class
+        if (!LCL_IN(tile, n_tiles)) continue;
+        if (pads) {
+            if (stroke_may_reach(st, lassos, a.tile_box, a.tiles_x, a.tiles_y, tx, ty)) mark(tile, false);
+        } else {
             const int4 *b = reinterpret_cast<const int4 *>(a.tile_box + 8 * tile);
             const int4 lo = b[0], hi = b[1];
-            if (lo.w == 0) continue;
-            if (st.kind == LCL_STROKE_SPHERE) {
-                hit = box_dist2(lo, hi, st.sphere) <= st.sphere.r2;
-                sure = hit && box_far2(lo, hi, st.sphere) <= st.sphere.r2;
-            } else {
-                const BLasso &L = lassos[st.lasso];
-                float4 sb;
-                if (box_may_touch(L.arg, lo, hi, L.depth, &sb)) {
-                    const int cls = lasso_tile_class<1>(L.arg, L.arg.vx, L.arg.vy, sb);
-                    hit = cls != kTileOut;
-                    sure = cls == kTileIn;
-                }
-            }
-        } else {
-            hit = stroke_may_reach(st, lassos, a.tile_box, a.tiles_x, a.tiles_y, tx, ty);
-        }
-        if (hit && LCL_IN(M.tile0 + tile, caps.tiles)) {
-            atomicOr(&tmask[M.tile0 + tile].x, 1ull << k);
-            if (sure) atomicOr(&tmask[M.tile0 + tile].y, 1ull << k);
+            if (lo.w > 0 && box_dist2(lo, hi, st.sphere) <= st.sphere.r2)
+                mark(tile, box_far2(lo, hi, st.sphere) <= st.sphere.r2);
         }
     }
 }

@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(kThreads) k_lasso_cull(AtlasDev a, const __gri
             const int4 *tb = reinterpret_cast<const int4 *>(a.tile_box + 8 * ((int64_t)ty * a.tiles_x + tx));
             const int4 lo = tb[0], hi = tb[1];
             if (lo.w > 0) {  // uniform over the group (one tile)
-                if (CLASSIFY) cand = box_may_touch_by<G, true>(p, lo, hi, depth, nullptr, svx, svy, &cls);
+                if (CLASSIFY) cand = box_may_touch_by<G, true>(p, lo, hi, depth, svx, svy, &cls);
                 else cand = box_may_touch_by<G>(p, lo, hi, depth);
             }
         }

@@ -377,12 +377,8 @@ __device__ __forceinline__ void stage_lasso(LassoShared &sh, const LassoArg &p) 
 //    minimum over the box is at a corner; if that minimum (less 1e-4 for FP32 rounding) exceeds
 //    the largest depth-map value over the box's widened pixel footprint plus the bias, every texel
 //    of the box fails the depth test.  Footprints above 1024 pixels are not scanned (kept).
-// sbox (optional): as for box_may_touch_by.
-__device__ inline bool box_may_touch(const LassoArg &p, int4 lo, int4 hi, const float *__restrict__ depth = nullptr,
-                                     float4 *sbox = nullptr) {
+__device__ inline bool box_may_touch(const LassoArg &p, int4 lo, int4 hi, const float *__restrict__ depth = nullptr) {
     float xmin = INFINITY, xmax = -INFINITY, ymin = INFINITY, ymax = -INFINITY, zmin = INFINITY;
-    bool finite = true;
-    if (sbox) *sbox = make_float4(NAN, NAN, NAN, NAN);
 #pragma unroll 1
     for (int c = 0; c < 8; ++c) {
         float x = (float)((c & 1) ? hi.x : lo.x), y = (float)((c & 2) ? hi.y : lo.y), z = (float)((c & 4) ? hi.z : lo.z);
@@ -390,14 +386,12 @@ __device__ inline bool box_may_touch(const LassoArg &p, int4 lo, int4 hi, const 
         if (!(cw > 0.0f)) return true;
         float xs = screen_of(div_rn(clip_row(p.m, x, y, z), cw), p.ws);
         float ys = screen_of(div_rn(clip_row(p.m + 4, x, y, z), cw), p.hs);
-        finite = finite && isfinite(xs) && isfinite(ys);
         float zn = div_rn(clip_row(p.m + 8, x, y, z), cw);
         xmin = fminf(xmin, xs); xmax = fmaxf(xmax, xs);
         ymin = fminf(ymin, ys); ymax = fmaxf(ymax, ys);
         zmin = fminf(zmin, zn);
     }
     if (xmax < p.bx0 || xmin > p.bx1 || ymax < p.by0 || ymin > p.by1) return false;
-    if (sbox && finite) *sbox = make_float4(xmin, xmax, ymin, ymax);
     if (!depth) return true;
     const float margin = 2.0f;
     const int ix0 = max(0, __float2int_rd(xmin - margin)), ix1 = min(p.w_s - 1, __float2int_rd(xmax + margin));
@@ -419,8 +413,6 @@ __device__ inline bool box_may_touch(const LassoArg &p, int4 lo, int4 hi, const 
 // gives up and keeps the box.  The scan looks for a pixel that the box's nearest corner does not lie
 // behind -- max(d) + bias >= z exactly if some d + bias >= z, rounding being monotone -- and stops
 // at the first group of pixels that holds one: visible boxes take one step, hidden ones all.
-// sbox (optional): the screen box {xmin, xmax, ymin, ymax} of the projected corners when every
-// corner lies in front of the camera and projects to finite coordinates, else NaNs.
 // Tile classes for a lasso (the texels of a box projected to screen box `sb`).
 enum : int { kTileOut = 0, kTileTest = 1, kTileIn = 2 };
 
@@ -453,19 +445,18 @@ __device__ __forceinline__ bool depth_reaches(const LassoArg &p, const float *__
 // polygon returns false at once, without the scan.
 template <int G, bool CLASSIFY = false>
 __device__ __forceinline__ bool box_may_touch_by(const LassoArg &p, int4 lo, int4 hi, const float *__restrict__ depth,
-                                                 float4 *sbox = nullptr, const float *vx = nullptr,
-                                                 const float *vy = nullptr, int *cls = nullptr) {
+                                                 const float *vx = nullptr, const float *vy = nullptr,
+                                                 int *cls = nullptr) {
     const unsigned lane = threadIdx.x & 31u, sub = lane & 7u;
     const unsigned gm = G == 32 ? 0xFFFFFFFFu : 0xFFu << (lane & 24u);
     const float x = (float)((sub & 1u) ? hi.x : lo.x), y = (float)((sub & 2u) ? hi.y : lo.y);
     const float z = (float)((sub & 4u) ? hi.z : lo.z);
     const float cw = clip_row(p.m + 12, x, y, z);
-    if (sbox) *sbox = make_float4(NAN, NAN, NAN, NAN);
     if (__any_sync(gm, !(cw > 0.0f))) return true;
     // each lane folds its corner into empty bounds exactly as the serial loop does (NaN ignored)
     const float xs = screen_of(div_rn(clip_row(p.m, x, y, z), cw), p.ws);
     const float ys = screen_of(div_rn(clip_row(p.m + 4, x, y, z), cw), p.hs);
-    const bool finite = __all_sync(gm, isfinite(xs) && isfinite(ys));
+    const bool finite = !CLASSIFY || __all_sync(gm, isfinite(xs) && isfinite(ys));
     float xmin = fminf(INFINITY, xs), xmax = fmaxf(-INFINITY, xs);
     float ymin = fminf(INFINITY, ys), ymax = fmaxf(-INFINITY, ys);
     float zmin = fminf(INFINITY, div_rn(clip_row(p.m + 8, x, y, z), cw));
@@ -477,7 +468,6 @@ __device__ __forceinline__ bool box_may_touch_by(const LassoArg &p, int4 lo, int
         zmin = fminf(zmin, __shfl_xor_sync(gm, zmin, o));
     }
     if (xmax < p.bx0 || xmin > p.bx1 || ymax < p.by0 || ymin > p.by1) return false;
-    if (sbox && finite) *sbox = make_float4(xmin, xmax, ymin, ymax);
     if (CLASSIFY) {
         *cls = finite ? lasso_tile_class<G>(p, vx, vy, make_float4(xmin, xmax, ymin, ymax)) : kTileTest;
         if (*cls == kTileOut) return false;  // outside the polygon: no texel can be selected
@@ -509,8 +499,7 @@ __device__ __forceinline__ bool box_may_touch_by(const LassoArg &p, int4 lo, int
 // same at every point of a region no edge meets -- the parity at the centre.  The segment-box test is
 // conservative: an FP32 side value whose magnitude is within its error bound counts as meeting.
 // vx, vy: the polygon's vertices (vertex nv = vertex 0), staged in shared memory by the caller so
-// that the lanes' different edges are not serialised on the parameter bank.  LANES = 1: one thread
-// does it alone.
+// that the lanes' different edges are not serialised on the parameter bank.
 template <int LANES>
 __device__ __forceinline__ int lasso_tile_class(const LassoArg &p, const float *vx, const float *vy, float4 sb) {
     const unsigned lane = threadIdx.x & 31u, sub = lane & (LANES - 1u);
@@ -597,8 +586,9 @@ __device__ __forceinline__ bool lasso_hit(const LassoArg &p, const Edges &sh, co
     if (cx < __fmul_rn(p.nx0, cw) || cx > __fmul_rn(p.nx1, cw)) return false;
     const float cy = clip_row(p.m + 4, fx, fy, fz);
     if (cy < __fmul_rn(p.ny0, cw) || cy > __fmul_rn(p.ny1, cw)) return false;
-    const float xs = screen_of(div_rn(cx, cw), p.ws);
-    const float ys = screen_of(div_rn(cy, cw), p.hs);
+    const Divisor dw = divisor(cw);
+    const float xs = screen_of(div_by(cx, dw), p.ws);
+    const float ys = screen_of(div_by(cy, dw), p.hs);
     if (!(xs >= 0.0f && xs < p.ws && ys >= 0.0f && ys < p.hs)) return false;
     if (!(ys >= p.ymin && ys < p.ymax)) return false;  // no edge straddles y
     int band = __float2int_rz(__fmul_rn(__fsub_rn(ys, p.band_y0), p.band_inv_h));
@@ -675,8 +665,9 @@ __device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const LassoSha
         if (!INSIDE && (cx < __fmul_rn(p.nx0, w) || cx > __fmul_rn(p.nx1, w))) continue;
         const float cy = clip_row(p.m + 4, fx, fy, fz);
         if (!INSIDE && (cy < __fmul_rn(p.ny0, w) || cy > __fmul_rn(p.ny1, w))) continue;
-        const float x = screen_of(div_rn(cx, w), p.ws);
-        const float y = screen_of(div_rn(cy, w), p.hs);
+        const Divisor dw = divisor(w);
+        const float x = screen_of(div_by(cx, dw), p.ws);
+        const float y = screen_of(div_by(cy, dw), p.hs);
         // INSIDE: the tile's class already settles the viewport, the polygon's box and its y-range
         // (the projected box widened by the margin lies on screen and inside the polygon)
         if (!INSIDE && !(x >= 0.0f && x < p.ws && y >= 0.0f && y < p.hs)) continue;
@@ -754,8 +745,9 @@ __device__ __forceinline__ bool tool_hit(const LassoArg &p, const ToolArg &t, co
     if (cx < __fmul_rn(p.nx0, cw) || cx > __fmul_rn(p.nx1, cw)) return false;
     const float cy = clip_row(p.m + 4, fx, fy, fz);
     if (cy < __fmul_rn(p.ny0, cw) || cy > __fmul_rn(p.ny1, cw)) return false;
-    const float xs = screen_of(div_rn(cx, cw), p.ws);
-    const float ys = screen_of(div_rn(cy, cw), p.hs);
+    const Divisor dw = divisor(cw);
+    const float xs = screen_of(div_by(cx, dw), p.ws);
+    const float ys = screen_of(div_by(cy, dw), p.hs);
     if (!(xs >= 0.0f && xs < p.ws && ys >= 0.0f && ys < p.hs)) return false;
     if (MASK) {
         const float fu = __fmul_rn(__fsub_rn(xs, t.x0), t.su), fv = __fmul_rn(__fsub_rn(ys, t.y0), t.sv);
@@ -792,16 +784,15 @@ inline int resident_grid(K kernel) {
 
 
 // y-bands of edges: band b lists the edges whose y-range comes within `slack` of it, in edge order.
-__host__ __device__ inline double lasso_band_height(const LassoArg &p) {
-    return fmax((double)p.ymax - (double)p.ymin, 1e-3) / kBands;
+// The slack is far above the rounding of a point's band (floor((y - band_y0) * band_inv_h), a few ulps)
+// and of the bounds below; an edge too many in a band changes nothing.
+__host__ __device__ inline float lasso_band_height(const LassoArg &p) {
+    return fmaxf(p.ymax - p.ymin, 1e-3f) * (1.0f / kBands);
 }
 
-// The lasso argument without its y-bands: matrix, screen, polygon (vertex nv repeated as vertex
-// 0), the widened bounding box in pixels and NDC, the band mapping.  Host and device run the same
-// code (batched edits build their lassos on the device), so both get identical fields.
-__host__ __device__ inline void lasso_arg_head(LassoArg &p, const float *m16, int32_t w_s, int32_t h_s,
-                                               const float *poly, int32_t nv, uint32_t label, float bias) {
-    for (int i = 0; i < 16; ++i) p.m[i] = m16[i];
+// The lasso argument's scalars but for the polygon's: matrix, screen, label, bias.
+__host__ __device__ inline void lasso_arg_scalars(LassoArg &p, int32_t w_s, int32_t h_s, int32_t nv, uint32_t label,
+                                                  float bias) {
     p.ws = (float)w_s;
     p.hs = (float)h_s;
     p.w_s = w_s;
@@ -809,6 +800,33 @@ __host__ __device__ inline void lasso_arg_head(LassoArg &p, const float *m16, in
     p.bias = bias;
     p.label = label;
     p.nv = nv;
+}
+
+// What follows from the polygon's bounding box: the widened box in pixels and NDC, the band mapping.
+__host__ __device__ inline void lasso_arg_box(LassoArg &p, float x0, float x1, float y0, float y1) {
+    // Culling and the division-free reject use the bbox widened by a margin far above the FP32
+    // rounding of projected points (well under a thousandth of a pixel at these sizes).
+    const float margin = 2.0f + 1e-3f * (float)(p.w_s > p.h_s ? p.w_s : p.h_s);
+    p.bx0 = fmaxf(x0, 0.0f) - margin;
+    p.bx1 = fminf(x1, (float)p.w_s) + margin;
+    p.by0 = fmaxf(y0, 0.0f) - margin;
+    p.by1 = fminf(y1, (float)p.h_s) + margin;
+    p.nx0 = (float)(2.0 * p.bx0 / p.w_s - 1.0);
+    p.nx1 = (float)(2.0 * p.bx1 / p.w_s - 1.0);
+    p.ny0 = (float)(2.0 * p.by0 / p.h_s - 1.0);
+    p.ny1 = (float)(2.0 * p.by1 / p.h_s - 1.0);
+    p.ymin = y0;
+    p.ymax = y1;
+    p.band_y0 = y0;
+    p.band_inv_h = 1.0f / lasso_band_height(p);
+}
+
+// The lasso argument without its y-bands (vertex nv repeated as vertex 0), on the host; batched edits
+// build theirs on the device, a lane per vertex (k_batch_prep).
+inline void lasso_arg_head(LassoArg &p, const float *m16, int32_t w_s, int32_t h_s, const float *poly, int32_t nv,
+                           uint32_t label, float bias) {
+    for (int i = 0; i < 16; ++i) p.m[i] = m16[i];
+    lasso_arg_scalars(p, w_s, h_s, nv, label, bias);
     float x0 = INFINITY, x1 = -INFINITY, y0 = INFINITY, y1 = -INFINITY;
     for (int i = 0; i < nv; ++i) {
         p.vx[i] = poly[2 * i];
@@ -822,36 +840,22 @@ __host__ __device__ inline void lasso_arg_head(LassoArg &p, const float *m16, in
         p.vx[i] = p.vx[0];
         p.vy[i] = p.vy[0];
     }
-    // Culling and the division-free reject use the bbox widened by a margin far above the FP32
-    // rounding of projected points (well under a thousandth of a pixel at these sizes).
-    const float margin = 2.0f + 1e-3f * (float)(w_s > h_s ? w_s : h_s);
-    p.bx0 = fmaxf(x0, 0.0f) - margin;
-    p.bx1 = fminf(x1, (float)w_s) + margin;
-    p.by0 = fmaxf(y0, 0.0f) - margin;
-    p.by1 = fminf(y1, (float)h_s) + margin;
-    p.nx0 = (float)(2.0 * p.bx0 / w_s - 1.0);
-    p.nx1 = (float)(2.0 * p.bx1 / w_s - 1.0);
-    p.ny0 = (float)(2.0 * p.by0 / h_s - 1.0);
-    p.ny1 = (float)(2.0 * p.by1 / h_s - 1.0);
-    p.ymin = y0;
-    p.ymax = y1;
-    p.band_y0 = y0;
-    p.band_inv_h = (float)(1.0 / lasso_band_height(p));
+    lasso_arg_box(p, x0, x1, y0, y1);
 }
 
-__host__ __device__ inline bool lasso_band_has(const LassoArg &p, int b, int e, double bh) {
-    const double slack = 1e-3 * bh + 1e-3;
-    const double lo = (double)p.ymin + b * bh - slack, hi = (double)p.ymin + (b + 1) * bh + slack;
-    const double ea = p.vy[e], eb = p.vy[e + 1];
+__host__ __device__ inline bool lasso_band_has(const LassoArg &p, int b, int e, float bh) {
+    const float slack = 2e-3f * bh + 2e-3f + 1e-6f * (fabsf(p.ymin) + fabsf(p.ymax));
+    const float lo = p.ymin + (float)b * bh - slack, hi = p.ymin + (float)(b + 1) * bh + slack;
+    const float ea = p.vy[e], eb = p.vy[e + 1];
     if (ea == eb) return false;  // horizontal edges never straddle
-    return fmin(ea, eb) <= hi && fmax(ea, eb) >= lo;
+    return fminf(ea, eb) <= hi && fmaxf(ea, eb) >= lo;
 }
 
 // The whole lasso argument, on the host.
 inline void fill_lasso_arg(LassoArg &p, const lcl_camera *cam, const float *poly, int32_t nv, uint32_t label,
                            float bias) {
     lasso_arg_head(p, cam->m, cam->width, cam->height, poly, nv, label, bias);
-    const double bh = lasso_band_height(p);
+    const float bh = lasso_band_height(p);
     int cnt = 0;
     for (int b = 0; b < kBands; ++b) {
         p.band_off[b] = (uint16_t)cnt;
