@@ -36,14 +36,16 @@
 namespace lcl {
 namespace {
 
-// Zeroes n counters and the first n_hits of `hits` (nullable).
-__global__ void k_sel_init(uint32_t *counters, int32_t n, unsigned long long *hits, int32_t n_hits) {
-    pdl_wait();  // launched as a dependent: the previous grid no longer reads the counters
+// Zeroes n counters, the first n_hits of `hits` (nullable) and n_flags tile flags.
+__global__ void k_sel_init(uint32_t *counters, int32_t n, unsigned long long *hits, int32_t n_hits, uint32_t *flags,
+                           int32_t n_flags) {
+    pdl_wait();  // launched as a dependent: the previous grid no longer uses the workspace
     pdl_allow_next();
-    const int32_t end = max(n, hits ? n_hits : 0);
+    const int32_t end = max(max(n, hits ? n_hits : 0), n_flags);
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < end; i += gridDim.x * blockDim.x) {
         if (i < n && LCL_IN(i, n)) counters[i] = 0;
         if (hits && i < n_hits) hits[i] = 0;
+        if (i < n_flags && LCL_IN(i, n_flags)) flags[i] = 0;
     }
 }
 
@@ -461,6 +463,8 @@ __global__ void __launch_bounds__(kThreads) k_lasso_cull(AtlasDev a, const __gri
 // its 3 x 3 neighbourhood is flagged.
 __global__ void __launch_bounds__(kThreads) k_dilate_candidates(AtlasDev a, const uint32_t *__restrict__ flags,
                                                                 uint32_t *counter, uint32_t *list) {
+    pdl_wait();  // the flags are complete
+    pdl_allow_next();
     const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     const int64_t n_tiles = (int64_t)a.tiles_x * a.tiles_y;
     bool cand = false;
@@ -534,6 +538,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_tool_apply(AtlasDev a, L *__res
                                                          const uint32_t *__restrict__ counter,
                                                          const uint32_t *__restrict__ list,
                                                          unsigned long long *hits, ValMask vm) {
+    pdl_wait();  // the candidate tiles are complete
+    pdl_allow_next();
     const uint32_t n = *counter;
     if (PAD) {
         __shared__ PadShared sh;
@@ -587,7 +593,8 @@ SelWs sel_ws(const lcl_atlas *a, int32_t n, void *ws) {
     return w;
 }
 
-// The cull's launches with G lanes per tile (launch_lasso_cull).
+// The cull's launches with G lanes per tile (launch_lasso_cull), each a programmatic dependent of the one
+// before.
 template <int G>
 int launch_lasso_cull_by(const AtlasDev &a, const lcl_atlas *atlas, const LassoArg &p, const float *depth,
                          const SelWs &w, bool pad, bool classify, cudaStream_t st) {
@@ -595,32 +602,28 @@ int launch_lasso_cull_by(const AtlasDev &a, const lcl_atlas *atlas, const LassoA
     const int n_super = atlas->supers_x * atlas->supers_y;
     const int grid = std::max(1, std::min(n_super * (LCL_SUPER * LCL_SUPER / (kThreads / G)), 8 * sm_count()));
     const uint32_t *const super_count = w.counters + 1, *const supers = w.list3;
-    if (!pad && classify) {  // the lasso's chain: each launch a programmatic dependent of the one before
-        launch_pdl(k_lasso_supers, dim3((n_super + kThreads / 8 - 1) / (kThreads / 8)), st, a, p, w.counters + 1,
-                   w.list3);
-        launch_pdl(k_lasso_cull<false, true, G>, dim3(grid), st, a, p, depth, super_count, supers, w.counters, w.list);
-        return 2;
-    }
-    k_lasso_supers<<<(n_super + kThreads / 8 - 1) / (kThreads / 8), kThreads, 0, st>>>(a, p, w.counters + 1, w.list3);
+    launch_pdl(k_lasso_supers, dim3((n_super + kThreads / 8 - 1) / (kThreads / 8)), st, a, p, w.counters + 1, w.list3);
     if (!pad) {
-        if (classify)
-            k_lasso_cull<false, true, G><<<grid, kThreads, 0, st>>>(a, p, depth, super_count, supers, w.counters, w.list);
-        else
-            k_lasso_cull<false, false, G><<<grid, kThreads, 0, st>>>(a, p, depth, super_count, supers, w.counters, w.list);
+        launch_pdl(classify ? k_lasso_cull<false, true, G> : k_lasso_cull<false, false, G>, dim3(grid), st, a, p, depth,
+                   super_count, supers, w.counters, w.list);
         return 2;
     }
     // padded edits: flags for every tile that may hold a selected texel (polygon-outside tiles of a
     // lasso hold none; tiles of super-tiles the lasso cannot reach keep the cleared 0), dilated to the
     // tiles padding can reach
     const int64_t tiles = (int64_t)atlas->tiles_x * atlas->tiles_y;
-    cudaMemsetAsync(w.list2, 0, (size_t)tiles * 4, st);
-    if (classify)
-        k_lasso_cull<true, true, G><<<grid, kThreads, 0, st>>>(a, p, depth, super_count, supers, w.counters, w.list2);
-    else
-        k_lasso_cull<true, false, G><<<grid, kThreads, 0, st>>>(a, p, depth, super_count, supers, w.counters, w.list2);
-    k_dilate_candidates<<<(unsigned)((tiles + kThreads - 1) / kThreads), kThreads, 0, st>>>(a, w.list2, w.counters,
-                                                                                        w.list);
+    launch_pdl(classify ? k_lasso_cull<true, true, G> : k_lasso_cull<true, false, G>, dim3(grid), st, a, p, depth,
+               super_count, supers, w.counters, w.list2);
+    launch_pdl(k_dilate_candidates, dim3((unsigned)((tiles + kThreads - 1) / kThreads)), st, a,
+               (const uint32_t *)w.list2, w.counters, w.list);
     return 3;
+}
+
+// Zeroes the counters and the hit count of a lasso or tool edit, and with padding its tile flags.
+void launch_edit_init(const lcl_atlas *atlas, const SelWs &w, unsigned long long *h, bool pad, cudaStream_t st) {
+    const int32_t n_flags = pad ? atlas->tiles_x * atlas->tiles_y : 0;
+    const int grid = std::max(1, std::min((n_flags + kThreads - 1) / kThreads, 2 * sm_count()));
+    launch_pdl(k_sel_init, dim3(grid), st, w.counters, 2, h, 1, w.list2, n_flags);
 }
 
 // Launches the cull of a lasso / tool into w.list (counter w.counters[0]); with padding, the flags
@@ -778,7 +781,7 @@ lcl_status select_sphere_run(const lcl_atlas *atlas, L *layer, uint32_t *mask, c
     for (int i = 0; i < 2; ++i)
         for (int j = 0; j < 2; ++j) grid[i][j] = resident_grid(step[i][j]);
     uint32_t *const inside = w.counters + (n + 1);
-    k_sel_init<<<(2 * (n + 1) + kThreads - 1) / kThreads, kThreads, 0, st>>>(w.counters, 2 * (n + 1), h, n);
+    k_sel_init<<<(2 * (n + 1) + kThreads - 1) / kThreads, kThreads, 0, st>>>(w.counters, 2 * (n + 1), h, n, nullptr, 0);
     const int n_super = atlas->supers_x * atlas->supers_y;
     cudaError_t e = launch_pdl(k_sphere_cull, dim3(std::min(n_super, grid[0][0])), st, a, arg(0), w.counters, w.list,
                                inside);
@@ -819,12 +822,9 @@ template <typename L, bool NUM>
 void launch_lasso_apply(bool pad, const AtlasDev &a, L *layer, const LassoArg &p, const float *depth,
                         const SelWs &w, unsigned long long *h, ValMask vm, int32_t pad_r, int32_t pad_t,
                         cudaStream_t st) {
-    if (pad)
-        k_lasso_apply<L, NUM, true><<<resident_grid(k_lasso_apply<L, NUM, true>), kThreads, 0, st>>>(
-            a, layer, p, depth, w.counters, w.list, h, vm, pad_r, pad_t);
-    else
-        launch_pdl(k_lasso_apply<L, NUM, false>, dim3(resident_grid(k_lasso_apply<L, NUM, false>)), st, a, layer, p,
-                   depth, (const uint32_t *)w.counters, (const uint32_t *)w.list, h, vm, 0, 0);
+    const auto kernel = pad ? k_lasso_apply<L, NUM, true> : k_lasso_apply<L, NUM, false>;
+    launch_pdl(kernel, dim3(resident_grid(kernel)), st, a, layer, p, depth, (const uint32_t *)w.counters,
+               (const uint32_t *)w.list, h, vm, pad_r, pad_t);
 }
 
 // Lasso on a label layer (mask NULL) or on a numeric layer (data bytes 1, 2 or 4 and its mask bits),
@@ -839,10 +839,7 @@ lcl_status lasso_run(const lcl_atlas *atlas, void *layer, int bytes, uint32_t *m
     fill_lasso_arg(p, cam, poly, nv, label, bias);
     const int32_t pad_r = (int32_t)(pad_flags & 15u), pad_t = (int32_t)((pad_flags >> 4) & 15u);
     const bool pad = pad_r > 0;
-    if (pad)
-        k_sel_init<<<1, kThreads, 0, st>>>(w.counters, 2, h, 1);
-    else
-        launch_pdl(k_sel_init, dim3(1), st, w.counters, 2, h, 1);
+    launch_edit_init(atlas, w, h, pad, st);
     const int n_cull = launch_lasso_cull(a, atlas, p, depth, w, pad, true, st);
     ValMask vm;
     vm.bits = mask;
@@ -884,24 +881,13 @@ lcl_status numeric_lasso_impl(const lcl_atlas *atlas, void *data, int data_bytes
 template <typename L, bool NUM>
 void launch_tool(int sel, const AtlasDev &a, L *layer, const LassoArg &p, const ToolArg &t, const float *depth,
                  const SelWs &w, unsigned long long *h, ValMask vm, cudaStream_t st) {
-    switch (sel) {  // bit 0: shape mask, bit 1: padding
-    case 0:
-        k_tool_apply<L, false, false, NUM><<<resident_grid(k_tool_apply<L, false, false, NUM>), kThreads, 0, st>>>(
-            a, layer, p, t, depth, w.counters, w.list, h, vm);
-        break;
-    case 1:
-        k_tool_apply<L, true, false, NUM><<<resident_grid(k_tool_apply<L, true, false, NUM>), kThreads, 0, st>>>(
-            a, layer, p, t, depth, w.counters, w.list, h, vm);
-        break;
-    case 2:
-        k_tool_apply<L, false, true, NUM><<<resident_grid(k_tool_apply<L, false, true, NUM>), kThreads, 0, st>>>(
-            a, layer, p, t, depth, w.counters, w.list, h, vm);
-        break;
-    default:
-        k_tool_apply<L, true, true, NUM><<<resident_grid(k_tool_apply<L, true, true, NUM>), kThreads, 0, st>>>(
-            a, layer, p, t, depth, w.counters, w.list, h, vm);
-        break;
-    }
+    // bit 0: shape mask, bit 1: padding
+    const auto kernel = sel == 0   ? k_tool_apply<L, false, false, NUM>
+                        : sel == 1 ? k_tool_apply<L, true, false, NUM>
+                        : sel == 2 ? k_tool_apply<L, false, true, NUM>
+                                   : k_tool_apply<L, true, true, NUM>;
+    launch_pdl(kernel, dim3(resident_grid(kernel)), st, a, layer, p, t, depth, (const uint32_t *)w.counters,
+               (const uint32_t *)w.list, h, vm);
 }
 
 // The tool on a label layer (mask NULL) or on a numeric layer.
@@ -914,8 +900,8 @@ lcl_status tool_run(const lcl_atlas *atlas, void *layer, int bytes, uint32_t *ma
     static thread_local LassoArg p;  // ~2.8 KB: kept off the stack
     ToolArg t;
     fill_tool_arg(t, p, cam, tool, label, bias);
-    k_sel_init<<<1, kThreads, 0, st>>>(w.counters, 2, h, 1);
     const bool pad = t.pad_r > 0;
+    launch_edit_init(atlas, w, h, pad, st);
     const int n_cull = launch_lasso_cull(a, atlas, p, depth, w, pad, false, st);
     const int sel = (tool->shape != nullptr ? 1 : 0) + (pad ? 2 : 0);
     ValMask vm;
