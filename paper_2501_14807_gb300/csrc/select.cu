@@ -480,8 +480,42 @@ __global__ void __launch_bounds__(kThreads) k_dilate_candidates(AtlasDev a, cons
 
 // A lasso's candidate-list entry: tile index, kInsideTile set when every texel of the tile that
 // projects lies inside the polygon (lasso_tile_class8).  Padded edits list plain tile indices.
+// An edit's CTAs take kEditQuads quads at a time, one per thread, of one tile or of several small ones
+// (a CTA per tile left threads idle where a tile has fewer quads: 105 -> 80 us for 3 lassos over tiles
+// of 16 on 2048^2).  The lasso's apply is bound by instruction issue and by the latency of its loads;
+// it reads the next item's positions ahead and projects the quads of inside tiles side by side
+// (lasso_quad_inside): with their culls, 5 lassos on a 16384^2 atlas 941 -> 884 us and 12 on 4096^2
+// 421 -> 417 us.  Four CTAs per SM, since few tiles are candidates on a small atlas: with three (and
+// no bound on the registers) 853 and 428 us.  CTAs of 64 and 128 threads were slower (462 and 426 us).
+constexpr int kEditQuads = 256;
+template <bool PAD>
+constexpr int edit_threads() {
+    return PAD ? kThreads : kEditQuads;
+}
+
+// The quad of this thread in item `i` of the candidate list; false if it has none.  entry: the tile's
+// list entry; l: the quad's first texel.
+__device__ __forceinline__ bool edit_quad(const AtlasDev &a, const uint32_t *__restrict__ list, uint32_t n, uint32_t i,
+                                          uint32_t &entry, int32_t &l) {
+    const int qlog = __ffs(a.T) - 3, nlog = 2 * qlog + 2;  // quads per row and per tile
+    const uint32_t g = i * kEditQuads + threadIdx.x, k = g >> nlog;
+    if (k >= n || !LCL_IN(k, (int64_t)a.tiles_x * a.tiles_y)) return false;
+    entry = __ldg(list + k);
+    int32_t tx, ty;
+    tile_xy(a, entry & ~kInsideTile, tx, ty);
+    const int32_t qd = (int32_t)(g & ((1u << nlog) - 1u));
+    const int32_t x = tx * a.T + 4 * (qd & ((1 << qlog) - 1)), y = ty * a.T + (qd >> qlog);
+    l = y * a.w + x;  // below 2^28
+    return x < a.w && y < a.h && LCL_IN((int64_t)y * a.w + x + 3, (int64_t)a.w * a.h);
+}
+// Items of n candidate tiles.
+__device__ __forceinline__ uint32_t edit_items(const AtlasDev &a, uint32_t n) {
+    const int nlog = 2 * (__ffs(a.T) - 3) + 2;
+    return (uint32_t)((((uint64_t)n << nlog) + kEditQuads - 1) / kEditQuads);  // an atlas has 2^26 quads
+}
+
 template <typename L, bool NUM, bool PAD>
-__global__ void __launch_bounds__(kThreads) k_lasso_apply(AtlasDev a, L *__restrict__ layer,
+__global__ void __launch_bounds__(edit_threads<PAD>(), 4) k_lasso_apply(AtlasDev a, L *__restrict__ layer,
                                                           const __grid_constant__ LassoArg p,
                                                           const float *__restrict__ depth,
                                                           const uint32_t *__restrict__ counter,
@@ -500,30 +534,35 @@ __global__ void __launch_bounds__(kThreads) k_lasso_apply(AtlasDev a, L *__restr
         add_hits(hits, pad_tiles<L, NUM>(a, layer, ps, n, list, pad_r, pad_t, p.label, vm, hit));
         return;
     }
-    const int32_t qpr = a.T / 4, nq = a.T * qpr;
     uint32_t cnt = 0;
     const int64_t n_tex = (int64_t)a.w * a.h;
-    for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
-        if (!LCL_IN(i, (int64_t)a.tiles_x * a.tiles_y)) break;
-        const uint32_t entry = list[i];
-        const bool inside = (entry & kInsideTile) != 0u;  // uniform over the CTA
-        const uint32_t tile = entry & ~kInsideTile;
-        int32_t tx, ty;
-        tile_xy(a, tile, tx, ty);
-        for (int32_t qd = threadIdx.x; qd < nq; qd += kThreads) {
-            const int32_t x = tx * a.T + 4 * (qd & (qpr - 1)), y = ty * a.T + (qd >> (__ffs(qpr) - 1));
-            if (x >= a.w || y >= a.h) continue;
-            const int64_t l = (int64_t)y * a.w + x;
-            if (!LCL_IN(l + 3, n_tex)) continue;
-            const int4 X = __ldg(reinterpret_cast<const int4 *>(a.px + l));
-            const int4 Y = __ldg(reinterpret_cast<const int4 *>(a.py + l));
-            const int4 Z = __ldg(reinterpret_cast<const int4 *>(a.pz + l));
-            const uint32_t m = inside ? lasso_quad<true>(p, sh, depth, X, Y, Z) : lasso_quad<false>(p, sh, depth, X, Y, Z);
-            if (m) {
-                store_hits<L>(layer, l, m, p.label);
-                if (NUM) valid_update_atomic(vm, l, m, n_tex);
-                cnt += __popc(m);
-            }
+    const uint32_t n_items = edit_items(a, n);
+    // the next item's positions are loaded while this one is tested
+    uint32_t next_entry = 0u;
+    int32_t next_l = -1;
+    int4 X, Y, Z;
+    auto load = [&](uint32_t i) {
+        if (!edit_quad(a, list, n, i, next_entry, next_l)) {
+            next_l = -1;
+            return;
+        }
+        X = __ldg(reinterpret_cast<const int4 *>(a.px + next_l));
+        Y = __ldg(reinterpret_cast<const int4 *>(a.py + next_l));
+        Z = __ldg(reinterpret_cast<const int4 *>(a.pz + next_l));
+    };
+    load(blockIdx.x);
+    for (uint32_t i = blockIdx.x; i < n_items; i += gridDim.x) {
+        const uint32_t entry = next_entry;
+        const int32_t l = next_l;
+        const int4 x = X, y = Y, z = Z;
+        load(i + gridDim.x);
+        if (l < 0) continue;
+        const uint32_t m = entry & kInsideTile ? lasso_quad_inside(p, sh, depth, x, y, z)
+                                               : lasso_quad(p, sh, depth, x, y, z);
+        if (m) {
+            store_hits<L>(layer, l, m, p.label);
+            if (NUM) valid_update_atomic(vm, l, m, n_tex);
+            cnt += __popc(m);
         }
     }
     add_hits(hits, cnt);
@@ -532,7 +571,7 @@ __global__ void __launch_bounds__(kThreads) k_lasso_apply(AtlasDev a, L *__restr
 // ---- the paper's editing tool -------------------------------------------------------------
 
 template <typename L, bool MASK, bool PAD, bool NUM>
-__global__ void __launch_bounds__(kThreads, 4) k_tool_apply(AtlasDev a, L *__restrict__ layer,
+__global__ void __launch_bounds__(edit_threads<PAD>(), 1024 / edit_threads<PAD>()) k_tool_apply(AtlasDev a, L *__restrict__ layer,
                                                          const __grid_constant__ LassoArg p, ToolArg t,
                                                          const float *__restrict__ depth,
                                                          const uint32_t *__restrict__ counter,
@@ -547,32 +586,25 @@ __global__ void __launch_bounds__(kThreads, 4) k_tool_apply(AtlasDev a, L *__res
         add_hits(hits, pad_tiles<L, NUM>(a, layer, sh, n, list, t.pad_r, t.pad_t, p.label, vm, hit));
         return;
     }
-    const int32_t qpr = a.T / 4, nq = a.T * qpr;
     uint32_t cnt = 0;
     const int64_t n_tex = (int64_t)a.w * a.h;
-    for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
-        if (!LCL_IN(i, (int64_t)a.tiles_x * a.tiles_y)) break;
-        const uint32_t tile = list[i] & ~kInsideTile;  // the tool's cull lists plain tiles
-        int32_t tx, ty;
-        tile_xy(a, tile, tx, ty);
-        for (int32_t qd = threadIdx.x; qd < nq; qd += kThreads) {
-            const int32_t x = tx * a.T + 4 * (qd & (qpr - 1)), y = ty * a.T + (qd >> (__ffs(qpr) - 1));
-            if (x >= a.w || y >= a.h) continue;
-            const int64_t l = (int64_t)y * a.w + x;
-            if (!LCL_IN(l + 3, n_tex)) continue;
-            const int4 X = __ldg(reinterpret_cast<const int4 *>(a.px + l));
-            const int4 Y = __ldg(reinterpret_cast<const int4 *>(a.py + l));
-            const int4 Z = __ldg(reinterpret_cast<const int4 *>(a.pz + l));
-            uint32_t m = 0;
-            m |= tool_hit<MASK>(p, t, depth, X.x, Y.x, Z.x) ? 1u : 0u;
-            m |= tool_hit<MASK>(p, t, depth, X.y, Y.y, Z.y) ? 2u : 0u;
-            m |= tool_hit<MASK>(p, t, depth, X.z, Y.z, Z.z) ? 4u : 0u;
-            m |= tool_hit<MASK>(p, t, depth, X.w, Y.w, Z.w) ? 8u : 0u;
-            if (m) {
-                store_hits<L>(layer, l, m, p.label);
-                if (NUM) valid_update_atomic(vm, l, m, n_tex);
-                cnt += __popc(m);
-            }
+    const uint32_t n_items = edit_items(a, n);
+    for (uint32_t i = blockIdx.x; i < n_items; i += gridDim.x) {
+        uint32_t entry;
+        int32_t l;
+        if (!edit_quad(a, list, n, i, entry, l)) continue;
+        const int4 X = __ldg(reinterpret_cast<const int4 *>(a.px + l));
+        const int4 Y = __ldg(reinterpret_cast<const int4 *>(a.py + l));
+        const int4 Z = __ldg(reinterpret_cast<const int4 *>(a.pz + l));
+        uint32_t m = 0;
+        m |= tool_hit<MASK>(p, t, depth, X.x, Y.x, Z.x) ? 1u : 0u;
+        m |= tool_hit<MASK>(p, t, depth, X.y, Y.y, Z.y) ? 2u : 0u;
+        m |= tool_hit<MASK>(p, t, depth, X.z, Y.z, Z.z) ? 4u : 0u;
+        m |= tool_hit<MASK>(p, t, depth, X.w, Y.w, Z.w) ? 8u : 0u;
+        if (m) {
+            store_hits<L>(layer, l, m, p.label);
+            if (NUM) valid_update_atomic(vm, l, m, n_tex);
+            cnt += __popc(m);
         }
     }
     add_hits(hits, cnt);
@@ -823,8 +855,9 @@ void launch_lasso_apply(bool pad, const AtlasDev &a, L *layer, const LassoArg &p
                         const SelWs &w, unsigned long long *h, ValMask vm, int32_t pad_r, int32_t pad_t,
                         cudaStream_t st) {
     const auto kernel = pad ? k_lasso_apply<L, NUM, true> : k_lasso_apply<L, NUM, false>;
-    launch_pdl(kernel, dim3(resident_grid(kernel)), st, a, layer, p, depth, (const uint32_t *)w.counters,
-               (const uint32_t *)w.list, h, vm, pad_r, pad_t);
+    const int threads = pad ? edit_threads<true>() : edit_threads<false>();
+    launch_pdl_shape(kernel, dim3(resident_per_sm(kernel, threads) * sm_count()), dim3(threads), st, a, layer, p, depth,
+                     (const uint32_t *)w.counters, (const uint32_t *)w.list, h, vm, pad_r, pad_t);
 }
 
 // Lasso on a label layer (mask NULL) or on a numeric layer (data bytes 1, 2 or 4 and its mask bits),
@@ -886,8 +919,9 @@ void launch_tool(int sel, const AtlasDev &a, L *layer, const LassoArg &p, const 
                         : sel == 1 ? k_tool_apply<L, true, false, NUM>
                         : sel == 2 ? k_tool_apply<L, false, true, NUM>
                                    : k_tool_apply<L, true, true, NUM>;
-    launch_pdl(kernel, dim3(resident_grid(kernel)), st, a, layer, p, t, depth, (const uint32_t *)w.counters,
-               (const uint32_t *)w.list, h, vm);
+    const int threads = t.pad_r > 0 ? edit_threads<true>() : edit_threads<false>();
+    launch_pdl_shape(kernel, dim3(resident_per_sm(kernel, threads) * sm_count()), dim3(threads), st, a, layer, p, t,
+                     depth, (const uint32_t *)w.counters, (const uint32_t *)w.list, h, vm);
 }
 
 // The tool on a label layer (mask NULL) or on a numeric layer.

@@ -638,13 +638,59 @@ __device__ __forceinline__ uint32_t lasso_depth_quad(const LassoArg &p, const fl
 // Candidate-list entry bit of a tile whose projecting texels all lie inside the lasso polygon.
 constexpr uint32_t kInsideTile = 0x80000000u;
 
+// lasso_hit for the texels of a quad whose tile lies inside the polygon (lasso_tile_class settles the
+// viewport, the polygon's box and the edge tests).  The four texels go through the projection side by
+// side, without branches, so that their chains of dependent operations overlap; what fails a condition
+// is masked.  A quad whose operands leave the window of the fast division goes texel by texel.
+__device__ __forceinline__ uint32_t lasso_quad_inside(const LassoArg &p, const LassoShared &sh,
+                                                      const float *__restrict__ depth, int4 X, int4 Y, int4 Z) {
+    const int32_t xq[4] = {X.x, X.y, X.z, X.w}, yq[4] = {Y.x, Y.y, Y.z, Y.w}, zq[4] = {Z.x, Z.y, Z.z, Z.w};
+    float t[4], cw[4], cz[4];
+    uint32_t live = 0u;
+    bool fast = true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float fx = (float)xq[k], fy = (float)yq[k], fz = (float)zq[k];
+        const float w = clip_row(p.m + 12, fx, fy, fz);
+        const float cx = clip_row(p.m, fx, fy, fz), cy = clip_row(p.m + 4, fx, fy, fz);
+        const bool l = xq[k] != INT32_MIN && w > 0.0f;
+        const Divisor dw = divisor(w);
+        fast = fast && (!l || (dw.in && div_window(cx) && div_window(cy)));
+        const int32_t ix = __float2int_rz(screen_of(div_in_window(cx, dw), p.ws));
+        const int32_t iy = __float2int_rz(screen_of(div_in_window(cy, dw), p.hs));
+        cw[k] = w;
+        cz[k] = clip_row(p.m + 8, fx, fy, fz);
+        live |= (l ? 1u : 0u) << k;
+        const int64_t i = (int64_t)iy * p.w_s + ix;
+        t[k] = __int_as_float(0x7fc00000);
+        if (l && fast && LCL_IN(i, (int64_t)p.w_s * p.h_s)) t[k] = __ldg(depth + i);
+    }
+    uint32_t m = 0u;
+    if (!fast) {
+#pragma unroll 1
+        for (int k = 0; k < 4; ++k) {  // selects, not a runtime index into the arrays
+            const int32_t qx = k == 0 ? X.x : k == 1 ? X.y : k == 2 ? X.z : X.w;
+            const int32_t qy = k == 0 ? Y.x : k == 1 ? Y.y : k == 2 ? Y.z : Y.w;
+            const int32_t qz = k == 0 ? Z.x : k == 1 ? Z.y : k == 2 ? Z.z : Z.w;
+            if (lasso_hit<true>(p, sh, depth, qx, qy, qz)) m |= 1u << k;
+        }
+        return m;
+    }
+    // the depth test (Fig. 3a): NDC depth RN(cz / cw) in [0, 1] and at most depth + bias, both upper
+    // bounds as one, the smaller (a NaN depth selects nothing)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float b = __fadd_rn(t[k], p.bias);
+        if (((live >> k) & 1u) && b == b && quot_ge0(cz[k], cw[k]) && quot_le(cz[k], cw[k], fminf(b, 1.0f)))
+            m |= 1u << k;
+    }
+    return m;
+}
+
 // lasso_hit for the four texels of a quad (bit k: texel k).  Each texel takes the steps of
 // lasso_hit up to its band; when the quad's live texels share a band (nearly always: they are
 // neighbours on the surface) one pass over that band's edge records tests all of them.  Texels
-// that failed a step carry ys = NaN, which straddles no edge.  INSIDE: the quad's tile is known to
-// lie inside the polygon (lasso_tile_class), so the edge tests are skipped: their outcome for
-// every texel that reaches them is "inside".
-template <bool INSIDE>
+// that failed a step carry ys = NaN, which straddles no edge.
 __device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const LassoShared &sh,
                                                const float *__restrict__ depth, int4 X, int4 Y, int4 Z) {
     const int32_t xq[4] = {X.x, X.y, X.z, X.w}, yq[4] = {Y.x, Y.y, Y.z, Y.w}, zq[4] = {Z.x, Z.y, Z.z, Z.w};
@@ -662,21 +708,16 @@ __device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const LassoSha
         const float w = clip_row(p.m + 12, fx, fy, fz);
         if (!(w > 0.0f)) continue;
         const float cx = clip_row(p.m, fx, fy, fz);
-        if (!INSIDE && (cx < __fmul_rn(p.nx0, w) || cx > __fmul_rn(p.nx1, w))) continue;
+        if (cx < __fmul_rn(p.nx0, w) || cx > __fmul_rn(p.nx1, w)) continue;
         const float cy = clip_row(p.m + 4, fx, fy, fz);
-        if (!INSIDE && (cy < __fmul_rn(p.ny0, w) || cy > __fmul_rn(p.ny1, w))) continue;
+        if (cy < __fmul_rn(p.ny0, w) || cy > __fmul_rn(p.ny1, w)) continue;
         const Divisor dw = divisor(w);
         const float x = screen_of(div_by(cx, dw), p.ws);
         const float y = screen_of(div_by(cy, dw), p.hs);
-        // INSIDE: the tile's class already settles the viewport, the polygon's box and its y-range
-        // (the projected box widened by the margin lies on screen and inside the polygon)
-        if (!INSIDE && !(x >= 0.0f && x < p.ws && y >= 0.0f && y < p.hs)) continue;
-        if (!INSIDE && !(y >= p.ymin && y < p.ymax)) continue;
-        int b = 0;
-        if (!INSIDE) {
-            b = __float2int_rz(__fmul_rn(__fsub_rn(y, p.band_y0), p.band_inv_h));
-            b = b < 0 ? 0 : (b >= kBands ? kBands - 1 : b);
-        }
+        if (!(x >= 0.0f && x < p.ws && y >= 0.0f && y < p.hs)) continue;
+        if (!(y >= p.ymin && y < p.ymax)) continue;
+        int b = __float2int_rz(__fmul_rn(__fsub_rn(y, p.band_y0), p.band_inv_h));
+        b = b < 0 ? 0 : (b >= kBands ? kBands - 1 : b);
         xs[k] = x;
         ys[k] = y;
         cw[k] = w;
@@ -684,7 +725,6 @@ __device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const LassoSha
         live |= 1u << k;
     }
     if (!live) return 0;
-    if (INSIDE) return lasso_depth_quad(p, depth, xq, yq, zq, xs, ys, cw, live);
     const int b0 = (live & 1u) ? band[0] : (live & 2u) ? band[1] : (live & 4u) ? band[2] : band[3];
     bool same = true;
 #pragma unroll
