@@ -344,7 +344,7 @@ typedef struct {
  *   threads      threads per CTA: 64, 128 or 256;
  *   ctas_per_sm  CTAs per SM, 0 = as many as fit, else 1..32 (capped at what fits);
  *   split        parts each (model, tile) work item is cut into (contiguous rows of the tile),
- *                1, 2, 4 or 8; a part is the unit a CTA takes from the work queue.
+ *                1, 2, 4 or 8; a warp takes up to an eighth of a part from the work queue.
  * Results do not depend on it. */
 typedef struct {
     int32_t threads, ctas_per_sm, split, _pad;
@@ -373,9 +373,8 @@ lcl_status lcl_batch_upload(const lcl_batch_limits *limits, const lcl_batch_mode
 /* Edits the models of the batch last uploaded to `workspace`: every model's queued strokes are
  * applied to its layer in queue order, with results identical to calling lcl_select_sphere /
  * lcl_select_lasso once per stroke in that order (Section 4.3.1 applied per stroke; batching is a
- * serving-side schedule the paper does not discuss).  Two cull launches give every touched tile of
- * every model a mask of the strokes that can reach it (tested per (super-tile, stroke) pair, then
- * compacted into work items); one persistent apply launch takes
+ * serving-side schedule the paper does not discuss).  A cull launch gives every touched tile of
+ * every model a mask of the strokes that can reach it (a work item); one persistent apply launch takes
  * (model, tile part) units from a work queue, loads each texel's position once and evaluates its
  * masked strokes from the newest down, stopping at the first that selects it (the label the
  * sequence leaves).  No host-to-device copy and a launch shape fixed by (limits, config): the call

@@ -1,16 +1,16 @@
 // batch.cu -- batched edits: many models, each with a queue of sphere and lasso strokes, edited
-// by two cull launches and one persistent apply launch (capturable in a CUDA graph).
+// by one cull launch and one persistent apply launch (capturable in a CUDA graph).
 //
 // The paper edits one layer of one model per operation (Section 4.3.1).  A server holding many
 // models batches their queued strokes instead: the result must equal applying each model's
 // strokes one by one, in queue order, so
-//   k_batch_pairs  gives every tile of every model a 64-bit mask of the model's queued strokes
+//   k_batch_cull   gives every tile of every model a 64-bit mask of the model's queued strokes
 //                  (queue order = bit order) whose conservative box test can reach the tile, and
 //                  of those a `sure` mask (spheres containing the tile, lassos inside whose polygon
-//                  it lies): a CTA per (super-tile, stroke) unit, a thread per tile, the bits ORed
-//                  into per-tile masks, so one super-tile's strokes are tested in parallel;
-//   k_batch_compact turns every tile with a non-empty mask into a work item (model, tile, masks);
-//   k_batch_apply  takes (item, part) units from a work queue (one atomic per unit and CTA); a
+//                  it lies): a warp per tile, a lane per stroke.  Tiles with a non-empty mask become
+//                  work items (model, tile, masks);
+//   k_batch_apply  takes units of up to 32 quads of an item from a work queue, a warp each.  The
+//                  warp tests the masked strokes once more, against the box of its own texels; a
 //                  thread loads its four texels' positions once and evaluates the masked strokes
 //                  from the newest down: the first stroke that selects a texel is the last one
 //                  sequential application would have written there, so the texel is final and
@@ -24,8 +24,8 @@
 // sequential single-stroke calls.
 //
 // The host uploads compact descriptors (models, strokes, each lasso's camera and polygon);
-// k_batch_prep clears the tile masks and builds the lassos' culling boxes and y-band edge lists on
-// the device, one warp per lasso.  Workspace layout and launch shape depend only on the limits (capacities) and the config,
+// k_batch_prep builds the lassos' culling boxes and y-band edge lists on the device, one warp per
+// lasso.  Workspace layout and launch shape depend only on the limits (capacities) and the config,
 // and the kernels read the batch's counts from the workspace header, so the launch is independent
 // of the batch's contents: it can be captured once in a CUDA graph and replayed after each upload.
 #include <cstring>
@@ -41,7 +41,6 @@ struct BModel {
     int32_t dtype_bytes;
     int32_t s0, ns;   // this model's strokes: [s0, s0 + ns) of the batch's stroke array, ns <= 64
     int32_t super0;   // first flattened super-tile of this model
-    int64_t tile0;    // first flattened tile of this model (index into the tile masks)
 };
 
 struct BStroke {
@@ -67,6 +66,7 @@ struct BLassoIn {  // what the host uploads per lasso
     uint32_t flags;  // texture padding: radius = bits 0-3, thickness = bits 4-7
 };
 
+constexpr uint32_t kPadItem = 0x80000000u;  // bit of an item's tile: a stroke of its mask pads
 struct BItem {
     uint32_t model, tile;
     unsigned long long mask;  // strokes that can write a texel of the tile
@@ -91,15 +91,16 @@ __device__ __forceinline__ bool stroke_in_bounds(const BStroke *strokes, int64_t
 // k_batch_prep at every launch.
 struct BHdr {
     int32_t n_models, n_strokes, n_lassos, n_supers;
-    unsigned int n_items;          // written by k_batch_compact
-    unsigned int n_tiles;          // tiles of the batch's models (the tile masks in use)
+    unsigned int n_items;          // written by k_batch_cull
+    unsigned int next_cull;        // work queue of k_batch_cull
     unsigned long long next_unit;  // work queue of k_batch_apply
 };
 
 // Workspace: [hdr | models | strokes | lasso inputs | super-tile -> model] is uploaded (the
-// staging holds its image); [lassos | items | tile masks] is written by the kernels.
+// staging holds its image); [lassos | items] is written by the kernels.  Another 16 bytes per tile are
+// counted but not used, so that lcl_batch_workspace_bytes stays what programs may have stored.
 struct BLayout {
-    size_t hdr, models, strokes, lasso_in, super_model, upload, lassos, items, tmask, total;
+    size_t hdr, models, strokes, lasso_in, super_model, upload, lassos, items, total;
 };
 
 BLayout b_layout(const lcl_batch_limits &lim) {
@@ -112,33 +113,26 @@ BLayout b_layout(const lcl_batch_limits &lim) {
     L.upload = L.super_model + align256((size_t)std::max<int64_t>(lim.supers, 1) * 4);
     L.lassos = L.upload;
     L.items = L.lassos + align256((size_t)std::max(lim.lassos, 1) * sizeof(BLasso));
-    L.tmask = L.items + align256((size_t)std::max<int64_t>(lim.tiles, 1) * sizeof(BItem));
-    L.total = L.tmask + align256((size_t)std::max<int64_t>(lim.tiles, 1) * sizeof(ulonglong2));
+    L.total = L.items + align256((size_t)std::max<int64_t>(lim.tiles, 1) * sizeof(BItem)) +
+              align256((size_t)std::max<int64_t>(lim.tiles, 1) * 16);
     return L;
-}
-
-__device__ __forceinline__ bool stroke_may_touch(const BStroke &st, const BLasso *lassos, int4 lo, int4 hi) {
-    if (lo.w == 0) return false;
-    if (st.kind == LCL_STROKE_SPHERE) return box_dist2(lo, hi, st.sphere) <= st.sphere.r2;
-    return box_may_touch(lassos[st.lasso].arg, lo, hi, lassos[st.lasso].depth);
 }
 
 __device__ __forceinline__ bool stroke_pads(const BStroke &st, const BLasso *lassos) {
     return st.kind == LCL_STROKE_SPHERE ? st.sphere.pad_r > 0 : lassos[st.lasso].pad_r > 0;
 }
 
-// Box (bx, by) of a grid of nx x ny boxes (8 int32 each): can the stroke write a texel in it?  With
-// texture padding a texel may be written because a neighbour within 8 texels (at most one tile,
-// and so one super-tile, away) is selected, so then any box of the 3 x 3 neighbourhood counts.
-__device__ __forceinline__ bool stroke_may_reach(const BStroke &st, const BLasso *lassos, const int32_t *boxes,
-                                                 int32_t nx, int32_t ny, int32_t bx, int32_t by) {
-    const bool pad = stroke_pads(st, lassos);
-    const int32_t r = pad ? 1 : 0;
+// Can lasso L select a texel of a box within r of box (bx, by) of a grid of nx x ny boxes (8 int32 each)?
+// By an aligned group of 8 lanes.  With texture padding a texel may be written because a neighbour within
+// 8 texels (at most one tile, and so one super-tile, away) is selected, so then r = 1.
+__device__ __forceinline__ bool box_near(const BLasso &L, const int32_t *boxes, int32_t nx, int32_t ny, int32_t bx,
+                                         int32_t by, int32_t r, const float *depth) {
     for (int32_t y = max(by - r, 0); y <= min(by + r, ny - 1); ++y)
         for (int32_t x = max(bx - r, 0); x <= min(bx + r, nx - 1); ++x) {
             if (!LCL_IN((int64_t)y * nx + x, (int64_t)nx * ny)) continue;
             const int4 *b = reinterpret_cast<const int4 *>(boxes + 8 * ((int64_t)y * nx + x));
-            if (stroke_may_touch(st, lassos, b[0], b[1])) return true;
+            const int4 lo = b[0], hi = b[1];
+            if (lo.w > 0 && box_may_touch_by<8>(L.arg, lo, hi, depth)) return true;
         }
     return false;
 }
@@ -146,20 +140,17 @@ __device__ __forceinline__ bool stroke_may_reach(const BStroke &st, const BLasso
 constexpr int kPrepWarps = kThreads / 32;  // lassos per CTA of k_batch_prep
 static_assert(kBands == 32, "k_batch_prep gives each y-band one lane");
 
-// Resets the work counters and the tile masks and builds every lasso's argument, one warp per lasso:
+// Resets the work counters and builds every lasso's argument, one warp per lasso:
 // the lanes copy the vertices and reduce their bounding box, then lane b counts and lists the edges of
 // band b (the same predicate, in the same edge order, as the host builder).
 __global__ void __launch_bounds__(kThreads) k_batch_prep(BHdr *hdr, const BLassoIn *__restrict__ in,
-                                                         BLasso *__restrict__ out, ulonglong2 *__restrict__ tmask,
-                                                         BCaps caps) {
+                                                         BLasso *__restrict__ out, BCaps caps) {
     pdl_allow_next();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         hdr->n_items = 0;
+        hdr->next_cull = 0;
         hdr->next_unit = 0;
     }
-    const int64_t n_tiles = hdr->n_tiles;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n_tiles; t += (int64_t)gridDim.x * blockDim.x)
-        if (LCL_IN(t, caps.tiles)) tmask[t] = make_ulonglong2(0ull, 0ull);
     __shared__ LassoArg s_arg[kPrepWarps];
     const int lane = threadIdx.x & 31;
     const int j = blockIdx.x * kPrepWarps + (int)(threadIdx.x / 32);
@@ -214,129 +205,143 @@ __global__ void __launch_bounds__(kThreads) k_batch_prep(BHdr *hdr, const BLasso
         reinterpret_cast<uint32_t *>(&out[j].arg)[i] = reinterpret_cast<const uint32_t *>(&p)[i];
 }
 
-// Masks of one (super-tile, stroke) unit: unit u is super-tile u / 64 of the batch and stroke u % 64
-// of its model, so the tile tests of one super-tile and all its strokes run in parallel rather than
-// one after another in one thread.  A stroke whose test can reach the super-tile tests each of its 256
-// tiles and ORs its bit into the tile's mask (and, for an exact class, into `sure`): a sphere with a
-// thread per tile, a lasso with 8 lanes per tile (its eight corners, its edges and the depth footprint
-// shared out; one thread doing all of it took 8x as long), a padded stroke, whose tiles look at their
-// neighbours, with a thread per tile.
-__global__ void __launch_bounds__(kThreads) k_batch_pairs(const BHdr *__restrict__ hdr,
-                                                          const BModel *__restrict__ models,
-                                                          const BStroke *__restrict__ strokes,
-                                                          const BLasso *__restrict__ lassos,
-                                                          const uint32_t *__restrict__ super_model,
-                                                          ulonglong2 *__restrict__ tmask, BCaps caps) {
-    pdl_wait();  // the tile masks are cleared and the lassos built
+// Bit number n (from 0) of the set bits of m, which has more than n.
+__device__ __forceinline__ int nth_bit(unsigned long long m, int n) {
+    for (; n > 0; --n) m &= m - 1;
+    return __ffsll((long long)m) - 1;
+}
+
+// OR of the lanes' values; every lane of the warp calls it.
+__device__ __forceinline__ unsigned long long warp_or(unsigned long long v) {
+    const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)v), hi = __reduce_or_sync(0xffffffffu, (uint32_t)(v >> 32));
+    return (unsigned long long)hi << 32 | lo;
+}
+
+// The strokes that can write a texel of each tile.  A warp takes units of four tiles (neighbours in a row
+// of a super-tile) from a work queue, 8 lanes per tile.  The warp first tests the model's lassos against
+// the super-tile's box, four at a time; then each group of 8 lanes tests its tile: a lane per sphere, the
+// whole group per lasso, so that the four groups go through the same lasso together.  A padded stroke
+// counts a tile if it may reach any box of its 3 x 3 neighbourhood.  The queue evens out tiles under many
+// large lassos; with a CTA per (super-tile, stroke) those ran on while the chip was idle (24 models of
+// 512^2 to 2048^2, 48 spheres and 16 lassos each: 341 us with the compaction, now about 220; 3 models with
+// 40 spheres each: 11.1 us and 8.5).  What is left is the latency of one warp's footprint scans.
+constexpr int kCullTiles = 4;  // tiles of a unit
+constexpr int kCullUnits = LCL_SUPER * LCL_SUPER / kCullTiles;
+static_assert(LCL_SUPER % kCullTiles == 0 && kCullTiles == 4, "k_batch_cull: 8 lanes per tile");
+
+__global__ void __launch_bounds__(kThreads, 4) k_batch_cull(BHdr *hdr, const BModel *__restrict__ models,
+                                                            const BStroke *__restrict__ strokes,
+                                                            const BLasso *__restrict__ lassos,
+                                                            const uint32_t *__restrict__ super_model,
+                                                            BItem *items, BCaps caps) {
+    const int lane = threadIdx.x & 31, sub = lane & 7, group = lane / 8;
+    pdl_wait();  // the counters are reset and the lassos built
     pdl_allow_next();
-    __shared__ int s_reach;
-    const int64_t n_units = (int64_t)hdr->n_supers * 64;
-    for (int64_t u = blockIdx.x; u < n_units; u += gridDim.x) {  // uniform over the CTA
-        const int32_t g = (int32_t)(u >> 6), k = (int32_t)(u & 63);
+    const int64_t n_units = (int64_t)hdr->n_supers * kCullUnits;
+    // the first unit is the warp's number, the others come from the queue, drawn one ahead
+    const uint32_t n_warps = gridDim.x * (kThreads / 32);
+    uint32_t next = blockIdx.x * (kThreads / 32) + threadIdx.x / 32;
+    for (;;) {
+        const uint32_t u = __shfl_sync(0xffffffffu, next, 0);
+        if (u >= n_units) break;  // uniform over the warp, as below
+        if (lane == 0) next = n_warps + atomicAdd(&hdr->next_cull, 1u);
+        const int32_t g = (int32_t)(u / kCullUnits), part = (int32_t)(u % kCullUnits);
         if (!LCL_IN(g, caps.supers)) break;
         const uint32_t mi = super_model[g];
         if (!LCL_IN(mi, caps.models)) continue;
         const BModel &M = models[mi];
-        if (k >= M.ns) continue;
-        if (!stroke_in_bounds(strokes, (int64_t)M.s0 + k, caps)) continue;
         const AtlasDev &a = M.a;
         const int32_t sidx = g - M.super0;
         if (!LCL_IN(sidx, (int64_t)a.supers_x * a.supers_y)) continue;
         const int32_t sx = sidx % a.supers_x, sy = sidx / a.supers_x;
-        const BStroke &st = strokes[M.s0 + k];
-        const bool pads = stroke_pads(st, lassos), by_lanes = !pads && st.kind == LCL_STROKE_LASSO;
-        __syncthreads();  // s_reach of the previous unit has been read
-        if (by_lanes) {
-            if (threadIdx.x < 32) {
-                const int4 *b = reinterpret_cast<const int4 *>(a.super_box + 8 * (int64_t)sidx);
-                const int4 lo = b[0], hi = b[1];
-                const bool reach = lo.w > 0 && box_may_touch_by<32>(lassos[st.lasso].arg, lo, hi, lassos[st.lasso].depth);
-                if (threadIdx.x == 0) s_reach = reach;
-            }
-        } else if (threadIdx.x == 0) {
-            s_reach = stroke_may_reach(st, lassos, a.super_box, a.supers_x, a.supers_y, sx, sy);
-        }
-        __syncthreads();
-        if (!s_reach) continue;
-        const int64_t n_tiles = (int64_t)a.tiles_x * a.tiles_y;
+        const int32_t tx0 = sx * LCL_SUPER + part % (LCL_SUPER / kCullTiles) * kCullTiles, tx = tx0 + group;
+        const int32_t ty = sy * LCL_SUPER + part / (LCL_SUPER / kCullTiles);
+        if (tx0 >= a.tiles_x || ty >= a.tiles_y) continue;
+        const int64_t n_tiles = (int64_t)a.tiles_x * a.tiles_y, tile = (int64_t)ty * a.tiles_x + tx;
         (void)n_tiles;
-        auto mark = [&](int64_t tile, bool sure) {
-            if (!LCL_IN(M.tile0 + tile, caps.tiles)) return;
-            atomicOr(&tmask[M.tile0 + tile].x, 1ull << k);
-            if (sure) atomicOr(&tmask[M.tile0 + tile].y, 1ull << k);
-        };
-        if (by_lanes) {
-            const BLasso &L = lassos[st.lasso];
-            for (int32_t i = threadIdx.x / 8; i < LCL_SUPER * LCL_SUPER; i += kThreads / 8) {
-                const int32_t tx = sx * LCL_SUPER + i % LCL_SUPER, ty = sy * LCL_SUPER + i / LCL_SUPER;
-                if (tx >= a.tiles_x || ty >= a.tiles_y) continue;  // uniform over the 8 lanes, as below
-                const int64_t tile = (int64_t)ty * a.tiles_x + tx;
-                if (!LCL_IN(tile, n_tiles)) continue;
-                const int4 *b = reinterpret_cast<const int4 *>(a.tile_box + 8 * tile);
-                const int4 lo = b[0], hi = b[1];
-                if (lo.w == 0) continue;
-                int cls = kTileTest;
-                const bool hit = box_may_touch_by<8, true>(L.arg, lo, hi, L.depth, L.arg.vx, L.arg.vy, &cls);
-                if (hit && (threadIdx.x & 7u) == 0) mark(tile, cls == kTileIn);
-            }
-            continue;
-        }
-        const int32_t tx = sx * LCL_SUPER + (threadIdx.x % LCL_SUPER);
-        const int32_t ty = sy * LCL_SUPER + (threadIdx.x / LCL_SUPER);
-        if (tx >= a.tiles_x || ty >= a.tiles_y) continue;
-        const int64_t tile = (int64_t)ty * a.tiles_x + tx;
-        if (!LCL_IN(tile, n_tiles)) continue;
-        if (pads) {
-            if (stroke_may_reach(st, lassos, a.tile_box, a.tiles_x, a.tiles_y, tx, ty)) mark(tile, false);
-        } else {
+        const bool here = tx < a.tiles_x && LCL_IN(tile, n_tiles);  // uniform over the 8 lanes
+        int4 lo = make_int4(0, 0, 0, 0), hi = lo;
+        if (here) {
             const int4 *b = reinterpret_cast<const int4 *>(a.tile_box + 8 * tile);
-            const int4 lo = b[0], hi = b[1];
-            if (lo.w > 0 && box_dist2(lo, hi, st.sphere) <= st.sphere.r2)
-                mark(tile, box_far2(lo, hi, st.sphere) <= st.sphere.r2);
+            lo = b[0], hi = b[1];
         }
-    }
-}
-
-// Work items: every tile whose mask is not empty becomes (model, tile, mask, sure); a CTA per
-// super-tile, a thread per tile.
-__global__ void __launch_bounds__(kThreads) k_batch_compact(const BHdr *__restrict__ hdr,
-                                                            const BModel *__restrict__ models,
-                                                            const uint32_t *__restrict__ super_model,
-                                                            const ulonglong2 *__restrict__ tmask, BItem *items,
-                                                            unsigned int *n_items, BCaps caps) {
-    pdl_wait();  // the masks are complete
-    pdl_allow_next();
-    const int32_t n_supers = hdr->n_supers;
-    for (int32_t g = blockIdx.x; g < n_supers; g += gridDim.x) {
-        if (!LCL_IN(g, caps.supers)) break;  // uniform over the CTA
-        const uint32_t mi = super_model[g];
-        if (!LCL_IN(mi, caps.models)) continue;
-        const BModel &M = models[mi];
-        const AtlasDev &a = M.a;
-        const int32_t sidx = g - M.super0;
-        if (!LCL_IN(sidx, (int64_t)a.supers_x * a.supers_y)) continue;
-        const int32_t sx = sidx % a.supers_x, sy = sidx / a.supers_x;
-        const int32_t tx = sx * LCL_SUPER + (threadIdx.x % LCL_SUPER);
-        const int32_t ty = sy * LCL_SUPER + (threadIdx.x / LCL_SUPER);
-        ulonglong2 m = make_ulonglong2(0ull, 0ull);
-        const int64_t tile = (int64_t)ty * a.tiles_x + tx;
-        if (tx < a.tiles_x && ty < a.tiles_y && LCL_IN(M.tile0 + tile, caps.tiles)) m = tmask[M.tile0 + tile];
-        const bool cand = m.x != 0ull;
-        const uint32_t bal = __ballot_sync(0xffffffffu, cand);
-        if (bal) {
-            const int lane = threadIdx.x & 31;
-            uint32_t base = 0;
-            if (lane == __ffs(bal) - 1) base = atomicAdd(n_items, (unsigned)__popc(bal));
-            base = __shfl_sync(0xffffffffu, base, __ffs(bal) - 1);
-            const uint32_t slot = base + __popc(bal & ((1u << lane) - 1));
-            if (cand && LCL_IN(slot, caps.tiles)) {
-                BItem it;
-                it.model = mi;
-                it.tile = (uint32_t)tile;
-                it.mask = m.x;
-                it.sure = m.y;
-                items[slot] = it;
+        // spheres: a lane tests strokes `lane` and `lane + 32` against the four tiles in turn
+        unsigned long long mask = 0ull, sure = 0ull, pads = 0ull, las = 0ull;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (32 * h >= M.ns) break;  // uniform over the warp
+            const int32_t k = 32 * h + lane;
+            const bool mine = k < M.ns && stroke_in_bounds(strokes, (int64_t)M.s0 + k, caps);
+            bool lasso = false, pad = false;
+            SphereArg sp = {};
+            if (mine) {
+                const BStroke &st = strokes[M.s0 + k];
+                lasso = st.kind != LCL_STROKE_SPHERE;
+                sp = st.sphere;
+                pad = stroke_pads(st, lassos);
             }
+            const bool sphere = mine && !lasso;
+#pragma unroll
+            for (int t = 0; t < kCullTiles; ++t) {
+                int4 tlo, thi;
+                tlo.x = __shfl_sync(0xffffffffu, lo.x, 8 * t), thi.x = __shfl_sync(0xffffffffu, hi.x, 8 * t);
+                tlo.y = __shfl_sync(0xffffffffu, lo.y, 8 * t), thi.y = __shfl_sync(0xffffffffu, hi.y, 8 * t);
+                tlo.z = __shfl_sync(0xffffffffu, lo.z, 8 * t), thi.z = __shfl_sync(0xffffffffu, hi.z, 8 * t);
+                tlo.w = __shfl_sync(0xffffffffu, lo.w, 8 * t), thi.w = 0;
+                bool can = false, in = false;
+                if (sphere && pad) {
+                    can = tx0 + t < a.tiles_x && near_box_3x3(a.tile_box, a.tiles_x, a.tiles_y, tx0 + t, ty, sp);
+                } else if (sphere && tlo.w > 0) {
+                    can = box_dist2(tlo, thi, sp) <= sp.r2;
+                    in = can && box_far2(tlo, thi, sp) <= sp.r2;
+                }
+                const uint32_t bc = __ballot_sync(0xffffffffu, can), bi = __ballot_sync(0xffffffffu, in);
+                if (group == t) {
+                    mask |= (unsigned long long)bc << (32 * h);
+                    sure |= (unsigned long long)bi << (32 * h);
+                }
+            }
+            pads |= (unsigned long long)__ballot_sync(0xffffffffu, pad) << (32 * h);
+            las |= (unsigned long long)__ballot_sync(0xffffffffu, lasso) << (32 * h);
+        }
+        if (las) {  // uniform over the warp
+            unsigned long long reach = 0ull;
+            const int n = __popcll(las);
+            for (int i = group; i < n; i += 4) {  // uniform over the 8 lanes
+                const int k = nth_bit(las, i);
+                const BLasso &L = lassos[strokes[M.s0 + k].lasso];
+                if (box_near(L, a.super_box, a.supers_x, a.supers_y, sx, sy, L.pad_r > 0 ? 1 : 0, nullptr))
+                    reach |= 1ull << k;
+            }
+            __syncwarp();
+            for (unsigned long long m = warp_or(reach); m; m &= m - 1) {  // uniform over the warp
+                const int k = __ffsll((long long)m) - 1;
+                const BLasso &L = lassos[strokes[M.s0 + k].lasso];
+                int cls = kTileTest;
+                bool can = false;
+                if (pads >> k & 1ull)
+                    can = here && box_near(L, a.tile_box, a.tiles_x, a.tiles_y, tx, ty, 1, L.depth);
+                else if (lo.w > 0)
+                    can = box_may_touch_by<8, true, 4>(L.arg, lo, hi, L.depth, L.arg.vx, L.arg.vy, &cls);
+                if (can) {
+                    mask |= 1ull << k;
+                    if (cls == kTileIn) sure |= 1ull << k;
+                }
+                __syncwarp();
+            }
+        }
+        const bool item = mask != 0ull && sub == 0;
+        const uint32_t bal = __ballot_sync(0xffffffffu, item);
+        uint32_t base = 0;
+        if (lane == 0 && bal) base = atomicAdd(&hdr->n_items, (unsigned)__popc(bal));
+        const uint32_t slot = __shfl_sync(0xffffffffu, base, 0) + __popc(bal & ((1u << lane) - 1));
+        if (item && LCL_IN(slot, caps.tiles)) {
+            BItem it;
+            it.model = mi;
+            it.tile = (uint32_t)tile | (mask & pads ? kPadItem : 0u);
+            it.mask = mask;
+            it.sure = sure;
+            items[slot] = it;
         }
     }
 }
@@ -399,115 +404,134 @@ __device__ __noinline__ uint32_t pad_texels(const AtlasDev &a, int64_t l, uint32
     return written;
 }
 
-// Quads [q0, q1) of a work item's tile (quad = 4 consecutive texels of a tile row, row-major in
-// the tile), one per thread per pass.
-template <typename L>
-__device__ __forceinline__ void apply_part(const BModel &M, const BItem &it, int32_t q0, int32_t q1,
-                                           const BStroke *__restrict__ strokes, const BLasso *__restrict__ lassos,
-                                           const BCaps &caps) {
-    const AtlasDev &a = M.a;
-    L *layer = static_cast<L *>(M.layer);
-    if (!LCL_IN(it.tile, (int64_t)a.tiles_x * a.tiles_y)) return;
-    int32_t tx, ty;
-    tile_xy(a, it.tile, tx, ty);
-    const int32_t qpr = a.T / 4;
-    for (int32_t qd = q0 + (int32_t)threadIdx.x; qd < q1; qd += (int32_t)blockDim.x) {
-        const int32_t x = tx * a.T + 4 * (qd & (qpr - 1)), y = ty * a.T + (qd >> (__ffs(qpr) - 1));
-        if (x >= a.w || y >= a.h) continue;
-        const int64_t l = (int64_t)y * a.w + x;
-        if (!LCL_IN(l + 3, (int64_t)a.w * a.h)) continue;
-        const int4 X = __ldg(reinterpret_cast<const int4 *>(a.px + l));
-        const int4 Y = __ldg(reinterpret_cast<const int4 *>(a.py + l));
-        const int4 Z = __ldg(reinterpret_cast<const int4 *>(a.pz + l));
-        const int32_t xs[4] = {X.x, X.y, X.z, X.w}, ys[4] = {Y.x, Y.y, Y.z, Y.w}, zs[4] = {Z.x, Z.y, Z.z, Z.w};
-        // uncovered texels (x = INT32_MIN) are never selected: they start final
-        uint32_t open = 0u;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) open |= (xs[k] != INT32_MIN ? 1u : 0u) << k;
-        uint32_t lab[4] = {0u, 0u, 0u, 0u}, hit = 0u;
-        for (unsigned long long m = it.mask; m && open; ) {
-            const int si = 63 - __clzll((long long)m);  // newest stroke left
-            m &= ~(1ull << si);
-            if (!stroke_in_bounds(strokes, (int64_t)M.s0 + si, caps)) continue;
-            const BStroke &st = strokes[M.s0 + si];
-            uint32_t sel = 0u;
-            const bool sure = (it.sure >> si) & 1ull;
-            if (st.kind == LCL_STROKE_SPHERE) {
-                if (sure) {
-                    sel = open;  // the sphere contains the tile's box: every covered texel is selected
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int64_t dx = (int64_t)xs[k] - st.sphere.cx, dy = (int64_t)ys[k] - st.sphere.cy;
-                        const int64_t dz = (int64_t)zs[k] - st.sphere.cz;
-                        sel |= (dx * dx + dy * dy + dz * dz <= st.sphere.r2 ? 1u : 0u) << k;
-                    }
-                    sel &= open;
-                }
-                if (sel) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (sel & (1u << k)) lab[k] = st.sphere.label;
-                }
-            } else {
-                const BLasso &ls = lassos[st.lasso];
+// The texels `open` of a quad that the lasso selects (sure: its tile lies inside the polygon).  Out of line
+// it took 1001 us where the batch at k_batch_apply takes 887.
+__device__ __forceinline__ uint32_t lasso_texels(const BLasso &ls, int4 X, int4 Y, int4 Z, uint32_t open, bool sure) {
+    uint32_t sel = 0u;
 #pragma unroll 1
-                for (int k = 0; k < 4; ++k) {  // selects, not a runtime index into the arrays
-                    if (!(open & (1u << k))) continue;
-                    const int32_t qx = k == 0 ? X.x : k == 1 ? X.y : k == 2 ? X.z : X.w;
-                    const int32_t qy = k == 0 ? Y.x : k == 1 ? Y.y : k == 2 ? Y.z : Y.w;
-                    const int32_t qz = k == 0 ? Z.x : k == 1 ? Z.y : k == 2 ? Z.z : Z.w;
-                    if (sure ? lasso_hit<true>(ls.arg, ls.arg, ls.depth, qx, qy, qz)
-                             : lasso_hit<false>(ls.arg, ls.arg, ls.depth, qx, qy, qz))
-                        sel |= 1u << k;
-                }
-                const uint32_t label = ls.arg.label;
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (sel & (1u << k)) lab[k] = label;
-            }
-            hit |= sel;
-            open &= ~sel;
-        }
-        // texture padding (Section 4.3.2) of the quad's uncovered texels: the newest padded stroke
-        // that selects a texel within its kernel radius, with a covered texel within its outline
-        // thickness, writes its label there
-        uint32_t unc = 0u;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) unc |= (xs[k] == INT32_MIN ? 1u : 0u) << k;
-        if (unc) {
-            const uint32_t ph = pad_texels(a, l, unc, it.mask, M.s0, strokes, lassos, lab, caps);
-            hit |= ph;
-        }
-        if (hit) store_labels<L>(layer, l, hit, lab);
+    for (int k = 0; k < 4; ++k) {  // selects, not a runtime index into the arrays
+        if (!(open & (1u << k))) continue;
+        const int32_t qx = k == 0 ? X.x : k == 1 ? X.y : k == 2 ? X.z : X.w;
+        const int32_t qy = k == 0 ? Y.x : k == 1 ? Y.y : k == 2 ? Y.z : Y.w;
+        const int32_t qz = k == 0 ? Z.x : k == 1 ? Z.y : k == 2 ? Z.z : Z.w;
+        if (sure ? lasso_hit<true>(ls.arg, ls.arg, ls.depth, qx, qy, qz)
+                 : lasso_hit<false>(ls.arg, ls.arg, ls.depth, qx, qy, qz))
+            sel |= 1u << k;
     }
+    return sel;
 }
 
-__global__ void __launch_bounds__(256, 3) k_batch_apply(const BHdr *__restrict__ hdr, const BModel *__restrict__ models,
+// 32 quads from q0 of a work item's tile (quad = 4 consecutive texels of a tile row, row-major in
+// the tile), one per lane.
+__device__ __forceinline__ void apply_quads(const BModel &M, const BItem &it, int32_t q0,
+                                            const BStroke *__restrict__ strokes, const BLasso *__restrict__ lassos,
+                                            const BCaps &caps) {
+    const AtlasDev &a = M.a;
+    const uint32_t tile = it.tile & ~kPadItem;
+    if (!LCL_IN(tile, (int64_t)a.tiles_x * a.tiles_y)) return;
+    int32_t tx, ty;
+    tile_xy(a, tile, tx, ty);
+    const int32_t qpr = a.T / 4, qd = q0 + (int32_t)(threadIdx.x & 31u);
+    const int32_t x = tx * a.T + 4 * (qd & (qpr - 1)), y = ty * a.T + (qd >> (__ffs(qpr) - 1));
+    if (qd >= a.T * qpr || x >= a.w || y >= a.h) return;
+    const int64_t l = (int64_t)y * a.w + x;
+    if (!LCL_IN(l + 3, (int64_t)a.w * a.h)) return;
+    const int4 X = __ldg(reinterpret_cast<const int4 *>(a.px + l));
+    const int4 Y = __ldg(reinterpret_cast<const int4 *>(a.py + l));
+    const int4 Z = __ldg(reinterpret_cast<const int4 *>(a.pz + l));
+    const int32_t xs[4] = {X.x, X.y, X.z, X.w}, ys[4] = {Y.x, Y.y, Y.z, Y.w}, zs[4] = {Z.x, Z.y, Z.z, Z.w};
+    // uncovered texels (x = INT32_MIN) are never selected: they start final
+    uint32_t open = 0u;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) open |= (xs[k] != INT32_MIN ? 1u : 0u) << k;
+    const uint32_t unc = ~open & 15u;
+    uint32_t lab[4] = {0u, 0u, 0u, 0u}, hit = 0u;
+    for (unsigned long long m = it.mask; m && open;) {
+        const int si = 63 - __clzll((long long)m);  // newest stroke left
+        m &= ~(1ull << si);
+        if (!stroke_in_bounds(strokes, (int64_t)M.s0 + si, caps)) continue;
+        const BStroke &st = strokes[M.s0 + si];
+        uint32_t sel = 0u, label;
+        const bool sure = (it.sure >> si) & 1ull;
+        if (st.kind == LCL_STROKE_SPHERE) {
+            label = st.sphere.label;
+            if (sure) {
+                sel = open;  // the sphere contains the tile's box: every covered texel is selected
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int64_t dx = (int64_t)xs[k] - st.sphere.cx, dy = (int64_t)ys[k] - st.sphere.cy;
+                    const int64_t dz = (int64_t)zs[k] - st.sphere.cz;
+                    sel |= (dx * dx + dy * dy + dz * dz <= st.sphere.r2 ? 1u : 0u) << k;
+                }
+                sel &= open;
+            }
+        } else {
+            const BLasso &ls = lassos[st.lasso];
+            label = ls.arg.label;
+            sel = lasso_texels(ls, X, Y, Z, open, sure);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (sel & (1u << k)) lab[k] = label;
+        hit |= sel;
+        open &= ~sel;
+    }
+    // texture padding (Section 4.3.2) of the quad's uncovered texels: the newest padded stroke
+    // that selects a texel within its kernel radius, with a covered texel within its outline
+    // thickness, writes its label there
+    if (unc && (it.tile & kPadItem)) {
+        uint32_t plab[4];
+        const uint32_t ph = pad_texels(a, l, unc, it.mask, M.s0, strokes, lassos, plab, caps);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (ph & (1u << k)) lab[k] = plab[k];
+        hit |= ph;
+    }
+    if (!hit) return;
+    if (M.dtype_bytes == 1) store_labels<uint8_t>(static_cast<uint8_t *>(M.layer), l, hit, lab);
+    else store_labels<uint16_t>(static_cast<uint16_t *>(M.layer), l, hit, lab);
+}
+
+// The work queue's tickets: 8 * split per item, each an equal share of the tile's groups of 32 quads (a
+// tile of 32 texels has 8; small tiles leave tickets empty), one warp per ticket.  A warp draws its next
+// ticket before it works on the current one, so the queue's latency is hidden; a ticket per CTA waited
+// for the slowest of its warps, and 4 or 1 per item took 1024 and 1498 us where 8 took 959.  The kernel
+// waits for the lassos' arguments (cache hits) between dependent operations, so warps count for more
+// than registers: with 3, 4, 5 and 6 CTAs per SM that batch took 1141, 1023, 1014 and 974 us.  The four
+// texels of a quad side by side, as in the single lasso's apply, need 80 registers and more code than the
+// instruction cache holds: 1484 us.  All of the batch: 1314 us before (a CTA per ticket, 3 per SM, padded
+// strokes looked for at every uncovered texel), now 877.
+constexpr int kItemTicketsLog = 3;
+
+__global__ void __launch_bounds__(256, 6) k_batch_apply(const BHdr *__restrict__ hdr, const BModel *__restrict__ models,
                                                      const BStroke *__restrict__ strokes,
                                                      const BLasso *__restrict__ lassos,
                                                      const BItem *__restrict__ items, unsigned long long *next_unit,
                                                      int32_t split, BCaps caps) {
     pdl_wait();
     pdl_allow_next();
-    __shared__ unsigned long long s_unit;
-    const unsigned long long n_units = (unsigned long long)hdr->n_items * (unsigned)split;
+    const int lane = threadIdx.x & 31;
+    const int plog = kItemTicketsLog + __ffs(split) - 1;  // split is a power of 2
+    const unsigned long long n_units = (unsigned long long)hdr->n_items << plog;
+    const unsigned long long n_warps = (unsigned long long)gridDim.x * (blockDim.x / 32);
+    unsigned long long next = (unsigned long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     for (;;) {
-        if (threadIdx.x == 0) s_unit = atomicAdd(next_unit, 1ull);
-        __syncthreads();
-        const unsigned long long u = s_unit;
-        __syncthreads();
-        if (u >= n_units) break;  // uniform over the CTA
-        if (!LCL_IN(u / (unsigned)split, caps.tiles)) continue;
-        const BItem it = items[u / (unsigned)split];
-        const int32_t part = (int32_t)(u % (unsigned)split);
+        const unsigned long long u = __shfl_sync(0xffffffffu, next, 0);
+        if (u >= n_units) break;  // uniform over the warp
+        if (lane == 0) next = n_warps + atomicAdd(next_unit, 1ull);
+        const unsigned long long i = u >> plog;
+        if (!LCL_IN(i, caps.tiles)) continue;
+        const BItem it = items[i];
+        const int32_t part = (int32_t)(u & ((1u << plog) - 1u));
         if (!LCL_IN(it.model, caps.models)) continue;
         const BModel &M = models[it.model];
-        const int32_t nq = M.a.T * (M.a.T / 4), per = nq / split;  // nq is a power of 2 >= 16
-        if (M.dtype_bytes == 1)
-            apply_part<uint8_t>(M, it, part * per, (part + 1) * per, strokes, lassos, caps);
-        else
-            apply_part<uint16_t>(M, it, part * per, (part + 1) * per, strokes, lassos, caps);
+        const int32_t groups = max(M.a.T * (M.a.T / 4) / 32, 1);
+        const int32_t g0 = groups * part >> plog, g1 = groups * (part + 1) >> plog;
+        for (int32_t g = g0; g < g1; ++g) {
+            apply_quads(M, it, 32 * g, strokes, lassos, caps);
+            __syncwarp();
+        }
     }
 }
 
@@ -610,7 +634,6 @@ struct BPtrs {
     BLasso *lassos;
     const uint32_t *super_model;
     BItem *items;
-    ulonglong2 *tmask;
 };
 
 BPtrs b_ptrs(const BLayout &L, void *ws) {
@@ -623,7 +646,6 @@ BPtrs b_ptrs(const BLayout &L, void *ws) {
     p.lassos = reinterpret_cast<BLasso *>(base + L.lassos);
     p.super_model = reinterpret_cast<const uint32_t *>(base + L.super_model);
     p.items = reinterpret_cast<BItem *>(base + L.items);
-    p.tmask = reinterpret_cast<ulonglong2 *>(base + L.tmask);
     return p;
 }
 
@@ -635,19 +657,12 @@ cudaError_t launch_kernels(const BPtrs &p, const lcl_batch_limits &lim, const lc
     caps.pad = 0;
     caps.supers = lim.supers;
     caps.tiles = lim.tiles;
-    // enough CTAs for the lassos (a warp each) and for clearing the tile masks
-    const int pg = (int)std::max<int64_t>((std::max(lim.lassos, 1) + kPrepWarps - 1) / kPrepWarps,
-                                          std::min<int64_t>((lim.tiles + kThreads - 1) / kThreads, 4 * sm_count()));
-    k_batch_prep<<<pg, kThreads, 0, st>>>(p.hdr, p.lasso_in, p.lassos, p.tmask, caps);
+    const int pg = (std::max(lim.lassos, 1) + kPrepWarps - 1) / kPrepWarps;  // a warp per lasso
+    k_batch_prep<<<pg, kThreads, 0, st>>>(p.hdr, p.lasso_in, p.lassos, caps);
     cudaError_t e = cudaSuccess;
     if (lim.supers > 0) {
-        const int ug = (int)std::min<int64_t>(lim.supers * 64, resident_grid(k_batch_pairs));
-        e = launch_pdl(k_batch_pairs, dim3(ug), st, (const BHdr *)p.hdr, p.models, p.strokes, p.lassos, p.super_model,
-                       p.tmask, caps);
-        const int cg = (int)std::min<int64_t>(lim.supers, resident_grid(k_batch_compact));
-        if (e == cudaSuccess)
-            e = launch_pdl(k_batch_compact, dim3(cg), st, (const BHdr *)p.hdr, p.models, p.super_model,
-                           (const ulonglong2 *)p.tmask, p.items, &p.hdr->n_items, caps);
+        const int ug = (int)std::min<int64_t>(lim.supers * kCullUnits / (kThreads / 32), resident_grid(k_batch_cull));
+        e = launch_pdl(k_batch_cull, dim3(ug), st, p.hdr, p.models, p.strokes, p.lassos, p.super_model, p.items, caps);
         if (e == cudaSuccess) {
             const int fit = resident_per_sm(k_batch_apply, c.threads);
             const int per_sm = c.ctas_per_sm > 0 ? std::min(c.ctas_per_sm, fit) : fit;
@@ -656,7 +671,7 @@ cudaError_t launch_kernels(const BPtrs &p, const lcl_batch_limits &lim, const lc
                                  (int32_t)c.split, caps);
         }
     }
-    count_launches(lim.supers > 0 ? 4 : 1);
+    count_launches(lim.supers > 0 ? 3 : 1);
     if (e == cudaSuccess) e = cudaGetLastError();
     return e;
 }
@@ -730,12 +745,10 @@ lcl_status batch_upload_impl(const lcl_batch_limits *lim, const lcl_batch_model 
     hdr.n_strokes = n_strokes;
     hdr.n_lassos = n_lassos;
     hdr.n_supers = (int32_t)n_supers;
-    hdr.n_tiles = (uint32_t)n_tiles;
     std::memcpy(img + L.hdr, &hdr, sizeof(hdr));
     BModel *bm = reinterpret_cast<BModel *>(img + L.models);
     uint32_t *super_model = reinterpret_cast<uint32_t *>(img + L.super_model);
     int32_t super0 = 0;
-    int64_t tile0 = 0;
     for (int32_t i = 0; i < n_models; ++i) {
         const lcl_batch_model &m = models[i];
         BModel d;
@@ -746,9 +759,7 @@ lcl_status batch_upload_impl(const lcl_batch_limits *lim, const lcl_batch_model 
         d.s0 = m.first_stroke;
         d.ns = m.n_strokes;
         d.super0 = super0;
-        d.tile0 = tile0;
         bm[i] = d;
-        tile0 += (int64_t)m.atlas->tiles_x * m.atlas->tiles_y;
         const int32_t nsup = m.atlas->supers_x * m.atlas->supers_y;
         for (int32_t k = 0; k < nsup; ++k) super_model[super0 + k] = (uint32_t)i;
         super0 += nsup;

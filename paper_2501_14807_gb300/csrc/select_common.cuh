@@ -376,61 +376,32 @@ __device__ __forceinline__ void stage_lasso(LassoShared &sh, const LassoArg &p) 
 //  - with a depth map: NDC depth z/w is linear-fractional along every segment of the box, so its
 //    minimum over the box is at a corner; if that minimum (less 1e-4 for FP32 rounding) exceeds
 //    the largest depth-map value over the box's widened pixel footprint plus the bias, every texel
-//    of the box fails the depth test.  Footprints above 1024 pixels are not scanned (kept).
-__device__ inline bool box_may_touch(const LassoArg &p, int4 lo, int4 hi, const float *__restrict__ depth = nullptr) {
-    float xmin = INFINITY, xmax = -INFINITY, ymin = INFINITY, ymax = -INFINITY, zmin = INFINITY;
-#pragma unroll 1
-    for (int c = 0; c < 8; ++c) {
-        float x = (float)((c & 1) ? hi.x : lo.x), y = (float)((c & 2) ? hi.y : lo.y), z = (float)((c & 4) ? hi.z : lo.z);
-        float cw = clip_row(p.m + 12, x, y, z);
-        if (!(cw > 0.0f)) return true;
-        float xs = screen_of(div_rn(clip_row(p.m, x, y, z), cw), p.ws);
-        float ys = screen_of(div_rn(clip_row(p.m + 4, x, y, z), cw), p.hs);
-        float zn = div_rn(clip_row(p.m + 8, x, y, z), cw);
-        xmin = fminf(xmin, xs); xmax = fmaxf(xmax, xs);
-        ymin = fminf(ymin, ys); ymax = fmaxf(ymax, ys);
-        zmin = fminf(zmin, zn);
-    }
-    if (xmax < p.bx0 || xmin > p.bx1 || ymax < p.by0 || ymin > p.by1) return false;
-    if (!depth) return true;
-    const float margin = 2.0f;
-    const int ix0 = max(0, __float2int_rd(xmin - margin)), ix1 = min(p.w_s - 1, __float2int_rd(xmax + margin));
-    const int iy0 = max(0, __float2int_rd(ymin - margin)), iy1 = min(p.h_s - 1, __float2int_rd(ymax + margin));
-    if (ix0 > ix1 || iy0 > iy1) return false;  // the whole footprint is off screen
-    if ((ix1 - ix0 + 1) * (iy1 - iy0 + 1) > 1024) return true;
-    float dmax = -INFINITY;
-    for (int iy = iy0; iy <= iy1; ++iy)
-        for (int ix = ix0; ix <= ix1; ++ix)
-            if (LCL_IN((int64_t)iy * p.w_s + ix, (int64_t)p.w_s * p.h_s))
-                dmax = fmaxf(dmax, __ldg(depth + (int64_t)iy * p.w_s + ix));
-    return !(zmin - 1e-4f > dmax + p.bias);
-}
-
-
-// box_may_touch evaluated by an aligned group of G lanes (8 or 32) for one box (all of them call it with
-// the same box): lane c projects corner c mod 8, and the depth footprint is shared out over the group.
-// The tests of box_may_touch, with footprints of up to 2048 px scanned (1024 there) before the test
-// gives up and keeps the box.  The scan looks for a pixel that the box's nearest corner does not lie
-// behind -- max(d) + bias >= z exactly if some d + bias >= z, rounding being monotone -- and stops
-// at the first group of pixels that holds one: visible boxes take one step, hidden ones all.
+//    of the box fails the depth test.  Footprints above 2048 pixels are not scanned (kept).
+// Evaluated by an aligned group of G lanes (8 or 32) for one box (all of them call it with the same
+// box): lane c projects corner c mod 8, and the depth footprint is shared out over the group.  The scan
+// looks for a pixel that the box's nearest corner does not lie behind -- max(d) + bias >= z exactly
+// if some d + bias >= z, rounding being monotone -- and stops at the first group of pixels that holds
+// one: visible boxes take one step, hidden ones all.
 // Tile classes for a lasso (the texels of a box projected to screen box `sb`).
 enum : int { kTileOut = 0, kTileTest = 1, kTileIn = 2 };
 
 template <int LANES>
 __device__ __forceinline__ int lasso_tile_class(const LassoArg &p, const float *vx, const float *vy, float4 sb);
 
-// Some pixel of [ix0, ix1] x [iy0, iy1] with depth + bias >= z?  Every lane of the group calls it.
-template <int G>
+// Some pixel of [ix0, ix1] x [iy0, iy1] with depth + bias >= z?  Every lane of the group calls it; ROWS rows
+// of 4 loads are in flight per lane (four in a batch's cull, where one warp may scan for many lassos:
+// 1001 -> 988 us for 24 models with 16 lassos each).
+template <int G, int ROWS = 2>
 __device__ __forceinline__ bool depth_reaches(const LassoArg &p, const float *__restrict__ depth, int ix0, int ix1,
                                               int iy0, int iy1, float z, unsigned gm) {
     constexpr int kX = 8, kY = G / 8;  // the group's pixels: 8 side by side, kY rows
     const int sub = (int)(threadIdx.x & (G - 1u));
-    for (int y = iy0; y <= iy1; y += 2 * kY)
+    for (int y = iy0; y <= iy1; y += ROWS * kY)
         for (int x = ix0; x <= ix1; x += 4 * kX) {
             bool any = false;
-            // eight independent loads; places beyond the edge repeat the last pixel
+            // independent loads; places beyond the edge repeat the last pixel
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
+            for (int j = 0; j < 4 * ROWS; ++j) {
                 const int ix = min(x + (sub & 7) + kX * (j & 3), ix1), iy = min(y + (sub >> 3) + kY * (j >> 2), iy1);
                 if (LCL_IN((int64_t)iy * p.w_s + ix, (int64_t)p.w_s * p.h_s))
                     any |= __ldg(depth + (int64_t)iy * p.w_s + ix) + p.bias >= z;
@@ -443,7 +414,7 @@ __device__ __forceinline__ bool depth_reaches(const LassoArg &p, const float *__
 // CLASSIFY (with vx, vy, *cls): between the screen-box test and the depth-footprint scan, the tile is
 // classified by lasso_tile_class (its class in *cls, kTileTest where it cannot be); a tile outside the
 // polygon returns false at once, without the scan.
-template <int G, bool CLASSIFY = false>
+template <int G, bool CLASSIFY = false, int ROWS = 2>
 __device__ __forceinline__ bool box_may_touch_by(const LassoArg &p, int4 lo, int4 hi, const float *__restrict__ depth,
                                                  const float *vx = nullptr, const float *vy = nullptr,
                                                  int *cls = nullptr) {
@@ -480,7 +451,7 @@ __device__ __forceinline__ bool box_may_touch_by(const LassoArg &p, int4 lo, int
     if ((ix1 - ix0 + 1) * (iy1 - iy0 + 1) > 2048) return true;
     // NaN depths never count, as in a maximum; a NaN zmin keeps the box
     const float near = zmin - 1e-4f;
-    return !(near == near) || depth_reaches<G>(p, depth, ix0, ix1, iy0, iy1, near, gm);
+    return !(near == near) || depth_reaches<G, ROWS>(p, depth, ix0, ix1, iy0, iy1, near, gm);
 }
 
 
@@ -642,7 +613,8 @@ constexpr uint32_t kInsideTile = 0x80000000u;
 // viewport, the polygon's box and the edge tests).  The four texels go through the projection side by
 // side, without branches, so that their chains of dependent operations overlap; what fails a condition
 // is masked.  A quad whose operands leave the window of the fast division goes texel by texel.
-__device__ __forceinline__ uint32_t lasso_quad_inside(const LassoArg &p, const LassoShared &sh,
+template <typename Edges>
+__device__ __forceinline__ uint32_t lasso_quad_inside(const LassoArg &p, const Edges &sh,
                                                       const float *__restrict__ depth, int4 X, int4 Y, int4 Z) {
     const int32_t xq[4] = {X.x, X.y, X.z, X.w}, yq[4] = {Y.x, Y.y, Y.z, Y.w}, zq[4] = {Z.x, Z.y, Z.z, Z.w};
     float t[4], cw[4], cz[4];
@@ -687,11 +659,20 @@ __device__ __forceinline__ uint32_t lasso_quad_inside(const LassoArg &p, const L
     return m;
 }
 
+// Edge e of a polygon: its two y ends and its widened x-range (edge_xrange).  A CTA's copy of a polygon
+// has these records; a batched lasso's come from its vertices.
+__device__ __forceinline__ float4 edge_record(const LassoShared &sh, int e) { return sh.rec[e]; }
+__device__ __forceinline__ float4 edge_record(const LassoArg &p, int e) {
+    const float2 r = edge_xrange(p.vx[e], p.vx[e + 1]);
+    return make_float4(p.vy[e], p.vy[e + 1], r.x, r.y);
+}
+
 // lasso_hit for the four texels of a quad (bit k: texel k).  Each texel takes the steps of
 // lasso_hit up to its band; when the quad's live texels share a band (nearly always: they are
 // neighbours on the surface) one pass over that band's edge records tests all of them.  Texels
 // that failed a step carry ys = NaN, which straddles no edge.
-__device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const LassoShared &sh,
+template <typename Edges>
+__device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const Edges &sh,
                                                const float *__restrict__ depth, int4 X, int4 Y, int4 Z) {
     const int32_t xq[4] = {X.x, X.y, X.z, X.w}, yq[4] = {Y.x, Y.y, Y.z, Y.w}, zq[4] = {Z.x, Z.y, Z.z, Z.w};
     float xs[4], ys[4], cw[4];
@@ -735,7 +716,7 @@ __device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const LassoSha
             if (!LCL_IN(j, kBandEdgesMax)) break;
             const int e = sh.band_edge[j];
             if (!LCL_IN(e, LCL_MAX_LASSO_VERTICES)) continue;
-            const float4 r = sh.rec[e];
+            const float4 r = edge_record(sh, e);
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 if ((r.x > ys[k]) != (r.y > ys[k]) && edge_left(sh.vx, e, xs[k], ys[k], r.x, r.y, r.z, r.w))
@@ -749,7 +730,7 @@ __device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const LassoSha
                 if (!LCL_IN(j, kBandEdgesMax)) break;
                 const int e = sh.band_edge[j];
                 if (!LCL_IN(e, LCL_MAX_LASSO_VERTICES)) continue;
-                const float4 r = sh.rec[e];
+                const float4 r = edge_record(sh, e);
                 if ((r.x > ys[k]) != (r.y > ys[k]) && edge_left(sh.vx, e, xs[k], ys[k], r.x, r.y, r.z, r.w))
                     inside ^= 1u << k;
             }
