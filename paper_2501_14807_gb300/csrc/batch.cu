@@ -49,11 +49,31 @@ struct BStroke {
     SphereArg sphere;
 };
 
-struct BLasso {  // built on the device by k_batch_prep
-    LassoArg arg;
+// Built on the device by k_batch_prep.  Every texel of a crossing tile goes through the edges of its y-band,
+// so the edges have records (as in LassoShared) and the bands bit masks of them; with lists of bytes, and
+// the records worked out from the vertices at each use, the batch at k_batch_apply took 859 us instead of 806.
+struct BLasso : LassoHead {
+    float4 rec[LCL_MAX_LASSO_VERTICES];  // {ay, by, lo, hi}
+    uint2 band[kBands];                  // edges 0-31 and 32-63 of the band
     const float *depth;
     int32_t pad_r, pad_t;  // texture padding: kernel radius and outline thickness (0: none)
 };
+static_assert(sizeof(BLasso) % 16 == 0, "k_batch_prep copies it by 16-byte words");
+constexpr size_t kBLassoRoom = 2792;  // bytes of the workspace per lasso, which programs may have stored
+static_assert(sizeof(BLasso) <= kBLassoRoom, "lcl_batch_workspace_bytes");
+
+template <typename F>
+__device__ __forceinline__ void band_edges(const BLasso &L, int band, F f) {
+    const uint2 b = L.band[band];
+    for (uint32_t m = b.x; m; m &= m - 1) {
+        const int e = __ffs(m) - 1;
+        f(e, L.rec[e]);
+    }
+    for (uint32_t m = b.y; m; m &= m - 1) {
+        const int e = 31 + __ffs(m);
+        f(e, L.rec[e]);
+    }
+}
 
 struct BLassoIn {  // what the host uploads per lasso
     float m[16];
@@ -112,7 +132,7 @@ BLayout b_layout(const lcl_batch_limits &lim) {
     L.super_model = L.lasso_in + align256((size_t)std::max(lim.lassos, 1) * sizeof(BLassoIn));
     L.upload = L.super_model + align256((size_t)std::max<int64_t>(lim.supers, 1) * 4);
     L.lassos = L.upload;
-    L.items = L.lassos + align256((size_t)std::max(lim.lassos, 1) * sizeof(BLasso));
+    L.items = L.lassos + align256((size_t)std::max(lim.lassos, 1) * kBLassoRoom);
     L.total = L.items + align256((size_t)std::max<int64_t>(lim.tiles, 1) * sizeof(BItem)) +
               align256((size_t)std::max<int64_t>(lim.tiles, 1) * 16);
     return L;
@@ -132,7 +152,7 @@ __device__ __forceinline__ bool box_near(const BLasso &L, const int32_t *boxes, 
             if (!LCL_IN((int64_t)y * nx + x, (int64_t)nx * ny)) continue;
             const int4 *b = reinterpret_cast<const int4 *>(boxes + 8 * ((int64_t)y * nx + x));
             const int4 lo = b[0], hi = b[1];
-            if (lo.w > 0 && box_may_touch_by<8>(L.arg, lo, hi, depth)) return true;
+            if (lo.w > 0 && box_may_touch_by<8>(L, lo, hi, depth)) return true;
         }
     return false;
 }
@@ -141,8 +161,8 @@ constexpr int kPrepWarps = kThreads / 32;  // lassos per CTA of k_batch_prep
 static_assert(kBands == 32, "k_batch_prep gives each y-band one lane");
 
 // Resets the work counters and builds every lasso's argument, one warp per lasso:
-// the lanes copy the vertices and reduce their bounding box, then lane b counts and lists the edges of
-// band b (the same predicate, in the same edge order, as the host builder).
+// the lanes copy the vertices and reduce their bounding box, then lane b collects the edges of
+// band b (the same predicate as the host builder).
 __global__ void __launch_bounds__(kThreads) k_batch_prep(BHdr *hdr, const BLassoIn *__restrict__ in,
                                                          BLasso *__restrict__ out, BCaps caps) {
     pdl_allow_next();
@@ -151,14 +171,14 @@ __global__ void __launch_bounds__(kThreads) k_batch_prep(BHdr *hdr, const BLasso
         hdr->next_cull = 0;
         hdr->next_unit = 0;
     }
-    __shared__ LassoArg s_arg[kPrepWarps];
+    __shared__ BLasso s_arg[kPrepWarps];
     const int lane = threadIdx.x & 31;
     const int j = blockIdx.x * kPrepWarps + (int)(threadIdx.x / 32);
     if (j >= hdr->n_lassos) return;  // uniform over the warp
     if (!LCL_IN(j, caps.lassos)) return;
     (void)caps;
     const BLassoIn &L = in[j];
-    LassoArg &p = s_arg[threadIdx.x / 32];
+    BLasso &p = s_arg[threadIdx.x / 32];
     const int nv = L.nv;
     float x0 = INFINITY, x1 = -INFINITY, y0 = INFINITY, y1 = -INFINITY;
     for (int i = lane; i <= LCL_MAX_LASSO_VERTICES; i += 32) {  // vertices nv and on repeat vertex 0
@@ -180,29 +200,23 @@ __global__ void __launch_bounds__(kThreads) k_batch_prep(BHdr *hdr, const BLasso
     if (lane == 0) {
         lasso_arg_scalars(p, L.w_s, L.h_s, nv, L.label, L.bias);
         lasso_arg_box(p, x0, x1, y0, y1);
-        out[j].depth = L.depth;
-        out[j].pad_r = (int32_t)(L.flags & 15u);
-        out[j].pad_t = (int32_t)((L.flags >> 4) & 15u);
+        p.depth = L.depth;
+        p.pad_r = (int32_t)(L.flags & 15u);
+        p.pad_t = (int32_t)((L.flags >> 4) & 15u);
     }
     __syncwarp();
     const float bh = lasso_band_height(p);
     unsigned long long has = 0ull;  // edges of band `lane`
     for (int e = 0; e < nv; ++e)
         if (lasso_band_has(p, lane, e, bh)) has |= 1ull << e;
-    const int c = __popcll(has);
-    int incl = c;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
+    p.band[lane] = make_uint2((uint32_t)has, (uint32_t)(has >> 32));
+    for (int e = lane; e < nv; e += 32) {
+        const float2 r = edge_xrange(p.vx[e], p.vx[e + 1]);
+        p.rec[e] = make_float4(p.vy[e], p.vy[e + 1], r.x, r.y);
     }
-    int k = incl - c;
-    p.band_off[lane] = (uint16_t)k;
-    if (lane == 31) p.band_off[kBands] = (uint16_t)incl;
-    for (; has; has &= has - 1) p.band_edge[k++] = (uint8_t)(__ffsll((long long)has) - 1);
     __syncwarp();
-    static_assert(sizeof(LassoArg) % 4 == 0, "LassoArg is copied by words");
-    for (int i = lane; i < (int)(sizeof(LassoArg) / 4); i += 32)
-        reinterpret_cast<uint32_t *>(&out[j].arg)[i] = reinterpret_cast<const uint32_t *>(&p)[i];
+    for (int i = lane; i < (int)(sizeof(BLasso) / 16); i += 32)
+        reinterpret_cast<uint4 *>(&out[j])[i] = reinterpret_cast<const uint4 *>(&p)[i];
 }
 
 // Bit number n (from 0) of the set bits of m, which has more than n.
@@ -322,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch_cull(BHdr *hdr, const BMo
                 if (pads >> k & 1ull)
                     can = here && box_near(L, a.tile_box, a.tiles_x, a.tiles_y, tx, ty, 1, L.depth);
                 else if (lo.w > 0)
-                    can = box_may_touch_by<8, true, 4>(L.arg, lo, hi, L.depth, L.arg.vx, L.arg.vy, &cls);
+                    can = box_may_touch_by<8, true, 4>(L, lo, hi, L.depth, L.vx, L.vy, &cls);
                 if (can) {
                     mask |= 1ull << k;
                     if (cls == kTileIn) sure |= 1ull << k;
@@ -355,7 +369,7 @@ __device__ __forceinline__ bool stroke_selects(const AtlasDev &a, const BStroke 
         return dx * dx + dy * dy + dz * dz <= st.sphere.r2;
     }
     const BLasso &ls = lassos[st.lasso];
-    return lasso_hit(ls.arg, ls.arg, ls.depth, qx, __ldg(a.py + n), __ldg(a.pz + n));
+    return lasso_hit(ls, ls, ls.depth, qx, __ldg(a.py + n), __ldg(a.pz + n));
 }
 
 // Texture padding of the uncovered texels `unc` of the quad at l: for each, the masked padded strokes
@@ -395,7 +409,7 @@ __device__ __noinline__ uint32_t pad_texels(const AtlasDev &a, int64_t l, uint32
                 }
             }
             if (outline && near) {
-                lab[k] = st.kind == LCL_STROKE_SPHERE ? st.sphere.label : lassos[st.lasso].arg.label;
+                lab[k] = st.kind == LCL_STROKE_SPHERE ? st.sphere.label : lassos[st.lasso].label;
                 written |= 1u << k;
                 break;
             }
@@ -414,8 +428,8 @@ __device__ __forceinline__ uint32_t lasso_texels(const BLasso &ls, int4 X, int4 
         const int32_t qx = k == 0 ? X.x : k == 1 ? X.y : k == 2 ? X.z : X.w;
         const int32_t qy = k == 0 ? Y.x : k == 1 ? Y.y : k == 2 ? Y.z : Y.w;
         const int32_t qz = k == 0 ? Z.x : k == 1 ? Z.y : k == 2 ? Z.z : Z.w;
-        if (sure ? lasso_hit<true>(ls.arg, ls.arg, ls.depth, qx, qy, qz)
-                 : lasso_hit<false>(ls.arg, ls.arg, ls.depth, qx, qy, qz))
+        if (sure ? lasso_hit<true>(ls, ls, ls.depth, qx, qy, qz)
+                 : lasso_hit<false>(ls, ls, ls.depth, qx, qy, qz))
             sel |= 1u << k;
     }
     return sel;
@@ -468,7 +482,7 @@ __device__ __forceinline__ void apply_quads(const BModel &M, const BItem &it, in
             }
         } else {
             const BLasso &ls = lassos[st.lasso];
-            label = ls.arg.label;
+            label = ls.label;
             sel = lasso_texels(ls, X, Y, Z, open, sure);
         }
 #pragma unroll
@@ -501,7 +515,7 @@ __device__ __forceinline__ void apply_quads(const BModel &M, const BItem &it, in
 // than registers: with 3, 4, 5 and 6 CTAs per SM that batch took 1141, 1023, 1014 and 974 us.  The four
 // texels of a quad side by side, as in the single lasso's apply, need 80 registers and more code than the
 // instruction cache holds: 1484 us.  All of the batch: 1314 us before (a CTA per ticket, 3 per SM, padded
-// strokes looked for at every uncovered texel), now 877.
+// strokes looked for at every uncovered texel), now 806.
 constexpr int kItemTicketsLog = 3;
 
 __global__ void __launch_bounds__(256, 6) k_batch_apply(const BHdr *__restrict__ hdr, const BModel *__restrict__ models,

@@ -308,18 +308,22 @@ cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, cudaStream_t st, A... ar
 constexpr int kBands = 32;                                    // y-bands of lasso edges
 constexpr int kBandEdgesMax = kBands * LCL_MAX_LASSO_VERTICES;
 
-struct LassoArg {
+struct alignas(16) LassoHead {  // in groups of four words, which the kernels load at once
     float m[16];
     float ws, hs;           // screen size as float
     int32_t w_s, h_s;
     float bias;
     uint32_t label;
-    int32_t nv;
+    int32_t nv, unused;
     float bx0, by0, bx1, by1;  // polygon bbox (clipped to the screen) widened by a margin, pixels
     float nx0, nx1, ny0, ny1;  // the same widened bbox in NDC, for the division-free reject
     float ymin, ymax;          // exact vertical extent of the polygon
     float band_y0, band_inv_h; // band of a point: floor((y - band_y0) * band_inv_h), clamped
     float vx[LCL_MAX_LASSO_VERTICES + 1], vy[LCL_MAX_LASSO_VERTICES + 1];  // vertex nv = vertex 0
+};
+
+// With the edges of each y-band: a kernel's argument.
+struct LassoArg : LassoHead {
     uint16_t band_off[kBands + 1];
     uint8_t band_edge[kBandEdgesMax];  // edge e runs from vertex e to vertex e + 1
 };
@@ -386,13 +390,13 @@ __device__ __forceinline__ void stage_lasso(LassoShared &sh, const LassoArg &p) 
 enum : int { kTileOut = 0, kTileTest = 1, kTileIn = 2 };
 
 template <int LANES>
-__device__ __forceinline__ int lasso_tile_class(const LassoArg &p, const float *vx, const float *vy, float4 sb);
+__device__ __forceinline__ int lasso_tile_class(const LassoHead &p, const float *vx, const float *vy, float4 sb);
 
 // Some pixel of [ix0, ix1] x [iy0, iy1] with depth + bias >= z?  Every lane of the group calls it; ROWS rows
 // of 4 loads are in flight per lane (four in a batch's cull, where one warp may scan for many lassos:
 // 1001 -> 988 us for 24 models with 16 lassos each).
 template <int G, int ROWS = 2>
-__device__ __forceinline__ bool depth_reaches(const LassoArg &p, const float *__restrict__ depth, int ix0, int ix1,
+__device__ __forceinline__ bool depth_reaches(const LassoHead &p, const float *__restrict__ depth, int ix0, int ix1,
                                               int iy0, int iy1, float z, unsigned gm) {
     constexpr int kX = 8, kY = G / 8;  // the group's pixels: 8 side by side, kY rows
     const int sub = (int)(threadIdx.x & (G - 1u));
@@ -415,7 +419,7 @@ __device__ __forceinline__ bool depth_reaches(const LassoArg &p, const float *__
 // classified by lasso_tile_class (its class in *cls, kTileTest where it cannot be); a tile outside the
 // polygon returns false at once, without the scan.
 template <int G, bool CLASSIFY = false, int ROWS = 2>
-__device__ __forceinline__ bool box_may_touch_by(const LassoArg &p, int4 lo, int4 hi, const float *__restrict__ depth,
+__device__ __forceinline__ bool box_may_touch_by(const LassoHead &p, int4 lo, int4 hi, const float *__restrict__ depth,
                                                  const float *vx = nullptr, const float *vy = nullptr,
                                                  int *cls = nullptr) {
     const unsigned lane = threadIdx.x & 31u, sub = lane & 7u;
@@ -472,7 +476,7 @@ __device__ __forceinline__ bool box_may_touch_by(const LassoArg &p, int4 lo, int
 // vx, vy: the polygon's vertices (vertex nv = vertex 0), staged in shared memory by the caller so
 // that the lanes' different edges are not serialised on the parameter bank.
 template <int LANES>
-__device__ __forceinline__ int lasso_tile_class(const LassoArg &p, const float *vx, const float *vy, float4 sb) {
+__device__ __forceinline__ int lasso_tile_class(const LassoHead &p, const float *vx, const float *vy, float4 sb) {
     const unsigned lane = threadIdx.x & 31u, sub = lane & (LANES - 1u);
     const unsigned gm = LANES == 32 ? 0xFFFFFFFFu : 0xFFu << (lane & 24u);
     if (!(isfinite(sb.x) && isfinite(sb.y) && isfinite(sb.z) && isfinite(sb.w))) return kTileTest;  // uniform
@@ -534,6 +538,16 @@ __device__ __forceinline__ bool quot_le(float a, float b, float t) {
     return div_rn(a, b) <= t;
 }
 
+// Calls f(e, record) for the edges of a y-band.
+template <typename F>
+__device__ __forceinline__ void band_edges(const LassoShared &sh, int band, F f) {
+    for (int k = sh.band_off[band]; k < sh.band_off[band + 1]; ++k) {
+        if (!LCL_IN(k, kBandEdgesMax)) break;
+        const int e = sh.band_edge[k];
+        if (LCL_IN(e, LCL_MAX_LASSO_VERTICES)) f(e, sh.rec[e]);
+    }
+}
+
 // The lasso test of one texel.  The conditions of the definition are all required, so they are
 // evaluated cheapest first; every value that decides the result is computed in the exact FP32
 // order of the definition.  Two shortcuts are exact as well:
@@ -547,7 +561,7 @@ __device__ __forceinline__ bool quot_le(float a, float b, float t) {
 // INSIDE: the texel's tile is known to lie inside the polygon (lasso_tile_class): the edge tests,
 // whose outcome would be "inside", are skipped.
 template <bool INSIDE = false, typename Edges>
-__device__ __forceinline__ bool lasso_hit(const LassoArg &p, const Edges &sh, const float *__restrict__ depth,
+__device__ __forceinline__ bool lasso_hit(const LassoHead &p, const Edges &sh, const float *__restrict__ depth,
                                           int32_t X, int32_t Y, int32_t Z) {
     if (X == INT32_MIN) return false;  // uncovered
     const float fx = (float)X, fy = (float)Y, fz = (float)Z;
@@ -565,16 +579,10 @@ __device__ __forceinline__ bool lasso_hit(const LassoArg &p, const Edges &sh, co
     int band = __float2int_rz(__fmul_rn(__fsub_rn(ys, p.band_y0), p.band_inv_h));
     band = band < 0 ? 0 : (band >= kBands ? kBands - 1 : band);
     bool inside = INSIDE;
-    for (int k = sh.band_off[band]; !INSIDE && k < sh.band_off[band + 1]; ++k) {
-        if (!LCL_IN(k, kBandEdgesMax)) break;
-        const int e = sh.band_edge[k];
-        if (!LCL_IN(e, LCL_MAX_LASSO_VERTICES)) continue;
-        const float ax = sh.vx[e], ay = sh.vy[e], bx = sh.vx[e + 1], by = sh.vy[e + 1];
-        if ((ay > ys) != (by > ys)) {
-            const float2 r = edge_xrange(ax, bx);
-            if (edge_left(sh.vx, e, xs, ys, ay, by, r.x, r.y)) inside = !inside;
-        }
-    }
+    if (!INSIDE)
+        band_edges(sh, band, [&](int e, float4 r) {
+            if ((r.x > ys) != (r.y > ys) && edge_left(p.vx, e, xs, ys, r.x, r.y, r.z, r.w)) inside = !inside;
+        });
     if (!inside) return false;
     // NDC depth zn = RN(cz / cw) in [0, 1] and zn <= depth + bias, decided as quot_* describes
     const float cz = clip_row(p.m + 8, fx, fy, fz);
@@ -588,7 +596,7 @@ __device__ __forceinline__ bool lasso_hit(const LassoArg &p, const Edges &sh, co
 
 // The depth test (Fig. 3a) of the texels `live` of a quad that passed the other steps: NDC depth in
 // [0, 1] and z <= depth[floor(ys)][floor(xs)] + bias.
-__device__ __forceinline__ uint32_t lasso_depth_quad(const LassoArg &p, const float *__restrict__ depth,
+__device__ __forceinline__ uint32_t lasso_depth_quad(const LassoHead &p, const float *__restrict__ depth,
                                                      const int32_t (&xq)[4], const int32_t (&yq)[4],
                                                      const int32_t (&zq)[4], const float (&xs)[4],
                                                      const float (&ys)[4], const float (&cw)[4], uint32_t live) {
@@ -613,8 +621,7 @@ constexpr uint32_t kInsideTile = 0x80000000u;
 // viewport, the polygon's box and the edge tests).  The four texels go through the projection side by
 // side, without branches, so that their chains of dependent operations overlap; what fails a condition
 // is masked.  A quad whose operands leave the window of the fast division goes texel by texel.
-template <typename Edges>
-__device__ __forceinline__ uint32_t lasso_quad_inside(const LassoArg &p, const Edges &sh,
+__device__ __forceinline__ uint32_t lasso_quad_inside(const LassoHead &p, const LassoShared &sh,
                                                       const float *__restrict__ depth, int4 X, int4 Y, int4 Z) {
     const int32_t xq[4] = {X.x, X.y, X.z, X.w}, yq[4] = {Y.x, Y.y, Y.z, Y.w}, zq[4] = {Z.x, Z.y, Z.z, Z.w};
     float t[4], cw[4], cz[4];
@@ -659,20 +666,11 @@ __device__ __forceinline__ uint32_t lasso_quad_inside(const LassoArg &p, const E
     return m;
 }
 
-// Edge e of a polygon: its two y ends and its widened x-range (edge_xrange).  A CTA's copy of a polygon
-// has these records; a batched lasso's come from its vertices.
-__device__ __forceinline__ float4 edge_record(const LassoShared &sh, int e) { return sh.rec[e]; }
-__device__ __forceinline__ float4 edge_record(const LassoArg &p, int e) {
-    const float2 r = edge_xrange(p.vx[e], p.vx[e + 1]);
-    return make_float4(p.vy[e], p.vy[e + 1], r.x, r.y);
-}
-
 // lasso_hit for the four texels of a quad (bit k: texel k).  Each texel takes the steps of
 // lasso_hit up to its band; when the quad's live texels share a band (nearly always: they are
 // neighbours on the surface) one pass over that band's edge records tests all of them.  Texels
 // that failed a step carry ys = NaN, which straddles no edge.
-template <typename Edges>
-__device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const Edges &sh,
+__device__ __forceinline__ uint32_t lasso_quad(const LassoHead &p, const LassoShared &sh,
                                                const float *__restrict__ depth, int4 X, int4 Y, int4 Z) {
     const int32_t xq[4] = {X.x, X.y, X.z, X.w}, yq[4] = {Y.x, Y.y, Y.z, Y.w}, zq[4] = {Z.x, Z.y, Z.z, Z.w};
     float xs[4], ys[4], cw[4];
@@ -716,7 +714,7 @@ __device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const Edges &s
             if (!LCL_IN(j, kBandEdgesMax)) break;
             const int e = sh.band_edge[j];
             if (!LCL_IN(e, LCL_MAX_LASSO_VERTICES)) continue;
-            const float4 r = edge_record(sh, e);
+            const float4 r = sh.rec[e];
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 if ((r.x > ys[k]) != (r.y > ys[k]) && edge_left(sh.vx, e, xs[k], ys[k], r.x, r.y, r.z, r.w))
@@ -730,7 +728,7 @@ __device__ __forceinline__ uint32_t lasso_quad(const LassoArg &p, const Edges &s
                 if (!LCL_IN(j, kBandEdgesMax)) break;
                 const int e = sh.band_edge[j];
                 if (!LCL_IN(e, LCL_MAX_LASSO_VERTICES)) continue;
-                const float4 r = edge_record(sh, e);
+                const float4 r = sh.rec[e];
                 if ((r.x > ys[k]) != (r.y > ys[k]) && edge_left(sh.vx, e, xs[k], ys[k], r.x, r.y, r.z, r.w))
                     inside ^= 1u << k;
             }
@@ -756,7 +754,7 @@ struct ToolArg {
 // Tool test of one texel: projection, viewport and depth test as for lassos (the window's
 // bounding box, widened, in p's division-free reject), then the shape (MASK) or the circle.
 template <bool MASK>
-__device__ __forceinline__ bool tool_hit(const LassoArg &p, const ToolArg &t, const float *__restrict__ depth,
+__device__ __forceinline__ bool tool_hit(const LassoHead &p, const ToolArg &t, const float *__restrict__ depth,
                                          int32_t X, int32_t Y, int32_t Z) {
     if (X == INT32_MIN) return false;  // uncovered
     const float fx = (float)X, fy = (float)Y, fz = (float)Z;
@@ -807,12 +805,12 @@ inline int resident_grid(K kernel) {
 // y-bands of edges: band b lists the edges whose y-range comes within `slack` of it, in edge order.
 // The slack is far above the rounding of a point's band (floor((y - band_y0) * band_inv_h), a few ulps)
 // and of the bounds below; an edge too many in a band changes nothing.
-__host__ __device__ inline float lasso_band_height(const LassoArg &p) {
+__host__ __device__ inline float lasso_band_height(const LassoHead &p) {
     return fmaxf(p.ymax - p.ymin, 1e-3f) * (1.0f / kBands);
 }
 
 // The lasso argument's scalars but for the polygon's: matrix, screen, label, bias.
-__host__ __device__ inline void lasso_arg_scalars(LassoArg &p, int32_t w_s, int32_t h_s, int32_t nv, uint32_t label,
+__host__ __device__ inline void lasso_arg_scalars(LassoHead &p, int32_t w_s, int32_t h_s, int32_t nv, uint32_t label,
                                                   float bias) {
     p.ws = (float)w_s;
     p.hs = (float)h_s;
@@ -824,7 +822,7 @@ __host__ __device__ inline void lasso_arg_scalars(LassoArg &p, int32_t w_s, int3
 }
 
 // What follows from the polygon's bounding box: the widened box in pixels and NDC, the band mapping.
-__host__ __device__ inline void lasso_arg_box(LassoArg &p, float x0, float x1, float y0, float y1) {
+__host__ __device__ inline void lasso_arg_box(LassoHead &p, float x0, float x1, float y0, float y1) {
     // Culling and the division-free reject use the bbox widened by a margin far above the FP32
     // rounding of projected points (well under a thousandth of a pixel at these sizes).
     const float margin = 2.0f + 1e-3f * (float)(p.w_s > p.h_s ? p.w_s : p.h_s);
@@ -844,7 +842,7 @@ __host__ __device__ inline void lasso_arg_box(LassoArg &p, float x0, float x1, f
 
 // The lasso argument without its y-bands (vertex nv repeated as vertex 0), on the host; batched edits
 // build theirs on the device, a lane per vertex (k_batch_prep).
-inline void lasso_arg_head(LassoArg &p, const float *m16, int32_t w_s, int32_t h_s, const float *poly, int32_t nv,
+inline void lasso_arg_head(LassoHead &p, const float *m16, int32_t w_s, int32_t h_s, const float *poly, int32_t nv,
                            uint32_t label, float bias) {
     for (int i = 0; i < 16; ++i) p.m[i] = m16[i];
     lasso_arg_scalars(p, w_s, h_s, nv, label, bias);
@@ -864,7 +862,7 @@ inline void lasso_arg_head(LassoArg &p, const float *m16, int32_t w_s, int32_t h
     lasso_arg_box(p, x0, x1, y0, y1);
 }
 
-__host__ __device__ inline bool lasso_band_has(const LassoArg &p, int b, int e, float bh) {
+__host__ __device__ inline bool lasso_band_has(const LassoHead &p, int b, int e, float bh) {
     const float slack = 2e-3f * bh + 2e-3f + 1e-6f * (fabsf(p.ymin) + fabsf(p.ymax));
     const float lo = p.ymin + (float)b * bh - slack, hi = p.ymin + (float)(b + 1) * bh + slack;
     const float ea = p.vy[e], eb = p.vy[e + 1];
