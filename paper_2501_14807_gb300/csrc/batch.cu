@@ -515,7 +515,7 @@ __device__ __forceinline__ void apply_quads(const BModel &M, const BItem &it, in
 // than registers: with 3, 4, 5 and 6 CTAs per SM that batch took 1141, 1023, 1014 and 974 us.  The four
 // texels of a quad side by side, as in the single lasso's apply, need 80 registers and more code than the
 // instruction cache holds: 1484 us.  All of the batch: 1314 us before (a CTA per ticket, 3 per SM, padded
-// strokes looked for at every uncovered texel), now 806.
+// strokes looked for at every uncovered texel), now 696.
 constexpr int kItemTicketsLog = 3;
 
 __global__ void __launch_bounds__(256, 6) k_batch_apply(const BHdr *__restrict__ hdr, const BModel *__restrict__ models,

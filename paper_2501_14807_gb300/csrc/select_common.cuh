@@ -549,8 +549,10 @@ __device__ __forceinline__ void band_edges(const LassoShared &sh, int band, F f)
 }
 
 // The lasso test of one texel.  The conditions of the definition are all required, so they are
-// evaluated cheapest first; every value that decides the result is computed in the exact FP32
-// order of the definition.  Two shortcuts are exact as well:
+// evaluated cheapest first -- the depth test before the polygon's edges, of which a band has about ten:
+// 24 models with 16 lassos each took 806 us with the edges first and 696 now, 12 lassos on a 4096^2
+// atlas 407 and 381, 5 on 16384^2 876 and 825.  Every value that decides the result is computed in the
+// exact FP32 order of the definition.  Two shortcuts are exact as well:
 //  - a point more than the margin outside the polygon's bounding box (clipped to the screen) is
 //    off screen or outside the polygon: left of every vertex each straddling edge counts, and a
 //    closed polygon has an even number of those; right of every vertex none counts.  The test
@@ -576,6 +578,13 @@ __device__ __forceinline__ bool lasso_hit(const LassoHead &p, const Edges &sh, c
     const float ys = screen_of(div_by(cy, dw), p.hs);
     if (!(xs >= 0.0f && xs < p.ws && ys >= 0.0f && ys < p.hs)) return false;
     if (!(ys >= p.ymin && ys < p.ymax)) return false;  // no edge straddles y
+    // NDC depth zn = RN(cz / cw) in [0, 1] and zn <= depth + bias, decided as quot_* describes
+    const float cz = clip_row(p.m + 8, fx, fy, fz);
+    if (!(quot_ge0(cz, cw) && quot_le(cz, cw, 1.0f))) return false;
+    const int32_t ix = __float2int_rz(xs), iy = __float2int_rz(ys);
+    if (!LCL_IN((int64_t)iy * p.w_s + ix, (int64_t)p.w_s * p.h_s)) return false;
+    const float d = __ldg(depth + (int64_t)iy * p.w_s + ix);
+    if (!quot_le(cz, cw, __fadd_rn(d, p.bias))) return false;
     int band = __float2int_rz(__fmul_rn(__fsub_rn(ys, p.band_y0), p.band_inv_h));
     band = band < 0 ? 0 : (band >= kBands ? kBands - 1 : band);
     bool inside = INSIDE;
@@ -583,14 +592,7 @@ __device__ __forceinline__ bool lasso_hit(const LassoHead &p, const Edges &sh, c
         band_edges(sh, band, [&](int e, float4 r) {
             if ((r.x > ys) != (r.y > ys) && edge_left(p.vx, e, xs, ys, r.x, r.y, r.z, r.w)) inside = !inside;
         });
-    if (!inside) return false;
-    // NDC depth zn = RN(cz / cw) in [0, 1] and zn <= depth + bias, decided as quot_* describes
-    const float cz = clip_row(p.m + 8, fx, fy, fz);
-    if (!(quot_ge0(cz, cw) && quot_le(cz, cw, 1.0f))) return false;
-    const int32_t ix = __float2int_rz(xs), iy = __float2int_rz(ys);
-    if (!LCL_IN((int64_t)iy * p.w_s + ix, (int64_t)p.w_s * p.h_s)) return false;
-    const float d = __ldg(depth + (int64_t)iy * p.w_s + ix);
-    return quot_le(cz, cw, __fadd_rn(d, p.bias));
+    return inside;
 }
 
 
@@ -669,7 +671,8 @@ __device__ __forceinline__ uint32_t lasso_quad_inside(const LassoHead &p, const 
 // lasso_hit for the four texels of a quad (bit k: texel k).  Each texel takes the steps of
 // lasso_hit up to its band; when the quad's live texels share a band (nearly always: they are
 // neighbours on the surface) one pass over that band's edge records tests all of them.  Texels
-// that failed a step carry ys = NaN, which straddles no edge.
+// that failed a step carry ys = NaN, which straddles no edge.  The depth test comes before the edges
+// (as in lasso_hit).
 __device__ __forceinline__ uint32_t lasso_quad(const LassoHead &p, const LassoShared &sh,
                                                const float *__restrict__ depth, int4 X, int4 Y, int4 Z) {
     const int32_t xq[4] = {X.x, X.y, X.z, X.w}, yq[4] = {Y.x, Y.y, Y.z, Y.w}, zq[4] = {Z.x, Z.y, Z.z, Z.w};
@@ -703,7 +706,14 @@ __device__ __forceinline__ uint32_t lasso_quad(const LassoHead &p, const LassoSh
         band[k] = b;
         live |= 1u << k;
     }
+    if (live) live = lasso_depth_quad(p, depth, xq, yq, zq, xs, ys, cw, live);
     if (!live) return 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (!(live & (1u << k))) {
+            ys[k] = __int_as_float(0x7fc00000);
+            band[k] = -1;
+        }
     const int b0 = (live & 1u) ? band[0] : (live & 2u) ? band[1] : (live & 4u) ? band[2] : band[3];
     bool same = true;
 #pragma unroll
@@ -734,7 +744,7 @@ __device__ __forceinline__ uint32_t lasso_quad(const LassoHead &p, const LassoSh
             }
         }
     }
-    return lasso_depth_quad(p, depth, xq, yq, zq, xs, ys, cw, live & inside);
+    return live & inside;
 }
 
 
