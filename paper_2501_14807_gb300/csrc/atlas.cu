@@ -15,7 +15,7 @@
 //                 small triangles; big triangles are split into 16x16-texel blocks appended to a
 //                 work list
 //   k_raster_big  one CTA per (triangle, block) entry
-//   k_resolve     one CTA per tile, one texel per thread and step: position of every covered texel
+//   k_resolve     one warp or CTA per tile, one texel per lane and step: position of every covered texel
 //                 (from the triangle's planes where their rounding cannot matter, else exact
 //                 barycentrics), coverage bits, tile box
 //   k_super       one CTA per super-tile: union of its tile boxes
@@ -627,23 +627,35 @@ __device__ __forceinline__ int3 plane_position(const TriPlane *__restrict__ plan
                      rc.z + (int32_t)__funnelshift_r((uint32_t)vz, (uint32_t)(vz >> 32), s));
 }
 
-// One CTA per tile.  WORDS (tile side 32 or more, width a multiple of 32): a warp takes 32-texel row
-// segments, each one aligned coverage word, a texel per lane.  Otherwise one texel per thread and
-// step, a tile row after the other.  Either way warps read the triangle plane and write the position
-// planes in long rows, and the texels of one triangle, which lie together, find its planes in L1.
-// Bound by the latency of the chain triangle id -> planes (47% of issue slots, a third of DRAM): 1.83 ms
-// at 16384^2 with 8 M triangles, where exact barycentrics for every texel (290 instructions) took 2.79.
-// Slower: planes in binary32 (their error sent a tenth of the warps to exact_position: 2.28 ms), four
-// segments in flight per warp (1.95 ms, spills), five or six CTAs per SM (spills).
-template <bool WORDS>
+// WORDS (tile side 32 or more, width a multiple of 32): a warp takes 32-texel row segments, each one
+// aligned coverage word, a texel per lane; otherwise one texel per thread and step, a tile row after the
+// other.  Either way warps read the triangle plane and write the position planes in long rows, and the
+// texels of one triangle, which lie together, find its planes in L1.  WARP: a tile per warp, all its
+// segments from top to bottom, else a tile per CTA.  Bound by the latency of the chain triangle id ->
+// planes and by issue (140 instructions per segment, 55% of the cycles): with a CTA per tile of 32 a warp
+// had four segments between the latency of its first ids and the reduction of the box.  16384^2, 8 M
+// triangles: 1.83 ms by CTAs, 1.39 by warps; exact barycentrics for every texel (290 instructions) took
+// 2.79.  Slower: planes in binary32 (their error sent a tenth of the warps to exact_position), four
+// segments in flight per warp (spills), three or five CTAs per SM (1.69 and 1.61 ms), planes prefetched
+// to L1 a segment ahead (no change by warps, 1.71 ms by CTAs).
+// The rule: enough tiles that each of the chip's 4864 warps gets several, weighed by their rows.  With
+// tiles of 32 the whole build takes 802 and 916 us (by warps, by CTAs) on 8192^2, 329 and 353 on 4096^2,
+// 222 and 225 on 2048^2 (4096 tiles: below the line); of 64 on 16384^2 2610 and 2733, on 8192^2 (16384
+// tiles: below the line) 838 and 832.
+constexpr int32_t kWarpTiles = 16384;  // of 32 texels
+
+template <bool WORDS, bool WARP>
 __global__ void __launch_bounds__(kThreads, 4) k_resolve(const TriPlane *__restrict__ planes,
                                                       const __grid_constant__ MeshRefs mesh, int32_t w, int32_t h,
-                                                      int32_t row0, int32_t T,
+                                                      int32_t row0, int32_t T, int32_t tiles_x, int32_t n_tiles,
                                                       const uint32_t *__restrict__ tri_plane,
                                                       int32_t *__restrict__ px, int32_t *__restrict__ py,
                                                       int32_t *__restrict__ pz, uint32_t *__restrict__ cover,
                                                       int32_t *__restrict__ tile_box) {
-    const int32_t tx = blockIdx.x, ty = blockIdx.y;
+    static_assert(WORDS || !WARP, "a warp per tile takes whole words");
+    const int32_t tile = WARP ? (int32_t)(blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) : (int32_t)blockIdx.x;
+    if (WARP && tile >= n_tiles) return;
+    const int32_t ty = tile / tiles_x, tx = tile - ty * tiles_x;
     int32_t mn[3] = {INT32_MAX, INT32_MAX, INT32_MAX}, mx[3] = {INT32_MIN, INT32_MIN, INT32_MIN};
     int32_t cnt = 0;
     const int tshift = __ffs(T) - 1;  // T is a power of two
@@ -670,14 +682,16 @@ __global__ void __launch_bounds__(kThreads, 4) k_resolve(const TriPlane *__restr
             y = (ty << tshift) + (i >> slog);
             return i < n_words && x < w && y < h;  // x < w implies x + 31 < w
         };
+        constexpr int kStep = WARP ? 1 : kThreads / 32;
+        const int i0 = WARP ? 0 : (int)(threadIdx.x >> 5);
         int32_t nx, ny;
-        bool nv = place((int)(threadIdx.x >> 5), nx, ny);
+        bool nv = place(i0, nx, ny);
         uint32_t nt = nv ? __ldcs(tri_plane + (ny * w + nx + lane)) : kNone;
-        for (int i = (int)(threadIdx.x >> 5); i < n_words; i += kThreads / 32) {  // uniform over the warp
+        for (int i = i0; i < n_words; i += kStep) {  // uniform over the warp
             const int32_t x = nx, y = ny;
             const bool v = nv;
             const uint32_t t = nt;
-            nv = place(i + kThreads / 32, nx, ny);
+            nv = place(i + kStep, nx, ny);
             nt = nv ? __ldcs(tri_plane + (ny * w + nx + lane)) : kNone;
             if (!v) continue;
             const int32_t l = y * w + x + lane;  // below 2^28
@@ -713,26 +727,26 @@ __global__ void __launch_bounds__(kThreads, 4) k_resolve(const TriPlane *__restr
     v[4] = __reduce_max_sync(0xffffffffu, mx[0]);
     v[5] = __reduce_max_sync(0xffffffffu, mx[1]);
     v[6] = __reduce_max_sync(0xffffffffu, mx[2]);
-    const int wid = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0)
-        for (int k = 0; k < 7; ++k) red[k][wid] = v[k];
-    __syncthreads();
-    if (threadIdx.x < 32) {  // lane j holds warp j's values
-        const int j = threadIdx.x & (kThreads / 32 - 1);
-        v[0] = __reduce_min_sync(0xffffffffu, red[0][j]);
-        v[1] = __reduce_min_sync(0xffffffffu, red[1][j]);
-        v[2] = __reduce_min_sync(0xffffffffu, red[2][j]);
-        v[3] = __reduce_add_sync(0xffffffffu, threadIdx.x < kThreads / 32 ? red[3][j] : 0);
-        v[4] = __reduce_max_sync(0xffffffffu, red[4][j]);
-        v[5] = __reduce_max_sync(0xffffffffu, red[5][j]);
-        v[6] = __reduce_max_sync(0xffffffffu, red[6][j]);
-    }
-    if (threadIdx.x == 0) {
-        if (LCL_IN((int64_t)ty * gridDim.x + tx, (int64_t)((w + T - 1) / T) * ((h + T - 1) / T))) {
-            int32_t *b = tile_box + 8 * ((int64_t)ty * gridDim.x + tx);
-            reinterpret_cast<int4 *>(b)[0] = make_int4(v[0], v[1], v[2], v[3]);
-            reinterpret_cast<int4 *>(b)[1] = make_int4(v[4], v[5], v[6], 0);
+    if (!WARP) {
+        const int wid = threadIdx.x >> 5;
+        if ((threadIdx.x & 31) == 0)
+            for (int k = 0; k < 7; ++k) red[k][wid] = v[k];
+        __syncthreads();
+        if (threadIdx.x < 32) {  // lane j holds warp j's values
+            const int j = threadIdx.x & (kThreads / 32 - 1);
+            v[0] = __reduce_min_sync(0xffffffffu, red[0][j]);
+            v[1] = __reduce_min_sync(0xffffffffu, red[1][j]);
+            v[2] = __reduce_min_sync(0xffffffffu, red[2][j]);
+            v[3] = __reduce_add_sync(0xffffffffu, threadIdx.x < kThreads / 32 ? red[3][j] : 0);
+            v[4] = __reduce_max_sync(0xffffffffu, red[4][j]);
+            v[5] = __reduce_max_sync(0xffffffffu, red[5][j]);
+            v[6] = __reduce_max_sync(0xffffffffu, red[6][j]);
         }
+    }
+    if ((WARP ? threadIdx.x & 31u : threadIdx.x) == 0 && LCL_IN(tile, n_tiles)) {
+        int32_t *b = tile_box + 8 * (int64_t)tile;
+        reinterpret_cast<int4 *>(b)[0] = make_int4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<int4 *>(b)[1] = make_int4(v[4], v[5], v[6], 0);
     }
 }
 
@@ -847,11 +861,16 @@ lcl_status atlas_build_impl(const lcl_mesh *mesh, lcl_atlas *at, void *ws, size_
     ra.big = big;
     ra.big_cap = (int64_t)big_capacity(mesh->n_tri, at->width, at->height);  // blocks of this atlas's rows
     const unsigned rg = (unsigned)((mesh->n_tri + 127) / 128);
-    const dim3 tg(at->tiles_x, at->tiles_y), sg(at->supers_x, at->supers_y);
+    const dim3 sg(at->supers_x, at->supers_y);
+    const int32_t n_tiles = at->tiles_x * at->tiles_y;
     auto resolve = [&]() {
-        auto kernel = at->tile >= 32 && (at->width & 31) == 0 ? k_resolve<true> : k_resolve<false>;
-        kernel<<<tg, kThreads, 0, st>>>(planes, mr, at->width, at->height, at->row0, at->tile, at->tri, at->pos_x,
-                                        at->pos_y, at->pos_z, at->cover, at->tile_box);
+        const bool words = at->tile >= 32 && (at->width & 31) == 0;
+        const bool by_warp = words && n_tiles >= kWarpTiles / 32 * at->tile;
+        auto kernel = by_warp ? k_resolve<true, true> : words ? k_resolve<true, false> : k_resolve<false, false>;
+        const int per_cta = by_warp ? kThreads / 32 : 1;
+        kernel<<<(n_tiles + per_cta - 1) / per_cta, kThreads, 0, st>>>(
+            planes, mr, at->width, at->height, at->row0, at->tile, at->tiles_x, n_tiles, at->tri, at->pos_x, at->pos_y,
+            at->pos_z, at->cover, at->tile_box);
         k_super<<<sg, kThreads, 0, st>>>(at->tile_box, at->tiles_x, at->tiles_y, at->super_box, &hdr->n_covered);
         count_launches(2);
     };
