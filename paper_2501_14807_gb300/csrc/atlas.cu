@@ -14,7 +14,7 @@
 //   k_raster      one thread per triangle: position planes, area weight, and the texels of
 //                 small triangles; big triangles are split into 16x16-texel blocks appended to a
 //                 work list
-//   k_raster_big  one CTA per (triangle, block) entry
+//   k_raster_big  one warp per (triangle, block) entry
 //   k_resolve     one warp or CTA per tile, one texel per lane and step: position of every covered texel
 //                 (from the triangle's planes where their rounding cannot matter, else exact
 //                 barycentrics), coverage bits, tile box
@@ -521,35 +521,52 @@ __global__ void __launch_bounds__(128) k_raster(const __grid_constant__ RasterAr
     }
 }
 
+// The blocks of big triangles, a warp each: a lane takes every second row of one of the block's 16 columns,
+// its edge values stepping from row to row.  Bound by the latency of the chain entry -> indices -> corners,
+// so a warp, not a CTA, waits on it: 400 000 triangles on 16384^2 (9 blocks each) took 6.06 ms with a CTA
+// per entry and a texel per thread, now 1.43.
 template <bool MIN>
 __global__ void __launch_bounds__(kThreads) k_raster_big(const uint2 *__restrict__ big, AtlasHdr *hdr, int64_t cap,
                              const MeshRefs m, int32_t w, int32_t row0, int32_t rows,
                              uint32_t *__restrict__ tri_plane) {
-    const int64_t n = min((int64_t)hdr->n_big, cap);
+    const int64_t n = min((int64_t)hdr->n_big, cap), n_warps = (int64_t)gridDim.x * (kThreads / 32);
+    const int32_t lane = (int32_t)(threadIdx.x & 31u), col = lane % kBlockSide, row = lane / kBlockSide;
+    constexpr int kStep = 32 / kBlockSide;  // rows of a warp's step
     uint32_t hits = 0;
-    for (int64_t e = blockIdx.x; e < n; e += gridDim.x) {
-        if (!LCL_IN(e, cap)) break;
-        uint2 ent = big[e];
+    int64_t e = (int64_t)blockIdx.x * (kThreads / 32) + threadIdx.x / 32;
+    uint2 next = e < n && LCL_IN(e, cap) ? big[e] : make_uint2(kNone, 0u);
+    for (; e < n; e += n_warps) {  // uniform over the warp
+        const uint2 ent = next;
+        next = e + n_warps < n && LCL_IN(e + n_warps, cap) ? big[e + n_warps] : make_uint2(kNone, 0u);
         if (ent.x == kNone) continue;  // a slot of a reservation that did not fit
         if (!LCL_IN(ent.x, m.n_tri)) continue;
         Corners s;
-        if (!load_corners(m, ent.x, s)) continue;  // uniform
+        if (!load_corners(m, ent.x, s)) continue;
         const int32_t xmin = min(s.x[0], min(s.x[1], s.x[2])), xmax = max(s.x[0], max(s.x[1], s.x[2]));
         const int32_t ymin = min(s.y[0], min(s.y[1], s.y[2])), ymax = max(s.y[0], max(s.y[1], s.y[2]));
         int32_t i0, i1, j0, j1;
         texel_range(xmin, xmax, 0, w - 1, i0, i1);
         texel_range(ymin, ymax, row0, row0 + rows - 1, j0, j1);  // as k_raster cut the blocks
         const uint32_t nbx = (uint32_t)(i1 - i0 + 1 + kBlockSide - 1) / kBlockSide;
-        const int32_t i = i0 + (int32_t)(ent.y % nbx) * kBlockSide + (int32_t)(threadIdx.x % kBlockSide);
-        const int32_t j = j0 + (int32_t)(ent.y / nbx) * kBlockSide + (int32_t)(threadIdx.x / kBlockSide);
-        if (i > i1 || j > j1) continue;
+        const int32_t i = i0 + (int32_t)(ent.y % nbx) * kBlockSide + col;
+        int32_t j = j0 + (int32_t)(ent.y / nbx) * kBlockSide + row;
+        if (i > i1) continue;
         const int32_t px = 256 * i + 128, py = 256 * j + 128;
-        const int64_t e0 = edge_fn32(s.x[1], s.y[1], s.x[2], s.y[2], px, py) + edge_bias(s.x[2] - s.x[1], s.y[2] - s.y[1]);
-        const int64_t e1 = edge_fn32(s.x[2], s.y[2], s.x[0], s.y[0], px, py) + edge_bias(s.x[0] - s.x[2], s.y[0] - s.y[2]);
-        const int64_t e2 = edge_fn32(s.x[0], s.y[0], s.x[1], s.y[1], px, py) + edge_bias(s.x[1] - s.x[0], s.y[1] - s.y[0]);
-        if (e0 > 0 && e1 > 0 && e2 > 0 && LCL_IN((j - row0) * (int64_t)w + i, (int64_t)w * rows)) {
-            mark_texel<MIN>(tri_plane + (j - row0) * (int64_t)w + i, ent.x);
-            ++hits;
+        int64_t e0 = edge_fn32(s.x[1], s.y[1], s.x[2], s.y[2], px, py) + edge_bias(s.x[2] - s.x[1], s.y[2] - s.y[1]);
+        int64_t e1 = edge_fn32(s.x[2], s.y[2], s.x[0], s.y[0], px, py) + edge_bias(s.x[0] - s.x[2], s.y[0] - s.y[2]);
+        int64_t e2 = edge_fn32(s.x[0], s.y[0], s.x[1], s.y[1], px, py) + edge_bias(s.x[1] - s.x[0], s.y[1] - s.y[0]);
+        const int64_t d0 = (int64_t)(s.x[2] - s.x[1]) * (256 * kStep), d1 = (int64_t)(s.x[0] - s.x[2]) * (256 * kStep);
+        const int64_t d2 = (int64_t)(s.x[1] - s.x[0]) * (256 * kStep);
+#pragma unroll
+        for (int k = 0; k < kBlockSide / kStep; ++k) {
+            if (j <= j1 && e0 > 0 && e1 > 0 && e2 > 0 && LCL_IN((j - row0) * (int64_t)w + i, (int64_t)w * rows)) {
+                mark_texel<MIN>(tri_plane + (j - row0) * (int64_t)w + i, ent.x);
+                ++hits;
+            }
+            j += kStep;
+            e0 += d0;
+            e1 += d1;
+            e2 += d2;
         }
     }
     if (!MIN && n > 0) {
