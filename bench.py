@@ -6,7 +6,7 @@ Workload (default): the roofline-size model -- a displaced vessel of 2828 x 1414
 through the C ABI:
   atlas build (quantise, UV rasterise, interpolate, boxes, area weights)
   1000 sphere strokes (radii log-uniform 1-30% of the bbox diagonal), one call per layer,
-      one launch per stroke (it applies its stroke and culls the next)
+      applied in one launch
   4 depth maps (2048^2) and 20 star lassos on them
   XOR(L0, L1) and OR(L2, L3) overlays, per-label area (256 labels) of the 4 layers
 
@@ -288,7 +288,7 @@ def run_ours(args):
                          device=dev)
     sphere_hits = [torch.zeros(max(len(r), 1), dtype=torch.int64, device=dev) for r in per_layer]
     inside_per_layer = [sphere_inside_texels(atlas, r, dev) for r in per_layer]
-    # every layer's strokes are one call of >= 2 unpadded strokes: the grouped path
+    # every layer's strokes are one unpadded call
     grouped = [sphere_group_bytes(atlas, r, dev, w.dtype_bytes) for r in per_layer]
     assert all(len(r) >= 2 and not (r["flags"] & 15).any() for r in per_layer)
     torch.cuda.empty_cache()
@@ -432,8 +432,8 @@ def run_ours(args):
                                     "all-reduce per step)") if world > 1 else "1 GPU, the whole texture"),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "peak_kind": peak_kind, "traffic": traffic,
-                     "kernel": f"sphere edit, grouped: k_group_cull + k_group_apply per {SPHERE_GROUP} consecutive "
-                               "strokes of a call (a launch = one group), timed over the whole sphere row",
+                     "kernel": f"sphere edit: one k_spheres launch per {SPHERE_GROUP} consecutive strokes of a call at "
+                               "most (a launch = one group), timed over the whole sphere row",
                      "algorithmic_bytes_per_launch": sph_bytes / max(n_groups, 1),
                      "bytes_model": "12 B position + label per selected texel, summed over the strokes (the scope's "
                                     "per-unit bytes).  The grouped apply reads a tile's positions once per group "
@@ -492,16 +492,16 @@ def sphere_inside_texels(atlas, records, dev, chunk=16):
     return out
 
 
-SPHERE_GROUP = 32  # strokes per grouped launch pair of the library (k_group_cull + k_group_apply)
+SPHERE_GROUP = 512  # strokes per launch of the library's k_spheres at most
 
 
 def sphere_group_bytes(atlas, records, dev, label_bytes, group=SPHERE_GROUP):
     """Bytes the grouped sphere apply moves at tile granularity for one call applying `records` (the
-    library applies a call of two or more unpadded strokes on a label layer `group` strokes per
-    launch): per group, every tile that some stroke of the group reaches costs its covered texels'
-    labels; a tile that some stroke's surface crosses also costs their 12-byte positions, a tile that
-    every stroke reaching it contains only their coverage bits.  Tile boxes against the strokes on
-    the device, one group at a time.  Returns (bytes, groups)."""
+    library applies an unpadded call's strokes `group` per launch): per group, every tile that some
+    stroke of the group reaches costs its covered texels' labels; a tile that some stroke's surface
+    crosses also costs their 12-byte positions, a tile that every stroke reaching it contains only
+    their coverage bits.  Tile boxes against the strokes on the device, one group at a time.  Returns
+    (bytes, groups)."""
     import torch
     tb = atlas.tile_box().to(torch.int64)
     lo, cnt, hi = tb[:, 0:3], tb[:, 3], tb[:, 4:7]
