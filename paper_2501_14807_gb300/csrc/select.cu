@@ -379,6 +379,301 @@ __global__ void __launch_bounds__(kThreads, 6) k_sphere_step(AtlasDev a, L *__re
     add_hits(hits, cnt);
 }
 
+// ---- grouped sphere strokes ----------------------------------------------------------------
+//
+// Middling calls of unpadded strokes on large label layers (by_lists): up to kGroup strokes are applied by
+// one cull and one apply launch.  Applying strokes one by one leaves each texel with
+// the label of the newest stroke that selects it (older labels are overwritten), so the apply walks a
+// texel's strokes from the newest down and writes it once; every stroke is still evaluated for its
+// hit count, which does not depend on the order.  Items are (tile, mask, sure): `mask` holds the
+// group's strokes whose sphere reaches the tile's box (bit k = stroke k of the group), `sure` those
+// of them whose sphere contains the box, so that every covered texel of the tile is selected.  Tiles
+// whose strokes are all sure need no positions: with whole-row layouts they go to the back of the
+// lists and a warp writes them from the coverage bits, one lane per 32-texel row segment.
+
+constexpr int kGroup = 32;
+
+struct GroupArg {
+    int32_t n;     // strokes in the group (<= kGroup)
+    int32_t rows;  // whole-row handling of all-sure tiles (tile side >= 32, width a multiple of 32)
+    SphereArg s[kGroup];
+};
+
+// The three lists hold an item's tile, mask and sure at the same index; front items from index 0
+// (count counters[0]), all-sure items from the last index down (count counters[1]).
+__device__ __forceinline__ void append_item(bool front, bool back, uint32_t tile, uint32_t mask, uint32_t sure,
+                                            uint32_t *counters, uint32_t *tiles, uint32_t *masks, uint32_t *sures,
+                                            int64_t cap) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t fm = __ballot_sync(0xffffffffu, front), bm = __ballot_sync(0xffffffffu, back);
+    uint32_t fb = 0, bb = 0;
+    if (fm && lane == __ffs(fm) - 1) fb = atomicAdd(counters, (uint32_t)__popc(fm));
+    if (bm && lane == __ffs(bm) - 1) bb = atomicAdd(counters + 1, (uint32_t)__popc(bm));
+    if (fm) fb = __shfl_sync(0xffffffffu, fb, __ffs(fm) - 1);
+    if (bm) bb = __shfl_sync(0xffffffffu, bb, __ffs(bm) - 1);
+    int64_t slot = -1;
+    if (front) slot = fb + __popc(fm & ((1u << lane) - 1));
+    if (back) slot = cap - 1 - (int64_t)(bb + __popc(bm & ((1u << lane) - 1)));
+    if ((front || back) && LCL_IN(slot, cap)) {
+        tiles[slot] = tile;
+        masks[slot] = mask;
+        sures[slot] = sure;
+    }
+}
+
+// ahead = 1 (every group but a call's first): the lists this cull writes were last read by the apply
+// two groups back, which had completed before the previous apply started, so the cull runs while the
+// previous group's apply is still writing the layer, and waits for it only at its end (the next
+// apply starts after this grid completes, hence after the previous apply).  The first group's cull
+// waits at once: its counters are being cleared by the grid before it.
+__global__ void __launch_bounds__(kThreads) k_group_cull(AtlasDev a, const __grid_constant__ GroupArg g,
+                                                         uint32_t *counters, uint32_t *tiles, uint32_t *masks,
+                                                         uint32_t *sures, int ahead) {
+    if (!ahead) pdl_wait();
+    __shared__ uint32_t s_mask;
+    const int32_t n_super = a.supers_x * a.supers_y;
+    const int64_t n_tiles = (int64_t)a.tiles_x * a.tiles_y;
+    for (int32_t sidx = blockIdx.x; sidx < n_super; sidx += gridDim.x) {
+        if (threadIdx.x == 0) s_mask = 0u;
+        __syncthreads();
+        if ((int)threadIdx.x < g.n && LCL_IN(sidx, (int64_t)n_super)) {  // one thread per stroke
+            const int4 *sb = reinterpret_cast<const int4 *>(a.super_box + 8 * (int64_t)sidx);
+            const int4 slo = sb[0], shi = sb[1];
+            const SphereArg &sp = g.s[threadIdx.x];
+            if (slo.w > 0 && box_dist2(slo, shi, sp) <= sp.r2) atomicOr(&s_mask, 1u << threadIdx.x);
+        }
+        __syncthreads();
+        const uint32_t smask = s_mask;
+        __syncthreads();
+        if (!smask) continue;  // uniform over the CTA
+        const int32_t sx = sidx % a.supers_x, sy = sidx / a.supers_x;
+        const int32_t tx = sx * LCL_SUPER + (threadIdx.x % LCL_SUPER);
+        const int32_t ty = sy * LCL_SUPER + (threadIdx.x / LCL_SUPER);
+        const int64_t tile = (int64_t)ty * a.tiles_x + tx;
+        uint32_t mask = 0u, sure = 0u;
+        if (tx < a.tiles_x && ty < a.tiles_y && LCL_IN(tile, n_tiles)) {
+            const int4 *tb = reinterpret_cast<const int4 *>(a.tile_box + 8 * tile);
+            const int4 lo = tb[0], hi = tb[1];
+            if (lo.w > 0) {
+                for (uint32_t m = smask; m; m &= m - 1) {
+                    const int k = __ffs(m) - 1;
+                    const SphereArg &sp = g.s[k];
+                    if (box_dist2(lo, hi, sp) > sp.r2) continue;
+                    mask |= 1u << k;
+                    if (box_far2(lo, hi, sp) <= sp.r2) sure |= 1u << k;
+                }
+            }
+        }
+        const bool back = g.rows && mask != 0u && mask == sure;
+        append_item(mask != 0u && !back, back, (uint32_t)tile, mask, sure, counters, tiles, masks, sures, n_tiles);
+    }
+    if (ahead) pdl_wait();
+    pdl_allow_next();
+}
+
+// A front item's list entry, loaded two items ahead; tile = kNone: none.
+struct GEnt {
+    uint32_t tile, mask, sure;
+};
+
+__device__ __forceinline__ GEnt load_gent(const AtlasDev &a, const uint32_t *__restrict__ tiles,
+                                          const uint32_t *__restrict__ masks, const uint32_t *__restrict__ sures,
+                                          uint32_t item, uint32_t n_items, int cpt_log2) {
+    GEnt e;
+    e.tile = kNone;
+    e.mask = e.sure = 0u;
+    const uint32_t idx = item >> cpt_log2;
+    if (item < n_items && LCL_IN(idx, (int64_t)a.tiles_x * a.tiles_y)) {
+        e.tile = __ldg(tiles + idx);
+        e.mask = __ldg(masks + idx);
+        e.sure = __ldg(sures + idx);
+    }
+    return e;
+}
+
+// A front item's quad for this thread, loaded one item ahead: the entry's masks and the raw data --
+// positions when some stroke of the item is not sure, else the coverage word -- with nothing that
+// waits for them (the coverage bits are taken out when the item is processed).
+struct GItem {
+    int64_t l;  // -1: no quad for this thread (the masks are still the item's)
+    uint32_t mask, sure, cw;
+    int4 X, Y, Z;
+};
+
+__device__ __forceinline__ GItem load_gquad(const AtlasDev &a, const GEnt &e, uint32_t item, int cpt_log2,
+                                            int32_t qpr, int32_t nq) {
+    GItem it;
+    it.l = -1;
+    it.mask = e.mask;
+    it.sure = e.sure;
+    it.cw = 0u;
+    it.X = it.Y = it.Z = make_int4(INT32_MIN, 0, 0, 0);
+    if (e.tile == kNone) return it;
+    const int32_t qd = (int32_t)((item & ((1u << cpt_log2) - 1)) * kThreads + threadIdx.x);
+    int32_t tx, ty;
+    tile_xy(a, e.tile, tx, ty);
+    const int32_t x = tx * a.T + 4 * (qd & (qpr - 1)), y = ty * a.T + (qd >> (__ffs(qpr) - 1));
+    const int64_t n_tex = (int64_t)a.w * a.h;
+    (void)n_tex;
+    if (qd < nq && x < a.w && y < a.h && LCL_IN((int64_t)y * a.w + x + 3, n_tex)) {
+        it.l = (int64_t)y * a.w + x;
+        if (it.mask & ~it.sure) {  // uniform over the item
+            it.X = __ldg(reinterpret_cast<const int4 *>(a.px + it.l));
+            it.Y = __ldg(reinterpret_cast<const int4 *>(a.py + it.l));
+            it.Z = __ldg(reinterpret_cast<const int4 *>(a.pz + it.l));
+        } else if (LCL_IN(it.l >> 5, (n_tex + 31) >> 5)) {
+            it.cw = __ldg(a.cover + (it.l >> 5));
+        }
+    }
+    return it;
+}
+
+// The quad's coverage bits (bit k: texel k) from its raw data.
+__device__ __forceinline__ uint32_t gquad_cov(const GItem &it) {
+    if (it.l < 0) return 0u;
+    if (it.mask & ~it.sure)
+        return (it.X.x != INT32_MIN ? 1u : 0u) | (it.X.y != INT32_MIN ? 2u : 0u) | (it.X.z != INT32_MIN ? 4u : 0u) |
+               (it.X.w != INT32_MIN ? 8u : 0u);
+    return (it.cw >> (it.l & 31)) & 0xFu;
+}
+
+template <typename L>
+__global__ void __launch_bounds__(kThreads, 5) k_group_apply(AtlasDev a, L *__restrict__ layer,
+                                                             const __grid_constant__ GroupArg g,
+                                                             const uint32_t *__restrict__ counters,
+                                                             const uint32_t *__restrict__ tiles,
+                                                             const uint32_t *__restrict__ masks,
+                                                             const uint32_t *__restrict__ sures,
+                                                             unsigned long long *hits) {
+    __shared__ unsigned long long s_hits[kGroup];
+    if (threadIdx.x < kGroup) s_hits[threadIdx.x] = 0ull;
+    __syncthreads();
+    pdl_wait();
+    pdl_allow_next();
+    const int lane = threadIdx.x & 31;
+    const int64_t n_tex = (int64_t)a.w * a.h;
+    (void)n_tex;
+    // front items: a CTA per tile (or 256-quad chunk of one), a thread per quad
+    const int32_t qpr = a.T / 4, nq = a.T * qpr;
+    const int cpt_log2 = nq > kThreads ? 31 - __clz(nq / kThreads) : 0;
+    const uint32_t n_items = counters[0] << cpt_log2;
+    // entries two items ahead, quads one item ahead: the position loads of the next item are issued
+    // as soon as this item starts, from an entry that arrived during the previous one
+    uint32_t item = blockIdx.x;
+    GItem cur = load_gquad(a, load_gent(a, tiles, masks, sures, item, n_items, cpt_log2), item, cpt_log2, qpr, nq);
+    GEnt e1 = load_gent(a, tiles, masks, sures, item + gridDim.x, n_items, cpt_log2);
+    for (; item < n_items; item += gridDim.x) {
+        const uint32_t after = item + gridDim.x;
+        const GEnt e2 = load_gent(a, tiles, masks, sures, after + gridDim.x, n_items, cpt_log2);
+        const GItem next = load_gquad(a, e1, after, cpt_log2, qpr, nq);
+        e1 = e2;
+        const int32_t xs[4] = {cur.X.x, cur.X.y, cur.X.z, cur.X.w}, ys[4] = {cur.Y.x, cur.Y.y, cur.Y.z, cur.Y.w},
+                      zs[4] = {cur.Z.x, cur.Z.y, cur.Z.z, cur.Z.w};
+        const uint32_t cov = gquad_cov(cur);
+        const int ks = cur.sure ? 31 - __clz(cur.sure) : -1;  // the newest stroke containing the tile
+        uint32_t open = cov;
+        uint32_t lab[4] = {0u, 0u, 0u, 0u};
+        // strokes whose surface crosses the tile, newest first (uniform over the CTA): each is tested
+        // per texel for its hit count; only those newer than stroke ks can give a texel its label
+        for (uint32_t m = cur.mask & ~cur.sure; m;) {
+            const int k = 31 - __clz(m);
+            m &= ~(1u << k);
+            if (!hits && k < ks) break;  // no counts wanted: stroke ks labels every open texel
+            const SphereArg &sp = g.s[k];
+            uint32_t sel = 0u;
+            if (cur.l >= 0) {
+                // The stroke reaches the tile's box (r <= 2^25 and the box inside [0, 2^21)^3), so for a
+                // covered texel every coordinate difference lies within +-(2^25 + 2^21) and its square
+                // is one 32 x 32 -> 64-bit product.  Uncovered texels (x = INT32_MIN) wrap around in
+                // the unsigned difference; the coverage bits drop them.
+                const uint32_t cx = (uint32_t)sp.cx, cy = (uint32_t)sp.cy, cz = (uint32_t)sp.cz;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int32_t dx = (int32_t)((uint32_t)xs[q] - cx), dy = (int32_t)((uint32_t)ys[q] - cy),
+                                  dz = (int32_t)((uint32_t)zs[q] - cz);
+                    const int64_t d2 = (int64_t)dx * dx + (int64_t)dy * dy + (int64_t)dz * dz;
+                    sel |= (d2 <= sp.r2 ? 1u : 0u) << q;
+                }
+                sel &= cov;
+            }
+            if (hits) {
+                const uint32_t c = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(sel));
+                if (lane == 0 && c) atomicAdd(&s_hits[k], (unsigned long long)c);
+            }
+            if (k > ks) {
+                const uint32_t nw = sel & open;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (nw & (1u << q)) lab[q] = sp.label;
+                open &= ~sel;
+            }
+        }
+        if (ks >= 0) {  // strokes containing the tile select every covered texel
+            const uint32_t label = g.s[ks].label;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (open & (1u << q)) lab[q] = label;
+            open = 0u;
+            if (hits) {
+                const uint32_t c = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(cov));
+                if (lane == 0 && c)
+                    for (uint32_t m = cur.sure; m; m &= m - 1) atomicAdd(&s_hits[__ffs(m) - 1], (unsigned long long)c);
+            }
+        }
+        const uint32_t written = cov & ~open;
+        if (written && LCL_IN(cur.l + 3, n_tex)) store_labels<L>(layer, cur.l, written, lab);
+        cur = next;
+    }
+    // all-sure items (whole-row layouts): a warp per tile from the far end of the grid, one lane per
+    // 32-texel row segment; the newest stroke's label goes to every covered texel
+    const uint32_t n_back = counters[1];
+    if (n_back) {  // uniform
+        const int64_t cap = (int64_t)a.tiles_x * a.tiles_y;
+        const int32_t wpr = a.T >> 5, words = a.T * wpr;
+        const uint32_t warps = gridDim.x * (kThreads / 32);
+        // the next tile's entry is loaded one tile ahead
+        auto entry = [&](uint32_t bb, uint32_t &t, uint32_t &m) {
+            t = kNone;
+            m = 0u;
+            if (bb < n_back && LCL_IN(cap - 1 - (int64_t)bb, cap)) {
+                t = __ldg(tiles + (cap - 1 - (int64_t)bb));
+                m = __ldg(masks + (cap - 1 - (int64_t)bb));
+            }
+        };
+        uint32_t b = (gridDim.x - 1 - blockIdx.x) * (kThreads / 32) + (threadIdx.x >> 5);
+        uint32_t next_tile, next_mask;
+        entry(b, next_tile, next_mask);
+        for (; b < n_back; b += warps) {
+            const uint32_t tile = next_tile, mask = next_mask;
+            entry(b + warps, next_tile, next_mask);
+            if (!mask || tile == kNone) continue;  // uniform over the warp
+            const uint32_t label = g.s[31 - __clz(mask)].label;
+            int32_t tx, ty;
+            tile_xy(a, tile, tx, ty);
+            uint32_t c = 0u;
+            for (int32_t wi = lane; wi < words; wi += 32) {
+                const int32_t x = tx * a.T + 32 * (wi % wpr), y = ty * a.T + wi / wpr;
+                if (x >= a.w || y >= a.h) continue;  // x < w implies x + 31 < w (w a multiple of 32)
+                const int64_t l = (int64_t)y * a.w + x;
+                if (!LCL_IN(l + 31, n_tex)) continue;
+                const uint32_t cov = __ldg(a.cover + (l >> 5));
+                if (!cov) continue;
+                store_word32<L>(layer, l, cov, label);
+                c += __popc(cov);
+            }
+            if (hits) {
+                c = __reduce_add_sync(0xffffffffu, c);
+                if (lane == 0 && c)
+                    for (uint32_t m = mask; m; m &= m - 1) atomicAdd(&s_hits[__ffs(m) - 1], (unsigned long long)c);
+            }
+        }
+    }
+    if (hits) {
+        __syncthreads();
+        if ((int)threadIdx.x < g.n && s_hits[threadIdx.x]) atomicAdd(hits + threadIdx.x, s_hits[threadIdx.x]);
+    }
+}
+
 // ---- lasso ---------------------------------------------------------------------------
 
 // Super-tiles a lasso (or tool window) can touch: 8 lanes per super-tile (box_may_touch_by without
@@ -611,7 +906,8 @@ __global__ void __launch_bounds__(edit_threads<PAD>(), 1024 / edit_threads<PAD>(
 }
 
 struct SelWs {
-    uint32_t *counters, *list, *list2, *list3;  // three candidate lists: padded sphere calls use list k mod 3 for stroke k
+    uint32_t *counters, *list, *list2, *list3;  // three candidate lists: a chain of strokes uses list k mod 3 for stroke k
+    uint32_t *list4, *list5, *list6;            // calls of two or more strokes: a second item set for groups
 };
 
 SelWs sel_ws(const lcl_atlas *a, int32_t n, void *ws) {
@@ -622,6 +918,12 @@ SelWs sel_ws(const lcl_atlas *a, int32_t n, void *ws) {
     w.list = reinterpret_cast<uint32_t *>(base + align256((size_t)2 * (n + 1) * 4));
     w.list2 = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(w.list) + lb);
     w.list3 = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(w.list2) + lb);
+    w.list4 = w.list5 = w.list6 = nullptr;
+    if (n >= 2) {
+        w.list4 = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(w.list3) + lb);
+        w.list5 = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(w.list4) + lb);
+        w.list6 = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(w.list5) + lb);
+    }
     return w;
 }
 
@@ -762,11 +1064,68 @@ lcl_status division_check_impl(uint64_t n, uint32_t seed, uint64_t *counts, cuda
     return LCL_OK;
 }
 
-// Two counters per stroke and three tile lists; calls of two or more strokes have room for three more
-// lists, which nothing uses since they stopped going through candidate lists: the size is part of
-// what callers (and the static scratch) allocate by, so it stays.
+// Two counters per stroke and three tile lists; calls of two or more strokes three more lists.
 size_t select_ws_bytes(const lcl_atlas *a, int32_t n) {
     return align256((size_t)2 * (n + 1) * 4) + (n >= 2 ? 6 : 3) * align256((size_t)a->tiles_x * a->tiles_y * 4);
+}
+
+// Unpadded strokes on a label layer, kGroup at a time (see k_group_apply): zeroing, then a cull and
+// an apply launch per group, chained with programmatic dependent launch.
+template <typename L, typename ArgOf>
+lcl_status select_sphere_grouped(const lcl_atlas *atlas, const AtlasDev &a, L *layer, const SelWs &w, int32_t n,
+                                 unsigned long long *h, const ArgOf &arg, cudaStream_t st) {
+    const int32_t n_groups = (n + kGroup - 1) / kGroup;
+    k_sel_init<<<(std::max(2 * n_groups, n) + kThreads - 1) / kThreads, kThreads, 0, st>>>(w.counters, 2 * n_groups,
+                                                                                          h, n, nullptr, 0);
+    static thread_local GroupArg g;  // ~1.5 KB: kept off the stack
+    g.rows = (a.T >= 32 && (a.w & 31) == 0) ? 1 : 0;
+    const int n_super = atlas->supers_x * atlas->supers_y;
+    const int cull_grid = std::min(n_super, resident_grid(k_group_cull));
+    const int apply_grid = resident_grid(k_group_apply<L>);
+    cudaError_t e = cudaSuccess;
+    for (int32_t gi = 0; gi < n_groups && e == cudaSuccess; ++gi) {
+        const int32_t k0 = gi * kGroup;
+        g.n = std::min(kGroup, n - k0);
+        for (int32_t k = 0; k < g.n; ++k) g.s[k] = arg(k0 + k);
+        uint32_t *const c = w.counters + 2 * gi;
+        // item sets alternate between groups, so a group's cull can run while the previous apply does
+        uint32_t *const t = (gi & 1) ? w.list4 : w.list, *const m = (gi & 1) ? w.list5 : w.list2,
+                        *const su = (gi & 1) ? w.list6 : w.list3;
+        e = launch_pdl(k_group_cull, dim3(cull_grid), st, a, g, c, t, m, su, gi > 0 ? 1 : 0);
+        if (e == cudaSuccess)
+            e = launch_pdl(k_group_apply<L>, dim3(apply_grid), st, a, layer, g, (const uint32_t *)c,
+                           (const uint32_t *)t, (const uint32_t *)m, (const uint32_t *)su, h ? h + k0 : nullptr);
+    }
+    count_launches(1 + 2 * n_groups);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "lcl_select_sphere launch");
+    return LCL_OK;
+}
+
+// Which unpadded calls go through candidate lists instead of spheres.cu's blocks.  A block is one CTA's, so
+// on a large texture a few strokes keep a few CTAs busy for long while the others only find their
+// blocks empty; lists spread the reached tiles over the chip.  Times per call, lists / blocks, radii 1-5%
+// of the diagonal (10-30% in brackets):
+//   a stroke, 16384^2 (262144 tiles of 32): 20.5 / 24.4 us (28.6 / 55.2), 8192^2: 20.8 / 15.7, 4096^2: 21 / 15;
+//   label layers, groups of 32 strokes: on 16384^2 2 strokes 21 / 25 (35 / 65), 32 33 / 59 (201 / 209), 64
+//   60 / 79 (409 / 278), 128 120 / 119, 256 239 / 179; on 8192^2 4 strokes 21 / 18, 8 21 / 21, 32 21 / 32,
+//   64 35 / 45, 128 65 / 60; on 4096^2 16 strokes 20 / 17, 64 26 / 23;
+//   value layers, a launch per stroke: on 16384^2 2 strokes 22 / 26, 4 27 / 30 (75 / 85), 8 41 / 41.
+constexpr int64_t kManyTiles1 = 131072, kManyTiles2 = 49152;  // tiles of a large texture, of a middling one
+constexpr int32_t kMidStrokes = 6;    // strokes at least, on a middling texture
+constexpr int32_t kGroupCall = 32;     // strokes at most, of any radius ...
+constexpr int32_t kGroupCallSmall = 96;  // ... or of radii up to an eighth of the grid
+constexpr int64_t kSmallR2 = int64_t(1) << 36;
+constexpr int32_t kChainValues = 4;
+
+template <bool NUM>
+bool by_lists(const lcl_sphere *strokes, int32_t n, int64_t n_tiles) {
+    if (NUM || n == 1) return n <= kChainValues && n_tiles >= kManyTiles1;
+    if (n_tiles < kManyTiles2 || (n < kMidStrokes && n_tiles < kManyTiles1) || n > kGroupCallSmall) return false;
+    if (n <= kGroupCall) return true;
+    for (int32_t k = 0; k < n; ++k)
+        if (strokes[k].r2 > kSmallR2) return false;
+    return true;
 }
 
 template <typename L>
@@ -800,7 +1159,10 @@ lcl_status select_sphere_run(const lcl_atlas *atlas, L *layer, uint32_t *mask, c
     };
     bool padded = false;
     for (int32_t k = 0; k < n; ++k) padded = padded || (strokes[k].flags & 15u) != 0;
-    if (!padded) {  // no stroke reads its neighbours' selections: all strokes in one pass (spheres.cu)
+    const bool lists = !padded && by_lists<NUM>(strokes, n, (int64_t)a.tiles_x * a.tiles_y);
+    if constexpr (!NUM)
+        if (lists && n >= 2) return select_sphere_grouped(atlas, a, layer, w, n, h, arg, st);
+    if (!padded && !lists) {  // all strokes in one pass (spheres.cu)
         cudaError_t e = spheres_run<L, NUM>(atlas, layer, mask, strokes, n, h, w.counters, st);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, NUM ? "lcl_numeric_sphere launch" : "lcl_select_sphere launch");

@@ -17,7 +17,7 @@
 //     newest containing stroke gives the texels left open their value.
 // No candidate lists pass through memory, and a call needs ceil(n / kManyStrokes) launches, where a
 // cull and an apply launch per 32 strokes (label layers) or one launch per stroke (numeric layers,
-// single strokes) ran before.
+// single strokes) ran before.  Those stay for few strokes on large textures (by_lists in select.cu).
 //
 // What bounds it: latency of the crossing tiles' loads, then issue of their 64-bit distance tests
 // (38% of issue slots, 21% of DRAM at 4096^2).  Measured on GB300, per call, before -> after: 250
