@@ -205,10 +205,10 @@ __global__ void __launch_bounds__(kThreads) k_batch_prep(BHdr *hdr, const BLasso
         p.pad_t = (int32_t)((L.flags >> 4) & 15u);
     }
     __syncwarp();
-    const float bh = lasso_band_height(p);
+    const float2 range = lasso_band_range(p, lane, lasso_band_height(p));
     unsigned long long has = 0ull;  // edges of band `lane`
     for (int e = 0; e < nv; ++e)
-        if (lasso_band_has(p, lane, e, bh)) has |= 1ull << e;
+        if (lasso_band_has(p, range, e)) has |= 1ull << e;
     p.band[lane] = make_uint2((uint32_t)has, (uint32_t)(has >> 32));
     for (int e = lane; e < nv; e += 32) {
         const float2 r = edge_xrange(p.vx[e], p.vx[e + 1]);

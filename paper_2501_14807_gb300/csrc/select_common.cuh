@@ -814,9 +814,11 @@ inline int resident_grid(K kernel) {
 
 // y-bands of edges: band b lists the edges whose y-range comes within `slack` of it, in edge order.
 // The slack is far above the rounding of a point's band (floor((y - band_y0) * band_inv_h), a few ulps)
-// and of the bounds below; an edge too many in a band changes nothing.
+// and of the bounds below; an edge too many in a band changes nothing.  Vertices may be any finite floats
+// (a polygon may span more than the largest one), so nothing here overflows to an infinity that would
+// lose an edge: the extent is taken after the division by the number of bands, the bounds by one FMA.
 __host__ __device__ inline float lasso_band_height(const LassoHead &p) {
-    return fmaxf(p.ymax - p.ymin, 1e-3f) * (1.0f / kBands);
+    return fmaxf(p.ymax * (1.0f / kBands) - p.ymin * (1.0f / kBands), 1e-3f / kBands);
 }
 
 // The lasso argument's scalars but for the polygon's: matrix, screen, label, bias.
@@ -872,12 +874,15 @@ inline void lasso_arg_head(LassoHead &p, const float *m16, int32_t w_s, int32_t 
     lasso_arg_box(p, x0, x1, y0, y1);
 }
 
-__host__ __device__ inline bool lasso_band_has(const LassoHead &p, int b, int e, float bh) {
-    const float slack = 2e-3f * bh + 2e-3f + 1e-6f * (fabsf(p.ymin) + fabsf(p.ymax));
-    const float lo = p.ymin + (float)b * bh - slack, hi = p.ymin + (float)(b + 1) * bh + slack;
+// The y-range {lo, hi} whose edges band b of height bh lists, and whether edge e is one of them.
+__host__ __device__ inline float2 lasso_band_range(const LassoHead &p, int b, float bh) {
+    const float slack = 2e-3f * bh + 2e-3f + 1e-6f * fabsf(p.ymin) + 1e-6f * fabsf(p.ymax);
+    return make_float2(fmaf((float)b, bh, p.ymin) - slack, fmaf((float)(b + 1), bh, p.ymin) + slack);
+}
+__host__ __device__ inline bool lasso_band_has(const LassoHead &p, float2 range, int e) {
     const float ea = p.vy[e], eb = p.vy[e + 1];
     if (ea == eb) return false;  // horizontal edges never straddle
-    return fminf(ea, eb) <= hi && fmaxf(ea, eb) >= lo;
+    return fminf(ea, eb) <= range.y && fmaxf(ea, eb) >= range.x;
 }
 
 // The whole lasso argument, on the host.
@@ -888,8 +893,9 @@ inline void fill_lasso_arg(LassoArg &p, const lcl_camera *cam, const float *poly
     int cnt = 0;
     for (int b = 0; b < kBands; ++b) {
         p.band_off[b] = (uint16_t)cnt;
+        const float2 range = lasso_band_range(p, b, bh);
         for (int e = 0; e < nv; ++e)
-            if (lasso_band_has(p, b, e, bh)) p.band_edge[cnt++] = (uint8_t)e;
+            if (lasso_band_has(p, range, e)) p.band_edge[cnt++] = (uint8_t)e;
     }
     p.band_off[kBands] = (uint16_t)cnt;
 }
