@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kThreads) k_batch_prep(BHdr *hdr, const BLasso
     }
     if (lane < 16) p.m[lane] = L.m[lane];
     if (lane == 0) {
-        lasso_arg_scalars(p, L.w_s, L.h_s, nv, L.label, L.bias);
+        lasso_arg_scalars(p, L.m, L.w_s, L.h_s, nv, L.label, L.bias);
         lasso_arg_box(p, x0, x1, y0, y1);
         p.depth = L.depth;
         p.pad_r = (int32_t)(L.flags & 15u);

@@ -314,7 +314,8 @@ struct alignas(16) LassoHead {  // in groups of four words, which the kernels lo
     int32_t w_s, h_s;
     float bias;
     uint32_t label;
-    int32_t nv, unused;
+    int32_t nv;
+    float w_safe;           // smallest clip w at which projections round by less than half a pixel (lasso_w_safe)
     float bx0, by0, bx1, by1;  // polygon bbox (clipped to the screen) widened by a margin, pixels
     float nx0, nx1, ny0, ny1;  // the same widened bbox in NDC, for the division-free reject
     float ymin, ymax;          // exact vertical extent of the polygon
@@ -374,7 +375,8 @@ __device__ __forceinline__ void stage_lasso(LassoShared &sh, const LassoArg &p) 
 }
 
 // Conservative: false only if no texel of the box can be selected by the lasso.  Two exact tests:
-//  - the box's projected corners (all with w > 0) bound the projection of every point of the box
+//  - the box's projected corners (all with w above w_safe, else the box is kept: close to the camera the
+//    binary32 projections of texels and corners may differ by more than the margins) bound the projection of every point of the box
 //    (a projective map keeps a convex box convex); if their bounding box, widened by the margin,
 //    misses the polygon's widened bounding box, no texel can be inside the polygon;
 //  - with a depth map: NDC depth z/w is linear-fractional along every segment of the box, so its
@@ -427,7 +429,7 @@ __device__ __forceinline__ bool box_may_touch_by(const LassoHead &p, int4 lo, in
     const float x = (float)((sub & 1u) ? hi.x : lo.x), y = (float)((sub & 2u) ? hi.y : lo.y);
     const float z = (float)((sub & 4u) ? hi.z : lo.z);
     const float cw = clip_row(p.m + 12, x, y, z);
-    if (__any_sync(gm, !(cw > 0.0f))) return true;
+    if (__any_sync(gm, !(cw > p.w_safe))) return true;
     // each lane folds its corner into empty bounds exactly as the serial loop does (NaN ignored)
     const float xs = screen_of(div_rn(clip_row(p.m, x, y, z), cw), p.ws);
     const float ys = screen_of(div_rn(clip_row(p.m + 4, x, y, z), cw), p.hs);
@@ -466,8 +468,8 @@ __device__ __forceinline__ bool box_may_touch_by(const LassoHead &p, int4 lo, in
 //   kTileIn    no edge comes near the box, its centre is inside and the box lies on screen: every
 //              texel of the box that projects is inside, so the texels skip the edge tests;
 //   kTileTest  otherwise (every texel is tested).
-// Why this is exact for the per-texel test in FP32: each texel's FP32 screen point lies in sb up to
-// far less than the margin m = 1 px (a few ulps of coordinates below 2^15), and no edge segment meets
+// Why this is exact for the per-texel test in FP32: with every corner's clip w above w_safe each texel's
+// FP32 screen point lies in sb up to less than the margin m = 1 px (lasso_w_safe), and no edge segment meets
 // sb widened by m, so along any straddled edge the crossing lies more than m - 0.05 px from the point,
 // beyond the error bound of the FP32 crossing (edge_xrange's 4.01 u (|ax| + |bx|) < 0.01 px); every
 // per-texel edge decision is then the exact one at that point, and the exact even-odd parity is the
@@ -821,9 +823,27 @@ __host__ __device__ inline float lasso_band_height(const LassoHead &p) {
     return fmaxf(p.ymax * (1.0f / kBands) - p.ymin * (1.0f / kBands), 1e-3f / kBands);
 }
 
-// The lasso argument's scalars but for the polygon's: matrix, screen, label, bias.
-__host__ __device__ inline void lasso_arg_scalars(LassoHead &p, int32_t w_s, int32_t h_s, int32_t nv, uint32_t label,
-                                                  float bias) {
+// Above this clip w a projected point's screen coordinates, in binary32, are within 0.4 px of the exact ones
+// wherever these lie within a screen's width of the screen (two projections then differ by less than the
+// 1 px margin of lasso_tile_class).  A row's value errs by at most E = 4.01 u (sum of its terms' magnitudes
+// over the grid, u = 2^-24: three roundings of products, three of sums), so cx / cw by (E_x + 2 E_w) / w for
+// |cx / cw| <= 2, which is 0.4 px at w = 1.25 width (E_x + 2 E_w).  A camera that looks at the model from
+// its own size away has w_safe at about 2^-8 of that; on a 16384-pixel screen texels closer than 1/2000 of
+// the model's size were off by 4 px, and those of tiles classed inside read the depth map without a check
+// of their place.
+__host__ __device__ inline float lasso_w_safe(const float *m, float ws, float hs) {
+    float e[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {  // rows x, y, w
+        const float *r = m + (k == 2 ? 12 : 4 * k);
+        e[k] = 2.3902e-7f * ((fabsf(r[0]) + fabsf(r[1]) + fabsf(r[2])) * (float)(1 << LCL_GRID_BITS) + fabsf(r[3]));
+    }
+    return 1.25f * fmaxf(ws * (e[0] + 2.0f * e[2]), hs * (e[1] + 2.0f * e[2]));
+}
+
+// The lasso argument's scalars but for the polygon's: screen, label, bias and what follows from the matrix m.
+__host__ __device__ inline void lasso_arg_scalars(LassoHead &p, const float *m, int32_t w_s, int32_t h_s, int32_t nv,
+                                                  uint32_t label, float bias) {
     p.ws = (float)w_s;
     p.hs = (float)h_s;
     p.w_s = w_s;
@@ -831,6 +851,7 @@ __host__ __device__ inline void lasso_arg_scalars(LassoHead &p, int32_t w_s, int
     p.bias = bias;
     p.label = label;
     p.nv = nv;
+    p.w_safe = lasso_w_safe(m, p.ws, p.hs);
 }
 
 // What follows from the polygon's bounding box: the widened box in pixels and NDC, the band mapping.
@@ -857,7 +878,7 @@ __host__ __device__ inline void lasso_arg_box(LassoHead &p, float x0, float x1, 
 inline void lasso_arg_head(LassoHead &p, const float *m16, int32_t w_s, int32_t h_s, const float *poly, int32_t nv,
                            uint32_t label, float bias) {
     for (int i = 0; i < 16; ++i) p.m[i] = m16[i];
-    lasso_arg_scalars(p, w_s, h_s, nv, label, bias);
+    lasso_arg_scalars(p, m16, w_s, h_s, nv, label, bias);
     float x0 = INFINITY, x1 = -INFINITY, y0 = INFINITY, y1 = -INFINITY;
     for (int i = 0; i < nv; ++i) {
         p.vx[i] = poly[2 * i];
