@@ -321,6 +321,7 @@ struct alignas(16) LassoHead {  // in groups of four words, which the kernels lo
     float ymin, ymax;          // exact vertical extent of the polygon
     float band_y0, band_inv_h; // band of a point: floor((y - band_y0) * band_inv_h), clamped
     float vx[LCL_MAX_LASSO_VERTICES + 1], vy[LCL_MAX_LASSO_VERTICES + 1];  // vertex nv = vertex 0
+    float z_err;               // z_err / w bounds the rounding of two points' NDC depths (clip_row_err)
 };
 
 // With the edges of each y-band: a kernel's argument.
@@ -380,7 +381,7 @@ __device__ __forceinline__ void stage_lasso(LassoShared &sh, const LassoArg &p) 
 //    (a projective map keeps a convex box convex); if their bounding box, widened by the margin,
 //    misses the polygon's widened bounding box, no texel can be inside the polygon;
 //  - with a depth map: NDC depth z/w is linear-fractional along every segment of the box, so its
-//    minimum over the box is at a corner; if that minimum (less 1e-4 for FP32 rounding) exceeds
+//    minimum over the box is at a corner; if that minimum (less z_err / w and 1e-4 for FP32 rounding) exceeds
 //    the largest depth-map value over the box's widened pixel footprint plus the bias, every texel
 //    of the box fails the depth test.  Footprints above 2048 pixels are not scanned (kept).
 // Evaluated by an aligned group of G lanes (8 or 32) for one box (all of them call it with the same
@@ -436,7 +437,8 @@ __device__ __forceinline__ bool box_may_touch_by(const LassoHead &p, int4 lo, in
     const bool finite = !CLASSIFY || __all_sync(gm, isfinite(xs) && isfinite(ys));
     float xmin = fminf(INFINITY, xs), xmax = fmaxf(-INFINITY, xs);
     float ymin = fminf(INFINITY, ys), ymax = fmaxf(-INFINITY, ys);
-    float zmin = fminf(INFINITY, div_rn(clip_row(p.m + 8, x, y, z), cw));
+    // less what rounding can take a texel's depth below its box's: (cz - z_err) / cw has its minimum at a corner too
+    float zmin = fminf(INFINITY, div_rn(__fsub_rn(clip_row(p.m + 8, x, y, z), p.z_err), cw));
     for (int o = 1; o < 8; o <<= 1) {
         xmin = fminf(xmin, __shfl_xor_sync(gm, xmin, o));
         xmax = fmaxf(xmax, __shfl_xor_sync(gm, xmax, o));
@@ -831,14 +833,12 @@ __host__ __device__ inline float lasso_band_height(const LassoHead &p) {
 // its own size away has w_safe at about 2^-8 of that; on a 16384-pixel screen texels closer than 1/2000 of
 // the model's size were off by 4 px, and those of tiles classed inside read the depth map without a check
 // of their place.
+__host__ __device__ inline float clip_row_err(const float *r) {
+    return 2.3902e-7f * ((fabsf(r[0]) + fabsf(r[1]) + fabsf(r[2])) * (float)(1 << LCL_GRID_BITS) + fabsf(r[3]));
+}
 __host__ __device__ inline float lasso_w_safe(const float *m, float ws, float hs) {
-    float e[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {  // rows x, y, w
-        const float *r = m + (k == 2 ? 12 : 4 * k);
-        e[k] = 2.3902e-7f * ((fabsf(r[0]) + fabsf(r[1]) + fabsf(r[2])) * (float)(1 << LCL_GRID_BITS) + fabsf(r[3]));
-    }
-    return 1.25f * fmaxf(ws * (e[0] + 2.0f * e[2]), hs * (e[1] + 2.0f * e[2]));
+    const float ew = 2.0f * clip_row_err(m + 12);
+    return 1.25f * fmaxf(ws * (clip_row_err(m) + ew), hs * (clip_row_err(m + 4) + ew));
 }
 
 // The lasso argument's scalars but for the polygon's: screen, label, bias and what follows from the matrix m.
@@ -852,6 +852,7 @@ __host__ __device__ inline void lasso_arg_scalars(LassoHead &p, const float *m, 
     p.label = label;
     p.nv = nv;
     p.w_safe = lasso_w_safe(m, p.ws, p.hs);
+    p.z_err = 2.6f * (clip_row_err(m + 8) + clip_row_err(m + 12));
 }
 
 // What follows from the polygon's bounding box: the widened box in pixels and NDC, the band mapping.
