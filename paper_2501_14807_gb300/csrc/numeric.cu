@@ -6,9 +6,9 @@
 //                 the 2, 4 or 8 lanes of its group, and the group's output word is merged with
 //                 shuffles and written by its first lane
 //   k_num_select  selection by value into a label layer (the lane owns its texels' label bytes)
-//   k_num_stats   zonal statistics: a contiguous range of quads per warp (a quad per lane and step);
-//                 runs of equal zone labels stay in registers, as integers, until the warp meets
-//                 another zone, then are reduced across the warp, rounded to double and flushed
+//   k_num_stats   zonal statistics: a warp walks down strips of 32 texels, four rows per step (a quad per
+//                 lane); two runs of equal zone labels stay in registers, as integers, until the warp
+//                 meets further zones, then are reduced across the warp, rounded to double and flushed
 //                 into a shared-memory table (or the output, for many zones); min / max through
 //                 order-preserving 64-bit keys
 #include <algorithm>
@@ -416,8 +416,12 @@ __device__ __forceinline__ __int128 warp_sum_i96(const Int96 &v) {
 // biased exponent is `base`.  A float32 value (significand m of 24 bits, exponent e) adds m << (e - base)
 // for exponents base .. base + kWindow; integer layers and float16 (multiples of 2^-24) have a fixed
 // unit.  A lane takes at most kRunTexels texels before a flush, so |s| < 2^(24 + kWindow + 10) and the
-// weighted sum (weights below 2^35) < 2^94.
+// weighted sum (weights below 2^35) < 2^94.  Float32 values below the unit, subnormals and infinities are
+// summed in binary64, per lane (OutSums).  The unit follows the values: it rises when a step holds a larger
+// one than the window, and falls when a step's largest value has fallen kFallen below the one it was set
+// for, kFallSteps steps at least after the last flush, so that it does not swing from step to step.
 constexpr int kWindow = 25, kRunTexels = 1024;
+constexpr int kHeadroom = 20, kFallen = 16, kFallSteps = 8;
 // Steps of a warp at least: a warp's zones and a CTA's table are written out at the end of its work.
 constexpr int kStatsSteps = 4;
 // Times a step lets zones take over runs; a step of more than twice as many zones is noise, whose texels
@@ -479,6 +483,72 @@ struct Quad4 {
     }
 };
 
+// m 2^e as a double, rounded to nearest, by integer operations (0 < m < 2^64, the result a normal double; an
+// FP64 operation costs a warp as much as 64 others on this part).
+__device__ __forceinline__ double scaled_to_double(uint64_t m, int e, uint32_t sign) {
+    const int lz = __clzll((long long)m);
+    m <<= lz;
+    const uint64_t q = (m >> 11) + ((m >> 10) & 1u);  // 53 bits, or 2^53, whose carry goes to the exponent
+    return __longlong_as_double((long long)((((uint64_t)(e - lz + 63 + 1022) << 52) + q) | ((uint64_t)sign << 63)));
+}
+
+// The binary64 sums of a thread's texels that do not fit their run's unit: value and weight x value, of one zone
+// for each of the two runs, until the end of a step in which a run changes its zone, or of the work.  They lie in
+// shared memory and are written to the table between steps, where registers are free: with a call in the
+// middle of a step or in the flush of a run, a layer without such texels took 7 to 80% more time.  8192^2
+// float32, one zone, of values near 1: 0.34 ms; with a value of 1e30 in each 4096 (256) texels 0.44 (0.58),
+// where an atomic per texel, 32 lanes to one address, took 16 (26) and binary64 sums throughout 0.58; of
+// values over 60 powers of two 0.60, and 17 with the atomics.
+struct OutSums {
+    double s[2][kThreads], w[2][kThreads];
+    uint32_t zone[2][kThreads];  // kNone: empty
+};
+// A texel of run i (zone `zone`): float32 bits v (not 0), weight w.  v and the product go to binary64 by their bits:
+// conversions and products on the FP64 pipe held layers of very wide range at 690 us for 8192^2, now 600.
+__device__ __forceinline__ void outs_add(OutSums &o, int i, uint32_t zone, uint32_t v, unsigned long long w, ZoneAcc *tab) {
+    const uint32_t e = (v >> 23) & 0xFFu, f = v & 0x7FFFFFu;
+    const double d = e - 1u < 254u ? __hiloint2double((int)((v & 0x80000000u) | ((e + 896u) << 20) | (f >> 3)), (int)(v << 29))
+                                   : (double)__uint_as_float(v);
+    const double wd = e < 255u && w ? scaled_to_double((uint64_t)(e ? f | 0x800000u : f) * w, (int)max(e, 1u) - 150, v >> 31)
+                                    : __dmul_rn(__ull2double_rn(w), d);
+    const uint32_t held = o.zone[i][threadIdx.x];
+    if (held == zone) {
+        o.s[i][threadIdx.x] = __dadd_rn(o.s[i][threadIdx.x], d);
+        o.w[i][threadIdx.x] = __dadd_rn(o.w[i][threadIdx.x], wd);
+    } else if (held == kNone) {
+        o.zone[i][threadIdx.x] = zone;
+        o.s[i][threadIdx.x] = d;
+        o.w[i][threadIdx.x] = wd;
+    } else {
+        atomicAdd(&tab[zone].sum, d);
+        atomicAdd(&tab[zone].wsum, wd);
+    }
+}
+// All of a warp's places into the table; every lane calls it.
+__device__ __noinline__ void outs_end(OutSums &o, ZoneAcc *tab) {
+#pragma unroll 1
+    for (int i = 0; i < 2; ++i) {
+        uint32_t zone = o.zone[i][threadIdx.x];
+        for (;;) {  // zone by zone
+            const uint32_t bal = __ballot_sync(0xffffffffu, zone != kNone);
+            if (!bal) break;
+            const int leader = __ffs(bal) - 1;
+            const uint32_t z = __shfl_sync(0xffffffffu, zone, leader);
+            double s = zone == z ? o.s[i][threadIdx.x] : 0.0, t = zone == z ? o.w[i][threadIdx.x] : 0.0;
+#pragma unroll 1
+            for (int k = 16; k; k >>= 1) {
+                s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, k));
+                t = __dadd_rn(t, __shfl_xor_sync(0xffffffffu, t, k));
+            }
+            if ((threadIdx.x & 31) == 0) {
+                atomicAdd(&tab[z].sum, s);
+                atomicAdd(&tab[z].wsum, t);
+            }
+            if (zone == z) o.zone[i][threadIdx.x] = zone = kNone;
+        }
+    }
+}
+
 // One texel into the table.
 template <int S, int KIND>
 __device__ __noinline__ void stats_single(ZoneAcc *tab, uint32_t n_zones, uint32_t zone, uint32_t v,
@@ -502,8 +572,11 @@ __device__ __noinline__ void stats_single(ZoneAcc *tab, uint32_t n_zones, uint32
 template <int S, int KIND, int ZB, bool SMEM>
 __global__ void __launch_bounds__(kThreads, 3) k_num_stats(StatsArgs p) {
     constexpr bool kF32 = KIND == kKindFloat && S == 4;
+    constexpr bool kFloat = KIND == kKindFloat;
     extern __shared__ ZoneAcc sh_zone[];
+    __shared__ OutSums outs;  // float layers only
     ZoneAcc *tab = SMEM ? sh_zone : p.out;
+    if (kFloat) outs.zone[0][threadIdx.x] = outs.zone[1][threadIdx.x] = kNone;
     if (SMEM) {
         for (uint32_t i = threadIdx.x; i < p.n_labels; i += blockDim.x) {
             sh_zone[i].count = 0;
@@ -550,10 +623,11 @@ __global__ void __launch_bounds__(kThreads, 3) k_num_stats(StatsArgs p) {
     run_reset(run[0]);
     run_reset(run[1]);
     run[0].zone = run[1].zone = kNone;
-    int base = kF32 ? 1 : KIND == kKindFloat ? 126 : 150;  // float32: raised to the values met; others: fixed
+    int base = kF32 ? 1 : KIND == kKindFloat ? 126 : 150;  // float32: follows the values met; others: fixed
     int since = 0;                                          // steps since the runs were last empty
-    // One run's sums into the table; every lane of the warp calls it.
-    auto flush = [&](StatsRun &r) {
+    // Run i's sums into the table; every lane of the warp calls it.
+    auto flush = [&](int i) {
+        StatsRun &r = run[i];
         const uint32_t cnt = __reduce_add_sync(0xffffffffu, r.cnt);
         if (cnt) {
             const __int128 area = warp_sum_i64((long long)r.area);
@@ -595,18 +669,22 @@ __global__ void __launch_bounds__(kThreads, 3) k_num_stats(StatsArgs p) {
             }
             ok |= (good ? 1u : 0u) << k;
         }
-        const bool above = kF32 && __any_sync(0xffffffffu, (int)emax > base + kWindow);
-        if (above || ++since > kRunTexels / 4) {  // uniform
-            flush(run[0]);
-            flush(run[1]);
+        const int top = kF32 ? (int)__reduce_max_sync(0xffffffffu, emax) : 0;  // 0: no normal value
+        ++since;
+        if (since > kRunTexels / 4 ||
+            (kF32 && (top > base + kWindow ||
+                      (top != 0 && base > 1 && top < base + kHeadroom - kFallen && since > kFallSteps)))) {  // uniform
+            flush(0);
+            flush(1);
             since = 1;
-            if (above) base = max((int)__reduce_max_sync(0xffffffffu, emax) - 20, 1);
+            if (kF32 && top != 0) base = max(top - kHeadroom, 1);
         }
 #pragma unroll
         for (int k = 1; k < 4; ++k)
             if (ts[k] == ts[k - 1]) w[k] = w[k - 1];
         // adds the texels take0 and take1 to the lane's shares of the two runs (with1: some lane has a take1)
         auto add = [&](uint32_t take0, uint32_t take1, bool with1) {
+            uint32_t miss = 0u;  // texels whose values do not fit the unit
             run[0].cnt += __popc(take0);
             run[1].cnt += __popc(take1);
 #pragma unroll
@@ -633,12 +711,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_num_stats(StatsArgs p) {
                     b0 = lo << sh;
                     b1 = __funnelshift_l(lo, hi, sh);
                     b2 = __funnelshift_l(hi, (uint32_t)((int32_t)hi >> 31), sh);
-                    if ((t0 || t1) && !fits && v[k] != 0u) {  // in binary64, into the table
-                        const double d = (double)__uint_as_float(v[k]);
-                        ZoneAcc &za = tab[t0 ? run[0].zone : run[1].zone];
-                        atomicAdd(&za.sum, d);
-                        atomicAdd(&za.wsum, __dmul_rn(__ull2double_rn(w[k]), d));
-                    }
+                    if (!fits && v[k] != 0u) miss |= 1u << k;
                 } else {
                     f = KIND == kKindSigned ? (long long)sext<S>(v[k]) : (long long)v[k];
                     if (S == 4) {
@@ -664,6 +737,15 @@ __global__ void __launch_bounds__(kThreads, 3) k_num_stats(StatsArgs p) {
                 acc(run[0], t0);
                 if (with1) acc(run[1], t1);
             }
+            if (kFloat) {  // rare: a loop, so that its code stands once and takes few registers
+#pragma unroll 1
+                for (miss &= take0 | take1; miss; miss &= miss - 1u) {
+                    const int k = __ffs(miss) - 1;
+                    const bool b = (take0 >> k) & 1u;
+                    outs_add(outs, b ? 0 : 1, b ? run[0].zone : run[1].zone, k & 2 ? (k & 1 ? v[3] : v[2]) : (k & 1 ? v[1] : v[0]),
+                             k & 2 ? (k & 1 ? w[3] : w[2]) : (k & 1 ? w[1] : w[0]), tab);
+                }
+            }
         };
         uint32_t in0 = 0u, in1 = 0u;
 #pragma unroll
@@ -673,15 +755,18 @@ __global__ void __launch_bounds__(kThreads, 3) k_num_stats(StatsArgs p) {
             else if (z[k] == run[1].zone) in1 |= b;
         }
         uint32_t odd = ok & ~(in0 | in1);
+        bool taken = false;  // a run has changed its zone
         // a zone not yet among the runs' takes over one that the step does not use (any more)
-        auto take_over = [&](StatsRun &r, uint32_t &in) {
+        auto take_over = [&](int i, uint32_t &in) {
+            StatsRun &r = run[i];
             const uint32_t bal = __ballot_sync(0xffffffffu, odd != 0u);
             if (!bal || __any_sync(0xffffffffu, in != 0u)) return;  // uniform
             uint32_t last = kNone;
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 if ((odd >> k) & 1u) last = z[k];
-            flush(r);
+            flush(i);
+            taken = true;
             r.zone = __shfl_sync(0xffffffffu, last, 31 - __clz(bal));
 #pragma unroll
             for (int k = 0; k < 4; ++k)
@@ -689,8 +774,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_num_stats(StatsArgs p) {
             odd &= ~in;
         };
         for (int round = 0; round < kZoneRounds; ++round) {
-            take_over(run[0], in0);
-            take_over(run[1], in1);
+            take_over(0, in0);
+            take_over(1, in1);
             if (__any_sync(0xffffffffu, (in0 | in1) != 0u)) add(in0, in1, __any_sync(0xffffffffu, in1 != 0u));
             in0 = in1 = 0u;
             if (!__any_sync(0xffffffffu, odd != 0u)) break;
@@ -698,10 +783,12 @@ __global__ void __launch_bounds__(kThreads, 3) k_num_stats(StatsArgs p) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)  // zones of a few texels: one by one, the lanes side by side
             if ((odd >> k) & 1u) stats_single<S, KIND>(tab, p.n_labels, z[k], v[k], w[k]);
+        if (kFloat && taken) outs_end(outs, tab);  // uniform
     }
     }
-    flush(run[0]);
-    flush(run[1]);
+    flush(0);
+    flush(1);
+    if (kFloat) outs_end(outs, tab);
     if (SMEM) {
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < p.n_labels; i += blockDim.x) {
@@ -730,7 +817,8 @@ void launch_select(const SelectArgs &p, cudaStream_t st) {
 template <int S, int KIND, int ZB, bool SMEM>
 void launch_stats_smem(const StatsArgs &p, size_t shb, cudaStream_t st) {
     auto kernel = k_num_stats<S, KIND, ZB, SMEM>;
-    if (SMEM && shb > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shb);
+    constexpr size_t kOuts = KIND == kKindFloat ? sizeof(OutSums) : 0;
+    if (SMEM && shb + kOuts > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shb);
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, shb) != cudaSuccess || per_sm < 1)
         per_sm = 1;
