@@ -492,42 +492,49 @@ __device__ __forceinline__ double scaled_to_double(uint64_t m, int e, uint32_t s
     return __longlong_as_double((long long)((((uint64_t)(e - lz + 63 + 1022) << 52) + q) | ((uint64_t)sign << 63)));
 }
 
-// The binary64 sums of a thread's texels that do not fit their run's unit: value and weight x value, of one zone
-// for each of the two runs, until the end of a step in which a run changes its zone, or of the work.  They lie in
-// shared memory and are written to the table between steps, where registers are free: with a call in the
+// The binary64 sums of a thread's texels that do not fit their run's unit: value and weight x value, by zone, until
+// the end of a step in which a run changes its zone, or of the work: such a step holds texels of two zones and of
+// the two before them (more go to the table one by one).  They lie in shared memory and are written to the table between steps, where registers are free: with a call in the
 // middle of a step or in the flush of a run, a layer without such texels took 7 to 80% more time.  8192^2
-// float32, one zone, of values near 1: 0.34 ms; with a value of 1e30 in each 4096 (256) texels 0.44 (0.58),
+// float32, one zone, of values near 1: 0.34 ms; with a value of 1e30 in each 4096 (256) texels 0.46 (0.61),
 // where an atomic per texel, 32 lanes to one address, took 16 (26) and binary64 sums throughout 0.58; of
-// values over 60 powers of two 0.60, and 17 with the atomics.
+// values over 60 powers of two 0.64, and 17 with the atomics.
+constexpr int kOutZones = 4;
 struct OutSums {
-    double s[2][kThreads], w[2][kThreads];
-    uint32_t zone[2][kThreads];  // kNone: empty
+    double s[kOutZones][kThreads], w[kOutZones][kThreads];
+    uint32_t zone[kOutZones][kThreads];  // filled from the first place on; kNone: empty
 };
-// A texel of run i (zone `zone`): float32 bits v (not 0), weight w.  v and the product go to binary64 by their bits:
-// conversions and products on the FP64 pipe held layers of very wide range at 690 us for 8192^2, now 600.
-__device__ __forceinline__ void outs_add(OutSums &o, int i, uint32_t zone, uint32_t v, unsigned long long w, ZoneAcc *tab) {
+// A texel of zone `zone`: float32 bits v (not 0), weight w.  v and the product go to binary64 by their bits: by
+// conversions and products on the FP64 pipe layers of very wide range took 690 us for 8192^2, not 610.
+__device__ __forceinline__ void outs_add(OutSums &o, uint32_t zone, uint32_t v, unsigned long long w, ZoneAcc *tab) {
     const uint32_t e = (v >> 23) & 0xFFu, f = v & 0x7FFFFFu;
     const double d = e - 1u < 254u ? __hiloint2double((int)((v & 0x80000000u) | ((e + 896u) << 20) | (f >> 3)), (int)(v << 29))
                                    : (double)__uint_as_float(v);
     const double wd = e < 255u && w ? scaled_to_double((uint64_t)(e ? f | 0x800000u : f) * w, (int)max(e, 1u) - 150, v >> 31)
                                     : __dmul_rn(__ull2double_rn(w), d);
-    const uint32_t held = o.zone[i][threadIdx.x];
-    if (held == zone) {
-        o.s[i][threadIdx.x] = __dadd_rn(o.s[i][threadIdx.x], d);
-        o.w[i][threadIdx.x] = __dadd_rn(o.w[i][threadIdx.x], wd);
-    } else if (held == kNone) {
-        o.zone[i][threadIdx.x] = zone;
-        o.s[i][threadIdx.x] = d;
-        o.w[i][threadIdx.x] = wd;
-    } else {
+    int i = 0;
+    uint32_t held = o.zone[0][threadIdx.x];
+#pragma unroll 1
+    while (held != zone && held != kNone && ++i < kOutZones) held = o.zone[i][threadIdx.x];
+    if (i == kOutZones) {
         atomicAdd(&tab[zone].sum, d);
         atomicAdd(&tab[zone].wsum, wd);
+        return;
+    }
+    double &s = o.s[i][threadIdx.x], &t = o.w[i][threadIdx.x];
+    if (held == zone) {
+        s = __dadd_rn(s, d);
+        t = __dadd_rn(t, wd);
+    } else {
+        o.zone[i][threadIdx.x] = zone;
+        s = d;
+        t = wd;
     }
 }
 // All of a warp's places into the table; every lane calls it.
 __device__ __noinline__ void outs_end(OutSums &o, ZoneAcc *tab) {
 #pragma unroll 1
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kOutZones; ++i) {
         uint32_t zone = o.zone[i][threadIdx.x];
         for (;;) {  // zone by zone
             const uint32_t bal = __ballot_sync(0xffffffffu, zone != kNone);
@@ -576,7 +583,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_num_stats(StatsArgs p) {
     extern __shared__ ZoneAcc sh_zone[];
     __shared__ OutSums outs;  // float layers only
     ZoneAcc *tab = SMEM ? sh_zone : p.out;
-    if (kFloat) outs.zone[0][threadIdx.x] = outs.zone[1][threadIdx.x] = kNone;
+    if (kFloat)
+        for (int i = 0; i < kOutZones; ++i) outs.zone[i][threadIdx.x] = kNone;
     if (SMEM) {
         for (uint32_t i = threadIdx.x; i < p.n_labels; i += blockDim.x) {
             sh_zone[i].count = 0;
@@ -742,7 +750,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_num_stats(StatsArgs p) {
                 for (miss &= take0 | take1; miss; miss &= miss - 1u) {
                     const int k = __ffs(miss) - 1;
                     const bool b = (take0 >> k) & 1u;
-                    outs_add(outs, b ? 0 : 1, b ? run[0].zone : run[1].zone, k & 2 ? (k & 1 ? v[3] : v[2]) : (k & 1 ? v[1] : v[0]),
+                    outs_add(outs, b ? run[0].zone : run[1].zone, k & 2 ? (k & 1 ? v[3] : v[2]) : (k & 1 ? v[1] : v[0]),
                              k & 2 ? (k & 1 ? w[3] : w[2]) : (k & 1 ? w[1] : w[0]), tab);
                 }
             }
