@@ -49,16 +49,22 @@ __global__ void k_sel_init(uint32_t *counters, int32_t n, unsigned long long *hi
     }
 }
 
+// Is every texel of tile (tx, ty) covered, `count` being the covered ones?  Padding writes uncovered texels only, so
+// such a tile goes through a padded edit as through one without padding.
+__device__ __forceinline__ bool tile_full(const AtlasDev &a, int32_t tx, int32_t ty, int32_t count) {
+    return count == min(a.T, a.w - tx * a.T) * min(a.T, a.h - ty * a.T);
+}
+
 // Culls stroke s against super-tile `sidx`, appending its candidate tiles.  Uniform per CTA.
 // With texture padding (PAD) a texel may be written because a neighbour within 8 texels was
-// selected, so a tile (super-tile) is then a candidate if any box of its 3 x 3 neighbourhood is
-// in reach.  PAD is a template parameter so that the common case carries no registers for it.
-// Tiles inside the sphere go to the back of the list (counter `inside_counter`) when whole-row
-// handling applies (`rows`: tile side >= 32 and width a multiple of 32), else to the front with
-// kInsideTile set.
+// selected, so a super-tile, and a tile with uncovered texels, is then a candidate if any box of its 3 x 3
+// neighbourhood is in reach; tiles with uncovered texels go to the back of the list (counter `back_counter`).
+// PAD is a template parameter so that the common case carries no registers for it.
+// Without padding tiles inside the sphere go to the back of the list when whole-row handling applies
+// (`rows`: tile side >= 32 and width a multiple of 32), else to the front with kInsideTile set.
 template <bool PAD>
 __device__ __forceinline__ void cull_super_sphere(const AtlasDev &a, const SphereArg &s, int32_t sidx,
-                                                  uint32_t *counter, uint32_t *list, uint32_t *inside_counter,
+                                                  uint32_t *counter, uint32_t *list, uint32_t *back_counter,
                                                   bool rows) {
     const int32_t sx = sidx % a.supers_x, sy = sidx / a.supers_x;
     bool in_reach;
@@ -74,35 +80,36 @@ __device__ __forceinline__ void cull_super_sphere(const AtlasDev &a, const Spher
     if (!in_reach) return;  // uniform over the CTA
     const int32_t tx = sx * LCL_SUPER + (threadIdx.x % LCL_SUPER);
     const int32_t ty = sy * LCL_SUPER + (threadIdx.x / LCL_SUPER);
-    bool cand = false, inside = false;
+    bool cand = false, inside = false, back = false;
     const int64_t n_tiles = (int64_t)a.tiles_x * a.tiles_y;
-    if (tx < a.tiles_x && ty < a.tiles_y) {
-        if (PAD) {
-            cand = near_box_3x3(a.tile_box, a.tiles_x, a.tiles_y, tx, ty, s);
-        } else if (LCL_IN((int64_t)ty * a.tiles_x + tx, n_tiles)) {
-            const int4 *tb = reinterpret_cast<const int4 *>(a.tile_box + 8 * ((int64_t)ty * a.tiles_x + tx));
-            const int4 lo = tb[0], hi = tb[1];
+    if (tx < a.tiles_x && ty < a.tiles_y && LCL_IN((int64_t)ty * a.tiles_x + tx, n_tiles)) {
+        const int4 *tb = reinterpret_cast<const int4 *>(a.tile_box + 8 * ((int64_t)ty * a.tiles_x + tx));
+        const int4 lo = tb[0], hi = tb[1];
+        if (PAD && !tile_full(a, tx, ty, lo.w)) {
+            back = near_box_3x3(a.tile_box, a.tiles_x, a.tiles_y, tx, ty, s);
+        } else {
             cand = lo.w > 0 && box_dist2(lo, hi, s) <= s.r2;
             // the sphere contains the tile's box: every covered texel of the tile is selected
             inside = cand && box_far2(lo, hi, s) <= s.r2;
+            if (!PAD) back = inside && rows;
         }
     }
     const uint32_t tile = (uint32_t)(ty * a.tiles_x + tx);
-    append_candidate(cand && !(inside && rows), tile | (inside ? kInsideTile : 0u), counter, list, n_tiles);
-    if (!PAD) append_candidate_back(inside && rows, tile, inside_counter, list, n_tiles);
+    append_candidate(cand && !back, tile | (inside ? kInsideTile : 0u), counter, list, n_tiles);
+    append_candidate_back(back, tile, back_counter, list, n_tiles);
 }
 
 // Culls the first stroke of a call.
 __global__ void __launch_bounds__(kThreads) k_sphere_cull(AtlasDev a, SphereArg s, uint32_t *counter,
-                                                          uint32_t *list, uint32_t *inside_counter) {
+                                                          uint32_t *list, uint32_t *back_counter) {
     pdl_wait();
     const int32_t n_super = a.supers_x * a.supers_y;
     const bool rows = a.T >= 32 && (a.w & 31) == 0;
     for (int32_t sidx = blockIdx.x; sidx < n_super; sidx += gridDim.x) {
         if (s.pad_r > 0)
-            cull_super_sphere<true>(a, s, sidx, counter, list, inside_counter, rows);
+            cull_super_sphere<true>(a, s, sidx, counter, list, back_counter, rows);
         else
-            cull_super_sphere<false>(a, s, sidx, counter, list, inside_counter, rows);
+            cull_super_sphere<false>(a, s, sidx, counter, list, back_counter, rows);
     }
     pdl_allow_next();
 }
@@ -163,7 +170,9 @@ __device__ __forceinline__ uint32_t sphere_mask(const Item &it, const SphereArg 
 // texel of the block and of a halo around it once, a texel per lane, and the ballots become rows of
 // coverage and selection bits in shared memory; both dilations are then shifts and ORs of whole rows.
 // Testing the neighbours of each uncovered texel over again, as before, took 73 us for one tool edit
-// (radius 70 px, padding 2) on an 8192^2 chart atlas.
+// (radius 70 px, padding 2) on an 8192^2 chart atlas.  Only tiles with uncovered texels come here: taking
+// covered ones too, halo and all, a padded stroke on a texture without gutters took up to 3.5 times as long
+// (3 strokes of 10-30% of the diagonal on 8192^2 with padding 8: 100 us before the bits, 349 so, now 47).
 struct PadShared {
     uint32_t hit0[48], hit1[48], cov0[48], cov1[48];  // per halo row: 32 and 16 texels from 8 left of the block
     uint32_t out_hit[32], out_pad[32];                // per block row: selected texels, padded texels
@@ -259,17 +268,18 @@ __device__ __forceinline__ uint32_t pad_block(const AtlasDev &a, L *__restrict__
     return cnt;
 }
 
-// pad_block over the n candidate tiles of `list`.
+// pad_block over the n candidate tiles at the back of `list`.
 template <typename L, bool NUM, typename Hit>
 __device__ __forceinline__ uint32_t pad_tiles(const AtlasDev &a, L *__restrict__ layer, PadShared &sh, uint32_t n,
                                               const uint32_t *__restrict__ list, int32_t pad_r, int32_t pad_t,
                                               uint32_t label, const ValMask &vm, const Hit &hit) {
     const int32_t B = min(a.T, 32);
     const int per_log = 2 * (__ffs(a.T) - __ffs(B));  // blocks per tile: 1 << per_log
+    const int64_t cap = (int64_t)a.tiles_x * a.tiles_y;
     uint32_t cnt = 0;
     for (uint32_t i = blockIdx.x; i < n << per_log; i += gridDim.x) {  // uniform over the CTA
-        if (!LCL_IN(i >> per_log, (int64_t)a.tiles_x * a.tiles_y)) break;
-        const uint32_t tile = list[i >> per_log] & ~kInsideTile;
+        if (!LCL_IN(cap - 1 - (int64_t)(i >> per_log), cap)) break;
+        const uint32_t tile = list[cap - 1 - (int64_t)(i >> per_log)];
         int32_t tx, ty;
         tile_xy(a, tile, tx, ty);
         const int32_t b = (int32_t)(i & ((1u << per_log) - 1u)), side = 1 << (per_log / 2);
@@ -283,38 +293,31 @@ __device__ __forceinline__ uint32_t pad_tiles(const AtlasDev &a, L *__restrict__
 // Applies stroke `s` from its candidate list and culls stroke `nxt` (if has_next) into the other list.
 // PAD: `s` pads the texture; NEXT_PAD: `nxt` does.  NUM: a numeric layer, whose mask bits (vm) are
 // set (or cleared) for every texel written.
-// Lists: candidate tiles the sphere's surface may cross at the front (`counter` entries), tiles
-// inside the sphere at the back (`inside_counter` entries, whole-row layouts only): a warp takes one
-// such tile, each lane one 32-texel row segment, whose coverage word says which texels get the label.
+// Lists: candidate tiles the sphere's surface may cross at the front (`counter` entries).  At the back
+// (`back_counter` entries) without padding tiles inside the sphere (whole-row layouts only): a warp takes one
+// such tile, each lane one 32-texel row segment, whose coverage word says which texels get the label; with
+// padding tiles that hold uncovered texels.
 template <typename L, bool PAD, bool NEXT_PAD, bool NUM>
 __global__ void __launch_bounds__(kThreads, 6) k_sphere_step(AtlasDev a, L *__restrict__ layer, SphereArg s,
                                                           const uint32_t *__restrict__ counter,
-                                                          const uint32_t *__restrict__ inside_counter,
+                                                          const uint32_t *__restrict__ back_counter,
                                                           const uint32_t *__restrict__ list,
                                                           unsigned long long *hits, int has_next, SphereArg nxt,
-                                                          uint32_t *next_counter, uint32_t *next_inside_counter,
+                                                          uint32_t *next_counter, uint32_t *next_back_counter,
                                                           uint32_t *next_list, ValMask vm) {
     const bool rows = a.T >= 32 && (a.w & 31) == 0;  // uniform
     // Cull of the next stroke: reads only the atlas boxes; its list is free (see the top of the file).
     if (has_next) {
         const int32_t n_super = a.supers_x * a.supers_y;
         for (int32_t sidx = blockIdx.x; sidx < n_super; sidx += gridDim.x)
-            cull_super_sphere<NEXT_PAD>(a, nxt, sidx, next_counter, next_list, next_inside_counter, rows);
+            cull_super_sphere<NEXT_PAD>(a, nxt, sidx, next_counter, next_list, next_back_counter, rows);
     }
     pdl_wait();
     pdl_allow_next();  // after the wait: grid k + 1 starts once every CTA of this grid got here
-    if (PAD) {
-        __shared__ PadShared sh;
-        const auto hit = [&](int32_t x, int32_t y, int32_t z) {
-            const int64_t dx = (int64_t)x - s.cx, dy = (int64_t)y - s.cy, dz = (int64_t)z - s.cz;
-            return dx * dx + dy * dy + dz * dz <= s.r2;
-        };
-        add_hits(hits, pad_tiles<L, NUM>(a, layer, sh, *counter, list, s.pad_r, s.pad_t, s.label, vm, hit));
-        return;
-    }
     const int32_t qpr = a.T / 4, nq = a.T * qpr;
     const int cpt_log2 = nq > kThreads ? 31 - __clz(nq / kThreads) : 0;
     const uint32_t n_items = *counter << cpt_log2;
+    const uint32_t n_pad = PAD ? *back_counter : 0u;
     const bool grouped = a.T >= 32 && (a.w & 31) == 0;  // uniform: see valid_update_warp
     const int64_t n_tex = (int64_t)a.w * a.h;
     (void)n_tex;
@@ -347,15 +350,20 @@ __global__ void __launch_bounds__(kThreads, 6) k_sphere_step(AtlasDev a, L *__re
         }
         cur = next;
     }
-    // tiles inside the sphere: one warp per tile, one lane per 32-texel row segment
-    const uint32_t n_in = *inside_counter;
-    if (n_in) {  // uniform
+    if (PAD) {  // tiles with uncovered texels
+        __shared__ PadShared sh;
+        const auto hit = [&](int32_t x, int32_t y, int32_t z) {
+            const int64_t dx = (int64_t)x - s.cx, dy = (int64_t)y - s.cy, dz = (int64_t)z - s.cz;
+            return dx * dx + dy * dy + dz * dz <= s.r2;
+        };
+        cnt += pad_tiles<L, NUM>(a, layer, sh, n_pad, list, s.pad_r, s.pad_t, s.label, vm, hit);
+    } else if (const uint32_t n_back = *back_counter) {  // uniform; tiles inside: a warp each, a 32-texel row segment per lane
         const int64_t cap = (int64_t)a.tiles_x * a.tiles_y;
         const int32_t wpr = a.T >> 5, words = a.T * wpr;  // row segments per tile row and per tile
         const uint32_t warps = gridDim.x * (kThreads / 32);
         // from the last CTA down: when the grid has CTAs to spare, the tiles above go to the first
         // CTAs and these to others, so that neither waits for the other
-        for (uint32_t b = (gridDim.x - 1 - blockIdx.x) * (kThreads / 32) + (threadIdx.x >> 5); b < n_in; b += warps) {
+        for (uint32_t b = (gridDim.x - 1 - blockIdx.x) * (kThreads / 32) + (threadIdx.x >> 5); b < n_back; b += warps) {
             if (!LCL_IN(cap - 1 - (int64_t)b, cap)) break;
             const uint32_t tile = __ldg(list + (cap - 1 - (int64_t)b));
             int32_t tx, ty;
@@ -696,8 +704,8 @@ __global__ void __launch_bounds__(kThreads) k_lasso_supers(AtlasDev a, const __g
 // Candidate tiles of a lasso (or tool window) in the super-tiles k_lasso_supers listed: the CTAs take
 // (super-tile, part) units, a part being kThreads / G tiles tested by G lanes each (box_may_touch_by
 // with the depth map), so the work spreads over the GPU however few super-tiles the lasso reaches.
-// FLAGS: write a 0/1 flag per tile instead of appending candidates (first pass of a padded edit; the
-// flags of tiles in other super-tiles were cleared before).  CLASSIFY (lassos): tiles that
+// FLAGS: write a flag per tile (0; 1: candidate; 2: inside the polygon) instead of appending candidates (first
+// pass of a padded edit; the flags of tiles in other super-tiles were cleared before).  CLASSIFY (lassos): tiles that
 // lasso_tile_class finds outside the polygon are dropped, and those it finds inside are listed with
 // kInsideTile set (their texels skip the edge tests).
 // G: a warp per tile where tiles are few, and so large on the screen: hidden ones have hundreds of
@@ -745,7 +753,8 @@ __global__ void __launch_bounds__(kThreads) k_lasso_cull(AtlasDev a, const __gri
         }
         const uint32_t tile = (uint32_t)(ty * a.tiles_x + tx);
         if (FLAGS) {
-            if (in_grid && (threadIdx.x & (G - 1u)) == 0 && LCL_IN(tile, n_tiles)) list[tile] = cand ? 1u : 0u;
+            if (in_grid && (threadIdx.x & (G - 1u)) == 0 && LCL_IN(tile, n_tiles))
+                list[tile] = !cand ? 0u : cls == kTileIn ? 2u : 1u;
         } else {
             append_candidate(cand && (threadIdx.x & (G - 1u)) == 0, tile | (cls == kTileIn ? kInsideTile : 0u), counter,
                              list, n_tiles);
@@ -754,27 +763,38 @@ __global__ void __launch_bounds__(kThreads) k_lasso_cull(AtlasDev a, const __gri
 }
 
 // Second pass of a padded edit: with texture padding a texel may be written because a neighbour
-// within 8 texels (at most one tile away) was selected, so a tile is a candidate if any tile of
-// its 3 x 3 neighbourhood is flagged.
+// within 8 texels (at most one tile away) was selected, so a tile with uncovered texels is a candidate if any
+// tile of its 3 x 3 neighbourhood is flagged: these go to the back of the list (counter `back_counter`).  A tile
+// without is one if its own flag is set, as without padding.
 __global__ void __launch_bounds__(kThreads) k_dilate_candidates(AtlasDev a, const uint32_t *__restrict__ flags,
-                                                                uint32_t *counter, uint32_t *list) {
+                                                                uint32_t *counter, uint32_t *back_counter,
+                                                                uint32_t *list) {
     pdl_wait();  // the flags are complete
     pdl_allow_next();
     const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     const int64_t n_tiles = (int64_t)a.tiles_x * a.tiles_y;
-    bool cand = false;
+    bool cand = false, back = false;
+    uint32_t own = 0u;
     if (t < n_tiles) {
         const int32_t tx = (int32_t)(t % a.tiles_x), ty = (int32_t)(t / a.tiles_x);
-        for (int32_t y = max(ty - 1, 0); y <= min(ty + 1, a.tiles_y - 1) && !cand; ++y)
+        bool near = false;
+        for (int32_t y = max(ty - 1, 0); y <= min(ty + 1, a.tiles_y - 1) && !near; ++y)
             for (int32_t x = max(tx - 1, 0); x <= min(tx + 1, a.tiles_x - 1); ++x)
-                if (LCL_IN((int64_t)y * a.tiles_x + x, n_tiles) && flags[(int64_t)y * a.tiles_x + x]) cand = true;
+                if (LCL_IN((int64_t)y * a.tiles_x + x, n_tiles) && flags[(int64_t)y * a.tiles_x + x]) near = true;
+        if (near && LCL_IN(t, n_tiles)) {
+            own = flags[t];
+            const bool full = tile_full(a, tx, ty, a.tile_box[8 * t + 3]);
+            cand = full && own;
+            back = !full;
+        }
     }
-    append_candidate(cand, (uint32_t)t, counter, list, n_tiles);
+    append_candidate(cand, (uint32_t)t | (own == 2u ? kInsideTile : 0u), counter, list, n_tiles);
+    append_candidate_back(back, (uint32_t)t, back_counter, list, n_tiles);
 }
 
 
 // A lasso's candidate-list entry: tile index, kInsideTile set when every texel of the tile that
-// projects lies inside the polygon (lasso_tile_class8).  Padded edits list plain tile indices.
+// projects lies inside the polygon (lasso_tile_class).
 // An edit's CTAs take kEditQuads quads at a time, one per thread, of one tile or of several small ones
 // (a CTA per tile left threads idle where a tile has fewer quads: 105 -> 80 us for 3 lassos over tiles
 // of 16 on 2048^2).  The lasso's apply is bound by instruction issue and by the latency of its loads;
@@ -783,6 +803,7 @@ __global__ void __launch_bounds__(kThreads) k_dilate_candidates(AtlasDev a, cons
 // 421 -> 417 us.  Four CTAs per SM, since few tiles are candidates on a small atlas: with three (and
 // no bound on the registers) 853 and 428 us.  CTAs of 64 and 128 threads were slower (462 and 426 us).
 constexpr int kEditQuads = 256;
+constexpr int kBackCounter = 2;  // of a lasso or tool edit's counters: list entries, super-tiles, entries at the back
 template <bool PAD>
 constexpr int edit_threads() {
     return PAD ? kThreads : kEditQuads;
@@ -822,13 +843,7 @@ __global__ void __launch_bounds__(edit_threads<PAD>(), 4) k_lasso_apply(AtlasDev
     __syncthreads();
     pdl_wait();  // the candidate tiles are complete
     pdl_allow_next();
-    const uint32_t n = *counter;
-    if (PAD) {
-        __shared__ PadShared ps;
-        const auto hit = [&](int32_t x, int32_t y, int32_t z) { return lasso_hit(p, sh, depth, x, y, z); };
-        add_hits(hits, pad_tiles<L, NUM>(a, layer, ps, n, list, pad_r, pad_t, p.label, vm, hit));
-        return;
-    }
+    const uint32_t n = *counter, n_back = PAD ? counter[kBackCounter] : 0u;
     uint32_t cnt = 0;
     const int64_t n_tex = (int64_t)a.w * a.h;
     const uint32_t n_items = edit_items(a, n);
@@ -860,6 +875,11 @@ __global__ void __launch_bounds__(edit_threads<PAD>(), 4) k_lasso_apply(AtlasDev
             cnt += __popc(m);
         }
     }
+    if (PAD) {  // tiles with uncovered texels
+        __shared__ PadShared ps;
+        const auto hit = [&](int32_t x, int32_t y, int32_t z) { return lasso_hit(p, sh, depth, x, y, z); };
+        cnt += pad_tiles<L, NUM>(a, layer, ps, n_back, list, pad_r, pad_t, p.label, vm, hit);
+    }
     add_hits(hits, cnt);
 }
 
@@ -874,13 +894,7 @@ __global__ void __launch_bounds__(edit_threads<PAD>(), 1024 / edit_threads<PAD>(
                                                          unsigned long long *hits, ValMask vm) {
     pdl_wait();  // the candidate tiles are complete
     pdl_allow_next();
-    const uint32_t n = *counter;
-    if (PAD) {
-        __shared__ PadShared sh;
-        const auto hit = [&](int32_t x, int32_t y, int32_t z) { return tool_hit<MASK>(p, t, depth, x, y, z); };
-        add_hits(hits, pad_tiles<L, NUM>(a, layer, sh, n, list, t.pad_r, t.pad_t, p.label, vm, hit));
-        return;
-    }
+    const uint32_t n = *counter, n_back = PAD ? counter[kBackCounter] : 0u;
     uint32_t cnt = 0;
     const int64_t n_tex = (int64_t)a.w * a.h;
     const uint32_t n_items = edit_items(a, n);
@@ -902,6 +916,11 @@ __global__ void __launch_bounds__(edit_threads<PAD>(), 1024 / edit_threads<PAD>(
             cnt += __popc(m);
         }
     }
+    if (PAD) {  // tiles with uncovered texels
+        __shared__ PadShared sh;
+        const auto hit = [&](int32_t x, int32_t y, int32_t z) { return tool_hit<MASK>(p, t, depth, x, y, z); };
+        cnt += pad_tiles<L, NUM>(a, layer, sh, n_back, list, t.pad_r, t.pad_t, p.label, vm, hit);
+    }
     add_hits(hits, cnt);
 }
 
@@ -914,7 +933,7 @@ SelWs sel_ws(const lcl_atlas *a, int32_t n, void *ws) {
     SelWs w;
     char *base = static_cast<char *>(ws);
     const size_t lb = align256((size_t)a->tiles_x * a->tiles_y * 4);
-    w.counters = reinterpret_cast<uint32_t *>(base);  // n + 1 front counters, then n + 1 inside counters
+    w.counters = reinterpret_cast<uint32_t *>(base);  // n + 1 front counters, then n + 1 back counters (lassos and the tool: three)
     w.list = reinterpret_cast<uint32_t *>(base + align256((size_t)2 * (n + 1) * 4));
     w.list2 = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(w.list) + lb);
     w.list3 = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(w.list2) + lb);
@@ -944,12 +963,12 @@ int launch_lasso_cull_by(const AtlasDev &a, const lcl_atlas *atlas, const LassoA
     }
     // padded edits: flags for every tile that may hold a selected texel (polygon-outside tiles of a
     // lasso hold none; tiles of super-tiles the lasso cannot reach keep the cleared 0), dilated to the
-    // tiles padding can reach
+    // tiles with uncovered texels that padding can reach
     const int64_t tiles = (int64_t)atlas->tiles_x * atlas->tiles_y;
     launch_pdl(classify ? k_lasso_cull<true, true, G> : k_lasso_cull<true, false, G>, dim3(grid), st, a, p, depth,
                super_count, supers, w.counters, w.list2);
     launch_pdl(k_dilate_candidates, dim3((unsigned)((tiles + kThreads - 1) / kThreads)), st, a,
-               (const uint32_t *)w.list2, w.counters, w.list);
+               (const uint32_t *)w.list2, w.counters, w.counters + kBackCounter, w.list);
     return 3;
 }
 
@@ -957,7 +976,7 @@ int launch_lasso_cull_by(const AtlasDev &a, const lcl_atlas *atlas, const LassoA
 void launch_edit_init(const lcl_atlas *atlas, const SelWs &w, unsigned long long *h, bool pad, cudaStream_t st) {
     const int32_t n_flags = pad ? atlas->tiles_x * atlas->tiles_y : 0;
     const int grid = std::max(1, std::min((n_flags + kThreads - 1) / kThreads, 2 * sm_count()));
-    launch_pdl(k_sel_init, dim3(grid), st, w.counters, 2, h, 1, w.list2, n_flags);
+    launch_pdl(k_sel_init, dim3(grid), st, w.counters, 3, h, 1, w.list2, n_flags);
 }
 
 // Launches the cull of a lasso / tool into w.list (counter w.counters[0]); with padding, the flags
@@ -1174,11 +1193,11 @@ lcl_status select_sphere_run(const lcl_atlas *atlas, L *layer, uint32_t *mask, c
     int grid[2][2];
     for (int i = 0; i < 2; ++i)
         for (int j = 0; j < 2; ++j) grid[i][j] = resident_grid(step[i][j]);
-    uint32_t *const inside = w.counters + (n + 1);
+    uint32_t *const back = w.counters + (n + 1);
     k_sel_init<<<(2 * (n + 1) + kThreads - 1) / kThreads, kThreads, 0, st>>>(w.counters, 2 * (n + 1), h, n, nullptr, 0);
     const int n_super = atlas->supers_x * atlas->supers_y;
     cudaError_t e = launch_pdl(k_sphere_cull, dim3(std::min(n_super, grid[0][0])), st, a, arg(0), w.counters, w.list,
-                               inside);
+                               back);
     for (int32_t k = 0; k < n && e == cudaSuccess; ++k) {
         uint32_t *const lists[3] = {w.list, w.list2, w.list3};
         uint32_t *cur_list = lists[k % 3], *next_list = lists[(k + 1) % 3];
@@ -1186,8 +1205,8 @@ lcl_status select_sphere_run(const lcl_atlas *atlas, L *layer, uint32_t *mask, c
         const SphereArg cur = arg(k), nxt = arg(has_next ? k + 1 : k);
         const int pi = cur.pad_r > 0, pj = has_next && nxt.pad_r > 0;
         e = launch_pdl(step[pi][pj], dim3(grid[pi][pj]), st, a, layer, cur, (const uint32_t *)(w.counters + k),
-                       (const uint32_t *)(inside + k), (const uint32_t *)cur_list, h ? h + k : nullptr, has_next, nxt,
-                       w.counters + k + 1, inside + k + 1, next_list, vmask(k));
+                       (const uint32_t *)(back + k), (const uint32_t *)cur_list, h ? h + k : nullptr, has_next, nxt,
+                       w.counters + k + 1, back + k + 1, next_list, vmask(k));
     }
     count_launches(2 + n);
     if (e == cudaSuccess) e = cudaGetLastError();
