@@ -9,7 +9,7 @@
 //   k_init        tri plane := none, coverage bits := 0, header reset
 //   k_bbox        float bbox of all positions (order-preserving integer atomics)
 //   k_scale       grid scale (2^21-1)/extent, one thread
-//   k_quant       every vertex to the grid (double, rounded once per operation)
+//   k_quant       every vertex to the grid (as in binary64, rounded once per operation)
 //   k_snap        every texture coordinate to 1/256 texel (round half to even)
 //   k_raster      one thread per triangle: position planes, area weight, and the texels of
 //                 small triangles; big triangles are split into 16x16-texel blocks appended to a
@@ -19,8 +19,6 @@
 //                 (from the triangle's planes where their rounding cannot matter, else exact
 //                 barycentrics), coverage bits, tile box
 //   k_super       one CTA per super-tile: union of its tile boxes
-// Where triangles overlap in the texture (found by counting), k_raster to k_super run once more, with
-// atomicMin: the smallest id wins.
 #include <algorithm>
 #include <cstring>
 
@@ -45,8 +43,6 @@ __global__ void k_init(uint32_t *__restrict__ tri, int64_t n_texels, uint32_t *_
         }
         hdr->flags = 0;
         hdr->n_big = 0;
-        hdr->n_covered = 0;
-        for (int a = 0; a < 8; ++a) hdr->n_hits[a] = 0;
     }
 }
 
@@ -345,21 +341,12 @@ __device__ __forceinline__ TriPlane make_plane(const Corners &c, int32_t ex, int
     return p;
 }
 
-// Marks a texel as covered by triangle t.  MIN: by the smallest id (texels that several triangles
-// cover); otherwise by whichever triangle comes last.
-template <bool MIN>
-__device__ __forceinline__ void mark_texel(uint32_t *texel, uint32_t t) {
-    if (MIN) atomicMin(texel, t);
-    else *texel = t;
-}
-
 // raster_rect for a triangle whose corners span at most 2^14 sub-pixels (64 texels) on each axis.
 // The scanned texel centres lie within the corners' bounding box (the texel range is cut from it),
 // and the values computed one texel past the last column or row within one texel of it, so with
 // ex, ey <= 2^14 the extents: |edge value| <= ex (ey + 256) + ey (ex + 256) + 1 < 2^30, and the
 // steps are at most 256 * 2^14.  The scan therefore runs in 32-bit integers after an exact start.
-template <bool MIN>
-__device__ __forceinline__ uint32_t raster_rect_small(const Corners &s, uint32_t t, int32_t i0, int32_t i1, int32_t j0, int32_t j1,
+__device__ __forceinline__ void raster_rect_small(const Corners &s, uint32_t t, int32_t i0, int32_t i1, int32_t j0, int32_t j1,
                                   int32_t w, int32_t row0, int32_t rows, uint32_t *__restrict__ tri_plane) {
     const int32_t X0 = s.x[0], X1 = s.x[1], X2 = s.x[2], Y0 = s.y[0], Y1 = s.y[1], Y2 = s.y[2];
     const int32_t px = 256 * i0 + 128, py = 256 * j0 + 128;
@@ -370,17 +357,14 @@ __device__ __forceinline__ uint32_t raster_rect_small(const Corners &s, uint32_t
     const int32_t dx1 = -(Y0 - Y2) * 256, dy1 = (X0 - X2) * 256;
     const int32_t dx2 = -(Y1 - Y0) * 256, dy2 = (X1 - X0) * 256;
     const int32_t n_i = i1 - i0;
-    uint32_t hits = 0;
 #pragma unroll 1
     for (int32_t j = j0; j <= j1; ++j) {
         int32_t r0 = e0, r1 = e1, r2 = e2;
         uint32_t *row = tri_plane + (j - row0) * (int64_t)w + i0;
 #pragma unroll 1
         for (int32_t i = 0; i <= n_i; ++i) {
-            if (min(r0, min(r1, r2)) > 0 && LCL_IN((j - row0) * (int64_t)w + i0 + i, (int64_t)w * rows)) {
-                mark_texel<MIN>(row + i, t);
-                ++hits;
-            }
+            if (min(r0, min(r1, r2)) > 0 && LCL_IN((j - row0) * (int64_t)w + i0 + i, (int64_t)w * rows))
+                atomicMin(row + i, t);
             r0 += dx0;
             r1 += dx1;
             r2 += dx2;
@@ -389,13 +373,11 @@ __device__ __forceinline__ uint32_t raster_rect_small(const Corners &s, uint32_t
         e1 += dy1;
         e2 += dy2;
     }
-    return hits;
 }
 
 // Rasterises texels [i0, i1] x [j0, j1] (texture rows j) of a set-up triangle into a plane that
-// holds rows [row0, row0 + rows).  Returns the texels it covers there.
-template <bool MIN>
-__device__ __noinline__ uint32_t raster_rect(const Corners &s, uint32_t t, int64_t i0, int64_t i1, int64_t j0, int64_t j1, int32_t w,
+// holds rows [row0, row0 + rows).
+__device__ __noinline__ void raster_rect(const Corners &s, uint32_t t, int64_t i0, int64_t i1, int64_t j0, int64_t j1, int32_t w,
                             int32_t row0, int32_t rows, uint32_t *__restrict__ tri_plane) {
     int64_t X0 = s.x[0], X1 = s.x[1], X2 = s.x[2], Y0 = s.y[0], Y1 = s.y[1], Y2 = s.y[2];
     int64_t px = 256 * i0 + 128, py = 256 * j0 + 128;
@@ -407,17 +389,14 @@ __device__ __noinline__ uint32_t raster_rect(const Corners &s, uint32_t t, int64
     int64_t dx0 = -(Y2 - Y1) * 256, dy0 = (X2 - X1) * 256;
     int64_t dx1 = -(Y0 - Y2) * 256, dy1 = (X0 - X2) * 256;
     int64_t dx2 = -(Y1 - Y0) * 256, dy2 = (X1 - X0) * 256;
-    uint32_t hits = 0;
 #pragma unroll 1
     for (int64_t j = j0; j <= j1; ++j) {
         int64_t r0 = e0, r1 = e1, r2 = e2;
         uint32_t *row = tri_plane + (j - row0) * (int64_t)w;
 #pragma unroll 1
         for (int64_t i = i0; i <= i1; ++i) {
-            if (r0 > 0 && r1 > 0 && r2 > 0 && LCL_IN((j - row0) * (int64_t)w + i, (int64_t)w * rows)) {
-                mark_texel<MIN>(row + i, t);
-                ++hits;
-            }
+            if (r0 > 0 && r1 > 0 && r2 > 0 && LCL_IN((j - row0) * (int64_t)w + i, (int64_t)w * rows))
+                atomicMin(row + i, t);
             r0 += dx0;
             r1 += dx1;
             r2 += dx2;
@@ -426,21 +405,18 @@ __device__ __noinline__ uint32_t raster_rect(const Corners &s, uint32_t t, int64
         e1 += dy1;
         e2 += dy2;
     }
-    return hits;
 }
 
-// Triangle t's planes and area weight (not MIN), and its texels: returns how many if it is a small
-// triangle (the texels of big ones are added to the header's counts).
-template <bool MIN>
-__device__ __forceinline__ uint32_t raster_triangle(const RasterArgs &a, int64_t t) {
+// Triangle t's planes and area weight, and its texels if it is a small triangle.
+__device__ __forceinline__ void raster_triangle(const RasterArgs &a, int64_t t) {
     Corners c;
     if (!load_corners(a.m, t, c)) {
         atomicOr(&a.hdr->flags, kBadIndex);
         a.area_w[t] = 0;
-        return 0;
+        return;
     }
     // area weight: 3D area over UV area, floor(isqrt(|n|^2) * 2^(16+F) / A), capped
-    if (!MIN) {
+    {
         const int32_t d1x = c.qx[1] - c.qx[0], d1y = c.qy[1] - c.qy[0], d1z = c.qz[1] - c.qz[0];
         const int32_t d2x = c.qx[2] - c.qx[0], d2y = c.qy[2] - c.qy[0], d2z = c.qz[2] - c.qz[0];
         const int64_t nx = (int64_t)d1y * d2z - (int64_t)d1z * d2y, ny = (int64_t)d1z * d2x - (int64_t)d1x * d2z,
@@ -468,71 +444,57 @@ __device__ __forceinline__ uint32_t raster_triangle(const RasterArgs &a, int64_t
         }
         a.area_w[t] = wgt;
     }
-    if (c.A == 0) return 0;
+    if (c.A == 0) return;
     const int32_t xmin = min(c.x[0], min(c.x[1], c.x[2])), xmax = max(c.x[0], max(c.x[1], c.x[2]));
     const int32_t ymin = min(c.y[0], min(c.y[1], c.y[2])), ymax = max(c.y[0], max(c.y[1], c.y[2]));
     int32_t i0, i1, j0, j1;
     texel_range(xmin, xmax, 0, a.w - 1, i0, i1);
     texel_range(ymin, ymax, a.row0, a.row0 + a.rows - 1, j0, j1);  // this atlas's rows only
-    if (i0 > i1 || j0 > j1) return 0;
-    if (!MIN) a.planes[t] = make_plane(c, xmax - xmin, ymax - ymin);
+    if (i0 > i1 || j0 > j1) return;
+    a.planes[t] = make_plane(c, xmax - xmin, ymax - ymin);
     const int32_t nx = i1 - i0 + 1, ny = j1 - j0 + 1;  // up to 2^14 each
     if (nx * ny <= kSmallRaster) {
         if (xmax - xmin <= (1 << 14) && ymax - ymin <= (1 << 14))
-            return raster_rect_small<MIN>(c, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
-        return raster_rect<MIN>(c, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
+            raster_rect_small(c, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
+        else
+            raster_rect(c, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
+        return;
     }
     const int64_t nb = (int64_t)((nx + kBlockSide - 1) / kBlockSide) * ((ny + kBlockSide - 1) / kBlockSide);
     unsigned long long base = atomicAdd(&a.hdr->n_big, (unsigned long long)nb);
     if ((int64_t)base + nb <= a.big_cap) {
         for (int64_t b = 0; b < nb; ++b)
             if (LCL_IN((int64_t)base + b, a.big_cap)) a.big[base + b] = make_uint2((uint32_t)t, (uint32_t)b);
-        return 0;
+        return;
     }
-    {
-        // list full: the reserved slots that lie below the capacity are read by k_raster_big, so they
-        // get empty entries, and this thread rasterises the triangle itself
-        for (int64_t b = 0; b < nb && (int64_t)base + b < a.big_cap; ++b)
-            if (LCL_IN((int64_t)base + b, a.big_cap)) a.big[base + b] = make_uint2(kNone, 0u);
-        const uint32_t hits = raster_rect<MIN>(c, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
-        if (!MIN) atomicAdd(&a.hdr->n_hits[0], (unsigned long long)hits);
-        return 0;
-    }
+    // list full: the reserved slots that lie below the capacity are read by k_raster_big, so they
+    // get empty entries, and this thread rasterises the triangle itself
+    for (int64_t b = 0; b < nb && (int64_t)base + b < a.big_cap; ++b)
+        if (LCL_IN((int64_t)base + b, a.big_cap)) a.big[base + b] = make_uint2(kNone, 0u);
+    raster_rect(c, (uint32_t)t, i0, i1, j0, j1, a.w, a.row0, a.rows, a.tri_plane);
 }
 
-// A thread per triangle.  Texels that no two triangles share, as in most unwraps, need no atomics, whose
-// rate of about one lane a cycle and SM bounds the scattered writes (268 M of them took 1.05 ms).  So
-// the first run (not MIN) stores ids as they come and counts the texels each triangle covers; when the
-// counts add up to the covered texels, every texel has one triangle and the plane is right.  Otherwise
-// atlas_build_impl runs MIN over the result: of the triangles that cover a texel the smallest id.
-template <bool MIN>
+// A thread per triangle.  Of the triangles that cover a texel the smallest id wins: atomicMin, whose rate of about
+// one lane a cycle and SM bounds the kernel (16384^2, 8 M triangles: 1.05 ms).  Plain stores take 0.87, with a
+// count of covered texels that shows whether two triangles share one, but then raster and resolve have to run
+// again: the whole build took 2.51 ms, and 4.9 to 7.6 with a single shared texel or a mirrored unwrap, where
+// it now takes 2.69, and 2.69 to 4.1; slivers that snapping folds over give nearly every unwrap such texels.
+// Four triangles at a time by eight lanes each, so that a row is one request: 2.67, on charts 2.78 (2.59).
 __global__ void __launch_bounds__(128) k_raster(const __grid_constant__ RasterArgs a) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    uint32_t hits = t < a.m.n_tri ? raster_triangle<MIN>(a, t) : 0u;
-    if (!MIN) {
-        __shared__ uint32_t s_hits[4];
-        hits = __reduce_add_sync(0xffffffffu, hits);
-        if ((threadIdx.x & 31) == 0) s_hits[threadIdx.x >> 5] = hits;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const unsigned long long n = (unsigned long long)s_hits[0] + s_hits[1] + s_hits[2] + s_hits[3];
-            if (n) atomicAdd(&a.hdr->n_hits[blockIdx.x & 7u], n);
-        }
-    }
+    if (t < a.m.n_tri) raster_triangle(a, t);
 }
 
 // The blocks of big triangles, a warp each: a lane takes every second row of one of the block's 16 columns,
 // its edge values stepping from row to row.  Bound by the latency of the chain entry -> indices -> corners,
 // so a warp, not a CTA, waits on it: 400 000 triangles on 16384^2 (9 blocks each) took 6.06 ms with a CTA
 // per entry and a texel per thread, now 1.43.
-template <bool MIN>
-__global__ void __launch_bounds__(kThreads) k_raster_big(const uint2 *__restrict__ big, AtlasHdr *hdr, int64_t cap,
+__global__ void __launch_bounds__(kThreads) k_raster_big(const uint2 *__restrict__ big, const AtlasHdr *hdr, int64_t cap,
                              const MeshRefs m, int32_t w, int32_t row0, int32_t rows,
                              uint32_t *__restrict__ tri_plane) {
     const int64_t n = min((int64_t)hdr->n_big, cap), n_warps = (int64_t)gridDim.x * (kThreads / 32);
     const int32_t lane = (int32_t)(threadIdx.x & 31u), col = lane % kBlockSide, row = lane / kBlockSide;
     constexpr int kStep = 32 / kBlockSide;  // rows of a warp's step
-    uint32_t hits = 0;
     int64_t e = (int64_t)blockIdx.x * (kThreads / 32) + threadIdx.x / 32;
     uint2 next = e < n && LCL_IN(e, cap) ? big[e] : make_uint2(kNone, 0u);
     for (; e < n; e += n_warps) {  // uniform over the warp
@@ -559,19 +521,13 @@ __global__ void __launch_bounds__(kThreads) k_raster_big(const uint2 *__restrict
         const int64_t d2 = (int64_t)(s.x[1] - s.x[0]) * (256 * kStep);
 #pragma unroll
         for (int k = 0; k < kBlockSide / kStep; ++k) {
-            if (j <= j1 && e0 > 0 && e1 > 0 && e2 > 0 && LCL_IN((j - row0) * (int64_t)w + i, (int64_t)w * rows)) {
-                mark_texel<MIN>(tri_plane + (j - row0) * (int64_t)w + i, ent.x);
-                ++hits;
-            }
+            if (j <= j1 && e0 > 0 && e1 > 0 && e2 > 0 && LCL_IN((j - row0) * (int64_t)w + i, (int64_t)w * rows))
+                atomicMin(tri_plane + (j - row0) * (int64_t)w + i, ent.x);
             j += kStep;
             e0 += d0;
             e1 += d1;
             e2 += d2;
         }
-    }
-    if (!MIN && n > 0) {
-        hits = __reduce_add_sync(0xffffffffu, hits);
-        if ((threadIdx.x & 31) == 0 && hits) atomicAdd(&hdr->n_hits[blockIdx.x & 7u], (unsigned long long)hits);
     }
 }
 
@@ -768,8 +724,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_resolve(const TriPlane *__restr
 }
 
 __global__ void __launch_bounds__(kThreads) k_super(const int32_t *__restrict__ tile_box, int32_t tiles_x,
-                                                    int32_t tiles_y, int32_t *__restrict__ super_box,
-                                                    unsigned long long *n_covered) {
+                                                    int32_t tiles_y, int32_t *__restrict__ super_box) {
     const int32_t sx = blockIdx.x, sy = blockIdx.y;
     const int32_t tx = sx * LCL_SUPER + (threadIdx.x % LCL_SUPER), ty = sy * LCL_SUPER + (threadIdx.x / LCL_SUPER);
     int32_t v[7] = {INT32_MAX, INT32_MAX, INT32_MAX, 0, INT32_MIN, INT32_MIN, INT32_MIN};
@@ -805,7 +760,6 @@ __global__ void __launch_bounds__(kThreads) k_super(const int32_t *__restrict__ 
             b[0] = make_int4(v[0], v[1], v[2], v[3]);
             b[1] = make_int4(v[4], v[5], v[6], 0);
         }
-        if (v[3]) atomicAdd(n_covered, (unsigned long long)v[3]);
         (void)n_sup;
     }
 }
@@ -877,46 +831,27 @@ lcl_status atlas_build_impl(const lcl_mesh *mesh, lcl_atlas *at, void *ws, size_
     ra.hdr = hdr;
     ra.big = big;
     ra.big_cap = (int64_t)big_capacity(mesh->n_tri, at->width, at->height);  // blocks of this atlas's rows
-    const unsigned rg = (unsigned)((mesh->n_tri + 127) / 128);
-    const dim3 sg(at->supers_x, at->supers_y);
-    const int32_t n_tiles = at->tiles_x * at->tiles_y;
-    auto resolve = [&]() {
-        const bool words = at->tile >= 32 && (at->width & 31) == 0;
-        const bool by_warp = words && n_tiles >= kWarpTiles / 32 * at->tile;
-        auto kernel = by_warp ? k_resolve<true, true> : words ? k_resolve<true, false> : k_resolve<false, false>;
-        const int per_cta = by_warp ? kThreads / 32 : 1;
-        kernel<<<(n_tiles + per_cta - 1) / per_cta, kThreads, 0, st>>>(
-            planes, mr, at->width, at->height, at->row0, at->tile, at->tiles_x, n_tiles, at->tri, at->pos_x, at->pos_y,
-            at->pos_z, at->cover, at->tile_box);
-        k_super<<<sg, kThreads, 0, st>>>(at->tile_box, at->tiles_x, at->tiles_y, at->super_box, &hdr->n_covered);
-        count_launches(2);
-    };
     if (mesh->n_tri > 0) {
-        k_raster<false><<<rg, 128, 0, st>>>(ra);
-        k_raster_big<false><<<sms * 8, kThreads, 0, st>>>(big, hdr, ra.big_cap, mr, at->width, at->row0, at->height,
-                                                          at->tri);
+        k_raster<<<(unsigned)((mesh->n_tri + 127) / 128), 128, 0, st>>>(ra);
+        k_raster_big<<<sms * 8, kThreads, 0, st>>>(big, hdr, ra.big_cap, mr, at->width, at->row0, at->height, at->tri);
         count_launches(2);
     }
-    resolve();
+    const int32_t n_tiles = at->tiles_x * at->tiles_y;
+    const bool words = at->tile >= 32 && (at->width & 31) == 0;
+    const bool by_warp = words && n_tiles >= kWarpTiles / 32 * at->tile;
+    const auto resolve = by_warp ? k_resolve<true, true> : words ? k_resolve<true, false> : k_resolve<false, false>;
+    const int per_cta = by_warp ? kThreads / 32 : 1;
+    resolve<<<(n_tiles + per_cta - 1) / per_cta, kThreads, 0, st>>>(planes, mr, at->width, at->height, at->row0, at->tile,
+                                                                    at->tiles_x, n_tiles, at->tri, at->pos_x, at->pos_y,
+                                                                    at->pos_z, at->cover, at->tile_box);
+    k_super<<<dim3(at->supers_x, at->supers_y), kThreads, 0, st>>>(at->tile_box, at->tiles_x, at->tiles_y, at->super_box);
+    count_launches(2);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "atlas build launch");
     AtlasHdr host;
     e = cudaMemcpyAsync(&host, hdr, sizeof(AtlasHdr), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "atlas build");
-    unsigned long long hits = 0;
-    for (const unsigned long long n : host.n_hits) hits += n;
-    if (hits != host.n_covered) {  // some texel has several triangles: the smallest id
-        // the big triangles' list is filled again from its start
-        e = cudaMemsetAsync(&hdr->n_big, 0, sizeof(hdr->n_big), st);
-        k_raster<true><<<rg, 128, 0, st>>>(ra);
-        k_raster_big<true><<<sms * 8, kThreads, 0, st>>>(big, hdr, ra.big_cap, mr, at->width, at->row0, at->height, at->tri);
-        count_launches(2);
-        resolve();
-        if (e == cudaSuccess) e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return cuda_fail(e, "atlas build");
-    }
     if (host.flags & kBadPos) return fail(LCL_ERR_INVALID_ARG, "mesh positions contain a non-finite value");
     if (host.flags & kFlatBBox) return fail(LCL_ERR_INVALID_ARG, "mesh bounding box has zero extent");
     if (host.flags & kBadIndex) return fail(LCL_ERR_INVALID_ARG, "triangle index out of range");
