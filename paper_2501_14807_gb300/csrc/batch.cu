@@ -235,7 +235,8 @@ __device__ __forceinline__ unsigned long long warp_or(unsigned long long v) {
 // of a super-tile) from a work queue, 8 lanes per tile.  The warp first tests the model's lassos against
 // the super-tile's box, four at a time; then each group of 8 lanes tests its tile: a lane per sphere, the
 // whole group per lasso, so that the four groups go through the same lasso together.  A padded stroke
-// counts a tile if it may reach any box of its 3 x 3 neighbourhood.  The queue evens out tiles under many
+// counts a tile if it may reach any box of its 3 x 3 neighbourhood: a padded sphere tests the 18 boxes around a unit
+// once each (nine per tile took 257 us for 4 models of 2048^2 with tiles of 8 and 16 padded spheres, now 90).  The queue evens out tiles under many
 // large lassos; with a CTA per (super-tile, stroke) those ran on while the chip was idle (24 models of
 // 512^2 to 2048^2, 48 spheres and 16 lassos each: 341 us with the compaction, now about 220; 3 models with
 // 40 spheres each: 11.1 us and 8.5).  What is left is the latency of one warp's footprint scans.
@@ -252,13 +253,21 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch_cull(BHdr *hdr, const BMo
     pdl_wait();  // the counters are reset and the lassos built
     pdl_allow_next();
     const int64_t n_units = (int64_t)hdr->n_supers * kCullUnits;
-    // the first unit is the warp's number, the others come from the queue, drawn one ahead
+    // a warp's first units are by its number, the others come from the queue, drawn one ahead
     const uint32_t n_warps = gridDim.x * (kThreads / 32);
-    uint32_t next = blockIdx.x * (kThreads / 32) + threadIdx.x / 32;
-    for (;;) {
-        const uint32_t u = __shfl_sync(0xffffffffu, next, 0);
-        if (u >= n_units) break;  // uniform over the warp, as below
-        if (lane == 0) next = n_warps + atomicAdd(&hdr->next_cull, 1u);
+    // Without lassos a unit is short, and a large model has more of them than the queue's one address serves
+    // in time (4 spheres on 16384^2 with tiles of 8: 784 us with one unit per draw, now 630): several per draw then.
+    const uint32_t chunk =
+        hdr->n_lassos ? 1u : (uint32_t)max((int64_t)1, min((int64_t)16, n_units / (4 * (int64_t)n_warps)));
+    uint32_t next = chunk * (blockIdx.x * (kThreads / 32) + threadIdx.x / 32);
+    uint32_t u = 0u, end = 0u;
+    for (;; ++u) {
+        if (u == end) {
+            u = __shfl_sync(0xffffffffu, next, 0);
+            if (u >= n_units) break;  // uniform over the warp, as below
+            end = min(u + chunk, (uint32_t)n_units);
+            if (lane == 0) next = chunk * n_warps + atomicAdd(&hdr->next_cull, chunk);
+        }
         const int32_t g = (int32_t)(u / kCullUnits), part = (int32_t)(u % kCullUnits);
         if (!LCL_IN(g, caps.supers)) break;
         const uint32_t mi = super_model[g];
@@ -295,6 +304,19 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch_cull(BHdr *hdr, const BMo
                 pad = stroke_pads(st, lassos);
             }
             const bool sphere = mine && !lasso;
+            uint32_t near = 0u;  // padded spheres: bit c, some box of column tx0 - 1 + c of the three rows is in reach
+            if (__any_sync(0xffffffffu, sphere && pad)) {
+#pragma unroll 1
+                for (int b = 0; b < 3 * (kCullTiles + 2); ++b) {  // uniform
+                    const int c = b % (kCullTiles + 2);
+                    const int32_t x = tx0 - 1 + c, y = ty - 1 + b / (kCullTiles + 2);
+                    if (x < 0 || x >= a.tiles_x || y < 0 || y >= a.tiles_y || !LCL_IN((int64_t)y * a.tiles_x + x, n_tiles))
+                        continue;
+                    const int4 *bp = reinterpret_cast<const int4 *>(a.tile_box + 8 * ((int64_t)y * a.tiles_x + x));
+                    const int4 blo = bp[0], bhi = bp[1];
+                    if (blo.w > 0 && box_dist2(blo, bhi, sp) <= sp.r2) near |= 1u << c;
+                }
+            }
 #pragma unroll
             for (int t = 0; t < kCullTiles; ++t) {
                 int4 tlo, thi;
@@ -304,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch_cull(BHdr *hdr, const BMo
                 tlo.w = __shfl_sync(0xffffffffu, lo.w, 8 * t), thi.w = 0;
                 bool can = false, in = false;
                 if (sphere && pad) {
-                    can = tx0 + t < a.tiles_x && near_box_3x3(a.tile_box, a.tiles_x, a.tiles_y, tx0 + t, ty, sp);
+                    can = tx0 + t < a.tiles_x && ((near >> t) & 7u);
                 } else if (sphere && tlo.w > 0) {
                     can = box_dist2(tlo, thi, sp) <= sp.r2;
                     in = can && box_far2(tlo, thi, sp) <= sp.r2;
