@@ -62,6 +62,7 @@ static_assert(sizeof(BLasso) % 16 == 0, "k_batch_prep copies it by 16-byte words
 constexpr size_t kBLassoRoom = 2792;  // bytes of the workspace per lasso, which programs may have stored
 static_assert(sizeof(BLasso) <= kBLassoRoom, "lcl_batch_workspace_bytes");
 
+// Kernels of batches whose limits hold no lassos leave out their code (LASSOS false).
 template <typename F>
 __device__ __forceinline__ void band_edges(const BLasso &L, int band, F f) {
     const uint2 b = L.band[band];
@@ -111,6 +112,7 @@ __device__ __forceinline__ bool stroke_in_bounds(const BStroke *strokes, int64_t
 // k_batch_prep at every launch.
 struct BHdr {
     int32_t n_models, n_strokes, n_lassos, n_supers;
+    int32_t groups_log, tickets_log;  // of the largest tiles: groups of 32 quads, and tickets per item, powers of 2
     unsigned int n_items;          // written by k_batch_cull
     unsigned int next_cull;        // work queue of k_batch_cull
     unsigned long long next_unit;  // work queue of k_batch_apply
@@ -383,9 +385,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch_cull(BHdr *hdr, const BMo
 }
 
 // Does stroke `st` select the covered texel n?
+template <bool LASSOS>
 __device__ __forceinline__ bool stroke_selects(const AtlasDev &a, const BStroke &st, const BLasso *__restrict__ lassos,
                                                int64_t n, int32_t qx) {
-    if (st.kind == LCL_STROKE_SPHERE) {
+    if (!LASSOS || st.kind == LCL_STROKE_SPHERE) {
         const int64_t dx = (int64_t)qx - st.sphere.cx, dy = (int64_t)__ldg(a.py + n) - st.sphere.cy;
         const int64_t dz = (int64_t)__ldg(a.pz + n) - st.sphere.cz;
         return dx * dx + dy * dy + dz * dz <= st.sphere.r2;
@@ -397,6 +400,7 @@ __device__ __forceinline__ bool stroke_selects(const AtlasDev &a, const BStroke 
 // Texture padding of the uncovered texels `unc` of the quad at l: for each, the masked padded strokes
 // from the newest down; the first whose outline (a covered texel within its thickness) and kernel
 // (a texel it selects within its radius) both hold gives the label.  Returns the texels written.
+template <bool LASSOS>
 __device__ __noinline__ uint32_t pad_texels(const AtlasDev &a, int64_t l, uint32_t unc, unsigned long long mask, int32_t s0,
                                const BStroke *__restrict__ strokes, const BLasso *__restrict__ lassos,
                                uint32_t lab[4], const BCaps &caps) {
@@ -410,9 +414,9 @@ __device__ __noinline__ uint32_t pad_texels(const AtlasDev &a, int64_t l, uint32
             m &= ~(1ull << si);
             if (!stroke_in_bounds(strokes, (int64_t)s0 + si, caps)) continue;
             const BStroke &st = strokes[s0 + si];
-            const int32_t pr = st.kind == LCL_STROKE_SPHERE ? st.sphere.pad_r : lassos[st.lasso].pad_r;
+            const int32_t pr = !LASSOS || st.kind == LCL_STROKE_SPHERE ? st.sphere.pad_r : lassos[st.lasso].pad_r;
             if (pr == 0) continue;
-            const int32_t pt = st.kind == LCL_STROKE_SPHERE ? st.sphere.pad_t : lassos[st.lasso].pad_t;
+            const int32_t pt = !LASSOS || st.kind == LCL_STROKE_SPHERE ? st.sphere.pad_t : lassos[st.lasso].pad_t;
             const int32_t reach = max(pr, pt);
             bool outline = false, near = false;
             for (int32_t dy = -reach; dy <= reach && !(outline && near); ++dy) {
@@ -427,11 +431,11 @@ __device__ __noinline__ uint32_t pad_texels(const AtlasDev &a, int64_t l, uint32
                     if (qx == INT32_MIN) continue;
                     const int32_t ax = abs(dx), ay = abs(dy);
                     if (ax <= pt && ay <= pt) outline = true;
-                    if (ax <= pr && ay <= pr && !near) near = stroke_selects(a, st, lassos, n, qx);
+                    if (ax <= pr && ay <= pr && !near) near = stroke_selects<LASSOS>(a, st, lassos, n, qx);
                 }
             }
             if (outline && near) {
-                lab[k] = st.kind == LCL_STROKE_SPHERE ? st.sphere.label : lassos[st.lasso].label;
+                lab[k] = !LASSOS || st.kind == LCL_STROKE_SPHERE ? st.sphere.label : lassos[st.lasso].label;
                 written |= 1u << k;
                 break;
             }
@@ -459,6 +463,7 @@ __device__ __forceinline__ uint32_t lasso_texels(const BLasso &ls, int4 X, int4 
 
 // 32 quads from q0 of a work item's tile (quad = 4 consecutive texels of a tile row, row-major in
 // the tile), one per lane.
+template <bool LASSOS>
 __device__ __forceinline__ void apply_quads(const BModel &M, const BItem &it, int32_t q0,
                                             const BStroke *__restrict__ strokes, const BLasso *__restrict__ lassos,
                                             const BCaps &caps) {
@@ -489,7 +494,7 @@ __device__ __forceinline__ void apply_quads(const BModel &M, const BItem &it, in
         const BStroke &st = strokes[M.s0 + si];
         uint32_t sel = 0u, label;
         const bool sure = (it.sure >> si) & 1ull;
-        if (st.kind == LCL_STROKE_SPHERE) {
+        if (!LASSOS || st.kind == LCL_STROKE_SPHERE) {
             label = st.sphere.label;
             if (sure) {
                 sel = open;  // the sphere contains the tile's box: every covered texel is selected
@@ -518,7 +523,7 @@ __device__ __forceinline__ void apply_quads(const BModel &M, const BItem &it, in
     // thickness, writes its label there
     if (unc && (it.tile & kPadItem)) {
         uint32_t plab[4];
-        const uint32_t ph = pad_texels(a, l, unc, it.mask, M.s0, strokes, lassos, plab, caps);
+        const uint32_t ph = pad_texels<LASSOS>(a, l, unc, it.mask, M.s0, strokes, lassos, plab, caps);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (ph & (1u << k)) lab[k] = plab[k];
@@ -529,18 +534,24 @@ __device__ __forceinline__ void apply_quads(const BModel &M, const BItem &it, in
     else store_labels<uint16_t>(static_cast<uint16_t *>(M.layer), l, hit, lab);
 }
 
-// The work queue's tickets: 8 * split per item, each an equal share of the tile's groups of 32 quads (a
-// tile of 32 texels has 8; small tiles leave tickets empty), one warp per ticket.  A warp draws its next
-// ticket before it works on the current one, so the queue's latency is hidden; a ticket per CTA waited
-// for the slowest of its warps, and 4 or 1 per item took 1024 and 1498 us where 8 took 959.  The kernel
-// waits for the lassos' arguments (cache hits) between dependent operations, so warps count for more
-// than registers: with 3, 4, 5 and 6 CTAs per SM that batch took 1141, 1023, 1014 and 974 us.  The four
-// texels of a quad side by side, as in the single lasso's apply, need 80 registers and more code than the
-// instruction cache holds: 1484 us.  All of the batch: 1314 us before (a CTA per ticket, 3 per SM, padded
-// strokes looked for at every uncovered texel), now 696.
-constexpr int kItemTicketsLog = 3;
+// The work queue's tickets: an item has up to 16 * split, each an equal share of the tile's groups of 32 quads and a
+// group at least (two where all strokes are spheres without padding, whose work is short), one warp per ticket.
+// A warp draws its next ticket before it works on the current one, so the queue's latency is hidden; a ticket
+// per CTA waited for the slowest of its warps.  24 models of 512^2 to 2048^2 with tiles of 32 (8 groups), 48 spheres
+// and 16 lassos each: 8 tickets 959 us, 4 1024, 1 1498.  Tiles of 64 (32 groups), 4 models of 2048^2 with 16 padded
+// spheres: 32 203, 16 264, 8 414; one of 16384^2 with 16 spheres and 4 lassos 934, 614, 614.  Tiles of 8 (one
+// group) with seven empty tickets each: one of 4096^2 with 64 spheres 502, without them 163.  A group or two per
+// ticket, 64 spheres on 4096^2 with tiles of 32: 72 and 61.
+// The kernel waits for the lassos' arguments (cache hits) between dependent operations, so warps count for more
+// than registers: with 3, 4, 5 and 6 CTAs per SM the batch of 24 took 1141, 1023, 1014 and 974 us.  Without
+// lassos (LASSOS false) six, whose 40 registers spill, cost a tenth of five.  The four texels of a quad side by
+// side, as in the single lasso's apply, need 80 registers and more code than the instruction cache holds: 1484
+// us.  All of the batch: 1314 us before (a CTA per ticket, 3 per SM, padded strokes looked for at every
+// uncovered texel), now 696.
+constexpr int kItemTicketsLog = 4;
 
-__global__ void __launch_bounds__(256, 6) k_batch_apply(const BHdr *__restrict__ hdr, const BModel *__restrict__ models,
+template <bool LASSOS>
+__global__ void __launch_bounds__(256, LASSOS ? 6 : 5) k_batch_apply(const BHdr *__restrict__ hdr, const BModel *__restrict__ models,
                                                      const BStroke *__restrict__ strokes,
                                                      const BLasso *__restrict__ lassos,
                                                      const BItem *__restrict__ items, unsigned long long *next_unit,
@@ -548,7 +559,7 @@ __global__ void __launch_bounds__(256, 6) k_batch_apply(const BHdr *__restrict__
     pdl_wait();
     pdl_allow_next();
     const int lane = threadIdx.x & 31;
-    const int plog = kItemTicketsLog + __ffs(split) - 1;  // split is a power of 2
+    const int plog = min(hdr->tickets_log + __ffs(split) - 1, hdr->groups_log);  // split is a power of 2
     const unsigned long long n_units = (unsigned long long)hdr->n_items << plog;
     const unsigned long long n_warps = (unsigned long long)gridDim.x * (blockDim.x / 32);
     unsigned long long next = (unsigned long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
@@ -565,7 +576,7 @@ __global__ void __launch_bounds__(256, 6) k_batch_apply(const BHdr *__restrict__
         const int32_t groups = max(M.a.T * (M.a.T / 4) / 32, 1);
         const int32_t g0 = groups * part >> plog, g1 = groups * (part + 1) >> plog;
         for (int32_t g = g0; g < g1; ++g) {
-            apply_quads(M, it, 32 * g, strokes, lassos, caps);
+            apply_quads<LASSOS>(M, it, 32 * g, strokes, lassos, caps);
             __syncwarp();
         }
     }
@@ -685,6 +696,10 @@ BPtrs b_ptrs(const BLayout &L, void *ws) {
     return p;
 }
 
+using ApplyKernel = void (*)(const BHdr *, const BModel *, const BStroke *, const BLasso *, const BItem *,
+                             unsigned long long *, int32_t, BCaps);
+ApplyKernel apply_kernel(const lcl_batch_limits &lim) { return lim.lassos > 0 ? k_batch_apply<true> : k_batch_apply<false>; }
+
 cudaError_t launch_kernels(const BPtrs &p, const lcl_batch_limits &lim, const lcl_batch_config &c, cudaStream_t st) {
     BCaps caps;
     caps.models = lim.models;
@@ -700,9 +715,10 @@ cudaError_t launch_kernels(const BPtrs &p, const lcl_batch_limits &lim, const lc
         const int ug = (int)std::min<int64_t>(lim.supers * kCullUnits / (kThreads / 32), resident_grid(k_batch_cull));
         e = launch_pdl(k_batch_cull, dim3(ug), st, p.hdr, p.models, p.strokes, p.lassos, p.super_model, p.items, caps);
         if (e == cudaSuccess) {
-            const int fit = resident_per_sm(k_batch_apply, c.threads);
+            const auto apply = apply_kernel(lim);
+            const int fit = resident_per_sm(apply, c.threads);
             const int per_sm = c.ctas_per_sm > 0 ? std::min(c.ctas_per_sm, fit) : fit;
-            e = launch_pdl_shape(k_batch_apply, dim3(per_sm * sm_count()), dim3(c.threads), st, (const BHdr *)p.hdr,
+            e = launch_pdl_shape(apply, dim3(per_sm * sm_count()), dim3(c.threads), st, (const BHdr *)p.hdr,
                                  p.models, p.strokes, p.lassos, (const BItem *)p.items, &p.hdr->next_unit,
                                  (int32_t)c.split, caps);
         }
@@ -781,6 +797,12 @@ lcl_status batch_upload_impl(const lcl_batch_limits *lim, const lcl_batch_model 
     hdr.n_strokes = n_strokes;
     hdr.n_lassos = n_lassos;
     hdr.n_supers = (int32_t)n_supers;
+    for (int32_t i = 0; i < n_models; ++i)
+        while ((32 << hdr.groups_log) < models[i].atlas->tile * models[i].atlas->tile / 4) ++hdr.groups_log;
+    bool spheres = true;  // nothing but spheres without padding
+    for (int32_t k = 0; k < n_strokes; ++k)
+        spheres = spheres && strokes[k].kind == LCL_STROKE_SPHERE && !(strokes[k].sphere.flags & 15u);
+    hdr.tickets_log = std::max(0, std::min(kItemTicketsLog, hdr.groups_log - (spheres ? 1 : 0)));
     std::memcpy(img + L.hdr, &hdr, sizeof(hdr));
     BModel *bm = reinterpret_cast<BModel *>(img + L.models);
     uint32_t *super_model = reinterpret_cast<uint32_t *>(img + L.super_model);
@@ -865,7 +887,6 @@ lcl_status batch_tune_impl(const lcl_batch_limits *lim, void *ws, size_t ws_byte
     const BLayout L = b_layout(*lim);
     if (!ws || ws_bytes < L.total) return fail(LCL_ERR_INVALID_ARG, "batch workspace NULL or smaller than the limits need");
     const BPtrs p = b_ptrs(L, ws);
-    const int fit256 = resident_per_sm(k_batch_apply, 256);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
@@ -878,10 +899,9 @@ lcl_status batch_tune_impl(const lcl_batch_limits *lim, void *ws, size_t ws_byte
                 lcl_batch_config c = default_config();
                 c.threads = threads[ti];
                 c.split = splits[si];
-                const int fit = resident_per_sm(k_batch_apply, c.threads);
+                const int fit = resident_per_sm(apply_kernel(*lim), c.threads);
                 c.ctas_per_sm = half ? std::max(1, fit / 2) : 0;
                 if (half && c.ctas_per_sm >= fit) continue;
-                (void)fit256;
                 e = launch_kernels(p, *lim, c, st);  // warm-up
                 if (e == cudaSuccess) e = cudaEventRecord(e0, st);
                 for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch_kernels(p, *lim, c, st);
