@@ -1121,30 +1121,45 @@ lcl_status select_sphere_grouped(const lcl_atlas *atlas, const AtlasDev &a, L *l
     return LCL_OK;
 }
 
-// Which unpadded calls go through candidate lists instead of spheres.cu's blocks.  A block is one CTA's, so
-// on a large texture a few strokes keep a few CTAs busy for long while the others only find their
-// blocks empty; lists spread the reached tiles over the chip.  Times per call, lists / blocks, radii 1-5%
-// of the diagonal (10-30% in brackets):
-//   a stroke, 16384^2 (262144 tiles of 32): 20.5 / 24.4 us (28.6 / 55.2), 8192^2: 20.8 / 15.7, 4096^2: 21 / 15;
-//   label layers, groups of 32 strokes: on 16384^2 2 strokes 21 / 25 (35 / 65), 32 33 / 59 (201 / 209), 64
-//   60 / 79 (409 / 278), 128 120 / 119, 256 239 / 179; on 8192^2 4 strokes 21 / 18, 8 21 / 21, 32 21 / 32,
-//   64 35 / 45, 128 65 / 60; on 4096^2 16 strokes 20 / 17, 64 26 / 23;
-//   value layers, a launch per stroke: on 16384^2 2 strokes 22 / 26, 4 27 / 30 (75 / 85), 8 41 / 41.
-constexpr int64_t kManyTiles1 = 131072, kManyTiles2 = 49152;  // tiles of a large texture, of a middling one
-constexpr int32_t kMidStrokes = 6;    // strokes at least, on a middling texture
-constexpr int32_t kGroupCall = 32;     // strokes at most, of any radius ...
-constexpr int32_t kGroupCallSmall = 96;  // ... or of radii up to an eighth of the grid
-constexpr int64_t kSmallR2 = int64_t(1) << 36;
-constexpr int32_t kChainValues = 4;
+// Which unpadded calls go through candidate lists instead of spheres.cu's blocks.  A block is one CTA's and its texels
+// grow with the texture, whatever the side of its tiles, so on a large texture a few strokes keep a few CTAs
+// busy for long while the others only find their blocks empty; lists spread the reached tiles over the chip, a CTA
+// per tile (of 32: a thread per quad; tiles of 16 and 8 leave three and fifteen threads of sixteen idle), and
+// take a cull and an apply per 32 strokes (label layers) or a launch per stroke (value layers).  Strokes with a
+// radius above an eighth of the grid ("wide" below) reach so many tiles that the idle threads count.
+// Measured per call, lists / blocks in us, radii of 1-5% of the diagonal and (wide) 10-30%:
+//   label layers, tiles of 32   4096^2    n 1: 17/17 (18/19)  8: 18/16 (19/25)  16: 17/17 (28/33)  32: 16/19 (38/38)
+//                               8192^2    n 1: 17/17 (18/34)  8: 17/21 (36/53)  32: 18/30 (81/87)  64: 29/39 (152/116)
+//                               16384^2   n 1: 17/27 (43/79)  8: 17/33 (107/138)  32: 29/56 (209/208)  128: 123/119
+//                 tiles of 128  4096^2    n 1: 18/17 (20/22)  8: 18/21 (40/44)  32: 26/30 (88/91)
+//                               8192^2    n 1: 16/23 (29/51)  32: 44/63 (180/164)  64: 82/81
+//                               16384^2   n 1: 18/53 (51/154)  32: 69/157 (381/401)  128: 257/285
+//                 tiles of 16   8192^2    n 1: 17/25 (66/104)  2: 17/21 (152/121)  32: 46/48 (533/265)  64: 88/74
+//                 tiles of 8    8192^2    n 1: 18/53 (242/161)  8: 42/60 (1067/272)  16: 110/81
+//   value layers, tiles of 32   8192^2    n 1: 16/19 (48/63)  2: 19/20 (77/70)  4: 26/20
+//                               16384^2   n 1: 16/35 (260/210)  4: 32/36  8: 79/46
+//                 tiles of 64   16384^2   n 1: 17/48 (227/246)  4: 43/52 (407/231)
+//                 tiles of 128  8192^2    n 1: 30/29 (61/85)  2: 49/33      16384^2   n 1: 35/71 (192/267)  2: 75/79
+//                 tiles of 16   8192^2    n 1: 17/25 (91/94)  4: 23/24  8: 33/29      16384^2   n 8: 59/78  (346/289)
+constexpr int64_t kMiddling = int64_t(3) << 22, kLarge = int64_t(3) << 24, kHuge = int64_t(3) << 26;  // texels
+constexpr int64_t kWideR2 = int64_t(1) << 36;
+constexpr int32_t kMostByLists = 128;
 
 template <bool NUM>
-bool by_lists(const lcl_sphere *strokes, int32_t n, int64_t n_tiles) {
-    if (NUM || n == 1) return n <= kChainValues && n_tiles >= kManyTiles1;
-    if (n_tiles < kManyTiles2 || (n < kMidStrokes && n_tiles < kManyTiles1) || n > kGroupCallSmall) return false;
-    if (n <= kGroupCall) return true;
-    for (int32_t k = 0; k < n; ++k)
-        if (strokes[k].r2 > kSmallR2) return false;
-    return true;
+bool by_lists(const lcl_sphere *strokes, int32_t n, int32_t T, int64_t n_texels) {
+    if (n > kMostByLists || n_texels < kMiddling) return false;
+    bool wide = false;
+    for (int32_t k = 0; k < n; ++k) wide = wide || strokes[k].r2 > kWideR2;
+    const bool large = n_texels >= kLarge, huge = n_texels >= kHuge;
+    if (NUM) {
+        if (wide) return n == 1 && T >= 32 && (T <= 64 || large) && (T > 32 || !huge);
+        const int32_t most = (T <= 16 ? 4 : T <= 64 ? 2 : 1) << (huge ? 1 : 0);
+        return n <= most && (large || T < 16);
+    }
+    if (T < 16) return !wide && n <= 8;
+    if (T == 16) return wide ? n == 1 : large && n <= 32;
+    if (large) return n <= (wide ? (T > 64 && !huge ? 16 : 32) : T > 32 && huge ? 128 : 96);
+    return wide ? n <= 16 : n >= (T > 32 ? 8 : 16) && n <= 32;
 }
 
 template <typename L>
@@ -1178,7 +1193,7 @@ lcl_status select_sphere_run(const lcl_atlas *atlas, L *layer, uint32_t *mask, c
     };
     bool padded = false;
     for (int32_t k = 0; k < n; ++k) padded = padded || (strokes[k].flags & 15u) != 0;
-    const bool lists = !padded && by_lists<NUM>(strokes, n, (int64_t)a.tiles_x * a.tiles_y);
+    const bool lists = !padded && by_lists<NUM>(strokes, n, a.T, (int64_t)a.w * a.h);
     if constexpr (!NUM)
         if (lists && n >= 2) return select_sphere_grouped(atlas, a, layer, w, n, h, arg, st);
     if (!padded && !lists) {  // all strokes in one pass (spheres.cu)
