@@ -1128,7 +1128,8 @@ lcl_status select_sphere_grouped(const lcl_atlas *atlas, const AtlasDev &a, L *l
 // take a cull and an apply per 32 strokes (label layers) or a launch per stroke (value layers).  Strokes with a
 // radius above an eighth of the grid ("wide" below) reach so many tiles that the idle threads count.
 // Measured per call, lists / blocks in us, radii of 1-5% of the diagonal and (wide) 10-30%:
-//   label layers, tiles of 32   4096^2    n 1: 17/17 (18/19)  8: 18/16 (19/25)  16: 17/17 (28/33)  32: 16/19 (38/38)
+//   label layers, tiles of 32   4096^2    n 1: 17/17 (18/19)  8: 18/16 (19/25)  16: 17/17 (28/33)  32: 16/19 (38/38), 20 of 0.5-30% on
+//                               5004 x 3310 43/55
 //                               8192^2    n 1: 17/17 (18/34)  8: 17/21 (36/53)  32: 18/30 (81/87)  64: 29/39 (152/116)
 //                               16384^2   n 1: 17/27 (43/79)  8: 17/33 (107/138)  32: 29/56 (209/208)  128: 123/119
 //                 tiles of 128  4096^2    n 1: 18/17 (20/22)  8: 18/21 (40/44)  32: 26/30 (88/91)
@@ -1159,7 +1160,7 @@ bool by_lists(const lcl_sphere *strokes, int32_t n, int32_t T, int64_t n_texels)
     if (T < 16) return !wide && n <= 8;
     if (T == 16) return wide ? n == 1 : large && n <= 32;
     if (large) return n <= (wide ? (T > 64 && !huge ? 16 : 32) : T > 32 && huge ? 128 : 96);
-    return wide ? n <= 16 : n >= (T > 32 ? 8 : 16) && n <= 32;
+    return n <= 32 && (wide || n >= (T > 32 ? 8 : 16));
 }
 
 template <typename L>
