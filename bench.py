@@ -289,7 +289,8 @@ def run_ours(args):
     sphere_hits = [torch.zeros(max(len(r), 1), dtype=torch.int64, device=dev) for r in per_layer]
     inside_per_layer = [sphere_inside_texels(atlas, r, dev) for r in per_layer]
     # every layer's strokes are one unpadded call
-    grouped = [sphere_group_bytes(atlas, r, dev, w.dtype_bytes) for r in per_layer]
+    sph_groups = {sphere_group(atlas, r) for r in per_layer}
+    grouped = [sphere_group_bytes(atlas, r, dev, w.dtype_bytes, sphere_group(atlas, r)) for r in per_layer]
     assert all(len(r) >= 2 and not (r["flags"] & 15).any() for r in per_layer)
     torch.cuda.empty_cache()
     cams = [lcl.lcl_camera_from_vp(atlas, c.vp, c.width, c.height) for c in w.cams]
@@ -432,8 +433,8 @@ def run_ours(args):
                                     "all-reduce per step)") if world > 1 else "1 GPU, the whole texture"),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "peak_kind": peak_kind, "traffic": traffic,
-                     "kernel": f"sphere edit: one k_spheres launch per {SPHERE_GROUP} consecutive strokes of a call at "
-                               "most (a launch = one group), timed over the whole sphere row",
+                     "kernel": "sphere edit: " + " and ".join(SPHERE_LAUNCHES[g] for g in sorted(sph_groups)) +
+                               " (a launch = one group), timed over the whole sphere row",
                      "algorithmic_bytes_per_launch": sph_bytes / max(n_groups, 1),
                      "bytes_model": "12 B position + label per selected texel, summed over the strokes (the scope's "
                                     "per-unit bytes).  The grouped apply reads a tile's positions once per group "
@@ -492,7 +493,29 @@ def sphere_inside_texels(atlas, records, dev, chunk=16):
     return out
 
 
-SPHERE_GROUP = 512  # strokes per launch of the library's k_spheres at most
+SPHERE_GROUP, SPHERE_LIST_GROUP = 512, 32  # strokes per launch of the library's k_spheres, k_group_apply at most
+SPHERE_LAUNCHES = {SPHERE_GROUP: f"one k_spheres launch per {SPHERE_GROUP} consecutive strokes of a call at most",
+                   SPHERE_LIST_GROUP: f"a cull and an apply launch (k_group_cull, k_group_apply) per {SPHERE_LIST_GROUP} "
+                                      "consecutive strokes of a call at most"}
+
+
+def sphere_group(atlas, records):
+    """Strokes per launch at most for a call of several unpadded strokes on a label layer: the library's rule
+    (by_lists in csrc/select.cu) for calls that go through candidate lists."""
+    n, tile, texels = len(records), atlas.tile, atlas.width * atlas.height
+    middling, large, huge = texels >= 3 << 22, texels >= 3 << 24, texels >= 3 << 26
+    wide = bool((records["r2"] > 1 << 36).any())
+    if n > 128 or not middling:
+        return SPHERE_GROUP
+    if tile < 16:
+        lists = not wide and n <= 8
+    elif tile == 16:
+        lists = n == 1 if wide else large and n <= 32
+    elif large:
+        lists = n <= ((16 if tile > 64 and not huge else 32) if wide else (128 if tile > 32 and huge else 96))
+    else:
+        lists = n <= 32 and (wide or n >= (8 if tile > 32 else 16))
+    return SPHERE_LIST_GROUP if lists else SPHERE_GROUP
 
 
 def sphere_group_bytes(atlas, records, dev, label_bytes, group=SPHERE_GROUP):

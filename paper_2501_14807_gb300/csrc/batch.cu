@@ -7,11 +7,10 @@
 //   k_batch_cull   gives every tile of every model a 64-bit mask of the model's queued strokes
 //                  (queue order = bit order) whose conservative box test can reach the tile, and
 //                  of those a `sure` mask (spheres containing the tile, lassos inside whose polygon
-//                  it lies): a warp per tile, a lane per stroke.  Tiles with a non-empty mask become
+//                  it lies): a warp per four tiles of a row.  Tiles with a non-empty mask become
 //                  work items (model, tile, masks);
-//   k_batch_apply  takes units of up to 32 quads of an item from a work queue, a warp each.  The
-//                  warp tests the masked strokes once more, against the box of its own texels; a
-//                  thread loads its four texels' positions once and evaluates the masked strokes
+//   k_batch_apply  takes units of one or more groups of 32 quads of an item from a work queue, a warp
+//                  each.  A thread loads its four texels' positions once and evaluates the masked strokes
 //                  from the newest down: the first stroke that selects a texel is the last one
 //                  sequential application would have written there, so the texel is final and
 //                  the thread stops once its four texels are final (or no stroke is left); each
@@ -238,7 +237,8 @@ __device__ __forceinline__ unsigned long long warp_or(unsigned long long v) {
 // the super-tile's box, four at a time; then each group of 8 lanes tests its tile: a lane per sphere, the
 // whole group per lasso, so that the four groups go through the same lasso together.  A padded stroke
 // counts a tile if it may reach any box of its 3 x 3 neighbourhood: a padded sphere tests the 18 boxes around a unit
-// once each (nine per tile took 257 us for 4 models of 2048^2 with tiles of 8 and 16 padded spheres, now 90).  The queue evens out tiles under many
+// once each (with nine per tile a batch of 4 models of 2048^2 with tiles of 8 and 16 padded spheres took 489 us, of
+// which the cull 257; now 262).  The queue evens out tiles under many
 // large lassos; with a CTA per (super-tile, stroke) those ran on while the chip was idle (24 models of
 // 512^2 to 2048^2, 48 spheres and 16 lassos each: 341 us with the compaction, now about 220; 3 models with
 // 40 spheres each: 11.1 us and 8.5).  What is left is the latency of one warp's footprint scans.

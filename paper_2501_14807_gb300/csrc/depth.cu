@@ -141,7 +141,8 @@ __device__ __forceinline__ void pixel_range(const DTri &d, int32_t w, int32_t h,
 //  - if qh + ql lies, with that margin and the binary64 one, strictly between the rounding boundaries
 //    around qh (half an ulp above, half an ulp below -- a quarter below a power of two), every value
 //    within the margins rounds to qh, the binary64 result included, so the result is qh.
-// Otherwise (near a boundary, about 2^-19 of the pixels, or A >= 2^24: triangles above 256 px^2)
+// Otherwise (near a boundary, about 2^-19 of the pixels, or A >= 2^24: triangles above 128 px^2, A being twice
+// the area in 1/65536 px^2)
 // the binary64 sequence itself runs.
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {  // s + e = a + b exactly
     s = __fadd_rn(a, b);

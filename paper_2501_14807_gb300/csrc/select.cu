@@ -19,14 +19,18 @@
 // branch that raises the kernel above 40 registers (5 instead of 6 CTAs per SM), cost 1.3-1.6 ms
 // per 1000 strokes, hence the separate template instances.
 //
-// Sphere strokes without padding take the passes of spheres.cu.  In a call with a padded stroke, whose
-// outcome depends on its neighbours' selections, strokes take one launch each: the kernel that applies
-// stroke k also culls stroke k + 1, and every launch is a programmatic dependent launch, so the next grid is scheduled while the
-// current one drains and waits (griddepcontrol.wait) only for its completion.  Stroke k's
-// candidates go to list k mod 3, and the cull of stroke k + 1 runs before the wait, in the
+// Sphere strokes without padding take the passes of spheres.cu, but for the calls that go by lists (by_lists):
+// several strokes on a label layer in groups (k_group_cull, k_group_apply), others as in a call with a padded
+// stroke, whose outcome depends on its neighbours' selections: there strokes take one launch each.  The kernel that
+// applies stroke k also culls stroke k + 1, and every launch is a programmatic dependent launch, so the next
+// grid is scheduled while the current one drains and waits (griddepcontrol.wait) only for its completion.
+// Stroke k's candidates go to list k mod 3, and the cull of stroke k + 1 runs before the wait, in the
 // shadow of stroke k - 1's tail: list (k + 1) mod 3 was last read by stroke k - 2, which has
 // completed, because grid k is only launched once every CTA of grid k - 1 has passed its own
-// wait.  Strokes of one call run in stream order, so a later stroke overwrites an earlier one.  Lassos take a cull and an apply launch (two culls with texture padding).  Hit counts are per-warp popcounts
+// wait.  Strokes of one call run in stream order, so a later stroke overwrites an earlier one.
+//
+// A lasso or a tool edit takes a chain of four launches, with texture padding five: zeroing, the super-tiles in
+// reach, the tiles, (with padding the tiles around them) and the apply.  Hit counts are per-warp popcounts
 // reduced per CTA into one 64-bit atomic.
 #include <algorithm>
 #include <cmath>
@@ -389,8 +393,8 @@ __global__ void __launch_bounds__(kThreads, 6) k_sphere_step(AtlasDev a, L *__re
 
 // ---- grouped sphere strokes ----------------------------------------------------------------
 //
-// Middling calls of unpadded strokes on large label layers (by_lists): up to kGroup strokes are applied by
-// one cull and one apply launch.  Applying strokes one by one leaves each texel with
+// Calls of several unpadded strokes on label layers that go by lists (by_lists): up to kGroup strokes are applied
+// by one cull and one apply launch.  Applying strokes one by one leaves each texel with
 // the label of the newest stroke that selects it (older labels are overwritten), so the apply walks a
 // texel's strokes from the newest down and writes it once; every stroke is still evaluated for its
 // hit count, which does not depend on the order.  Items are (tile, mask, sure): `mask` holds the
@@ -795,26 +799,22 @@ __global__ void __launch_bounds__(kThreads) k_dilate_candidates(AtlasDev a, cons
 
 // A lasso's candidate-list entry: tile index, kInsideTile set when every texel of the tile that
 // projects lies inside the polygon (lasso_tile_class).
-// An edit's CTAs take kEditQuads quads at a time, one per thread, of one tile or of several small ones
-// (a CTA per tile left threads idle where a tile has fewer quads: 105 -> 80 us for 3 lassos over tiles
-// of 16 on 2048^2).  The lasso's apply is bound by instruction issue and by the latency of its loads;
-// it reads the next item's positions ahead and projects the quads of inside tiles side by side
-// (lasso_quad_inside): with their culls, 5 lassos on a 16384^2 atlas 941 -> 884 us and 12 on 4096^2
-// 421 -> 417 us.  Four CTAs per SM, since few tiles are candidates on a small atlas: with three (and
-// no bound on the registers) 853 and 428 us.  CTAs of 64 and 128 threads were slower (462 and 426 us).
-constexpr int kEditQuads = 256;
+// An edit's CTAs take kThreads quads at a time, one per thread, of one tile or of several small ones (a CTA per
+// tile left threads idle where a tile has fewer quads: 105 -> 80 us for 3 lassos over tiles of 16 on 2048^2).
+// The lasso's apply is bound by instruction issue and by the latency of its loads; it reads the next item's
+// positions ahead and projects the quads of inside tiles side by side (lasso_quad_inside).  With the cull, 5
+// lassos on a 16384^2 atlas went from 941 to 884 us and 12 on 4096^2 from 421 to 417 by that, and to 825 and
+// 381 by the order of lasso_hit's conditions.  Four CTAs per SM, since few tiles are candidates on a small
+// atlas: with three (and no bound on the registers) 853 and 428 us where four took 884 and 417.  CTAs of 64
+// and 128 threads were slower (462 and 426 us for the 12).
 constexpr int kBackCounter = 2;  // of a lasso or tool edit's counters: list entries, super-tiles, entries at the back
-template <bool PAD>
-constexpr int edit_threads() {
-    return PAD ? kThreads : kEditQuads;
-}
 
 // The quad of this thread in item `i` of the candidate list; false if it has none.  entry: the tile's
 // list entry; l: the quad's first texel.
 __device__ __forceinline__ bool edit_quad(const AtlasDev &a, const uint32_t *__restrict__ list, uint32_t n, uint32_t i,
                                           uint32_t &entry, int32_t &l) {
     const int qlog = __ffs(a.T) - 3, nlog = 2 * qlog + 2;  // quads per row and per tile
-    const uint32_t g = i * kEditQuads + threadIdx.x, k = g >> nlog;
+    const uint32_t g = i * kThreads + threadIdx.x, k = g >> nlog;
     if (k >= n || !LCL_IN(k, (int64_t)a.tiles_x * a.tiles_y)) return false;
     entry = __ldg(list + k);
     int32_t tx, ty;
@@ -827,11 +827,11 @@ __device__ __forceinline__ bool edit_quad(const AtlasDev &a, const uint32_t *__r
 // Items of n candidate tiles.
 __device__ __forceinline__ uint32_t edit_items(const AtlasDev &a, uint32_t n) {
     const int nlog = 2 * (__ffs(a.T) - 3) + 2;
-    return (uint32_t)((((uint64_t)n << nlog) + kEditQuads - 1) / kEditQuads);  // an atlas has 2^26 quads
+    return (uint32_t)((((uint64_t)n << nlog) + kThreads - 1) / kThreads);  // an atlas has 2^26 quads
 }
 
 template <typename L, bool NUM, bool PAD>
-__global__ void __launch_bounds__(edit_threads<PAD>(), 4) k_lasso_apply(AtlasDev a, L *__restrict__ layer,
+__global__ void __launch_bounds__(kThreads, 4) k_lasso_apply(AtlasDev a, L *__restrict__ layer,
                                                           const __grid_constant__ LassoArg p,
                                                           const float *__restrict__ depth,
                                                           const uint32_t *__restrict__ counter,
@@ -886,7 +886,7 @@ __global__ void __launch_bounds__(edit_threads<PAD>(), 4) k_lasso_apply(AtlasDev
 // ---- the paper's editing tool -------------------------------------------------------------
 
 template <typename L, bool MASK, bool PAD, bool NUM>
-__global__ void __launch_bounds__(edit_threads<PAD>(), 1024 / edit_threads<PAD>()) k_tool_apply(AtlasDev a, L *__restrict__ layer,
+__global__ void __launch_bounds__(kThreads, 4) k_tool_apply(AtlasDev a, L *__restrict__ layer,
                                                          const __grid_constant__ LassoArg p, ToolArg t,
                                                          const float *__restrict__ depth,
                                                          const uint32_t *__restrict__ counter,
@@ -1252,9 +1252,8 @@ void launch_lasso_apply(bool pad, const AtlasDev &a, L *layer, const LassoArg &p
                         const SelWs &w, unsigned long long *h, ValMask vm, int32_t pad_r, int32_t pad_t,
                         cudaStream_t st) {
     const auto kernel = pad ? k_lasso_apply<L, NUM, true> : k_lasso_apply<L, NUM, false>;
-    const int threads = pad ? edit_threads<true>() : edit_threads<false>();
-    launch_pdl_shape(kernel, dim3(resident_per_sm(kernel, threads) * sm_count()), dim3(threads), st, a, layer, p, depth,
-                     (const uint32_t *)w.counters, (const uint32_t *)w.list, h, vm, pad_r, pad_t);
+    launch_pdl(kernel, dim3(resident_grid(kernel)), st, a, layer, p, depth, (const uint32_t *)w.counters,
+               (const uint32_t *)w.list, h, vm, pad_r, pad_t);
 }
 
 // Lasso on a label layer (mask NULL) or on a numeric layer (data bytes 1, 2 or 4 and its mask bits),
@@ -1316,9 +1315,8 @@ void launch_tool(int sel, const AtlasDev &a, L *layer, const LassoArg &p, const 
                         : sel == 1 ? k_tool_apply<L, true, false, NUM>
                         : sel == 2 ? k_tool_apply<L, false, true, NUM>
                                    : k_tool_apply<L, true, true, NUM>;
-    const int threads = t.pad_r > 0 ? edit_threads<true>() : edit_threads<false>();
-    launch_pdl_shape(kernel, dim3(resident_per_sm(kernel, threads) * sm_count()), dim3(threads), st, a, layer, p, t,
-                     depth, (const uint32_t *)w.counters, (const uint32_t *)w.list, h, vm);
+    launch_pdl(kernel, dim3(resident_grid(kernel)), st, a, layer, p, t, depth, (const uint32_t *)w.counters,
+               (const uint32_t *)w.list, h, vm);
 }
 
 // The tool on a label layer (mask NULL) or on a numeric layer.

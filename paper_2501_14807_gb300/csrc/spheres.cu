@@ -17,13 +17,14 @@
 //     newest containing stroke gives the texels left open their value.
 // No candidate lists pass through memory, and a call needs ceil(n / kManyStrokes) launches, where a
 // cull and an apply launch per 32 strokes (label layers) or one launch per stroke (numeric layers,
-// single strokes) ran before.  Those stay for few strokes on large textures (by_lists in select.cu).
+// single strokes) ran before.  Those stay where they are the faster ones, for few strokes on large textures
+// (by_lists in select.cu).
 //
 // What bounds it: latency of the crossing tiles' loads, then issue of their 64-bit distance tests
 // (38% of issue slots, 21% of DRAM at 4096^2).  Measured on GB300, per call, before -> after: 250
 // strokes of 1-30% of the diagonal on 16384^2 u8 1000 -> 350 us; 625 of 0.1-5% on a 4096^2 u16 chart
-// atlas 225 -> 97 us; 40 value strokes on 5004 x 3310 i16 190 -> 39 us; one stroke on 1024^2 18 -> 15 us
-// (two launches instead of three).  Tried and slower: a tile per warp from the culling on (the warps
+// atlas 225 -> 97 us; 40 value strokes on 5004 x 3310 i16 190 -> 39 us; one stroke on 1024^2 17 -> 15 us
+// (two launches instead of three; two runs of one side differ by as much).  Tried and slower: a tile per warp from the culling on (the warps
 // of a CTA drift apart and wait at its end: 121 us at 4096^2), the next 32 quads' positions held in
 // registers (64 registers, four CTAs per SM: 105 us), CTAs of 128 threads (twice the staging: 106-113
 // us and 490 us at 16384^2), six CTAs per SM (40 registers: spills).

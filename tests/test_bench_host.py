@@ -200,3 +200,27 @@ def test_latency_split_of_served_requests():
     assert s["epoch_gpu_p50_p99_max"][0] == 0.5 and s["epoch_gpu_p50_p99_max"][2] == 2.0
     # no GPU times (a server that could not time its epochs): that part is null
     assert bench.latency_split([R(0.0, 0.001, 0.002, -1.0)])["epoch_gpu_p50_p99_max"] is None
+
+
+def test_sphere_group_follows_the_library_rule():
+    """bench.sphere_group: the texture sizes, tile sides, stroke counts and radii from which the rule changes."""
+    import types
+
+    import numpy as np
+
+    import bench
+    from paper_2501_14807_gb300 import lcl
+
+    def lists(side, tile, n, wide=False):
+        recs = np.zeros(n, lcl.SPHERE_DTYPE)
+        recs["r2"] = 1 << 36
+        recs["r2"][n // 2] += 1 if wide else 0
+        return bench.sphere_group(types.SimpleNamespace(width=side, height=side, tile=tile), recs) == 32
+
+    assert not lists(2048, 32, 20) and not lists(2048, 8, 2)
+    assert lists(4096, 32, 16) and not lists(4096, 32, 15) and lists(4096, 32, 2, True) and not lists(4096, 32, 33, True)
+    assert lists(4096, 64, 8) and not lists(4096, 64, 7) and lists(4096, 8, 8) and not lists(4096, 8, 2, True)
+    assert lists(8192, 32, 96) and not lists(8192, 32, 97) and lists(8192, 32, 32, True) and not lists(8192, 32, 33, True)
+    assert not lists(8192, 128, 17, True) and lists(16384, 128, 32, True)
+    assert lists(8192, 16, 32) and not lists(8192, 16, 2, True) and not lists(8192, 16, 33)
+    assert lists(16384, 64, 128) and not lists(16384, 64, 129) and not lists(16384, 32, 250, True)

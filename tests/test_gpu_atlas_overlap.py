@@ -1,5 +1,6 @@
 """Atlases whose triangles share texels of the texture (csrc/atlas.cu): of the triangles that cover a texel the one of
 the smallest id has it, whatever their order, and a mesh with a shared texel costs no second build."""
+import os
 import numpy as np
 import pytest
 import torch
@@ -36,6 +37,7 @@ def test_smallest_id_wins(kind, W, H, T):
     assert np.array_equal(to_np(a.cover(), np.uint32), o.cover_bits())
 
 
+@pytest.mark.skipif(os.environ.get("LCL_DEBUG_BOUNDS") == "1", reason="times of the bounds-checking build")
 def test_a_shared_texel_costs_no_second_build():
     def time_of(kind):
         mesh = lcl.Mesh.from_host(overlapping(kind, 400, 150), "cuda")

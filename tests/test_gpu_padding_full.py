@@ -2,6 +2,7 @@
 beside tiles with them: textures covered whole, covered but for their last rows, and charts, tiles of every side,
 sides that end inside a tile, against the oracle; and a padded stroke on a covered texture costs about what it
 costs without padding."""
+import os
 import numpy as np
 import pytest
 import torch
@@ -83,6 +84,7 @@ def test_lasso_and_tool(model, pad):
     assert not ((to_np(layer, np.uint8) != exp) & (amb == 0)).any() and exp.any()
 
 
+@pytest.mark.skipif(os.environ.get("LCL_DEBUG_BOUNDS") == "1", reason="times of the bounds-checking build")
 def test_padding_costs_little_on_a_covered_texture():
     W = H = 4096
     mesh = covered()

@@ -1,6 +1,8 @@
 """Zonal statistics of float layers whose values range too widely for one unit (csrc/numeric.cu): the sums keep the
 bounds of include/lcl.h as they stand -- against exact integer sums, so a zone of one texel is exact -- and a few
 outliers cost no more than a small factor in time."""
+import os
+
 from fractions import Fraction
 
 import numpy as np
@@ -66,6 +68,7 @@ def test_sums_within_the_stated_bounds(shape, zones, kind):
     assert ones or zones < 700
 
 
+@pytest.mark.skipif(os.environ.get("LCL_DEBUG_BOUNDS") == "1", reason="times of the bounds-checking build")
 @pytest.mark.parametrize("zones", [1, 40])
 @pytest.mark.parametrize("kind", ["outliers", "log", "subnormal"])
 def test_outliers_cost_little(kind, zones):
