@@ -344,7 +344,7 @@ typedef struct {
  *   threads      threads per CTA: 64, 128 or 256;
  *   ctas_per_sm  CTAs per SM, 0 = as many as fit, else 1..32 (capped at what fits);
  *   split        parts each (model, tile) work item is cut into (contiguous rows of the tile),
- *                1, 2, 4 or 8; a warp takes up to an eighth of a part from the work queue.
+ *                1, 2, 4 or 8; a warp takes a sixteenth of a part or more from the work queue.
  * Results do not depend on it. */
 typedef struct {
     int32_t threads, ctas_per_sm, split, _pad;

@@ -2,7 +2,6 @@
 bounds of include/lcl.h as they stand -- against exact integer sums, so a zone of one texel is exact -- and a few
 outliers cost no more than a small factor in time."""
 import os
-
 from fractions import Fraction
 
 import numpy as np
