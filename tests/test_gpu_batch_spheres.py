@@ -1,6 +1,8 @@
 """Batches without lassos (csrc/batch.cu), whose kernels leave out the lassos' code, against the same strokes one call
 at a time: all models of one tile side, so that an item has one ticket up to sixteen, with and without texture
 padding, for every split of the launch, and a texture with more units than the cull's warps draw one by one."""
+import os
+
 import numpy as np
 import pytest
 import torch
@@ -56,3 +58,27 @@ def test_splits(T, split, threads):
 @pytest.mark.parametrize("pads", [False, True])
 def test_more_units_than_warps_draw(pads):
     check([(4100, 4090)], 8, 5, pads, r_hi=0.2)
+
+
+@pytest.mark.skipif(os.environ.get("LCL_DEBUG_BOUNDS") == "1", reason="times of the bounds-checking build")
+def test_small_tiles_leave_no_tickets_empty():
+    mesh = synth.vessel_cylindrical(200, 100, noise_amp=0.03, seed=5)
+    o = oracle.Atlas(mesh, 64, 64, tile=32)  # the grid only
+    recs = sphere_recs(o, synth.sphere_strokes(mesh, 64, 17, 0.005, 0.1, 1, 255))
+
+    def time_of(T):
+        _, a = gpu_atlas(mesh, 4096, 4096, T)
+        batch = lcl.Batch([(a, torch.zeros((4096, 4096), dtype=torch.uint8, device="cuda"))], [[("sphere", r) for r in recs]])
+        lcl.lcl_batch_upload(batch)
+        best = float("inf")
+        for _ in range(6):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            for _ in range(10):
+                lcl.lcl_batch_launch(batch)
+            t1.record()
+            t1.synchronize()
+            best = min(best, t0.elapsed_time(t1))
+        return best
+
+    assert time_of(8) < 4.5 * time_of(32)  # 6.5 with eight tickets per item whatever its tile

@@ -1,6 +1,8 @@
 """Sphere calls on both sides of the rule that sends some through candidate lists (by_lists in csrc/select.cu), by texture
 size, tile side, number of strokes and radius, on label and value layers, against the definition on the
 atlas's planes: textures just above the sizes from which the rule changes, with tiles of every side."""
+import os
+
 import numpy as np
 import pytest
 import torch
@@ -50,3 +52,27 @@ def test_every_route_is_the_definition(mesh, side, T):
         assert torch.equal(value.data, exp) and h.tolist() == want, (n, wide, "value")
         known = np.unpackbits(value.mask.cpu().numpy().view(np.uint8), bitorder="little")[:side * side]
         assert np.array_equal(known.reshape(side, side).astype(bool), (exp > 0).cpu().numpy())
+
+
+@pytest.mark.skipif(os.environ.get("LCL_DEBUG_BOUNDS") == "1", reason="times of the bounds-checking build")
+def test_one_wide_stroke_costs_the_same_with_larger_tiles(mesh):
+    o = oracle.Atlas(mesh, 64, 64, tile=32)  # the grid only
+    recs = sphere_recs(o, synth.sphere_strokes(mesh, 1, 17, 0.2, 0.2, 1, 255))
+
+    def time_of(T):
+        side = 16384
+        _, a = gpu_atlas(mesh, side, side, T)
+        layer = torch.zeros((side, side), dtype=torch.uint8, device="cuda")
+        ws = torch.empty(lcl.lcl_select_workspace_bytes(a, 1), dtype=torch.uint8, device="cuda")
+        best = float("inf")
+        for _ in range(6):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            for _ in range(20):
+                lcl.lcl_select_sphere(a, layer, recs, workspace=ws)
+            t1.record()
+            t1.synchronize()
+            best = min(best, t0.elapsed_time(t1))
+        return best
+
+    assert time_of(64) < 1.8 * time_of(32)  # three times by blocks, as a rule that counted tiles had it
